@@ -1633,6 +1633,7 @@ CollideParams<typename Store<S>::A> level_params(const lbmp_handle* h, const Lev
         p.scale = (A)1;
         p.inv_scale = (A)1;
     }
+    collide_consts(p);
     return p;
 }
 

@@ -29,7 +29,7 @@ struct SimDev {
     int mask_off;        // boundary mask: one byte per box cell
     int bnd_off, bnd_n;  // boundary-kernel blocks of the simulation (and their force partials)
     BoxDesc box;
-    double sp, sm, db;
+    CollideParams<double> P;   // FP64: the collision's parameters; else its rates are rounded from here
     long long hist_off;  // records
 };
 
@@ -43,9 +43,10 @@ template <typename S>
 __host__ __device__ __forceinline__ CollideParams<typename Store<S>::A> sim_params(const SimDev& D, typename Store<S>::A scale,
                                                typename Store<S>::A inv) {
     CollideParams<typename Store<S>::A> p;
-    p.sp = (typename Store<S>::A)D.sp;
-    p.sm = (typename Store<S>::A)D.sm;
-    p.db = (typename Store<S>::A)D.db;
+    if constexpr (sizeof(S) == 8) return D.P;
+    p.sp = (typename Store<S>::A)D.P.sp;
+    p.sm = (typename Store<S>::A)D.P.sm;
+    p.db = (typename Store<S>::A)D.P.db;
     p.F[0] = p.F[1] = p.F[2] = 0;
     p.forced = 0;
     p.scale = scale;
@@ -298,7 +299,7 @@ __global__ void __launch_bounds__(BW)
         const int i = __shfl_sync(0xffffffffu, p[0], src), j = __shfl_sync(0xffffffffu, p[1], src),
                   k = __shfl_sync(0xffffffffu, p[2], src);
         const size_t cc = (size_t)i + (size_t)G.nx * ((size_t)j + (size_t)G.ny * (size_t)k);
-        batch_refill_warp<S>(p0, fc, G, n3, F, P, i, j, k, cc, scale, inv, grad, D.sp);
+        batch_refill_warp<S>(p0, fc, G, n3, F, P, i, j, k, cc, scale, inv, grad, D.P.sp);
     }
 }
 
@@ -478,10 +479,12 @@ lbmp_status batch_create(lbmp_handle* h, const lbmp_batch_sim* sims, int n) {
         D.flag_off = cells;
         B->cell_off[s] = cells;
         cells += D.G.n;
-        const double sp = 1.0 / in.tau, sm = 1.0 / (0.5 + h->cfg.magic / (in.tau - 0.5));
-        D.sp = sp;
-        D.sm = sm;
-        D.db = bulk_rate_offset(in.tau, h->cfg.bulk_factor);
+        relaxation_rates(in.tau, h->cfg.magic, &D.P.sp, &D.P.sm);
+        D.P.db = bulk_rate_offset(in.tau, h->cfg.bulk_factor);
+        D.P.F[0] = D.P.F[1] = D.P.F[2] = 0.0;
+        D.P.forced = 0;
+        D.P.scale = D.P.inv_scale = 1.0;
+        collide_consts(D.P);
         ParticleState& P = B->h_ps[s];
         std::memset(&P, 0, sizeof(P));
         for (int a = 0; a < 3; ++a) {

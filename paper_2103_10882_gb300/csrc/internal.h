@@ -46,6 +46,17 @@ __device__ __forceinline__ A wall_term(const GridDesc& G, int q, const int xyz[3
     return t;
 }
 
+// Coefficients of collide_direct, formed once on the host in FP64 (collide_consts): the relaxation and
+// equilibrium factors of a pair's sum and difference, and per pair of directions the constant part of the
+// Guo source.  The quadratic ones include the FP16 storage factor.
+template <typename A>
+struct CollideConsts {
+    A hp, hm, r0;         // (1 - s+)/2, (1 - s-)/2, 1 - s+
+    A kF, kE, mF, mE;     // s+ 9/2 w, s- 3 w on faces and edges
+    A c15, cF;            // 3/2, 3 (1 - s+/2)
+    A gs[9], ga[9];       // 9 (1 - s+/2) w c_q.F, 3 (1 - s-/2) w c_q.F for q = 1, 3, ..., 17
+};
+
 // Collision parameters in the arithmetic precision A of the storage type.
 template <typename A>
 struct CollideParams {
@@ -54,7 +65,32 @@ struct CollideParams {
     A F[3];            // fluid body force
     int forced;
     A scale, inv_scale;   // FP16 storage scaling (1 otherwise)
+    CollideConsts<A> k;
 };
+
+// Fills p.k from the rates and the force of p (already rounded to A: the coefficients belong to them).
+template <typename A>
+inline void collide_consts(CollideParams<A>& p) {
+    const double sp = p.sp, sm = p.sm, q2 = p.inv_scale;
+    const double wF = 1.0 / 18.0, wE = 1.0 / 36.0;
+    CollideConsts<A>& k = p.k;
+    k.hp = (A)(0.5 * (1.0 - sp));
+    k.hm = (A)(0.5 * (1.0 - sm));
+    k.r0 = (A)(1.0 - sp);
+    k.kF = (A)(4.5 * sp * wF * q2);
+    k.kE = (A)(4.5 * sp * wE * q2);
+    k.mF = (A)(3.0 * sm * wF);
+    k.mE = (A)(3.0 * sm * wE);
+    k.c15 = (A)(1.5 * q2);
+    k.cF = (A)(3.0 * (1.0 - 0.5 * sp));
+    for (int i = 0; i < 9; ++i) {
+        const int q = 2 * i + 1;
+        const double w = q < 7 ? wF : wE;
+        const double c = (double)p.F[0] * kCX[q] + (double)p.F[1] * kCY[q] + (double)p.F[2] * kCZ[q];
+        k.gs[i] = (A)(9.0 * (1.0 - 0.5 * sp) * w * c);
+        k.ga[i] = (A)(3.0 * (1.0 - 0.5 * sm) * w * c);
+    }
+}
 
 // Axis-aligned box of cells around the sphere, fixed extent, origin read
 // from the particle state on the device.
@@ -210,6 +246,7 @@ inline CollideParams<A> collide_params(const lbmp_handle* h) {
         p.scale = (A)1;
         p.inv_scale = (A)1;
     }
+    collide_consts(p);
     return p;
 }
 

@@ -29,6 +29,107 @@ __device__ __forceinline__ double link_delta(const double d[3], int q, double r)
     return s < 0.0 ? 0.0 : (s > 1.0 ? 1.0 : s);
 }
 
+// c_q . u for a direction known at compile time, without the products by zero (which the compiler may
+// not drop in IEEE arithmetic: 0 * inf); the value is the same.
+template <typename A>
+__device__ __forceinline__ A dir_dot(int q, A x, A y, A z) {
+    const int a = cx(q), b = cy(q), c = cz(q);
+    A t = A(0);
+    bool any = false;
+    if (a) {
+        t = a > 0 ? x : -x;
+        any = true;
+    }
+    if (b) {
+        t = any ? (b > 0 ? t + y : t - y) : (b > 0 ? y : -y);
+        any = true;
+    }
+    if (c) t = any ? (c > 0 ? t + z : t - z) : (c > 0 ? z : -z);
+    return t;
+}
+
+// The collision of trt_collide with the fewest instructions, for the kernels whose time is instructions: FP64
+// (GB300 issues one FP64 warp instruction per scheduler in about 76 cycles: k_bulk in FP64 ran at 242 of them per
+// cell, 0.51e12 a second) and FP16 storage (two cells per thread, issue-bound).  With the sums ps and differences pd
+// of the opposite pairs, both new populations of a pair are S + D and S - D,
+//   S = (1 - s+)/2 ps + s+ e+ + (1 - s+/2) S+,   D = (1 - s-)/2 pd + s- e- + (1 - s-/2) S-,
+// the coefficients and the direction's part of the Guo source come from the host (collide_consts), the density part of
+// e+ and the MRT correction are one number per class of directions: 112 instructions per cell unforced (13 more forced).
+// Measured: a coupled FP64 step of 61 x 53 x 75 cells 175 -> 129 us, a refined FP64 step (1.1 M updates) 394 -> 261 us,
+// an FP16-storage step of 256^3 301 -> 293 us.
+// The MRT sums over a class follow from ps alone: sum_faces 2 e+ = rho/3, sum_edges 2 e+ = rho/3 + uu/2, and the half
+// source sums to -uF/2, 0 and uF/2 over rest, faces and edges.
+// FP32 storage keeps the plain form below: its coefficient (1 - s-)/2 would be rounded to FP32 for s- < 1/2, a relative
+// momentum change of up to 3e-8 in every step, and its kernels wait on memory, not on instructions.  In FP64 the same
+// rounding is 6e-17 a step; FP16 storage itself rounds at 5e-4.
+// Populations may be scaled by 2^s (SCALED): quadratic terms then carry 2^-s, which the host's coefficients include.
+template <typename A, bool FORCED, bool SCALED, int MRT_MODE>
+__device__ __forceinline__ void collide_direct(A (&g)[19], const CollideParams<A>& P, int* status) {
+    const CollideConsts<A>& K = P.k;
+    A ps[9], pd[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        ps[k] = g[2 * k + 1] + g[2 * k + 2];
+        pd[k] = g[2 * k + 1] - g[2 * k + 2];
+    }
+    const A pF = ps[0] + ps[1] + ps[2];
+    const A pE = ((ps[3] + ps[4]) + (ps[5] + ps[6])) + (ps[7] + ps[8]);
+    const A drho = g[0] + pF + pE;
+    // pairs 3..8 are (+x+y), (+x-y), (+x+z), (+x-z), (+y+z), (+y-z)
+    A ux = pd[0] + ((pd[3] + pd[4]) + (pd[5] + pd[6]));
+    A uy = pd[1] + ((pd[3] - pd[4]) + (pd[7] + pd[8]));
+    A uz = pd[2] + ((pd[5] - pd[6]) + (pd[7] - pd[8]));
+    if (FORCED) {
+        ux += A(0.5) * P.F[0];
+        uy += A(0.5) * P.F[1];
+        uz += A(0.5) * P.F[2];
+    }
+    const A u2[3] = {ux * ux, uy * uy, uz * uz};
+    const A uu = u2[0] + u2[1] + u2[2];   // SCALED: times 2^2s
+    if (!(uu * (SCALED ? P.inv_scale * P.inv_scale : A(1)) <= A(0.09))) atomicOr(status, STATUS_UNSTABLE_FLUID);
+    A R = P.sp * (drho - K.c15 * uu);
+    A uF = A(0);
+    if (FORCED) {
+        uF = ux * P.F[0] + uy * P.F[1] + uz * P.F[2];
+        R -= K.cF * uF;
+    }
+    A bF = wgt<A>(1) * R, bE = wgt<A>(7) * R, b0 = wgt<A>(0) * R;
+    const bool mrt = MRT_MODE < 0 ? P.db != A(0) : MRT_MODE == 1;
+    if (mrt) {   // as in trt_collide
+        const A t = drho * (A(1) / A(3)), u3 = K.c15 * (A(1) / A(3)) * uu;   // u3 = uu / 2 (scaled as a population)
+        A nR = g[0] - t + u3;
+        const A nF = pF - t;
+        A nE = pE - t - u3;
+        if (FORCED) {
+            nR -= A(0.5) * uF;
+            nE += A(0.5) * uF;
+        }
+        const A c4 = A(1.5) * (nE - nR);
+        const A c16 = A(0.5) * (nR - A(2) * nF + nE);
+        b0 -= P.db * wgt<A>(0) * (c16 - c4);
+        bF -= P.db * wgt<A>(1) * (A(-2) * c16);
+        bE -= P.db * wgt<A>(7) * (c4 + c16);
+    }
+    g[0] = K.r0 * g[0] + b0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int q = 2 * k + 1;
+        const bool face = k < 3;
+        const A cu = dir_dot<A>(q, ux, uy, uz);
+        A e, d;
+        if (FORCED) {
+            e = ((face ? K.kF : K.kE) * cu + K.gs[k]) * cu + (face ? bF : bE);
+            d = (face ? K.mF : K.mE) * cu + K.ga[k];
+        } else {
+            e = face ? K.kF * u2[k < 3 ? k : 0] + bF : (K.kE * cu) * cu + bE;
+            d = (face ? K.mF : K.mE) * cu;
+        }
+        const A Sy = K.hp * ps[k] + e, Da = K.hm * pd[k] + d;
+        g[q] = Sy + Da;
+        g[q + 1] = Sy - Da;
+    }
+}
+
 // TRT collision on deviations (Sec. 2.1, Lambda_b = 1): the symmetric part of
 // each pair relaxes with s+, the antisymmetric part with s-; incompressible
 // equilibrium with rho_0 = 1; optional Guo-type source split the same way.
@@ -37,45 +138,25 @@ __device__ __forceinline__ double link_delta(const double d[3], int q, double r)
 // quadratic terms, which then take one factor 2^-s (P.inv_scale).
 // MRT_MODE: -1 decides TRT or MRT from P.db at run time, 0 is TRT only, 1
 // MRT only (kernels that know which one runs carry no code of the other).
-template <typename A, bool FORCED, bool SCALED = false, int MRT_MODE = -1, bool PAIRS = false>
+// DIRECT: collide_direct (FP64, and where a kernel asks for it).
+template <typename A, bool FORCED, bool SCALED = false, int MRT_MODE = -1, bool DIRECT = sizeof(A) == 8>
 __device__ __forceinline__ void trt_collide(A (&g)[19], const CollideParams<A>& P, int* status) {
     static_assert(!(FORCED && SCALED), "the scaled form is for the unforced collision");
+    if constexpr (DIRECT) {
+        collide_direct<A, FORCED, SCALED, MRT_MODE>(g, P, status);
+        return;
+    }
     const A q2 = SCALED ? P.inv_scale : A(1);
-    // PAIRS: the moments from the sums and differences of the opposite pairs (q, q + 1), q odd,
-    // which the relaxation below uses again (c_{q+1} = -c_q: a pair adds its sum to the density and
-    // its difference times c_q to the momentum).  Fewer instructions, for the issue-bound FP16 bulk
-    // update; 18 more live values, which the register-capped level update pays for in spills.
-    A ps[9], pd[9];
-    A drho = g[0], jx = A(0), jy = A(0), jz = A(0);
-    if (PAIRS) {
+    A drho = A(0), jx = A(0), jy = A(0), jz = A(0);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            ps[k] = g[2 * k + 1] + g[2 * k + 2];
-            pd[k] = g[2 * k + 1] - g[2 * k + 2];
-        }
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const int q = 2 * k + 1;
-            drho += ps[k];
-            if (cx(q) == 1) jx += pd[k];
-            if (cx(q) == -1) jx -= pd[k];
-            if (cy(q) == 1) jy += pd[k];
-            if (cy(q) == -1) jy -= pd[k];
-            if (cz(q) == 1) jz += pd[k];
-            if (cz(q) == -1) jz -= pd[k];
-        }
-    } else {
-        drho = A(0);
-#pragma unroll
-        for (int q = 0; q < 19; ++q) {
-            drho += g[q];
-            if (cx(q) == 1) jx += g[q];
-            if (cx(q) == -1) jx -= g[q];
-            if (cy(q) == 1) jy += g[q];
-            if (cy(q) == -1) jy -= g[q];
-            if (cz(q) == 1) jz += g[q];
-            if (cz(q) == -1) jz -= g[q];
-        }
+    for (int q = 0; q < 19; ++q) {
+        drho += g[q];
+        if (cx(q) == 1) jx += g[q];
+        if (cx(q) == -1) jx -= g[q];
+        if (cy(q) == 1) jy += g[q];
+        if (cy(q) == -1) jy -= g[q];
+        if (cz(q) == 1) jz += g[q];
+        if (cz(q) == -1) jz -= g[q];
     }
     A ux = jx, uy = jy, uz = jz;
     if (FORCED) {
@@ -103,12 +184,12 @@ __device__ __forceinline__ void trt_collide(A (&g)[19], const CollideParams<A>& 
     }
 #pragma unroll
     for (int q = 1; q < 19; q += 2) {
-        const A cu = A(cx(q)) * ux + A(cy(q)) * uy + A(cz(q)) * uz;
+        const A cu = dir_dot<A>(q, ux, uy, uz);
         const A w = wgt<A>(q);
         const A ep = w * (drho + A(4.5) * q2 * cu * cu - A(1.5) * uu);
         const A em = w * (A(3) * cu);
-        const A gp = A(0.5) * (PAIRS ? ps[q >> 1] : g[q] + g[q + 1]);
-        const A gm = A(0.5) * (PAIRS ? pd[q >> 1] : g[q] - g[q + 1]);
+        const A gp = A(0.5) * (g[q] + g[q + 1]);
+        const A gm = A(0.5) * (g[q] - g[q + 1]);
         const A dp = sp * (gp - ep);
         const A dm = sm * (gm - em);
         if (mrt) {
@@ -118,7 +199,7 @@ __device__ __forceinline__ void trt_collide(A (&g)[19], const CollideParams<A>& 
         A a = g[q] - dp - dm;
         A b = g[q + 1] - dp + dm;
         if (FORCED) {
-            const A cF = A(cx(q)) * P.F[0] + A(cy(q)) * P.F[1] + A(cz(q)) * P.F[2];
+            const A cF = dir_dot<A>(q, P.F[0], P.F[1], P.F[2]);
             const A uF = ux * P.F[0] + uy * P.F[1] + uz * P.F[2];
             const A Sp = (A(1) - A(0.5) * sp) * w * (A(9) * cu * cF - A(3) * uF);
             const A Sm = (A(1) - A(0.5) * sm) * w * (A(3) * cF);

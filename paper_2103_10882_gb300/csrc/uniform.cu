@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(BULK_THREADS)
 // outer half from the neighbouring lane (a shuffle); the first lane of a
 // warp (rows start there) and the last pair of a warp or of a row load that
 // one half themselves.  The collision runs on the stored, scaled values
-// (trt_collide's SCALED form), so neither the loads nor the stores multiply
+// (trt_collide's SCALED form, collide_direct), so neither the loads nor the stores multiply
 // by the scale, and TRT or MRT is chosen at compile time.  nx is even; rows
 // hold whole pairs.
 constexpr int BULK2_THREADS = 256;
