@@ -424,15 +424,6 @@ __global__ void __launch_bounds__(AT)
     for (int a = 0; a < 3; ++a) grad_u0[(size_t)a * n + x] = s * (3.0 * L1[a] + 9.0 * L2u[a] - 3.0 * L0 * u[a]);
 }
 
-// Force of the step from the boundary kernel's partials (fixed block order).
-__global__ void k_adj_force(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
-    if (threadIdx.x < 3) {
-        double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += partials[(size_t)b * 6 + threadIdx.x];
-        out[threadIdx.x] = s;
-    }
-}
-
 __global__ void k_adj_mean(const double* __restrict__ forces, int nsteps, int axis, double* __restrict__ J) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         double s = 0.0;
@@ -506,16 +497,10 @@ struct AdjointEngine {
 
 namespace {
 
+// One forward step with the sphere held at rest; the force of the step into force_out (null: not wanted).
 template <typename S>
 void forward_step(lbmp_handle* h, const S* src, S* dst, double* force_out) {
-    using A = typename Store<S>::A;
-    const CollideParams<A> p = collide_params<A>(h);
-    launch_bulk<S>(src, dst, h->G, p, h->status, h->stream);
-    int nb = 0;
-    launch_boundary<S>(src, dst, h->flags[h->fcur], h->list, h->count, h->list_cap, h->G, p, h->d_ps,
-                       h->cfg.boundary == LBMP_CLI ? 1 : 0, h->partials, &nb, h->status, h->stream);
-    launch_refill<S>(dst, h->flags[h->fcur], h->flags[h->fcur], h->G, h->box, h->d_ps, A(1), A(1), A(0), h->stream);
-    if (force_out) k_adj_force<<<1, 32, 0, h->stream>>>(h->partials, nb, force_out);
+    launch_step<S>(h, src, dst, collide_params<typename Store<S>::A>(h), force_out ? 1 : 2, force_out, h->stream);
 }
 
 template <typename S>
@@ -651,6 +636,11 @@ lbmp_status adjoint_forward(lbmp_handle* h, const double* u0, int nsteps, int in
         E->graph_axis = axis;
         for (int a = 0; a < 3; ++a) E->graph_F[a] = h->body_force[a];
     }
+    if (h->frames_stale) {   // the host changed the record: the step's frames first
+        launch_frames(h, h->stream);
+        h->frames_stale = false;
+        h->launches += 1;
+    }
     if (!E->geometry_done) {   // cells of the reverse step next to the (fixed) sphere
         const unsigned gb = (unsigned)E->plain_blocks;
         k_adj_kind<<<gb, AT, 0, h->stream>>>(h->flags[h->fcur], h->G, E->kind, E->blk);
@@ -687,7 +677,7 @@ lbmp_status adjoint_forward(lbmp_handle* h, const double* u0, int nsteps, int in
     if (st != LBMP_OK) return st;
     h->cur = (par + nsteps) & 1;
     h->steps += nsteps;
-    h->launches += 1 + 4LL * nsteps;
+    h->launches += 1 + (long long)nsteps;
     h->updates += (long long)nsteps * h->G.n;
     k_adj_mean<<<1, 32, 0, h->stream>>>(E->forces, nsteps, axis, J);
     h->launches += 1;
@@ -744,7 +734,7 @@ lbmp_status adjoint_backward(lbmp_handle* h, const double* dJ, double* grad_tau,
                 }
             }
         });
-        h->launches += 3LL * (N - E->nckpt) + 2LL * N;
+        h->launches += (long long)(N - E->nckpt) + 2LL * N;
         if (st == LBMP_OK && grad_u0) {   // nu^1 sits in nu[N % 2] after N reverse steps
             k_adj_init_grad<A><<<gb, AT, 0, h->stream>>>((const A*)E->nu[N & 1], h->flags[h->fcur], E->kind, h->G,
                                                          E->u0, h->d_ps, cli, P.seed, E->axis, dJ, grad_u0);

@@ -360,57 +360,11 @@ constexpr int BND_CHUNK = 128;     // box cells per boundary CTA (sizes the grid
 // instead of 1,024.
 template <typename S>
 constexpr int BND_MAXREG = sizeof(S) == 8 ? 128 : (sizeof(S) == 4 ? 56 : 64);
-constexpr int LINK_THREADS = 64;   // box cells per run of the boundary mask (one count per run)
 constexpr int REMAP_THREADS = 256;   // remap blocks: their uncovered cells are spread over the eight warps
-
-// Exclusive prefix of n counts into pre[0..n] (pre[n] = total), computed by
-// the whole CTA (NT threads, two consecutive counts per thread and pass);
-// every thread must call it.  first0, first1: counts 2 threadIdx.x and
-// 2 threadIdx.x + 1 (0 beyond n), loaded by the caller ahead.
-template <int NT>
-__device__ __forceinline__ int block_prefix(const int* __restrict__ count, int n, int* pre, int first0, int first1) {
-    __shared__ int wsum[NT / 32];
-    __shared__ int carry;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int base = 0; base < n; base += 2 * NT) {
-        const int i = base + 2 * (int)threadIdx.x;
-        const int c0 = base == 0 ? first0 : (i < n ? count[i] : 0);
-        const int c1 = base == 0 ? first1 : (i + 1 < n ? count[i + 1] : 0);
-        int v = c0 + c1;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, v, off);
-            if (lane >= off) v += y;
-        }
-        if (lane == 31) wsum[wid] = v;
-        __syncthreads();
-        if (wid == 0) {
-            int w = lane < NT / 32 ? wsum[lane] : 0;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, w, off);
-                if (lane >= off) w += y;
-            }
-            if (lane < NT / 32) wsum[lane] = w;
-        }
-        __syncthreads();
-        const int incl = carry + (wid > 0 ? wsum[wid - 1] : 0) + v;   // through count i + 1
-        if (i < n) pre[i + 1] = incl - c1;
-        if (i + 1 < n) pre[i + 2] = incl;
-        __syncthreads();
-        if (threadIdx.x == 0) carry += wsum[NT / 32 - 1];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) pre[0] = 0;
-    __syncthreads();
-    return pre[n];
-}
 
 // Boundary cells of the finest level (flag 2: fluid with a solid
 // neighbour), from the mask the remap wrote in box order and its count of
-// marked cells per run of LINK_THREADS box cells.  The marked cells are
+// marked cells per run of LINK_RUN box cells.  The marked cells are
 // spread evenly over all warps of the grid: every CTA turns the counts into
 // a prefix, and warp w of W takes the marked cells w, w + W, ... (box
 // order), one cell per warp at a time, lane q handling population q (CLI
@@ -430,7 +384,7 @@ __global__ void __maxnreg__(BND_MAXREG<S>)
     extern __shared__ int pre[];   // [runs + 1]
     __shared__ LinkFrame<A> Fr;
     __shared__ BoxFrame Bf;
-    const int runs = (int)((B.cells + LINK_THREADS - 1) / LINK_THREADS);
+    const int runs = (int)((B.cells + LINK_RUN - 1) / LINK_RUN);
     const int i2 = 2 * (int)threadIdx.x;   // this thread's first two counts, in flight during the set-up
     const int first0 = i2 < runs ? run_count[i2] : 0, first1 = i2 + 1 < runs ? run_count[i2 + 1] : 0;
     if (threadIdx.x == 0) Fr = pframe_link<A>(*frames);   // formed by the last particle update
@@ -441,27 +395,7 @@ __global__ void __maxnreg__(BND_MAXREG<S>)
     const int W = (int)gridDim.x * (BNDW_THREADS / 32);
     LinkSums<A> acc;
     for (int j = (int)blockIdx.x * (BNDW_THREADS / 32) + wib; j < total; j += W) {
-        // run r holding marked cell j: the largest r with pre[r] <= j
-        int lo = 0, hi = runs;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (pre[mid] <= j) lo = mid;
-            else hi = mid;
-        }
-        const long long r0 = (long long)lo * LINK_THREADS;
-        const bool m0 = r0 + lane < B.cells && mask[r0 + lane] != 0;
-        const bool m1 = r0 + 32 + lane < B.cells && mask[r0 + 32 + lane] != 0;
-        const unsigned b0 = __ballot_sync(0xffffffffu, m0), b1 = __ballot_sync(0xffffffffu, m1);
-        int k = j - pre[lo];
-        unsigned bits = b0;
-        int base = 0;
-        if (k >= __popc(b0)) {
-            k -= __popc(b0);
-            bits = b1;
-            base = 32;
-        }
-        for (; k > 0; --k) bits &= bits - 1u;   // drop the k lowest marked cells
-        const int t = (int)(r0 + base + __ffs((int)bits) - 1);
+        const int t = marked_cell(pre, runs, mask, B.cells, j);
         int g[3], c;
         if (!box_cell(t, D.n, D.periodic, B, Bf, g)) continue;   // marked cells are inside the domain
         const int b = locate(D, g, &c);
@@ -609,7 +543,7 @@ __global__ void k_pframes(const ParticleState* __restrict__ ps, PFrames* __restr
 // the block in turn (refill_cell_warp: it reads only cells that are fluid
 // before and after the move, which nothing here writes); fluid cells with a
 // solid neighbour are marked for the boundary list (counts per run of
-// LINK_THREADS box cells for the ordered compaction).  Neighbour flags are
+// LINK_RUN box cells for the ordered compaction).  Neighbour flags are
 // evaluated from the same predicate instead of being read back, so no
 // second pass is needed.
 template <typename S>
@@ -675,10 +609,10 @@ __global__ void __launch_bounds__(REMAP_THREADS)
     __shared__ int wsum[REMAP_THREADS / 32];
     if ((threadIdx.x & 31) == 0) wsum[wid] = __popc(ballot);
     __syncthreads();
-    constexpr int RUNS = REMAP_THREADS / LINK_THREADS, WPR = LINK_THREADS / 32;
+    constexpr int RUNS = REMAP_THREADS / LINK_RUN, WPR = LINK_RUN / 32;
     if ((int)threadIdx.x < RUNS) {
         const long long run = (long long)blockIdx.x * RUNS + threadIdx.x;
-        if (run * LINK_THREADS < B.cells) {
+        if (run * LINK_RUN < B.cells) {
             int s = 0;
             for (int w = 0; w < WPR; ++w) s += wsum[threadIdx.x * WPR + w];
             block_count[run] = s;
@@ -686,24 +620,24 @@ __global__ void __launch_bounds__(REMAP_THREADS)
     }
 }
 
-__global__ void __launch_bounds__(LINK_THREADS)
+__global__ void __launch_bounds__(LINK_RUN)
     k_amr_links_emit(LevelView D, const uint8_t* __restrict__ mask, const int* __restrict__ block_count, BoxDesc B,
                      const ParticleState* __restrict__ ps, int* __restrict__ list, int* __restrict__ count,
                      int capacity, int* __restrict__ status) {
-    __shared__ int red[LINK_THREADS];
-    __shared__ int wsum[LINK_THREADS / 32];
+    __shared__ int red[LINK_RUN];
+    __shared__ int wsum[LINK_RUN / 32];
     __shared__ BoxFrame F;
     if (threadIdx.x == 0) box_frame_init(F, D.n, D.periodic, B, *ps);
     int s = 0;
-    for (int b = threadIdx.x; b < (int)blockIdx.x; b += LINK_THREADS) s += block_count[b];
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += LINK_RUN) s += block_count[b];
     red[threadIdx.x] = s;
     __syncthreads();
-    for (int h = LINK_THREADS / 2; h > 0; h >>= 1) {
+    for (int h = LINK_RUN / 2; h > 0; h >>= 1) {
         if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
         __syncthreads();
     }
     const int base = red[0];
-    const int t = blockIdx.x * LINK_THREADS + threadIdx.x;
+    const int t = blockIdx.x * LINK_RUN + threadIdx.x;
     const int is_b = t < B.cells ? mask[t] : 0;
     const unsigned ballot = __ballot_sync(0xffffffffu, is_b);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -721,7 +655,7 @@ __global__ void __launch_bounds__(LINK_THREADS)
     }
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
         int tot = base;
-        for (int w = 0; w < LINK_THREADS / 32; ++w) tot += wsum[w];
+        for (int w = 0; w < LINK_RUN / 32; ++w) tot += wsum[w];
         *count = tot < capacity ? tot : capacity;
     }
 }
@@ -1731,7 +1665,7 @@ void enqueue_advance(lbmp_handle* h, int l, int sub) {
         }
         cudaEventRecord(E->ev_fork, st);
         cudaStreamWaitEvent(E->side, E->ev_fork, 0);
-        const size_t pre_bytes = sizeof(int) * (size_t)((h->box.cells + LINK_THREADS - 1) / LINK_THREADS + 1);
+        const size_t pre_bytes = sizeof(int) * (size_t)((h->box.cells + LINK_RUN - 1) / LINK_RUN + 1);
         k_amr_boundary<S><<<E->boundary_blocks, BNDW_THREADS, pre_bytes, E->side>>>(
             D, U.src, U.dst, U.solid, h->link_mask, h->link_blocks, h->box, P, h->d_ps, h->cfg.boundary == LBMP_CLI ? 1 : 0,
             h->partials, E->d_done, G, h->history, h->cfg.history_capacity, h->status, E->d_frames);
@@ -1874,10 +1808,10 @@ lbmp_status amr_add_sphere(lbmp_handle* h) {
     if (!E->d_frames) E->d_frames = (PFrames*)handle_alloc(h, sizeof(PFrames));
     if (!E->d_frames) return LBMP_ERR_OOM;
     h->link_mask = (uint8_t*)handle_alloc(h, (size_t)B.cells);
-    h->link_blocks = (int*)handle_alloc(h, sizeof(int) * (size_t)((B.cells + LINK_THREADS - 1) / LINK_THREADS));
+    h->link_blocks = (int*)handle_alloc(h, sizeof(int) * (size_t)((B.cells + LINK_RUN - 1) / LINK_RUN));
     if (!h->list || !h->partials || !h->link_mask || !h->link_blocks) return LBMP_ERR_OOM;
     // the boundary kernel keeps a prefix of the remap's run counts in dynamic shared memory
-    const int pre_bytes = (int)(sizeof(int) * ((B.cells + LINK_THREADS - 1) / LINK_THREADS + 1));
+    const int pre_bytes = (int)(sizeof(int) * ((B.cells + LINK_RUN - 1) / LINK_RUN + 1));
     bool attr_ok = true;
     with_storage_amr(h->cfg.precision, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
@@ -2277,8 +2211,8 @@ lbmp_status amr_links(lbmp_handle* h, int64_t* cell, int32_t* q, double* delta, 
     // the step keeps the boundary cells as a mask in box order; compact it for the export
     {
         const Level& Vf = E->lv[E->L - 1];
-        const unsigned nl = (unsigned)((h->box.cells + LINK_THREADS - 1) / LINK_THREADS);
-        k_amr_links_emit<<<nl, LINK_THREADS, 0, h->stream>>>(view(E, Vf), h->link_mask, h->link_blocks, h->box,
+        const unsigned nl = (unsigned)((h->box.cells + LINK_RUN - 1) / LINK_RUN);
+        k_amr_links_emit<<<nl, LINK_RUN, 0, h->stream>>>(view(E, Vf), h->link_mask, h->link_blocks, h->box,
                                                              h->d_ps, h->list, h->count, h->list_cap, h->status);
     }
     int cnt = 0;

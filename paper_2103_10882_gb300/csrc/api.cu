@@ -89,34 +89,42 @@ void enqueue_step(lbmp_handle* h) {
         const S* src = (const S*)h->pops[h->cur];
         S* dst = (S*)h->pops[1 - h->cur];
         const CollideParams<A> p = collide_params<A>(h);
-        // 1. stream + collide every cell (LBM step)
+        if (h->has_particle && h->frames_stale) {   // the host changed the record: its frames first
+            launch_frames(h, h->stream);
+            h->frames_stale = false;
+            h->launches += 1;
+        }
+        // stream + collide every cell; beside it the cells next to the sphere (CLI links, momentum-exchange force)
+        // and the particle update (force average, gravity, virtual mass, Velocity Verlet)
         const long long ev_bulk = profile_mark(h);
-        launch_bulk<S>(src, dst, h->G, p, h->status, h->stream);
+        launch_step<S>(h, src, dst, p, 0, nullptr, h->stream);
         profile_kernel(h, ev_bulk, profile_mark(h), 38.0 * sizeof(S) * (double)h->G.n, (double)h->G.n);
         h->launches += 1;
         if (h->has_particle) {
-            // 2. cells next to the sphere: CLI links + momentum-exchange force partials
-            int nb = 0;
-            launch_boundary<S>(src, dst, h->flags[h->fcur], h->list, h->count, h->list_cap, h->G, p, h->d_ps,
-                               h->cfg.boundary == LBMP_CLI ? 1 : 0, h->partials, &nb, h->status, h->stream);
-            // 3. force average, gravity, virtual mass, Velocity Verlet
-            launch_particle_update(h->d_ps, h->partials, nb, h->G, h->history, h->cfg.history_capacity, h->status,
-                                   h->stream);
-            // 4. remap: new flags in the box, refill/zero, new boundary list
-            uint8_t* fnext = h->flags[1 - h->fcur];
-            launch_flags_box(fnext, h->G, h->box, h->d_ps, h->stream);
-            launch_refill<S>(dst, h->flags[h->fcur], fnext, h->G, h->box, h->d_ps, (A)fp16_scale(h, false),
-                             (A)fp16_scale(h, true), (A)grad_refill_coef(h->cfg.refill, h->tau), h->stream);
-            launch_build_links(fnext, h->G, h->box, h->d_ps, h->link_mask, h->link_blocks, h->list, h->count,
-                               h->list_cap, h->status, h->stream);
+            // remap: new flags in the box, refill and zeroing, boundary marks
+            h->frame_cur = 1 - h->frame_cur;
+            h->launches += launch_remap<S>(h, dst, h->flags[h->fcur], h->flags[1 - h->fcur], h->frame_cur, false,
+                                           (A)fp16_scale(h, false), (A)fp16_scale(h, true),
+                                           (A)grad_refill_coef(h->cfg.refill, h->tau), h->stream);
             h->fcur = 1 - h->fcur;
-            h->launches += 6;
         }
     });
     profile_step(h, ev_step, profile_mark(h));
     h->cur = 1 - h->cur;
     h->steps += 1;
     h->updates += h->G.n;
+}
+
+// Frames, boundary marks and counts of the sphere's current position (uniform grids).
+void mark_boundary(lbmp_handle* h) {
+    launch_frames(h, h->stream);
+    h->frames_stale = false;
+    with_storage(h->cfg.precision, [&](auto tag) {
+        using S = std::remove_pointer_t<decltype(tag)>;
+        using A = typename Store<S>::A;
+        launch_remap<S>(h, (S*)h->pops[h->cur], h->flags[h->fcur], h->flags[1 - h->fcur], h->frame_cur, true, (A)1, (A)1,
+                        (A)0, h->stream);
+    });
 }
 
 lbmp_status read_status(lbmp_handle* h) {
@@ -385,22 +393,24 @@ lbmp_status lbmp_add_sphere(lbmp_handle* h, const double pos[3], double diameter
     const double shell = 4.0 / 3.0 * M_PI * (ro * ro * ro - ri * ri * ri);
     h->list_cap = (int)std::min<double>((double)B.cells, std::ceil(shell) + 64.0);
     h->list = (int*)dev_alloc(h, sizeof(int) * (size_t)h->list_cap);
-    const int max_blocks = boundary_grid(h->list_cap);
+    const int max_blocks = step_boundary_blocks(B, h->list_cap);
     h->partials = (double*)dev_alloc(h, sizeof(double) * 6 * (size_t)max_blocks);
     h->link_mask = (uint8_t*)dev_alloc(h, (size_t)B.cells);
-    h->link_blocks = (int*)dev_alloc(h, sizeof(int) * (size_t)((B.cells + 255) / 256));
-    if (!h->list || !h->partials || !h->link_mask || !h->link_blocks)
+    h->link_blocks = (int*)dev_alloc(h, sizeof(int) * (size_t)((B.cells + 63) / 64));
+    h->frames = (PFrames*)dev_alloc(h, frames_bytes());
+    h->d_done = (int*)dev_alloc(h, sizeof(int));
+    if (!h->list || !h->partials || !h->link_mask || !h->link_blocks || !h->frames || !h->d_done)
         return fail(h, LBMP_ERR_OOM, "lbmp_add_sphere: device allocation failed");
     lbmp_status s = upload_particle(h);
     if (s != LBMP_OK) return s;
     launch_flags_full(h->flags[h->fcur], h->G, h->d_ps, h->stream);
     launch_flags_full(h->flags[1 - h->fcur], h->G, h->d_ps, h->stream);
+    LBMP_CK(h, cudaMemsetAsync(h->d_done, 0, sizeof(int), h->stream));
     with_storage(h->cfg.precision, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
         launch_zero_solid<S>((S*)h->pops[h->cur], h->flags[h->fcur], h->G, h->stream);
     });
-    launch_build_links(h->flags[h->fcur], h->G, h->box, h->d_ps, h->link_mask, h->link_blocks, h->list, h->count,
-                       h->list_cap, h->status, h->stream);
+    mark_boundary(h);
     LBMP_CK(h, cudaGetLastError());
     LBMP_CK(h, cudaStreamSynchronize(h->stream));
     h->has_particle = true;
@@ -733,8 +743,9 @@ lbmp_status lbmp_get_links(lbmp_handle* h, int64_t* cell, int32_t* q, double* de
         const lbmp_status st = amr_links(h, cell, q, delta, cap, n);
         return st == LBMP_OK ? LBMP_OK : fail(h, st, "lbmp_get_links: failed");
     }
-    if (!h->has_particle) return LBMP_OK;
+    if (!h->has_particle || h->batch) return LBMP_OK;
     int cnt = 0;
+    launch_links_emit(h, h->frame_cur, h->stream);
     LBMP_CK(h, cudaMemcpyAsync(&cnt, h->count, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     LBMP_CK(h, cudaStreamSynchronize(h->stream));
     if (cnt == 0) return LBMP_OK;
@@ -914,7 +925,7 @@ lbmp_status lbmp_updates_per_step(lbmp_handle* h, int64_t* updates, int32_t* lau
         if (launches) *launches = amr_launches_per_coarse_step(h);
     } else {
         if (updates) *updates = h->G.n;
-        if (launches) *launches = h->has_particle ? 7 : 1;
+        if (launches) *launches = h->has_particle ? (step_uses_list(h->box) ? 3 : 2) : 1;
     }
     return LBMP_OK;
 }
@@ -1101,9 +1112,7 @@ lbmp_status lbmp_load(lbmp_handle* h, const char* path) {
     LBMP_CK(h, cudaMemcpy(h->flags[h->fcur], buf.data(), (size_t)h->G.n, cudaMemcpyHostToDevice));
     LBMP_CK(h, cudaMemcpy(h->flags[1 - h->fcur], buf.data(), (size_t)h->G.n, cudaMemcpyHostToDevice));
     h->h2d += (long long)(pb + 2 * (size_t)h->G.n);
-    if (h->has_particle)
-        launch_build_links(h->flags[h->fcur], h->G, h->box, h->d_ps, h->link_mask, h->link_blocks, h->list, h->count,
-                           h->list_cap, h->status, h->stream);
+    if (h->has_particle) mark_boundary(h);
     LBMP_CK(h, cudaStreamSynchronize(h->stream));
     return read_status(h);
 }

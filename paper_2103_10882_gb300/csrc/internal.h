@@ -51,7 +51,7 @@ __device__ __forceinline__ A wall_term(const GridDesc& G, int q, const int xyz[3
 // Guo source.  The quadratic ones include the FP16 storage factor.
 template <typename A>
 struct CollideConsts {
-    A hp, hm, r0;         // (1 - s+)/2, (1 - s-)/2, 1 - s+
+    A hp, hm, hsm, r0;    // (1 - s+)/2, (1 - s-)/2, s-/2, 1 - s+
     A kF, kE, mF, mE;     // s+ 9/2 w, s- 3 w on faces and edges
     A c15, cF;            // 3/2, 3 (1 - s+/2)
     A gs[9], ga[9];       // 9 (1 - s+/2) w c_q.F, 3 (1 - s-/2) w c_q.F for q = 1, 3, ..., 17
@@ -76,6 +76,7 @@ inline void collide_consts(CollideParams<A>& p) {
     CollideConsts<A>& k = p.k;
     k.hp = (A)(0.5 * (1.0 - sp));
     k.hm = (A)(0.5 * (1.0 - sm));
+    k.hsm = (A)(0.5 * sm);
     k.r0 = (A)(1.0 - sp);
     k.kF = (A)(4.5 * sp * wF * q2);
     k.kE = (A)(4.5 * sp * wE * q2);
@@ -100,39 +101,34 @@ struct BoxDesc {
     long long cells;
 };
 
-// Grid of the warp-per-cell boundary kernels (8 warps per block, grid-stride
-// over the boundary list); also the number of force partials.  The list
-// capacity is about three times the boundary cells of the sphere, so one
-// block per 32 entries of capacity gives each warp one or two cells: enough
-// warps to hide the gathers' latency, few enough that the per-block set-up
-// and the FP64 reduction stay small.  At most eight blocks per SM.
-inline int boundary_grid(int capacity) {
-    const int b = (capacity + 31) / 32;
-    return b < 1 ? 1 : (b > 1216 ? 1216 : b);
+// Boundary CTAs of a coupled uniform step, also the number of force partials (8 warps each, taking the boundary
+// cells in turn).  A prefix of the counts per run of box cells finds them (MARK_CELLS_MAX bounds its shared memory,
+// 8 KB, spheres up to about 43 cells): one CTA per 128 box cells gives each warp one or two cells, enough
+// warps to hide the gathers' latency, few enough that the per-CTA set-up and the sums stay small.  Larger boxes
+// read a list: one CTA per 32 entries of its capacity (about three times the boundary cells), at most eight per SM.
+constexpr long long MARK_CELLS_MAX = 1 << 17;
+inline bool step_uses_list(const BoxDesc& b) { return b.cells > MARK_CELLS_MAX; }
+inline int step_boundary_blocks(const BoxDesc& b, int list_capacity) {
+    const long long n = step_uses_list(b) ? (list_capacity + 31) / 32 : (b.cells + 127) / 128;
+    return (int)(n < 1 ? 1 : (n > 1216 ? 1216 : n));
 }
+
+struct PFrames;
 
 // Launchers (uniform.cu).  All are asynchronous on `stream`.
 template <typename S>
-void launch_bulk(const S* src, S* dst, const GridDesc& g, const CollideParams<typename Store<S>::A>& p,
-                 int* status, cudaStream_t stream);
-template <typename S>
-void launch_boundary(const S* src, S* dst, const uint8_t* flags, const int* list, const int* count, int max_cells,
-                     const GridDesc& g, const CollideParams<typename Store<S>::A>& p, const ParticleState* ps,
-                     int cli, double* partials, int* nblocks_out, int* status, cudaStream_t stream);
-void launch_particle_update(ParticleState* ps, const double* partials, int nblocks, const GridDesc& g,
-                            double* history, int hist_cap, int* status, cudaStream_t stream);
+void launch_step(const lbmp_handle* h, const S* src, S* dst, const CollideParams<typename Store<S>::A>& p, int finish,
+                 double* force_out, cudaStream_t stream);
 void launch_flags_full(uint8_t* flags, const GridDesc& g, const ParticleState* ps, cudaStream_t stream);
-void launch_flags_box(uint8_t* flags_next, const GridDesc& g, const BoxDesc& b, const ParticleState* ps,
-                      cudaStream_t stream);
+void launch_frames(const lbmp_handle* h, cudaStream_t stream);
+size_t frames_bytes();
+// Returns the number of launches.
 template <typename S>
-void launch_refill(S* pops, const uint8_t* flags_cur, const uint8_t* flags_next, const GridDesc& g,
-                   const BoxDesc& b, const ParticleState* ps, typename Store<S>::A scale,
-                   typename Store<S>::A inv_scale, typename Store<S>::A gcoef, cudaStream_t stream);
-// Boundary-cell list of the box; mask (b.cells bytes) and block_count
-// (ceil(b.cells / 256) ints) are scratch.
-void launch_build_links(const uint8_t* flags, const GridDesc& g, const BoxDesc& b, const ParticleState* ps,
-                        uint8_t* mask, int* block_count, int* list, int* count, int capacity, int* status,
-                        cudaStream_t stream);
+int launch_remap(const lbmp_handle* h, S* pops, const uint8_t* fcur, uint8_t* fnext, int frame, bool mark_only,
+                 typename Store<S>::A scale, typename Store<S>::A inv_scale, typename Store<S>::A gcoef,
+                 cudaStream_t stream);
+// Boundary cells of the current marks as a list (h->list, h->count).
+void launch_links_emit(const lbmp_handle* h, int frame, cudaStream_t stream);
 void launch_export_links(const uint8_t* flags, const int* list, const int* count, int max_cells,
                          const GridDesc& g, const ParticleState* ps, int cli, int32_t* q_out, double* delta_out,
                          cudaStream_t stream);
@@ -177,10 +173,12 @@ struct lbmp_handle {
     int* list = nullptr;                 // boundary cells
     int* count = nullptr;
     int list_cap = 0;
-    uint8_t* link_mask = nullptr;        // scratch of the link compaction (one byte per box cell)
-    int* link_blocks = nullptr;          // scratch: per-block counts
+    uint8_t* link_mask = nullptr;        // marks of the box cells around the sphere (one byte each)
+    int* link_blocks = nullptr;          // boundary cells per run of box cells
     double* partials = nullptr;
-    int partial_blocks = 0;
+    int* d_done = nullptr;               // last-block-done counter of the boundary CTAs (uniform grids)
+    lbmp::PFrames* frames = nullptr;     // uniform grids: two copies of the sphere's frames, a step reads one
+    int frame_cur = 0;                   // (frame_cur) while its particle update writes the other
     lbmp::ParticleState* d_ps = nullptr;
     lbmp::ParticleState h_ps;                  // host copy of the parameters
     double* history = nullptr;

@@ -54,14 +54,15 @@ __device__ __forceinline__ A dir_dot(int q, A x, A y, A z) {
 // of the opposite pairs, both new populations of a pair are S + D and S - D,
 //   S = (1 - s+)/2 ps + s+ e+ + (1 - s+/2) S+,   D = (1 - s-)/2 pd + s- e- + (1 - s-/2) S-,
 // the coefficients and the direction's part of the Guo source come from the host (collide_consts), the density part of
-// e+ and the MRT correction are one number per class of directions: 112 instructions per cell unforced (13 more forced).
+// e+ and the MRT correction are one number per class of directions: 121 instructions per cell unforced (13 more forced).
+// (1 - s+)/2 is exact for s+ in [1/2, 2]; (1 - s-)/2 is not for s- < 1/2, and its rounding would change every cell's
+// momentum by the same relative 6e-17 in every step, so FP64 takes pd/2 - (s-/2) pd in two operations.
 // Measured: a coupled FP64 step of 61 x 53 x 75 cells 175 -> 129 us, a refined FP64 step (1.1 M updates) 394 -> 261 us,
 // an FP16-storage step of 256^3 301 -> 293 us.
 // The MRT sums over a class follow from ps alone: sum_faces 2 e+ = rho/3, sum_edges 2 e+ = rho/3 + uu/2, and the half
 // source sums to -uF/2, 0 and uF/2 over rest, faces and edges.
-// FP32 storage keeps the plain form below: its coefficient (1 - s-)/2 would be rounded to FP32 for s- < 1/2, a relative
-// momentum change of up to 3e-8 in every step, and its kernels wait on memory, not on instructions.  In FP64 the same
-// rounding is 6e-17 a step; FP16 storage itself rounds at 5e-4.
+// FP32 storage keeps the plain form below: its kernels wait on memory, not on instructions, and there the rounded
+// coefficient would be a relative 3e-8 a step.  FP16 storage itself rounds at 5e-4 and takes (1 - s-)/2 in one.
 // Populations may be scaled by 2^s (SCALED): quadratic terms then carry 2^-s, which the host's coefficients include.
 template <typename A, bool FORCED, bool SCALED, int MRT_MODE>
 __device__ __forceinline__ void collide_direct(A (&g)[19], const CollideParams<A>& P, int* status) {
@@ -124,7 +125,8 @@ __device__ __forceinline__ void collide_direct(A (&g)[19], const CollideParams<A
             e = face ? K.kF * u2[k < 3 ? k : 0] + bF : (K.kE * cu) * cu + bE;
             d = (face ? K.mF : K.mE) * cu;
         }
-        const A Sy = K.hp * ps[k] + e, Da = K.hm * pd[k] + d;
+        const A Sy = K.hp * ps[k] + e;
+        const A Da = sizeof(A) == 8 ? (A(0.5) * pd[k] + d) - K.hsm * pd[k] : K.hm * pd[k] + d;
         g[q] = Sy + Da;
         g[q + 1] = Sy - Da;
     }
@@ -812,6 +814,31 @@ __device__ __forceinline__ void particle_advance_axis(ParticleState& P, int a, d
     }
 }
 
+// Sum of component comp over the nblocks force partials by one warp, in a fixed order (every lane gets it).
+__device__ __forceinline__ double sum_partials(const double* partials, int nblocks, int comp) {
+    const int lane = threadIdx.x & 31;
+    // Lane l sums partials l, l + 64, ... into s0 and l + 32, l + 96, ... into s1, in that
+    // order; eight loads at a time are issued before their sums
+    double s0 = 0.0, s1 = 0.0;
+    for (int base = 0; base < nblocks; base += 256) {
+        double v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int b = base + lane + 32 * k;
+            v[k] = b < nblocks ? __ldcg(partials + (size_t)b * 6 + comp) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) {
+            if (base + lane + 32 * k < nblocks) s0 += v[k];
+            if (base + lane + 32 * (k + 1) < nblocks) s1 += v[k + 1];
+        }
+    }
+    double t = s0 + s1;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+    return t;
+}
+
 // Particle update by one block of NT >= 256 threads once the nblocks force
 // partials are complete: warps 0..5 sum one component each in a fixed
 // order (lane l takes partials l, l + 32, ... in two alternating sums, then
@@ -831,25 +858,7 @@ __device__ __forceinline__ void particle_block_update(ParticleState* __restrict_
     __shared__ ParticleState sP;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (wid < 6) {
-        // lane l sums partials l, l + 64, ... into s0 and l + 32, l + 96, ... into s1, in that
-        // order; eight loads at a time are issued before their sums
-        double s0 = 0.0, s1 = 0.0;
-        for (int base = 0; base < nblocks; base += 256) {
-            double v[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int b = base + lane + 32 * k;
-                v[k] = b < nblocks ? __ldcg(partials + (size_t)b * 6 + wid) : 0.0;
-            }
-#pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-                if (base + lane + 32 * k < nblocks) s0 += v[k];
-                if (base + lane + 32 * (k + 1) < nblocks) s1 += v[k + 1];
-            }
-        }
-        double t = s0 + s1;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+        const double t = sum_partials(partials, nblocks, wid);
         if (lane == 0) sFT[wid] = t;
     } else if (wid == 6) {
         if (lane < 2) sinv[lane] = inv ? inv[lane] : 1.0 / (lane == 0 ? particle_mass(*ps) : particle_inertia(*ps));
@@ -931,6 +940,82 @@ __device__ __forceinline__ bool last_block_done(int* counter, int nblocks) {
     }
     __syncthreads();
     return last != 0;
+}
+
+constexpr int LINK_RUN = 64;   // box cells per run of the boundary marks (one count per run)
+
+// Exclusive prefix of n counts into pre[0..n] (pre[n] = total), computed by
+// the whole CTA (NT threads, two consecutive counts per thread and pass);
+// every thread must call it.  first0, first1: counts 2 threadIdx.x and
+// 2 threadIdx.x + 1 (0 beyond n), loaded by the caller ahead.
+template <int NT>
+__device__ __forceinline__ int block_prefix(const int* __restrict__ count, int n, int* pre, int first0, int first1) {
+    __shared__ int wsum[NT / 32];
+    __shared__ int carry;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (threadIdx.x == 0) carry = 0;
+    __syncthreads();
+    for (int base = 0; base < n; base += 2 * NT) {
+        const int i = base + 2 * (int)threadIdx.x;
+        const int c0 = base == 0 ? first0 : (i < n ? count[i] : 0);
+        const int c1 = base == 0 ? first1 : (i + 1 < n ? count[i + 1] : 0);
+        int v = c0 + c1;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, v, off);
+            if (lane >= off) v += y;
+        }
+        if (lane == 31) wsum[wid] = v;
+        __syncthreads();
+        if (wid == 0) {
+            int w = lane < NT / 32 ? wsum[lane] : 0;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, w, off);
+                if (lane >= off) w += y;
+            }
+            if (lane < NT / 32) wsum[lane] = w;
+        }
+        __syncthreads();
+        const int incl = carry + (wid > 0 ? wsum[wid - 1] : 0) + v;   // through count i + 1
+        if (i < n) pre[i + 1] = incl - c1;
+        if (i + 1 < n) pre[i + 2] = incl;
+        __syncthreads();
+        if (threadIdx.x == 0) carry += wsum[NT / 32 - 1];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) pre[0] = 0;
+    __syncthreads();
+    return pre[n];
+}
+
+// Box cell of the j-th marked one (mask byte 1, box order): the run r that holds it is the largest with
+// pre[r] <= j (pre: the prefix of the runs' counts), the cell the (j - pre[r])-th marked one of that run.  The whole
+// warp calls it with the same j.
+__device__ __forceinline__ int marked_cell(const int* pre, int runs, const uint8_t* __restrict__ mask, long long cells,
+                                           int j) {
+    static_assert(LINK_RUN == 64, "two ballots per run");
+    const int lane = threadIdx.x & 31;
+    int lo = 0, hi = runs;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (pre[mid] <= j) lo = mid;
+        else hi = mid;
+    }
+    const long long r0 = (long long)lo * LINK_RUN;
+    const bool m0 = r0 + lane < cells && mask[r0 + lane] == 1;
+    const bool m1 = r0 + 32 + lane < cells && mask[r0 + 32 + lane] == 1;
+    const unsigned b0 = __ballot_sync(0xffffffffu, m0), b1 = __ballot_sync(0xffffffffu, m1);
+    int k = j - pre[lo];
+    unsigned bits = b0;
+    int base = 0;
+    if (k >= __popc(b0)) {
+        k -= __popc(b0);
+        bits = b1;
+        base = 32;
+    }
+    for (; k > 0; --k) bits &= bits - 1u;   // drop the k lowest marked cells
+    return (int)(r0 + base + __ffs((int)bits) - 1);
 }
 
 // Box cells of [t0, t0 + chunk) whose mask byte is set, in box order, into

@@ -1,9 +1,9 @@
-// Uniform-grid kernels of the coupled step (Algorithm 1):
-//   k_bulk       stream (pull) + TRT collide of every cell         Sec. 2.1, Eq. LBE
-//   k_boundary   re-does the cells next to the sphere with CLI links and
-//                sums the momentum-exchange force/torque in FP64     Sec. 2.3
-//   k_particle   force averaging, gravity, virtual mass, Velocity Verlet   Sec. 2.2, 3.3
-//   k_flags_box, k_refill, k_build_links   remap after the sphere moved    Sec. 2.3
+// Uniform-grid kernels of the coupled step (Algorithm 1), two launches per step:
+//   k_step       stream (pull) + TRT collide of every cell (Sec. 2.1, Eq. LBE); its first CTAs take the cells
+//                next to the sphere (CLI links, momentum-exchange force and torque, Sec. 2.3), and the last of
+//                those to finish runs the particle update (force averaging, gravity, virtual mass, Velocity
+//                Verlet, Sec. 2.2, 3.3)
+//   k_remap      flags, refill and marks of the boundary cells after the sphere moved (Sec. 2.3)
 // Populations are stored as deviations g = f - w in SoA layout [q][z][y][x].
 #include <cuda_fp16.h>
 
@@ -15,27 +15,91 @@
 namespace lbmp {
 namespace {
 
-constexpr int BULK_THREADS = 256;
+constexpr int STEP_THREADS = 256;
+// Marks of the box cells around the sphere, written by the remap: plain fluid cell, fluid cell with a solid
+// D3Q19 neighbour (taken by the boundary CTAs), cell with its centre inside the sphere.
+constexpr uint8_t MARK_PLAIN = 0, MARK_BOUNDARY = 1, MARK_SOLID = 2;
+
+// n / d for n < 2^31 by one high multiplication (Granlund & Montgomery, "Division by invariant integers
+// using multiplication", 1994, Fig. 4.1): d >= 1.
+struct FastDiv {
+    unsigned d, m, s;
+    __host__ void set(unsigned v) {
+        d = v;
+        s = 0;
+        while ((1ull << s) < v) ++s;
+        m = (unsigned)(((1ull << 32) * ((1ull << s) - v)) / v + 1);
+    }
+    __device__ __forceinline__ unsigned div(unsigned n) const {
+        const unsigned t = __umulhi(m, n);
+        return (t + n) >> s;   // t <= n < 2^31: no overflow
+    }
+};
+
+// One coupled step of a uniform grid.
+template <typename S>
+struct StepArgs {
+    using A = typename Store<S>::A;
+    const S* src;
+    S* dst;
+    GridDesc G;
+    CollideParams<A> P;
+    FastDiv dx, dy;        // by nx (FP16 pairs: nx / 2) and ny
+    unsigned items;        // cells (FP16 pairs: pairs of cells)
+    int per_cta;           // of them per bulk CTA
+    int* status;
+    // the sphere's part (bblocks = 0 without a sphere)
+    int bblocks;           // boundary CTAs, first in the grid
+    int finish;            // last boundary CTA: 0 the particle update, 1 the force into force_out, 2 nothing
+    int cli, hist_cap;
+    const uint8_t* flags;
+    const uint8_t* mark;
+    const int* run_count;
+    const int* list;       // boundary cells as a list, for boxes of more than MARK_CELLS_MAX cells; else null
+    const int* count;
+    BoxDesc B;
+    ParticleState* ps;
+    double* partials;
+    int* done;
+    double* history;
+    const PFrames* frames;   // of the sphere's position in this step
+    PFrames* frames_next;    // of the position that the particle update reaches
+    double* force_out;
+};
+
+// Mark of cell (x, y, z): outside the sphere's box every cell is plain.  The box origin lies on the device;
+// o, n and E per axis as in box_cell.
+__device__ __forceinline__ int box_coord(int v, int o, int n, int periodic, int E) {
+    int t = v - o;
+    if (periodic) t = t < 0 ? t + n : (t >= n ? t - n : t);
+    return (t >= 0 && t < E) ? t : -1;
+}
+
+template <typename S>
+__device__ __forceinline__ uint8_t cell_mark(const StepArgs<S>& T, int x, int y, int z) {
+    if (T.bblocks == 0) return MARK_PLAIN;
+    const int* o = T.frames->bf.o;
+    const int tz = box_coord(z, o[2], T.G.nz, T.G.periodic[2], T.B.E[2]);
+    const int ty = box_coord(y, o[1], T.G.ny, T.G.periodic[1], T.B.E[1]);
+    const int tx = box_coord(x, o[0], T.G.nx, T.G.periodic[0], T.B.E[0]);
+    if ((tx | ty | tz) < 0) return MARK_PLAIN;
+    return T.mark[tx + T.B.E[0] * (ty + T.B.E[1] * tz)];
+}
 
 // ------------------------------------------------------------------ bulk
-// One thread per cell, pull form: g_q(x, t+1) = g~_q(x - c_q, t), then TRT.
-// WALLS: some axis has no-slip walls (bounce-back at the domain edge);
-// FORCED: fluid body force present.  Both are compile-time so the common
-// periodic, unforced case carries no per-population branches.  Spatial
-// offsets are 32-bit (cells < 2^31); each population array is addressed
-// from its own base pointer.
+// One thread per cell, pull form: g_q(x, t+1) = g~_q(x - c_q, t), then TRT; solid cells are stored as zero and
+// boundary cells left to the boundary CTAs.  Cells are taken in memory order, so full warps touch whole lines
+// whatever the extents (a 2-D tile of a 75-cell row left two threads in five idle).  WALLS: some axis has
+// no-slip walls (bounce-back at the domain edge); FORCED: fluid body force present.
 template <typename S, bool WALLS, bool FORCED>
-__global__ void __launch_bounds__(BULK_THREADS)
-    k_bulk(const S* __restrict__ src, S* __restrict__ dst, GridDesc G, CollideParams<typename Store<S>::A> P,
-           int* __restrict__ status) {
+__device__ __forceinline__ void bulk_cells(const StepArgs<S>& T, unsigned item) {
     using A = typename Store<S>::A;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
+    const GridDesc& G = T.G;
     const int nx = G.nx, ny = G.ny, nz = G.nz;
-    if (x >= nx || y >= ny) return;
+    const unsigned row = T.dx.div(item), plane = T.dy.div(row);
+    const int x = (int)(item - row * (unsigned)nx), y = (int)(row - plane * (unsigned)ny), z = (int)plane;
     const size_t n = (size_t)G.n;
-    const int cell = x + nx * (y + ny * z);
+    const int cell = (int)item;
     // source coordinate x - c for c = -1, 0, +1 (-1 marks a wall)
     int xs[3], ys[3], zs[3];
     xs[1] = x;
@@ -53,40 +117,43 @@ __global__ void __launch_bounds__(BULK_THREADS)
         const int sx = xs[cx(q) + 1], sy = ys[cy(q) + 1], sz = zs[cz(q) + 1];
         if (WALLS && (sx < 0 || sy < 0 || sz < 0)) {   // no-slip wall: bounce-back (moving: Ladd's term)
             const int xyz[3] = {x, y, z};
-            g[q] = Store<S>::load(src + (size_t)opp(q) * n + cell, P.inv_scale) + wall_term<A>(G, q, xyz);
+            g[q] = Store<S>::load(T.src + (size_t)opp(q) * n + cell, T.P.inv_scale) + wall_term<A>(G, q, xyz);
         } else {
             const int off = sx + nx * (sy + ny * sz);
-            g[q] = Store<S>::load(src + (size_t)q * n + off, P.inv_scale);
+            g[q] = Store<S>::load(T.src + (size_t)q * n + off, T.P.inv_scale);
         }
     }
-    trt_collide<A, FORCED>(g, P, status);
+    const uint8_t mark = cell_mark<S>(T, x, y, z);   // beside the pulls, not before them
+    if (mark != MARK_PLAIN) {
+        if (mark == MARK_SOLID)
 #pragma unroll
-    for (int q = 0; q < 19; ++q) Store<S>::store(dst + (size_t)q * n + cell, g[q], P.scale);
+            for (int q = 0; q < 19; ++q) Store<S>::store(T.dst + (size_t)q * n + cell, A(0), T.P.scale);
+        return;
+    }
+    trt_collide<A, FORCED>(g, T.P, T.status);
+#pragma unroll
+    for (int q = 0; q < 19; ++q) Store<S>::store(T.dst + (size_t)q * n + cell, g[q], T.P.scale);
 }
 
-// FP16 storage, unforced: the same update as k_bulk, two cells (x, x + 1,
-// x even) per thread.  Every population is read as the aligned pair of
-// halves of its source row; the populations shifted along x take their
-// outer half from the neighbouring lane (a shuffle); the first lane of a
-// warp (rows start there) and the last pair of a warp or of a row load that
-// one half themselves.  The collision runs on the stored, scaled values
-// (trt_collide's SCALED form, collide_direct), so neither the loads nor the stores multiply
-// by the scale, and TRT or MRT is chosen at compile time.  nx is even; rows
-// hold whole pairs.
-constexpr int BULK2_THREADS = 256;
+// FP16 storage, unforced: the same update, two cells (x, x + 1, x even) per
+// thread.  Every population is read as the aligned pair of halves of its
+// source row; the populations shifted along x take their outer half from the
+// neighbouring lane (a shuffle); the first lane of a warp or row and the last
+// pair of a warp or row load that one half themselves.  The collision runs on
+// the stored, scaled values (trt_collide's SCALED form, collide_direct), so
+// neither the loads nor the stores multiply by the scale, and TRT or MRT is
+// chosen at compile time.  nx is even; rows hold whole pairs.  Every lane of
+// the warp calls it (valid: the lane has a pair).
 template <bool WALLS, bool MRT>
-__global__ void __launch_bounds__(BULK2_THREADS)
-    k_bulk_h2(const __half* __restrict__ src, __half* __restrict__ dst, GridDesc G, CollideParams<float> P,
-              int* __restrict__ status) {
-    const int xp = blockIdx.x * blockDim.x + threadIdx.x;   // pair index
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
+__device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, unsigned pair, bool valid) {
+    const GridDesc& G = T.G;
     const int nx = G.nx, ny = G.ny, nz = G.nz;
-    const int lane = threadIdx.x & 31;   // blockDim.x is a multiple of 32: a warp is one run of a row
-    const bool valid = 2 * xp < nx && y < ny;
-    const int x = valid ? 2 * xp : 0;
-    const int yy = valid ? y : 0;
+    const int lane = threadIdx.x & 31;
+    const unsigned item = valid ? pair : 0u;
+    const unsigned row0 = T.dx.div(item), plane = T.dy.div(row0);
+    const int x = 2 * (int)(item - row0 * T.dx.d), yy = (int)(row0 - plane * (unsigned)ny), z = (int)plane;
     const size_t n = (size_t)G.n;
+    const __half* src = T.src;
     const int cell = x + nx * (yy + ny * z);
     int ys[3], zs[3];
     ys[1] = yy;
@@ -98,6 +165,7 @@ __global__ void __launch_bounds__(BULK2_THREADS)
     // x - 1 of the pair's first cell and x + 2 of its second (-1: beyond a wall)
     const int xm = x > 0 ? x - 1 : (WALLS && !G.periodic[0] ? -1 : nx - 1);
     const int xq = x + 2 < nx ? x + 2 : (WALLS && !G.periodic[0] ? -1 : 0);
+    const bool first = lane == 0 || x == 0, last = lane == 31 || x + 2 >= nx;   // warp or row ends
     // all loads first (the pairs, then the outer halves of the shifted populations, every lane
     // loading one: the lanes that need none read their own pair's first half), then the shuffles
     __half2 pr[19];
@@ -112,10 +180,11 @@ __global__ void __launch_bounds__(BULK2_THREADS)
         pr[q] = __ldg(reinterpret_cast<const __half2*>(pq + row + x));
         if (cx(q) != 0) {
             const int xe = cx(q) == 1 ? xm : xq;
-            const bool need = cx(q) == 1 ? lane == 0 : (lane == 31 || x + 2 >= nx);   // warp or row end
+            const bool need = cx(q) == 1 ? first : last;
             ex[q] = __ldg(pq + row + ((need && xe >= 0) ? xe : x));
         }
     }
+    const uint8_t mark0 = cell_mark<__half>(T, x, yy, z), mark1 = cell_mark<__half>(T, x + 1, yy, z);
     float g0[19], g1[19];
 #pragma unroll
     for (int q = 0; q < 19; ++q) {
@@ -126,12 +195,12 @@ __global__ void __launch_bounds__(BULK2_THREADS)
             b = __high2float(p);
         } else if (cx(q) == 1) {   // sources x - 1 and x
             const float prev = __shfl_up_sync(0xffffffffu, __high2float(p), 1);
-            a = lane == 0 ? __half2float(ex[q]) : prev;
+            a = first ? __half2float(ex[q]) : prev;
             b = __low2float(p);
         } else {                   // sources x + 1 and x + 2
             const float next = __shfl_down_sync(0xffffffffu, __low2float(p), 1);
             a = __high2float(p);
-            b = (lane == 31 || x + 2 >= nx) ? __half2float(ex[q]) : next;
+            b = last ? __half2float(ex[q]) : next;
         }
         if (WALLS) {   // bounce-back (moving walls: Ladd's term, scaled like the stored values)
             const bool wa = yw[q] || (cx(q) == 1 && xm < 0);
@@ -139,57 +208,80 @@ __global__ void __launch_bounds__(BULK2_THREADS)
             if (wa || wb) {
                 const __half2 o = *reinterpret_cast<const __half2*>(src + (size_t)opp(q) * n + cell);
                 const int xyz0[3] = {x, yy, z}, xyz1[3] = {x + 1, yy, z};
-                if (wa) a = __low2float(o) + wall_term<float>(G, q, xyz0) * P.scale;
-                if (wb) b = __high2float(o) + wall_term<float>(G, q, xyz1) * P.scale;
+                if (wa) a = __low2float(o) + wall_term<float>(G, q, xyz0) * T.P.scale;
+                if (wb) b = __high2float(o) + wall_term<float>(G, q, xyz1) * T.P.scale;
             }
         }
         g0[q] = a;
         g1[q] = b;
     }
     if (!valid) return;
-    trt_collide<float, false, true, MRT ? 1 : 0, true>(g0, P, status);
-    trt_collide<float, false, true, MRT ? 1 : 0, true>(g1, P, status);
+    __half* dst = T.dst;
+    if ((mark0 | mark1) == MARK_PLAIN) {
+        trt_collide<float, false, true, MRT ? 1 : 0, true>(g0, T.P, T.status);
+        trt_collide<float, false, true, MRT ? 1 : 0, true>(g1, T.P, T.status);
 #pragma unroll
-    for (int q = 0; q < 19; ++q)
-        __stcs(reinterpret_cast<__half2*>(dst + (size_t)q * n + cell), __floats2half2_rn(g0[q], g1[q]));
+        for (int q = 0; q < 19; ++q)
+            __stcs(reinterpret_cast<__half2*>(dst + (size_t)q * n + cell), __floats2half2_rn(g0[q], g1[q]));
+        return;
+    }
+    // one of the two is solid or a boundary cell: each by itself
+    if (mark0 == MARK_PLAIN) trt_collide<float, false, true, MRT ? 1 : 0, true>(g0, T.P, T.status);
+    if (mark1 == MARK_PLAIN) trt_collide<float, false, true, MRT ? 1 : 0, true>(g1, T.P, T.status);
+#pragma unroll
+    for (int q = 0; q < 19; ++q) {
+        if (mark0 != MARK_BOUNDARY) dst[(size_t)q * n + cell] = __float2half_rn(mark0 == MARK_SOLID ? 0.0f : g0[q]);
+        if (mark1 != MARK_BOUNDARY) dst[(size_t)q * n + cell + 1] = __float2half_rn(mark1 == MARK_SOLID ? 0.0f : g1[q]);
+    }
 }
 
 // -------------------------------------------------------------- boundary
-// One warp per fluid cell that has a solid neighbour, lane q handling
-// population q: pulls from solid cells are replaced by the CLI rule of
-// Sec. 2.3 (link geometry in the population arithmetic, force and torque
-// summed in FP64), then the warp collides the cell cooperatively and writes
-// it.  Each block covers 8 list entries per pass; blocks past the end of the
-// list write zero partials.
-constexpr int BNDW_THREADS = 256;
+// The cells next to the sphere, one warp per cell, lane q handling population q: pulls from solid cells are
+// replaced by the CLI rule of Sec. 2.3 (link geometry in the population arithmetic), then the warp collides the
+// cell cooperatively and writes it.  The marked cells are spread evenly over the warps of the boundary CTAs:
+// every CTA turns the remap's counts per run into a prefix, and warp w of W takes the marked cells w, w + W, ...
+// in box order (or the entries of the list, for large boxes).  The block sums of force and torque go into one
+// FP64 partial per CTA; the CTA that finishes last sums them.  Runs beside the bulk CTAs, which skip these cells.
 template <typename S, bool FORCED>
-__global__ void __launch_bounds__(BNDW_THREADS)
-    k_boundary(const S* __restrict__ src, S* __restrict__ dst, const uint8_t* __restrict__ flags,
-               const int* __restrict__ list, const int* __restrict__ count, GridDesc G,
-               CollideParams<typename Store<S>::A> P, const ParticleState* __restrict__ ps, int cli,
-               double* __restrict__ partials, int* __restrict__ status) {
+__device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int* pre) {
     using A = typename Store<S>::A;
+    const GridDesc& G = T.G;
+    const CollideParams<A>& P = T.P;
+    const S* src = T.src;
     __shared__ LinkFrame<A> Fr;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int nwarps = gridDim.x * (BNDW_THREADS / 32);
-    const int cnt = *count;
-    if ((int)blockIdx.x * (BNDW_THREADS / 32) >= cnt) {   // uniform across the block
-        if (threadIdx.x < 6) partials[(size_t)blockIdx.x * 6 + threadIdx.x] = 0.0;
-        return;
+    __shared__ BoxFrame Bf;
+    const int runs = (int)((T.B.cells + LINK_RUN - 1) / LINK_RUN);
+    const int i2 = 2 * (int)threadIdx.x;   // this thread's first two counts, in flight during the set-up
+    int first0 = 0, first1 = 0;
+    if (!T.list) {
+        if (i2 < runs) first0 = T.run_count[i2];
+        if (i2 + 1 < runs) first1 = T.run_count[i2 + 1];
     }
-    if (threadIdx.x == 0) Fr.init(*ps);
+    if (threadIdx.x == 0) Fr = pframe_link<A>(*T.frames);
+    if (threadIdx.x == 32) Bf = T.frames->bf;
     __syncthreads();
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int total = T.list ? *T.count : block_prefix<STEP_THREADS>(T.run_count, runs, pre, first0, first1);
+    const int W = T.bblocks * (STEP_THREADS / 32);
     const size_t n = (size_t)G.n;
     const int n3[3] = {G.nx, G.ny, G.nz};
     LinkSums<A> acc;
-    for (int w = blockIdx.x * (BNDW_THREADS / 32) + wib; w < cnt; w += nwarps) {
-        const int cell = list[w];
-        const int x = cell % G.nx, y = (cell / G.nx) % G.ny, z = cell / (G.nx * G.ny);
+    for (int j = (int)blockIdx.x * (STEP_THREADS / 32) + wib; j < total; j += W) {
+        int xyz[3];
+        if (T.list) {
+            const int c = T.list[j];
+            xyz[0] = c % G.nx;
+            xyz[1] = (c / G.nx) % G.ny;
+            xyz[2] = c / (G.nx * G.ny);
+        } else {
+            const int t = marked_cell(pre, runs, T.mark, T.B.cells, j);
+            if (!box_cell(t, n3, G.periodic, T.B, Bf, xyz)) continue;   // marked cells are inside the domain
+        }
+        const size_t cell = (size_t)xyz[0] + (size_t)G.nx * ((size_t)xyz[1] + (size_t)G.ny * (size_t)xyz[2]);
         A gq = A(0);
         if (lane < 19) {
             const int q = lane;
             const int c[3] = {cx(q), cy(q), cz(q)};
-            const int xyz[3] = {x, y, z};
             int s3[3], f3[3];
             bool wall = false, far_ok = true;
 #pragma unroll
@@ -203,14 +295,13 @@ __global__ void __launch_bounds__(BNDW_THREADS)
                 gq = Store<S>::load(src + (size_t)opp(q) * n + cell, P.inv_scale) + wall_term<A>(G, q, xyz);
             } else {
                 const size_t sidx = (size_t)s3[0] + (size_t)G.nx * ((size_t)s3[1] + (size_t)G.ny * (size_t)s3[2]);
-                if (q == 0 || flags[sidx] == 0) {
-                    gq = Store<S>::load(src + (size_t)q * n + sidx, P.inv_scale);
-                } else {
+                gq = Store<S>::load(src + (size_t)q * n + sidx, P.inv_scale);   // beside the flag; dropped on a link
+                if (q != 0 && T.flags[sidx] != 0) {
                     const int k = opp(q);
                     size_t far = 0;
                     if (far_ok) {
                         far = (size_t)f3[0] + (size_t)G.nx * ((size_t)f3[1] + (size_t)G.ny * (size_t)f3[2]);
-                        far_ok = flags[far] == 0;
+                        far_ok = T.flags[far] == 0;
                     }
                     A d[3], fl[3], tl[3];
                     int pu[3];
@@ -218,28 +309,58 @@ __global__ void __launch_bounds__(BNDW_THREADS)
                     const A gt_k = Store<S>::load(src + (size_t)k * n + cell, P.inv_scale);
                     const A gt_q = Store<S>::load(src + (size_t)q * n + cell, P.inv_scale);
                     const A gt_far = far_ok ? Store<S>::load(src + (size_t)k * n + far, P.inv_scale) : A(0);
-                    gq = cli_link<A>(q, d, cli && far_ok, gt_k, gt_q, gt_far, Fr, fl, tl);
+                    gq = cli_link<A>(q, d, T.cli && far_ok, gt_k, gt_q, gt_far, Fr, fl, tl);
                     acc.add(k, pu, fl, tl);
                 }
             }
         }
-        gq = warp_trt_collide<A, FORCED>(gq, lane, P, status);
-        if (lane < 19) Store<S>::store(dst + (size_t)lane * n + cell, gq, P.scale);
+        gq = warp_trt_collide<A, FORCED>(gq, lane, P, T.status);
+        if (lane < 19) Store<S>::store(T.dst + (size_t)lane * n + cell, gq, P.scale);
     }
-    block_link_sums<BNDW_THREADS>(acc, ps->x, partials + (size_t)blockIdx.x * 6);
+    if (T.finish == 2) return;   // the force is not wanted
+    block_link_sums<STEP_THREADS>(acc, T.ps->x, T.partials + (size_t)blockIdx.x * 6);
+    if (!last_block_done(T.done, T.bblocks)) return;
+    if (T.finish == 1) {
+        if (wib < 3) {
+            const double f = sum_partials(T.partials, T.bblocks, wib);
+            if (lane == 0) T.force_out[wib] = f;
+        }
+        return;
+    }
+    particle_block_update<STEP_THREADS>(T.ps, T.partials, T.bblocks, G, T.history, T.hist_cap, T.status, T.frames->inv);
+    __syncthreads();
+    // frames of the moved sphere, in the other copy: bulk CTAs of this launch still read this one
+    if (threadIdx.x < 3) pframes_axis(T.frames_next, *T.ps, n3, T.B, threadIdx.x);
 }
 
-// -------------------------------------------------------------- particle
-// Sums the per-block partial forces in a fixed order, then Algorithm 1:
-// average over two steps, gravity/buoyancy F_g = (rho_p - rho_f) g V,
-// virtual force/torque from the previous accelerations, and Velocity
-// Verlet (kick-drift-kick) with m = (rho_p + C_v) V, I = 2/5 (rho_p + C_vw) V r^2.
-constexpr int PART_THREADS = 256;
+// One launch: bblocks boundary CTAs, then the bulk CTAs.  The chain boundary cells -> force sum -> particle update
+// (11 + 5 us as two launches of their own) runs beside the bulk update instead of after it.
+// Registers: 5 CTAs of 256 threads per SM (48 registers) where the bulk update waits on memory.
+template <typename S>
+constexpr int STEP_MIN_CTAS = sizeof(S) == 4 ? 5 : (sizeof(S) == 2 ? 4 : 2);
 
-__global__ void __launch_bounds__(PART_THREADS)
-    k_particle(ParticleState* __restrict__ ps, const double* __restrict__ partials, int nblocks, GridDesc G,
-               double* __restrict__ history, int hist_cap, int* __restrict__ status) {
-    particle_block_update<PART_THREADS>(ps, partials, nblocks, G, history, hist_cap, status);
+template <typename S, bool WALLS, bool FORCED>
+__global__ void __launch_bounds__(STEP_THREADS, STEP_MIN_CTAS<S>) k_step(const __grid_constant__ StepArgs<S> T) {
+    extern __shared__ int pre[];   // prefix of the run counts (boundary CTAs)
+    if ((int)blockIdx.x < T.bblocks) {
+        boundary_cells<S, FORCED>(T, pre);
+        return;
+    }
+    const unsigned item = (blockIdx.x - (unsigned)T.bblocks) * (unsigned)T.per_cta + threadIdx.x;
+    if ((int)threadIdx.x >= T.per_cta || item >= T.items) return;
+    bulk_cells<S, WALLS, FORCED>(T, item);
+}
+
+template <bool WALLS, bool MRT>
+__global__ void __launch_bounds__(STEP_THREADS, 3) k_step_h2(const __grid_constant__ StepArgs<__half> T) {
+    extern __shared__ int pre[];
+    if ((int)blockIdx.x < T.bblocks) {
+        boundary_cells<__half, false>(T, pre);
+        return;
+    }
+    if ((int)threadIdx.x >= T.per_cta) return;   // whole warps
+    const unsigned item = (blockIdx.x - (unsigned)T.bblocks) * (unsigned)T.per_cta + threadIdx.x;
+    bulk_pairs<WALLS, MRT>(T, item, item < T.items);
 }
 
 // ------------------------------------------------------------------ remap
@@ -251,37 +372,30 @@ __global__ void k_flags_full(uint8_t* __restrict__ flags, GridDesc G, const Part
     flags[c] = (ps->present && inside_ball(i, j, k, G, *ps)) ? 1 : 0;
 }
 
-__global__ void k_flags_box(uint8_t* __restrict__ flags_next, GridDesc G, BoxDesc B,
-                            const ParticleState* __restrict__ ps) {
-    __shared__ BoxFrame F;
+// Both copies of the frames of the current record, after the host changed it (128 threads).
+__global__ void k_frames(const ParticleState* __restrict__ ps, PFrames* __restrict__ frames, GridDesc G, BoxDesc B) {
     const int n3[3] = {G.nx, G.ny, G.nz};
-    if (threadIdx.x == 0) box_frame_init(F, n3, G.periodic, B, *ps);
-    __syncthreads();
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B.cells) return;
-    int p[3];
-    if (!box_cell(t, n3, G.periodic, B, F, p)) return;
-    const size_t c = (size_t)p[0] + (size_t)G.nx * ((size_t)p[1] + (size_t)G.ny * (size_t)p[2]);
-    flags_next[c] = ball_flag(p, n3, G.periodic, F, *ps) ? 1 : 0;
+    pframes_form(frames, *ps, n3, G.periodic, B);
+    pframes_form(frames + 1, *ps, n3, G.periodic, B);
 }
 
 // Refill of the uncovered cell (i, j, k) = index c by the whole warp
 // (Sec. 2.3): lane q = 1..18 takes the neighbour (i, j, k) + c_q (wrapped on
 // periodic axes; none beyond a wall), counted when it is fluid before (fcur)
-// and after (fnext) the move, with its density 1 + sum_p g_p and momentum
-// sum_p c_p g_p (for Grad's strain rate from the face neighbours).  The mean
-// density and the rigid-body velocity u_p + omega_p x (x - x_p) give the
-// equilibrium, plus Grad's term when gcoef != 0; lane q < 19 writes
+// and after (the ball predicate) the move, with its density 1 + sum_p g_p and
+// momentum sum_p c_p g_p (for Grad's strain rate from the face neighbours).
+// The mean density and the rigid-body velocity u_p + omega_p x (x - x_p) give
+// the equilibrium, plus Grad's term when gcoef != 0; lane q < 19 writes
 // population q.  Every lane calls it with the same cell.
 template <typename S>
-__device__ __forceinline__ void refill_warp(S* __restrict__ pops, const uint8_t* __restrict__ fcur,
-                                            const uint8_t* __restrict__ fnext, const GridDesc& G, const int n3[3],
-                                            const ParticleState& P, int i, int j, int k, size_t c,
-                                            typename Store<S>::A scale, typename Store<S>::A inv_scale,
+__device__ __forceinline__ void refill_warp(S* __restrict__ pops, const uint8_t* __restrict__ fcur, const GridDesc& G,
+                                            const int n3[3], const BoxFrame& F, const ParticleState& P, int i, int j,
+                                            int k, typename Store<S>::A scale, typename Store<S>::A inv_scale,
                                             typename Store<S>::A gcoef) {
     using A = typename Store<S>::A;
     const int lane = threadIdx.x & 31;
     const size_t n = (size_t)G.n;
+    const size_t c = (size_t)i + (size_t)G.nx * ((size_t)j + (size_t)G.ny * (size_t)k);
     bool ok = false;
     A r = A(0), mo[3] = {A(0), A(0), A(0)};
     if (lane >= 1 && lane < 19) {
@@ -294,22 +408,21 @@ __device__ __forceinline__ void refill_warp(S* __restrict__ pops, const uint8_t*
                 v[a] = (v[a] + n3[a]) % n3[a];
             }
         }
-        if (in) {
+        if (in && !ball_flag(v, n3, G.periodic, F, P)) {
             const size_t y = (size_t)v[0] + (size_t)G.nx * ((size_t)v[1] + (size_t)G.ny * (size_t)v[2]);
-            if (fcur[y] == 0 && fnext[y] == 0) {
-                ok = true;
-                A gp[19];
+            // the populations are loaded beside the flag (not after it): a solid neighbour's are dropped
+            A gp[19];
 #pragma unroll
-                for (int q = 0; q < 19; ++q) gp[q] = Store<S>::load(pops + (size_t)q * n + y, inv_scale);
-                r = A(1);
+            for (int q = 0; q < 19; ++q) gp[q] = Store<S>::load(pops + (size_t)q * n + y, inv_scale);
+            ok = fcur[y] == 0;
+            r = A(1);
 #pragma unroll
-                for (int q = 0; q < 19; ++q) r += gp[q];
+            for (int q = 0; q < 19; ++q) r += gp[q];
 #pragma unroll
-                for (int q = 1; q < 19; ++q) {
-                    mo[0] += A(cx(q)) * gp[q];
-                    mo[1] += A(cy(q)) * gp[q];
-                    mo[2] += A(cz(q)) * gp[q];
-                }
+            for (int q = 1; q < 19; ++q) {
+                if (cx(q)) mo[0] += cx(q) > 0 ? gp[q] : -gp[q];
+                if (cy(q)) mo[1] += cy(q) > 0 ? gp[q] : -gp[q];
+                if (cz(q)) mo[2] += cz(q) > 0 ? gp[q] : -gp[q];
             }
         }
     }
@@ -344,110 +457,101 @@ __device__ __forceinline__ void refill_warp(S* __restrict__ pops, const uint8_t*
     }
 }
 
-// Cells now solid are zeroed; cells the sphere uncovered are refilled
-// afterwards, one at a time by their whole warp (refill_warp).  blockDim.x
-// is a multiple of 32.
+// Remap of Sec. 2.3 after the particle moved, one pass over the box: the new flag of every box cell (the exact
+// ball predicate) and its mark; newly covered cells drop their populations (the step stores the cells that were
+// solid before as zero); uncovered cells are listed in shared memory and refilled afterwards, each by one warp
+// of the block in turn (refill_warp reads only cells that are fluid before and after the move, which nothing
+// here writes).  Neighbour flags are evaluated from the same predicate instead of being read back, so flags,
+// refill and boundary marks (four launches of 4 to 6 us before) take one pass.  mark_only: only marks and counts
+// (flags and populations already belong to the current position).
+constexpr int REMAP_THREADS = 256;
 template <typename S>
-__global__ void k_refill(S* __restrict__ pops, const uint8_t* __restrict__ fcur, const uint8_t* __restrict__ fnext,
-                         GridDesc G, BoxDesc B, const ParticleState* __restrict__ ps,
-                         typename Store<S>::A scale, typename Store<S>::A inv_scale, typename Store<S>::A gcoef) {
+__global__ void __launch_bounds__(REMAP_THREADS)
+    k_remap(S* __restrict__ pops, const uint8_t* __restrict__ fcur, uint8_t* __restrict__ fnext, GridDesc G, BoxDesc B,
+            const ParticleState* __restrict__ ps, const PFrames* __restrict__ frames, typename Store<S>::A scale,
+            typename Store<S>::A inv_scale, typename Store<S>::A gcoef, uint8_t* __restrict__ mark,
+            int* __restrict__ run_count, int mark_only) {
     using A = typename Store<S>::A;
     __shared__ BoxFrame F;
+    __shared__ int s_n;
+    __shared__ int s_g[3][REMAP_THREADS];   // uncovered cells
+    __shared__ int wsum[REMAP_THREADS / 32];
     const int n3[3] = {G.nx, G.ny, G.nz};
-    if (threadIdx.x == 0) box_frame_init(F, n3, G.periodic, B, *ps);
+    if (threadIdx.x == 0) {
+        F = frames->bf;
+        s_n = 0;
+    }
     __syncthreads();
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const ParticleState& P = *ps;
     const size_t n = (size_t)G.n;
-    bool uncovered = false;
-    int p[3] = {0, 0, 0};
-    if (t < B.cells && box_cell(t, n3, G.periodic, B, F, p)) {
-        const size_t c = (size_t)p[0] + (size_t)G.nx * ((size_t)p[1] + (size_t)G.ny * (size_t)p[2]);
-        if (fnext[c] != 0) {
-#pragma unroll
-            for (int q = 0; q < 19; ++q) Store<S>::store(pops + (size_t)q * n + c, A(0), scale);
-        } else {
-            uncovered = fcur[c] != 0;
-        }
-    }
-    for (unsigned todo = __ballot_sync(0xffffffffu, uncovered); todo != 0u; todo &= todo - 1u) {
-        const int src = __ffs((int)todo) - 1;
-        const int i = __shfl_sync(0xffffffffu, p[0], src), j = __shfl_sync(0xffffffffu, p[1], src),
-                  k = __shfl_sync(0xffffffffu, p[2], src);
-        const size_t c = (size_t)i + (size_t)G.nx * ((size_t)j + (size_t)G.ny * (size_t)k);
-        refill_warp<S>(pops, fcur, fnext, G, n3, *ps, i, j, k, c, scale, inv_scale, gcoef);
-    }
-}
-
-// Ordered compaction of the fluid cells with a solid neighbour inside the
-// box, in two passes over the box: k_links_mark flags each box cell and
-// counts per block; k_links_emit gives every block its offset (sum of the
-// counts of the blocks before it) and writes its cells in traversal order.
-// The order is the box traversal order, identical in every run.
-constexpr int LINK_THREADS = 256;
-
-__device__ __forceinline__ int wrap_idx(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
-
-__global__ void __launch_bounds__(LINK_THREADS)
-    k_links_mark(const uint8_t* __restrict__ flags, GridDesc G, BoxDesc B, const ParticleState* __restrict__ ps,
-                 uint8_t* __restrict__ mask, int* __restrict__ block_count) {
-    __shared__ BoxFrame F;
-    const int n3[3] = {G.nx, G.ny, G.nz};
-    if (threadIdx.x == 0) box_frame_init(F, n3, G.periodic, B, *ps);
-    __syncthreads();
-    const int t = blockIdx.x * LINK_THREADS + threadIdx.x;
+    const int t = blockIdx.x * REMAP_THREADS + threadIdx.x;
     int is_b = 0;
     if (t < B.cells) {
+        uint8_t m = MARK_PLAIN;
         int p[3];
         if (box_cell(t, n3, G.periodic, B, F, p)) {
-            const int i = p[0], j = p[1], k = p[2];
-            const int nx = G.nx, ny = G.ny;
-            const int c = i + nx * (j + ny * k);
-            if (flags[c] == 0) {
+            const size_t c = (size_t)p[0] + (size_t)G.nx * ((size_t)p[1] + (size_t)G.ny * (size_t)p[2]);
+            const bool was_solid = fcur[c] != 0;
+            bool any_nb = false;
+            const bool solid = ball_flag_and_neighbours(p, n3, G.periodic, F, P, &any_nb);
+            is_b = (!solid && any_nb) ? 1 : 0;
+            m = solid ? MARK_SOLID : (is_b ? MARK_BOUNDARY : MARK_PLAIN);
+            if (!mark_only) {
+                fnext[c] = solid ? 1 : 0;
+                if (solid && !was_solid) {
 #pragma unroll
-                for (int q = 1; q < 19; ++q) {
-                    const int a = i + cx(q), b = j + cy(q), d = k + cz(q);
-                    if ((!G.periodic[0] && (a < 0 || a >= nx)) || (!G.periodic[1] && (b < 0 || b >= ny)) ||
-                        (!G.periodic[2] && (d < 0 || d >= G.nz)))
-                        continue;
-                    const int y = wrap_idx(a, nx) + nx * (wrap_idx(b, ny) + ny * wrap_idx(d, G.nz));
-                    is_b |= flags[y] != 0;
+                    for (int q = 0; q < 19; ++q) Store<S>::store(pops + (size_t)q * n + c, A(0), scale);
+                } else if (!solid && was_solid) {
+                    const int k = atomicAdd(&s_n, 1);
+                    s_g[0][k] = p[0];
+                    s_g[1][k] = p[1];
+                    s_g[2][k] = p[2];
                 }
             }
         }
-        mask[t] = (uint8_t)is_b;
+        mark[t] = m;
     }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned ballot = __ballot_sync(0xffffffffu, is_b);
-    __shared__ int wsum[LINK_THREADS / 32];
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = __popc(ballot);
+    if (lane == 0) wsum[wid] = __popc(ballot);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int s = 0;
-        for (int w = 0; w < LINK_THREADS / 32; ++w) s += wsum[w];
-        block_count[blockIdx.x] = s;
+    constexpr int RUNS = REMAP_THREADS / LINK_RUN, WPR = LINK_RUN / 32;
+    if ((int)threadIdx.x < RUNS) {
+        const long long run = (long long)blockIdx.x * RUNS + threadIdx.x;
+        if (run * LINK_RUN < B.cells) {
+            int s = 0;
+#pragma unroll
+            for (int w = 0; w < WPR; ++w) s += wsum[threadIdx.x * WPR + w];
+            run_count[run] = s;
+        }
     }
+    for (int k = wid; k < s_n; k += REMAP_THREADS / 32)
+        refill_warp<S>(pops, fcur, G, n3, F, P, s_g[0][k], s_g[1][k], s_g[2][k], scale, inv_scale, gcoef);
 }
 
-__global__ void __launch_bounds__(LINK_THREADS)
-    k_links_emit(const uint8_t* __restrict__ mask, const int* __restrict__ block_count, GridDesc G, BoxDesc B,
-                 const ParticleState* __restrict__ ps, int* __restrict__ list, int* __restrict__ count, int capacity,
+// The marked cells as a list in box order (linear cell indices): every block takes 256 box cells and adds up the
+// runs before them.  Read back for inspection, and by the step itself for boxes too large for a prefix of the run
+// counts in shared memory (MARK_CELLS_MAX).
+constexpr int EMIT_THREADS = 256;
+__global__ void __launch_bounds__(EMIT_THREADS)
+    k_links_emit(const uint8_t* __restrict__ mark, const int* __restrict__ run_count, GridDesc G, BoxDesc B,
+                 const PFrames* __restrict__ frames, int* __restrict__ list, int* __restrict__ count, int capacity,
                  int* __restrict__ status) {
-    __shared__ int red[LINK_THREADS];
-    __shared__ int wsum[LINK_THREADS / 32];
-    __shared__ BoxFrame F;
+    __shared__ int red[EMIT_THREADS];
+    __shared__ int wsum[EMIT_THREADS / 32];
     const int n3[3] = {G.nx, G.ny, G.nz};
-    if (threadIdx.x == 0) box_frame_init(F, n3, G.periodic, B, *ps);
-    // offset of this block: sum of the counts of all earlier blocks
+    const int before = (int)blockIdx.x * (EMIT_THREADS / LINK_RUN);
     int s = 0;
-    for (int b = threadIdx.x; b < (int)blockIdx.x; b += LINK_THREADS) s += block_count[b];
+    for (int b = threadIdx.x; b < before; b += EMIT_THREADS) s += run_count[b];
     red[threadIdx.x] = s;
     __syncthreads();
-    for (int h = LINK_THREADS / 2; h > 0; h >>= 1) {
+    for (int h = EMIT_THREADS / 2; h > 0; h >>= 1) {
         if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
         __syncthreads();
     }
     const int base = red[0];
-    const int t = blockIdx.x * LINK_THREADS + threadIdx.x;
-    const int is_b = (t < B.cells) ? mask[t] : 0;
+    const int t = blockIdx.x * EMIT_THREADS + threadIdx.x;
+    const int is_b = t < B.cells && mark[t] == MARK_BOUNDARY;
     const unsigned ballot = __ballot_sync(0xffffffffu, is_b);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lane == 0) wsum[warp] = __popc(ballot);
@@ -456,14 +560,14 @@ __global__ void __launch_bounds__(LINK_THREADS)
     for (int w = 0; w < warp; ++w) wbase += wsum[w];
     if (is_b) {
         int p[3];
-        const bool in = box_cell(t, n3, G.periodic, B, F, p);
+        const bool in = box_cell(t, n3, G.periodic, B, frames->bf, p);
         const int pos = base + wbase + __popc(ballot & ((1u << lane) - 1u));
         if (pos >= capacity) atomicOr(status, STATUS_LINK_OVERFLOW);
         else if (in) list[pos] = p[0] + G.nx * (p[1] + G.ny * p[2]);
     }
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
         int tot = base;
-        for (int w = 0; w < LINK_THREADS / 32; ++w) tot += wsum[w];
+        for (int w = 0; w < EMIT_THREADS / 32; ++w) tot += wsum[w];
         *count = tot < capacity ? tot : capacity;
     }
 }
@@ -565,79 +669,96 @@ inline unsigned blocks_for(long long n, int t) { return (unsigned)((n + t - 1) /
 }  // namespace
 
 // ------------------------------------------------------------- launchers
+// One coupled step (StepArgs); without a sphere only its bulk part.
 template <typename S>
-void launch_bulk(const S* src, S* dst, const GridDesc& g, const CollideParams<typename Store<S>::A>& p,
-                 int* status, cudaStream_t stream) {
-    int bx = 32;
-    while (bx < g.nx && bx < 128) bx *= 2;
-    const int by = BULK_THREADS / bx;
-    dim3 block(bx, by, 1);
-    dim3 grid((g.nx + bx - 1) / bx, (g.ny + by - 1) / by, g.nz);
+void launch_step(const lbmp_handle* h, const S* src, S* dst, const CollideParams<typename Store<S>::A>& p, int finish,
+                 double* force_out, cudaStream_t stream) {
+    const GridDesc& g = h->G;
+    StepArgs<S> T;
+    T.src = src;
+    T.dst = dst;
+    T.G = g;
+    T.P = p;
+    T.status = h->status;
+    T.bblocks = 0;
+    T.finish = finish;
+    T.cli = h->cfg.boundary == LBMP_CLI ? 1 : 0;
+    T.hist_cap = h->cfg.history_capacity;
+    T.flags = h->flags[h->fcur];
+    T.mark = h->link_mask;
+    T.run_count = h->link_blocks;
+    T.list = nullptr;
+    T.count = h->count;
+    T.B = h->box;
+    T.ps = h->d_ps;
+    T.partials = h->partials;
+    T.done = h->d_done;
+    T.history = h->history;
+    T.frames = h->frames + h->frame_cur;
+    T.frames_next = h->frames + (1 - h->frame_cur);
+    T.force_out = force_out;
+    size_t smem = 0;
+    if (h->has_particle) {
+        T.bblocks = step_boundary_blocks(h->box, h->list_cap);
+        if (step_uses_list(h->box)) T.list = h->list;
+        else smem = sizeof(int) * (size_t)((h->box.cells + LINK_RUN - 1) / LINK_RUN + 1);
+    }
     const bool walls = !(g.periodic[0] && g.periodic[1] && g.periodic[2]);
-    if constexpr (std::is_same<S, __half>::value) {   // FP16, unforced, whole pairs: two cells per thread
-        if (!p.forced && g.nx % 2 == 0) {
-            const int pairs = g.nx / 2;
-            int px = 32;
-            while (px < pairs && px < 128) px *= 2;
-            dim3 b2(px, BULK2_THREADS / px, 1);
-            dim3 g2((pairs + px - 1) / px, (g.ny + b2.y - 1) / b2.y, g.nz);
+    const bool pairs = std::is_same<S, __half>::value && !p.forced && g.nx % 2 == 0;   // FP16: two cells per thread
+    T.dx.set((unsigned)(pairs ? g.nx / 2 : g.nx));
+    T.dy.set((unsigned)g.ny);
+    T.items = (unsigned)(pairs ? g.n / 2 : g.n);
+    // Small grids are spread over the SMs: CTAs of fewer cells until there are two per SM (FP64 in particular is
+    // bound by each scheduler's own FP64 rate, so idle SMs cost in proportion).
+    T.per_cta = STEP_THREADS;
+    while (T.per_cta > 32 && T.items / (unsigned)T.per_cta < 2 * 152) T.per_cta /= 2;
+    const unsigned grid = (unsigned)T.bblocks + (T.items + (unsigned)T.per_cta - 1) / (unsigned)T.per_cta;
+    if constexpr (std::is_same<S, __half>::value) {
+        if (pairs) {
             const bool mrt = p.db != 0.0f;
-            if (walls && mrt) k_bulk_h2<true, true><<<g2, b2, 0, stream>>>(src, dst, g, p, status);
-            else if (walls) k_bulk_h2<true, false><<<g2, b2, 0, stream>>>(src, dst, g, p, status);
-            else if (mrt) k_bulk_h2<false, true><<<g2, b2, 0, stream>>>(src, dst, g, p, status);
-            else k_bulk_h2<false, false><<<g2, b2, 0, stream>>>(src, dst, g, p, status);
+            if (walls && mrt) k_step_h2<true, true><<<grid, STEP_THREADS, smem, stream>>>(T);
+            else if (walls) k_step_h2<true, false><<<grid, STEP_THREADS, smem, stream>>>(T);
+            else if (mrt) k_step_h2<false, true><<<grid, STEP_THREADS, smem, stream>>>(T);
+            else k_step_h2<false, false><<<grid, STEP_THREADS, smem, stream>>>(T);
             return;
         }
     }
     if (walls) {
-        if (p.forced) k_bulk<S, true, true><<<grid, block, 0, stream>>>(src, dst, g, p, status);
-        else k_bulk<S, true, false><<<grid, block, 0, stream>>>(src, dst, g, p, status);
+        if (p.forced) k_step<S, true, true><<<grid, STEP_THREADS, smem, stream>>>(T);
+        else k_step<S, true, false><<<grid, STEP_THREADS, smem, stream>>>(T);
     } else {
-        if (p.forced) k_bulk<S, false, true><<<grid, block, 0, stream>>>(src, dst, g, p, status);
-        else k_bulk<S, false, false><<<grid, block, 0, stream>>>(src, dst, g, p, status);
+        if (p.forced) k_step<S, false, true><<<grid, STEP_THREADS, smem, stream>>>(T);
+        else k_step<S, false, false><<<grid, STEP_THREADS, smem, stream>>>(T);
     }
-}
-
-template <typename S>
-void launch_boundary(const S* src, S* dst, const uint8_t* flags, const int* list, const int* count, int max_cells,
-                     const GridDesc& g, const CollideParams<typename Store<S>::A>& p, const ParticleState* ps,
-                     int cli, double* partials, int* nblocks_out, int* status, cudaStream_t stream) {
-    const int nb = boundary_grid(max_cells);
-    *nblocks_out = nb;
-    if (p.forced)
-        k_boundary<S, true><<<nb, BNDW_THREADS, 0, stream>>>(src, dst, flags, list, count, g, p, ps, cli, partials, status);
-    else
-        k_boundary<S, false><<<nb, BNDW_THREADS, 0, stream>>>(src, dst, flags, list, count, g, p, ps, cli, partials, status);
-}
-
-void launch_particle_update(ParticleState* ps, const double* partials, int nblocks, const GridDesc& g,
-                            double* history, int hist_cap, int* status, cudaStream_t stream) {
-    k_particle<<<1, PART_THREADS, 0, stream>>>(ps, partials, nblocks, g, history, hist_cap, status);
 }
 
 void launch_flags_full(uint8_t* flags, const GridDesc& g, const ParticleState* ps, cudaStream_t stream) {
     k_flags_full<<<blocks_for(g.n, 256), 256, 0, stream>>>(flags, g, ps);
 }
 
-void launch_flags_box(uint8_t* flags_next, const GridDesc& g, const BoxDesc& b, const ParticleState* ps,
-                      cudaStream_t stream) {
-    k_flags_box<<<blocks_for(b.cells, 256), 256, 0, stream>>>(flags_next, g, b, ps);
+size_t frames_bytes() { return 2 * sizeof(PFrames); }
+
+void launch_frames(const lbmp_handle* h, cudaStream_t stream) {
+    k_frames<<<1, 128, 0, stream>>>(h->d_ps, h->frames, h->G, h->box);
 }
 
+// Remap to the position of frames[frame] (fcur -> fnext); mark_only for the marks alone.  Large boxes: also the list.
 template <typename S>
-void launch_refill(S* pops, const uint8_t* flags_cur, const uint8_t* flags_next, const GridDesc& g,
-                   const BoxDesc& b, const ParticleState* ps, typename Store<S>::A scale,
-                   typename Store<S>::A inv_scale, typename Store<S>::A gcoef, cudaStream_t stream) {
-    k_refill<S><<<blocks_for(b.cells, 128), 128, 0, stream>>>(pops, flags_cur, flags_next, g, b, ps, scale,
-                                                               inv_scale, gcoef);
+int launch_remap(const lbmp_handle* h, S* pops, const uint8_t* fcur, uint8_t* fnext, int frame, bool mark_only,
+                 typename Store<S>::A scale, typename Store<S>::A inv_scale, typename Store<S>::A gcoef,
+                 cudaStream_t stream) {
+    const PFrames* F = h->frames + frame;
+    k_remap<S><<<blocks_for(h->box.cells, REMAP_THREADS), REMAP_THREADS, 0, stream>>>(
+        pops, fcur, fnext, h->G, h->box, h->d_ps, F, scale, inv_scale, gcoef, h->link_mask, h->link_blocks,
+        mark_only ? 1 : 0);
+    if (!step_uses_list(h->box)) return 1;
+    launch_links_emit(h, frame, stream);
+    return 2;
 }
 
-void launch_build_links(const uint8_t* flags, const GridDesc& g, const BoxDesc& b, const ParticleState* ps,
-                        uint8_t* mask, int* block_count, int* list, int* count, int capacity, int* status,
-                        cudaStream_t stream) {
-    const unsigned nb = blocks_for(b.cells, LINK_THREADS);
-    k_links_mark<<<nb, LINK_THREADS, 0, stream>>>(flags, g, b, ps, mask, block_count);
-    k_links_emit<<<nb, LINK_THREADS, 0, stream>>>(mask, block_count, g, b, ps, list, count, capacity, status);
+void launch_links_emit(const lbmp_handle* h, int frame, cudaStream_t stream) {
+    k_links_emit<<<blocks_for(h->box.cells, EMIT_THREADS), EMIT_THREADS, 0, stream>>>(
+        h->link_mask, h->link_blocks, h->G, h->box, h->frames + frame, h->list, h->count, h->list_cap, h->status);
 }
 
 void launch_export_links(const uint8_t* flags, const int* list, const int* count, int max_cells, const GridDesc& g,
@@ -677,13 +798,10 @@ void launch_zero_solid(S* pops, const uint8_t* flags, const GridDesc& g, cudaStr
 }
 
 #define LBMP_INSTANTIATE(S)                                                                                        \
-    template void launch_bulk<S>(const S*, S*, const GridDesc&, const CollideParams<Store<S>::A>&, int*,           \
+    template void launch_step<S>(const lbmp_handle*, const S*, S*, const CollideParams<Store<S>::A>&, int, double*, \
                                  cudaStream_t);                                                                    \
-    template void launch_boundary<S>(const S*, S*, const uint8_t*, const int*, const int*, int, const GridDesc&,   \
-                                     const CollideParams<Store<S>::A>&, const ParticleState*, int, double*, int*,  \
-                                     int*, cudaStream_t);                                                          \
-    template void launch_refill<S>(S*, const uint8_t*, const uint8_t*, const GridDesc&, const BoxDesc&,            \
-                                   const ParticleState*, Store<S>::A, Store<S>::A, Store<S>::A, cudaStream_t);     \
+    template int launch_remap<S>(const lbmp_handle*, S*, const uint8_t*, uint8_t*, int, bool, Store<S>::A,         \
+                                 Store<S>::A, Store<S>::A, cudaStream_t);                                          \
     template void launch_init_equilibrium<S>(S*, const uint8_t*, const GridDesc&, double, const double*,           \
                                              const double*, Store<S>::A, cudaStream_t);                            \
     template void launch_to_f64<S>(const S*, double*, long long, Store<S>::A, cudaStream_t);                       \

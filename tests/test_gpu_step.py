@@ -1,0 +1,33 @@
+"""The coupled uniform step at the edges of its launch: boundary cells found from the marks' run counts (boxes of up to
+131,072 cells) and from the list (larger ones), boxes that span a periodic axis or exceed a walled one, grids of a few
+cells, rows that begin inside a warp.  Tolerances of test_gpu_uniform.py: FP64 1e-10, FP16 5e-3 of max|g|."""
+import numpy as np
+import pytest
+
+from test_gpu_uniform import assert_links_equal, assert_pops_close, lib, make_pair  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+P, N = "periodic", "noslip"
+
+
+@pytest.mark.parametrize("precision,shape,d,bc,steps", [
+    ("fp64", (53, 52, 51), 41.0, (P, P, P), 6),     # 50^3 box cells, 1,954 runs: the largest prefixes
+    ("fp64", (56, 58, 57), 46.0, (P, P, P), 6),     # 54^3 box cells: the list
+    ("fp64", (9, 9, 9), 5.0, (P, P, P), 40),        # the box spans every axis
+    ("fp64", (7, 40, 9), 3.0, (N, P, N), 40),       # the box exceeds two walled axes
+    ("fp64", (8, 8, 257), 4.0, (P, N, P), 40),
+    ("fp16", (22, 9, 11), 5.0, (P, N, P), 60),      # pairs of several rows in one warp
+    ("fp16", (10, 13, 9), 5.0, (N, P, P), 60),
+    ("fp16", (56, 57, 54), 46.0, (P, P, P), 6),
+])
+def test_step_edges(orc, lib, precision, shape, d, bc, steps):  # noqa: F811
+    pos = np.array(shape, dtype=float) / 2 + np.array([0.23, -0.31, 0.17])
+    u = np.array([0.03, -0.04, 0.05]) * (0.2 if min(shape) < 10 else 1.0)
+    o, g = make_pair(orc, lib, shape, precision=precision, tau=0.7, bc=bc, sphere=(pos, d, 0.6, 0.5),
+                     gravity=(0, 0, -2e-5), velocity=(u, (0.001, -0.002, 0.0005)))
+    o.step(steps)
+    g.step(steps)
+    assert_pops_close(o, g, 1e-10 if precision == "fp64" else 5e-3)
+    if precision == "fp64":
+        assert np.array_equal(o.flags(), g.flags())
+        assert_links_equal(o, g)
