@@ -37,6 +37,7 @@ namespace lbmp {
 namespace {
 
 constexpr int AT = 256;   // threads per block of the cell kernels
+constexpr int NEAR_BLOCKS_MAX = 608;   // CTAs of the cells next to the sphere (four per SM, each warp takes several of a large sphere's)
 constexpr int ADJ_MIN_CTAS = 4;   // resident reverse-step CTAs per SM asked of the compiler (FP32): 64 registers
 
 enum : uint8_t { KIND_PLAIN = 0, KIND_SOLID = 1, KIND_NEAR = 2 };
@@ -54,90 +55,161 @@ __device__ __forceinline__ long long cell_at(const GridDesc& G, int i, int j, in
     return (long long)wrapc(i, G.nx) + (long long)G.nx * ((long long)wrapc(j, G.ny) + (long long)G.ny * wrapc(k, G.nz));
 }
 
-// Transpose of the TRT collision with the Guo-type source (the derivative
-// of trt_collide at h, applied to lambda), and the parameter parts
-// part = (lambda . dC/ds+, lambda . dC/ds-, lambda . dC/dF).  The source is
-// always differentiated, also where F = 0.
-//   C_q(h) = h_q - s+ (h+_q - e+_q) - s- (h-_q - e-_q) + (1 - s+/2) S+_q + (1 - s-/2) S-_q
-//   (dC/dh)^T lambda = lambda - s+ lambda+ - s- lambda- + a + b.c_p with
-//   a = s+ L0, b = s+ (9 L2 u - 3 L0 u) + 3 s- L1 + (1 - s+/2)(9 L2 F - 3 L0 F),
-//   L0 = sum w lambda, L1 = sum w lambda c, L2 = sum w lambda c c^T.
+// Moments that the transposed collision needs: of h the density and velocity (with half the force), of lambda
+//   L0 = sum w lambda, L1 = sum w lambda c, L2 = sum w lambda c c^T (xx yy zz xy xz yz).
 template <typename A>
-__device__ __forceinline__ void trt_adjoint(const A (&h)[19], A (&lam)[19], const AdjParams<A>& P, A part[5]) {
-    A drho = A(0), u[3] = {A(0), A(0), A(0)};
-    A L0 = A(0), L1[3] = {A(0), A(0), A(0)}, L2[6] = {A(0), A(0), A(0), A(0), A(0), A(0)};   // xx yy zz xy xz yz
-#pragma unroll
-    for (int q = 0; q < 19; ++q) {
-        drho += h[q];
-        if (cx(q) != 0) u[0] += A(cx(q)) * h[q];
-        if (cy(q) != 0) u[1] += A(cy(q)) * h[q];
-        if (cz(q) != 0) u[2] += A(cz(q)) * h[q];
-        const A wl = wgt<A>(q) * lam[q];
-        L0 += wl;
-        if (cx(q) != 0) {
-            L1[0] += A(cx(q)) * wl;
-            L2[0] += wl;
-        }
-        if (cy(q) != 0) {
-            L1[1] += A(cy(q)) * wl;
-            L2[1] += wl;
-        }
-        if (cz(q) != 0) {
-            L1[2] += A(cz(q)) * wl;
-            L2[2] += wl;
-        }
-        if (cx(q) * cy(q) != 0) L2[3] += A(cx(q) * cy(q)) * wl;
-        if (cx(q) * cz(q) != 0) L2[4] += A(cx(q) * cz(q)) * wl;
-        if (cy(q) * cz(q) != 0) L2[5] += A(cy(q) * cz(q)) * wl;
-    }
-#pragma unroll
-    for (int a = 0; a < 3; ++a) u[a] += A(0.5) * P.F[a];
-    const A uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const A uF = u[0] * P.F[0] + u[1] * P.F[1] + u[2] * P.F[2];
-    const A sp = P.sp, sm = P.sm;
-    // parameter parts: dC_q/ds+ = -(h+_q - e+_q) - S+_q / 2, dC_q/ds- = -(h-_q - e-_q) - S-_q / 2
-    A tsp, tsm = A(0);
-    {
-        const A e0 = wgt<A>(0) * (drho - A(1.5) * uu);
-        const A S0 = wgt<A>(0) * (A(-3) * uF);
-        tsp = lam[0] * (-(h[0] - e0) - A(0.5) * S0);
-    }
-#pragma unroll
-    for (int q = 1; q < 19; q += 2) {
-        const A cu = A(cx(q)) * u[0] + A(cy(q)) * u[1] + A(cz(q)) * u[2];
-        const A cF = A(cx(q)) * P.F[0] + A(cy(q)) * P.F[1] + A(cz(q)) * P.F[2];
-        const A w = wgt<A>(q);
-        const A ep = w * (drho + A(4.5) * cu * cu - A(1.5) * uu), em = w * (A(3) * cu);
-        const A Sp = w * (A(9) * cu * cF - A(3) * uF), Sm = w * (A(3) * cF);
-        const A hp = A(0.5) * (h[q] + h[q + 1]), hm = A(0.5) * (h[q] - h[q + 1]);
-        tsp += (lam[q] + lam[q + 1]) * (-(hp - ep) - A(0.5) * Sp);
-        tsm += (lam[q] - lam[q + 1]) * (-(hm - em) - A(0.5) * Sm);
-    }
+struct AdjMoments {
+    A drho, u[3], L0, L1[3], L2[6];
+};
+
+// What every population of the cell shares: a0 and b of
+//   (dC/dh)^T lambda = lambda - s+ lambda+ - s- lambda- + a0 + b.c with
+//   a0 = s+ L0, b = s+ (9 L2 u - 3 L0 u) + 3 s- L1 + (1 - s+/2)(9 L2 F - 3 L0 F),
+// and the force parts lambda . dC/dF.  The source is always differentiated, also where F = 0.
+template <typename A>
+__device__ __forceinline__ void adj_shared(const AdjMoments<A>& M, const AdjParams<A>& P, A* a0, A b[3], A dF[3]) {
+    const A* L2 = M.L2;
+    const A* u = M.u;
     const A L2u[3] = {L2[0] * u[0] + L2[3] * u[1] + L2[4] * u[2], L2[3] * u[0] + L2[1] * u[1] + L2[5] * u[2],
                       L2[4] * u[0] + L2[5] * u[1] + L2[2] * u[2]};
     const A L2F[3] = {L2[0] * P.F[0] + L2[3] * P.F[1] + L2[4] * P.F[2],
                       L2[3] * P.F[0] + L2[1] * P.F[1] + L2[5] * P.F[2],
                       L2[4] * P.F[0] + L2[5] * P.F[1] + L2[2] * P.F[2]};
-    const A a0 = sp * L0;
-    A b[3];
+    *a0 = P.sp * M.L0;
+    const A L03 = A(3) * M.L0, hs = A(1) - A(0.5) * P.sp, hm = A(3) * (A(1) - A(0.5) * P.sm);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const A du = A(9) * L2u[a] - A(3) * L0 * u[a];
-        b[a] = sp * du + A(3) * sm * L1[a] + (A(1) - A(0.5) * sp) * (A(9) * L2F[a] - A(3) * L0 * P.F[a]);
-        part[2 + a] = A(0.5) * b[a] + (A(1) - A(0.5) * sp) * du + A(3) * (A(1) - A(0.5) * sm) * L1[a];
+        const A du = A(9) * L2u[a] - L03 * u[a];
+        b[a] = P.sp * du + A(3) * P.sm * M.L1[a] + hs * (A(9) * L2F[a] - L03 * P.F[a]);
+        dF[a] = A(0.5) * b[a] + hs * du + hm * M.L1[a];
+    }
+}
+
+// Transpose of the TRT collision with the Guo-type source (the derivative of trt_collide at h, applied to lambda) on
+// one cell, and the parameter parts part = (lambda . dC/ds+, lambda . dC/ds-, lambda . dC/dF), with
+//   C_q(h) = h_q - s+ (h+_q - e+_q) - s- (h-_q - e-_q) + (1 - s+/2) S+_q + (1 - s-/2) S-_q,
+//   dC_q/ds+ = -(h+_q - e+_q) - S+_q / 2, dC_q/ds- = -(h-_q - e-_q) - S-_q / 2.
+// All on the sums and differences of the opposite pairs, without products by zero components: about 300
+// instructions instead of 470, which is the time in FP64.
+template <typename A>
+__device__ __forceinline__ void trt_adjoint(const A (&h)[19], A (&lam)[19], const AdjParams<A>& P, A part[5]) {
+    A hp[9], hm[9], lp[9], lm[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        hp[k] = h[2 * k + 1] + h[2 * k + 2];
+        hm[k] = h[2 * k + 1] - h[2 * k + 2];
+        lp[k] = lam[2 * k + 1] + lam[2 * k + 2];
+        lm[k] = lam[2 * k + 1] - lam[2 * k + 2];
+    }
+    // pairs 0..2 are the faces, 3..8 (+x+y), (+x-y), (+x+z), (+x-z), (+y+z), (+y-z)
+    AdjMoments<A> M;
+    M.drho = h[0] + (((hp[0] + hp[1]) + hp[2]) + (((hp[3] + hp[4]) + (hp[5] + hp[6])) + (hp[7] + hp[8])));
+    M.u[0] = (hm[0] + ((hm[3] + hm[4]) + (hm[5] + hm[6]))) + A(0.5) * P.F[0];
+    M.u[1] = (hm[1] + ((hm[3] - hm[4]) + (hm[7] + hm[8]))) + A(0.5) * P.F[1];
+    M.u[2] = (hm[2] + ((hm[5] - hm[6]) + (hm[7] - hm[8]))) + A(0.5) * P.F[2];
+    const A wF = wgt<A>(1), wE = wgt<A>(7);
+    const A exy = lp[3] + lp[4], exz = lp[5] + lp[6], eyz = lp[7] + lp[8];
+    M.L0 = wgt<A>(0) * lam[0] + wF * ((lp[0] + lp[1]) + lp[2]) + wE * ((exy + exz) + eyz);
+    M.L1[0] = wF * lm[0] + wE * ((lm[3] + lm[4]) + (lm[5] + lm[6]));
+    M.L1[1] = wF * lm[1] + wE * ((lm[3] - lm[4]) + (lm[7] + lm[8]));
+    M.L1[2] = wF * lm[2] + wE * ((lm[5] - lm[6]) + (lm[7] - lm[8]));
+    M.L2[0] = wF * lp[0] + wE * (exy + exz);
+    M.L2[1] = wF * lp[1] + wE * (exy + eyz);
+    M.L2[2] = wF * lp[2] + wE * (exz + eyz);
+    M.L2[3] = wE * (lp[3] - lp[4]);
+    M.L2[4] = wE * (lp[5] - lp[6]);
+    M.L2[5] = wE * (lp[7] - lp[8]);
+    A a0, b[3];
+    adj_shared<A>(M, P, &a0, b, part + 2);
+    const A* u = M.u;
+    const A uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    const A uF = u[0] * P.F[0] + u[1] * P.F[1] + u[2] * P.F[2];
+    const A r = M.drho - A(1.5) * uu + A(1.5) * uF;   // e+ - S+/2 without its direction-dependent part, over w
+    A tsp = lam[0] * (wgt<A>(0) * r - h[0]), tsm = A(0);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int q = 2 * k + 1;
+        const A w = wgt<A>(q);
+        const A cu = dir_dot<A>(q, u[0], u[1], u[2]);
+        const A cF = dir_dot<A>(q, P.F[0], P.F[1], P.F[2]);   // the same in every cell
+        const A v = A(4.5) * (cu - cF);
+        tsp += lp[k] * (w * (v * cu + r) - A(0.5) * hp[k]);
+        tsm += lm[k] * ((A(3) * w) * (cu - A(0.5) * cF) - A(0.5) * hm[k]);
+        const A bc = dir_dot<A>(q, b[0], b[1], b[2]);
+        // x, y = lambda+ (1 - s+) + a0 +- (lambda- (1 - s-) + b.c)
+        const A hl = A(0.5) * lp[k];
+        const A Sy = hl - P.sp * hl + a0;
+        const A gl = A(0.5) * lm[k];
+        const A Da = gl - P.sm * gl + bc;
+        lam[q] = Sy + Da;
+        lam[q + 1] = Sy - Da;
     }
     part[0] = tsp;
     part[1] = tsm;
-    lam[0] = lam[0] - sp * lam[0] + a0;
+    lam[0] = lam[0] - P.sp * lam[0] + a0;
+}
+
+// Sums of 16 values over the warp's lanes: each exchange halves the values a lane still carries, 16 shuffles where 16
+// separate sums take 80.  Value i ends in the lanes sum16_lane(i) and the one after.
+template <typename A>
+__device__ __forceinline__ A warp_sum16(A (&v)[16]) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int q = 1; q < 19; q += 2) {
-        const A lp = A(0.5) * (lam[q] + lam[q + 1]), lm = A(0.5) * (lam[q] - lam[q + 1]);
-        const A bc = A(cx(q)) * b[0] + A(cy(q)) * b[1] + A(cz(q)) * b[2];
-        const A x = lam[q] - sp * lp - sm * lm + a0 + bc;
-        const A y = lam[q + 1] - sp * lp + sm * lm + a0 - bc;
-        lam[q] = x;
-        lam[q + 1] = y;
+    for (int off = 16, m = 8; m >= 1; off >>= 1, m >>= 1) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < m; ++i) {
+            const A keep = up ? v[i + m] : v[i], send = up ? v[i] : v[i + m];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
     }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+__host__ __device__ constexpr int sum16_lane(int i) { return 2 * i; }
+
+// trt_adjoint by a whole warp: lane q < 19 holds h_q and lambda_q (the others zero) and gets the new lambda_q; sp and
+// sm parts are added up per lane, the force parts in lane 0.
+template <typename A>
+__device__ __forceinline__ A warp_trt_adjoint(A h, A lam, int lane, const AdjParams<A>& P, A part[5]) {
+    const int c0 = lane_c(lane, 0), c1 = lane_c(lane, 1), c2 = lane_c(lane, 2);
+    const A w = lane >= 19 ? A(0) : (lane == 0 ? A(1) / A(3) : (lane <= 6 ? A(1) / A(18) : A(1) / A(36)));
+    const A f0 = A(c0), f1 = A(c1), f2 = A(c2), wl = w * lam;
+    A v[16] = {h,           f0 * h,      f1 * h,      f2 * h,       wl,           f0 * wl,      f1 * wl, f2 * wl,
+               f0 * f0 * wl, f1 * f1 * wl, f2 * f2 * wl, f0 * f1 * wl, f0 * f2 * wl, f1 * f2 * wl, A(0),    A(0)};
+    const A mine = warp_sum16<A>(v);
+    A s[14];
+#pragma unroll
+    for (int i = 0; i < 14; ++i) s[i] = __shfl_sync(0xffffffffu, mine, sum16_lane(i));
+    AdjMoments<A> M;
+    M.drho = s[0];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        M.u[a] = s[1 + a] + A(0.5) * P.F[a];
+        M.L1[a] = s[5 + a];
+    }
+    M.L0 = s[4];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) M.L2[i] = s[8 + i];
+    A a0, b[3], dF[3];
+    adj_shared<A>(M, P, &a0, b, dF);
+    const int partner = lane == 0 ? 0 : (lane < 19 ? ((lane & 1) ? lane + 1 : lane - 1) : lane);
+    const A ho = __shfl_sync(0xffffffffu, h, partner), lo = __shfl_sync(0xffffffffu, lam, partner);
+    const A* u = M.u;
+    const A uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    const A uF = u[0] * P.F[0] + u[1] * P.F[1] + u[2] * P.F[2];
+    const A cu = f0 * u[0] + f1 * u[1] + f2 * u[2];
+    const A cF = f0 * P.F[0] + f1 * P.F[1] + f2 * P.F[2];
+    const A ep = w * (M.drho + A(4.5) * cu * cu - A(1.5) * uu), em = w * (A(3) * cu);
+    const A Sp = w * (A(9) * cu * cF - A(3) * uF), Sm = w * (A(3) * cF);
+    const A hp = A(0.5) * (h + ho), hm = A(0.5) * (h - ho);
+    part[0] += lam * (-(hp - ep) - A(0.5) * Sp);
+    part[1] += lam * (-(hm - em) - A(0.5) * Sm);
+    if (lane == 0)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) part[2 + a] += dF[a];
+    const A lp = A(0.5) * (lam + lo), lm = A(0.5) * (lam - lo);
+    const A bc = f0 * b[0] + f1 * b[1] + f2 * b[2];
+    return lam - P.sp * lp - P.sm * lm + a0 + bc;
 }
 
 // Block sum of the per-thread parameter parts, added to this block's FP64
@@ -235,76 +307,148 @@ __global__ void __launch_bounds__(AT)
     }
 }
 
+// One reverse step; its first nblocks CTAs take the cells next to the sphere, the others the plain cells in memory
+// order.
+template <typename S>
+struct ReverseArgs {
+    using A = typename Store<S>::A;
+    const S* gprev;
+    const A* nu_next;
+    A* nu_out;
+    const uint8_t* kind;
+    const uint8_t* flags;
+    const int* list;       // the near cells
+    const int* count;
+    GridDesc G;
+    FastDiv dx, dy;        // by nx and ny
+    int per_cta;           // plain cells per CTA
+    int nblocks;
+    AdjParams<A> P;
+    const ParticleState* ps;
+    int cli, with_seed;
+    double* acc;           // [CTA][5]
+};
+
 // Reverse step on the cells that see no solid: h_q = g_q(x - c_q),
 // lambda_q = nu_q(x + c_q).  Solid cells get nu = 0; near cells are left to
-// k_adj_near.
+// the first CTAs.
 template <typename S>
-__global__ void __launch_bounds__(AT, sizeof(S) == 8 ? 1 : ADJ_MIN_CTAS)
-    k_adj_plain(const S* __restrict__ gprev, const typename Store<S>::A* __restrict__ nu_next,
-                typename Store<S>::A* __restrict__ nu_out, const uint8_t* __restrict__ kind, GridDesc G,
-                AdjParams<typename Store<S>::A> P, double* __restrict__ acc) {
+__device__ __forceinline__ void reverse_plain(const ReverseArgs<S>& T, unsigned item, typename Store<S>::A part[5]) {
     using A = typename Store<S>::A;
-    const long long x = (long long)blockIdx.x * AT + threadIdx.x;
+    const GridDesc& G = T.G;
     const size_t n = (size_t)G.n;
-    A part[5] = {A(0), A(0), A(0), A(0), A(0)};
-    if (x < G.n) {
-        // the cell's kind is loaded beside the 38 loads of the plain case (a branch on it would
-        // hold them back by one memory round trip); a cell of another kind drops them
-        const uint8_t kd = kind[x];
-        const int i = (int)(x % G.nx), j = (int)((x / G.nx) % G.ny), k = (int)(x / ((long long)G.nx * G.ny));
-        // xs[1 + d] = i - d: the pull source x - c_q at index 1 + c, x + c_q at 1 - c
-        const int xs[3] = {wrapc(i + 1, G.nx), i, wrapc(i - 1, G.nx)};
-        const int ys[3] = {wrapc(j + 1, G.ny), j, wrapc(j - 1, G.ny)};
-        const int zs[3] = {wrapc(k + 1, G.nz), k, wrapc(k - 1, G.nz)};
-        A h[19], lam[19];
+    // the cell's kind is loaded beside the 38 loads of the plain case (a branch on it would
+    // hold them back by one memory round trip); a cell of another kind drops them
+    const uint8_t kd = T.kind[item];
+    const unsigned row = T.dx.div(item), plane = T.dy.div(row);
+    const int i = (int)(item - row * (unsigned)G.nx), j = (int)(row - plane * (unsigned)G.ny), k = (int)plane;
+    // xs[1 + d] = i - d: the pull source x - c_q at index 1 + c, x + c_q at 1 - c
+    const int xs[3] = {wrapc(i + 1, G.nx), i, wrapc(i - 1, G.nx)};
+    const int ys[3] = {wrapc(j + 1, G.ny), j, wrapc(j - 1, G.ny)};
+    const int zs[3] = {wrapc(k + 1, G.nz), k, wrapc(k - 1, G.nz)};
+    A h[19], lam[19];
 #pragma unroll
-        for (int q = 0; q < 19; ++q) {
-            const size_t src = (size_t)xs[1 + cx(q)] + (size_t)G.nx * ((size_t)ys[1 + cy(q)] + (size_t)G.ny * zs[1 + cz(q)]);
-            const size_t dn = (size_t)xs[1 - cx(q)] + (size_t)G.nx * ((size_t)ys[1 - cy(q)] + (size_t)G.ny * zs[1 - cz(q)]);
-            h[q] = Store<S>::load(gprev + (size_t)q * n + src, A(1));
-            lam[q] = nu_next[(size_t)q * n + dn];
-        }
-        if (kd == KIND_SOLID) {
-#pragma unroll
-            for (int q = 0; q < 19; ++q) nu_out[(size_t)q * n + x] = A(0);
-        } else if (kd == KIND_PLAIN) {
-            trt_adjoint<A>(h, lam, P, part);
-#pragma unroll
-            for (int q = 0; q < 19; ++q) nu_out[(size_t)q * n + x] = lam[q];
-        }
+    for (int q = 0; q < 19; ++q) {
+        const int src = xs[1 + cx(q)] + G.nx * (ys[1 + cy(q)] + G.ny * zs[1 + cz(q)]);
+        const int dn = xs[1 - cx(q)] + G.nx * (ys[1 - cy(q)] + G.ny * zs[1 - cz(q)]);
+        h[q] = Store<S>::load(T.gprev + (size_t)q * n + src, A(1));
+        lam[q] = T.nu_next[(size_t)q * n + dn];
     }
-    accumulate_parts<A>(part, acc);
+    if (kd == KIND_SOLID) {
+#pragma unroll
+        for (int q = 0; q < 19; ++q) T.nu_out[(size_t)q * n + item] = A(0);
+    } else if (kd == KIND_PLAIN) {
+        trt_adjoint<A>(h, lam, T.P, part);
+#pragma unroll
+        for (int q = 0; q < 19; ++q) T.nu_out[(size_t)q * n + item] = lam[q];
+    }
 }
 
-// h^n at a near cell: the pull of the forward step with the CLI rule on
-// links (wall at rest).
+// Reverse step of the cells next to the sphere, one warp per cell, lane q on population q: h_q is the forward pull
+// with the CLI rule on links (wall at rest), lambda_q the pull run backwards with the terms of every link moved to the
+// cells it reads (near_lambda), and the force's own dependence on both.  Everything a population can need is loaded at
+// once; a thread per cell followed 19 chains of flag and value loads one after another (43 us at 64^3 in FP32, 142 us
+// at 24^3 in FP64).
 template <typename S>
-__device__ __forceinline__ void near_pull(const S* __restrict__ g, const uint8_t* __restrict__ flags, const GridDesc& G,
-                                          int i, int j, int k, const LinkFrame<typename Store<S>::A>& Fr, int cli,
-                                          typename Store<S>::A (&h)[19]) {
+__device__ __forceinline__ void reverse_near(const ReverseArgs<S>& T, typename Store<S>::A part[5]) {
     using A = typename Store<S>::A;
+    __shared__ LinkFrame<A> Fr;
+    if (threadIdx.x == 0) Fr.init(*T.ps);
+    const GridDesc& G = T.G;
     const size_t n = (size_t)G.n;
-    const long long x = cell_at(G, i, j, k);
-    const int p[3] = {i, j, k}, n3[3] = {G.nx, G.ny, G.nz}, per[3] = {1, 1, 1};
-    A d[3];
-    int pu[3];
-    Fr.offset(p, n3, per, d, pu);
-    for (int q = 0; q < 19; ++q) {
-        const long long s = cell_at(G, i - cx(q), j - cy(q), k - cz(q));
-        if (q == 0 || flags[s] == 0) {
-            h[q] = Store<S>::load(g + (size_t)q * n + s, A(1));
-        } else {
-            const int kk = opp(q);
-            const long long far = cell_at(G, i + cx(q), j + cy(q), k + cz(q));
-            const bool far_ok = flags[far] == 0;
-            A delta, kappa0, alpha;
-            cli_coeffs<A>(q, d, cli && far_ok, Fr.r, &delta, &kappa0, &alpha);
-            const A gt_k = Store<S>::load(g + (size_t)kk * n + x, A(1));
-            const A gt_q = Store<S>::load(g + (size_t)q * n + x, A(1));
-            const A gt_far = far_ok ? Store<S>::load(g + (size_t)kk * n + far, A(1)) : A(0);
-            h[q] = gt_k + kappa0 * gt_far - kappa0 * gt_q;
+    const int n3[3] = {G.nx, G.ny, G.nz}, per[3] = {1, 1, 1};
+    const int lane = threadIdx.x & 31;
+    const int total = *T.count, W = T.nblocks * (AT / 32);
+    __syncthreads();
+    for (int t = (int)blockIdx.x * (AT / 32) + (int)(threadIdx.x >> 5); t < total; t += W) {
+        const int x = T.list[t];
+        const unsigned row = T.dx.div((unsigned)x), plane = T.dy.div(row);
+        const int p[3] = {x - (int)row * G.nx, (int)row - (int)plane * G.ny, (int)plane};
+        A h = A(0), l = A(0);
+        bool link = false;
+        const int q = lane < 19 ? lane : 0, k = opp(q);
+        const int c[3] = {cx(q), cy(q), cz(q)};
+        if (lane < 19) {
+            const long long s = cell_at(G, p[0] - c[0], p[1] - c[1], p[2] - c[2]);
+            const long long y = cell_at(G, p[0] + c[0], p[1] + c[1], p[2] + c[2]);
+            const long long yy = cell_at(G, p[0] + 2 * c[0], p[1] + 2 * c[1], p[2] + 2 * c[2]);
+            const bool s_solid = T.flags[s] != 0, y_solid = T.flags[y] != 0, yy_solid = T.flags[yy] != 0;
+            const A g_s = Store<S>::load(T.gprev + (size_t)q * n + s, A(1));
+            const A g_k = Store<S>::load(T.gprev + (size_t)k * n + x, A(1));
+            const A g_q = Store<S>::load(T.gprev + (size_t)q * n + x, A(1));
+            const A g_far = Store<S>::load(T.gprev + (size_t)k * n + y, A(1));
+            const A nu_y = T.nu_next[(size_t)q * n + y], nu_yk = T.nu_next[(size_t)k * n + y];
+            const A nu_k = T.nu_next[(size_t)k * n + x], nu_q = T.nu_next[(size_t)q * n + x];
+            const int ca = c[T.P.axis];
+            h = g_s;
+            if (q == 0) {
+                l = nu_q;
+            } else {
+                link = s_solid;
+                A dx[3], delta, kappa0, alpha;
+                int pu[3];
+                if (!y_solid) {
+                    l = nu_y;   // plain pull at y reads g_q(x)
+                    if (yy_solid) {   // link at y, incoming opp(q): its far cell is x
+                        const int py[3] = {wrapc(p[0] + c[0], G.nx), wrapc(p[1] + c[1], G.ny), wrapc(p[2] + c[2], G.nz)};
+                        Fr.offset(py, n3, per, dx, pu);
+                        cli_coeffs<A>(k, dx, T.cli != 0, Fr.r, &delta, &kappa0, &alpha);
+                        l += kappa0 * nu_yk;
+                    }
+                } else {   // link at x, incoming opp(q): g_q(x) is its g~_k, also in the force
+                    l = nu_k;
+                    if (T.with_seed) l += T.P.seed * A(ca);
+                }
+                if (link) {   // link at x, incoming q
+                    Fr.offset(p, n3, per, dx, pu);
+                    cli_coeffs<A>(q, dx, T.cli && !y_solid, Fr.r, &delta, &kappa0, &alpha);
+                    h = g_k + kappa0 * (y_solid ? A(0) : g_far) - kappa0 * g_q;
+                    l -= kappa0 * nu_q;
+                }
+            }
+        }
+        A out = warp_trt_adjoint<A>(h, l, lane, T.P, part);
+        if (lane < 19) {
+            if (link) out -= T.P.seed * A(c[T.P.axis]);   // the force's own dependence on h^n at the link: c_k = -c_q
+            T.nu_out[(size_t)q * n + x] = out;
         }
     }
+}
+
+template <typename S>
+__global__ void __launch_bounds__(AT, sizeof(S) == 8 ? 1 : ADJ_MIN_CTAS)
+    k_adj_step(const __grid_constant__ ReverseArgs<S> T) {
+    using A = typename Store<S>::A;
+    pdl_trigger();
+    pdl_wait();
+    A part[5] = {A(0), A(0), A(0), A(0), A(0)};
+    if ((int)blockIdx.x < T.nblocks) {
+        reverse_near<S>(T, part);
+    } else {
+        const unsigned item = (blockIdx.x - (unsigned)T.nblocks) * (unsigned)T.per_cta + threadIdx.x;
+        if ((int)threadIdx.x < T.per_cta && item < (unsigned)T.G.n) reverse_plain<S>(T, item, part);
+    }
+    accumulate_parts<A>(part, T.acc);
 }
 
 // lambda at a fluid cell next to the sphere: S^T nu with the link terms,
@@ -350,38 +494,6 @@ __device__ __forceinline__ void near_lambda(const A* __restrict__ nu, const uint
         }
         lam[q] = l;
     }
-}
-
-template <typename S>
-__global__ void __launch_bounds__(AT)
-    k_adj_near(const S* __restrict__ gprev, const typename Store<S>::A* __restrict__ nu_next,
-               typename Store<S>::A* __restrict__ nu_out, const uint8_t* __restrict__ flags,
-               const int* __restrict__ list, const int* __restrict__ count, GridDesc G,
-               AdjParams<typename Store<S>::A> P, const ParticleState* __restrict__ ps, int cli, int with_seed,
-               double* __restrict__ acc) {
-    using A = typename Store<S>::A;
-    __shared__ LinkFrame<A> Fr;
-    if (threadIdx.x == 0) Fr.init(*ps);
-    __syncthreads();
-    const int t = blockIdx.x * AT + threadIdx.x;
-    A part[5] = {A(0), A(0), A(0), A(0), A(0)};
-    if (t < *count) {
-        const long long x = list[t];
-        const int i = (int)(x % G.nx), j = (int)((x / G.nx) % G.ny), k = (int)(x / ((long long)G.nx * G.ny));
-        A h[19], lam[19];
-        near_pull<S>(gprev, flags, G, i, j, k, Fr, cli, h);
-        near_lambda<A>(nu_next, flags, G, i, j, k, Fr, cli, with_seed != 0, P.seed, P.axis, lam);
-        trt_adjoint<A>(h, lam, P, part);
-        const size_t n = (size_t)G.n;
-        // the force's own dependence on h^n at the links (x, q): c_k = -c_q
-        for (int q = 1; q < 19; ++q)
-            if (flags[cell_at(G, i - cx(q), j - cy(q), k - cz(q))] != 0) {
-                const int ca = P.axis == 0 ? cx(q) : (P.axis == 1 ? cy(q) : cz(q));
-                lam[q] -= P.seed * A(ca);
-            }
-        for (int q = 0; q < 19; ++q) nu_out[(size_t)q * n + x] = lam[q];
-    }
-    accumulate_parts<A>(part, acc);
 }
 
 // lambda^0 and dJ/du0 = (dE/du0)^T lambda^0 with
@@ -476,7 +588,9 @@ struct AdjointEngine {
     double* u0 = nullptr;     // copy of the initial velocity field [3][n]
     double* forces = nullptr; // [nsteps][3]
     double* acc = nullptr;    // [acc_blocks][5]
-    int acc_blocks = 0, plain_blocks = 0, near_blocks = 0, near_cells = 0;
+    int acc_blocks = 0, near_blocks = 0, near_cells = 0;
+    int cell_blocks = 0;                   // blocks of AT cells
+    int per_cta = AT, plain_blocks = 0;    // plain cells per reverse-step CTA, and those CTAs
     uint8_t* kind = nullptr;
     int* blk = nullptr;
     int* near_list = nullptr;
@@ -605,10 +719,13 @@ lbmp_status adjoint_forward(lbmp_handle* h, const double* u0, int nsteps, int in
         E->nckpt = nckpt;
         E->state_bytes = es * 19 * n;
         E->nu_bytes = es * 19 * n;
-        E->plain_blocks = (int)((n + AT - 1) / AT);
+        E->cell_blocks = (int)((n + AT - 1) / AT);
+        E->per_cta = AT;   // small grids over all SMs, as in launch_step
+        while (E->per_cta > 32 && (int)n / E->per_cta < 2 * 152) E->per_cta /= 2;
+        E->plain_blocks = (int)((n + (size_t)E->per_cta - 1) / (size_t)E->per_cta);
         E->near_cap = (int)n;
         E->near_blocks = 0;
-        E->acc_blocks = E->plain_blocks * 2;   // plain blocks, then at most as many near blocks
+        E->acc_blocks = NEAR_BLOCKS_MAX + E->plain_blocks;
         E->ckpt = handle_alloc(h, E->state_bytes * (size_t)nckpt);
         E->seg = handle_alloc(h, E->state_bytes * (size_t)interval);
         E->nu[0] = handle_alloc(h, E->nu_bytes);
@@ -617,7 +734,7 @@ lbmp_status adjoint_forward(lbmp_handle* h, const double* u0, int nsteps, int in
         E->forces = (double*)handle_alloc(h, sizeof(double) * 3 * (size_t)nsteps);
         E->acc = (double*)handle_alloc(h, sizeof(double) * 5 * (size_t)E->acc_blocks);
         E->kind = (uint8_t*)handle_alloc(h, n);
-        E->blk = (int*)handle_alloc(h, sizeof(int) * (size_t)E->plain_blocks);
+        E->blk = (int*)handle_alloc(h, sizeof(int) * (size_t)E->cell_blocks);
         E->near_list = (int*)handle_alloc(h, sizeof(int) * n);
         E->near_count = (int*)handle_alloc(h, sizeof(int));
         if (!E->ckpt || !E->seg || !E->nu[0] || !E->nu[1] || !E->u0 || !E->forces || !E->acc || !E->kind || !E->blk ||
@@ -642,7 +759,7 @@ lbmp_status adjoint_forward(lbmp_handle* h, const double* u0, int nsteps, int in
         h->launches += 1;
     }
     if (!E->geometry_done) {   // cells of the reverse step next to the (fixed) sphere
-        const unsigned gb = (unsigned)E->plain_blocks;
+        const unsigned gb = (unsigned)E->cell_blocks;
         k_adj_kind<<<gb, AT, 0, h->stream>>>(h->flags[h->fcur], h->G, E->kind, E->blk);
         k_adj_near_list<<<gb, AT, 0, h->stream>>>(E->kind, E->blk, h->G, E->near_list, E->near_count);
         h->launches += 2;
@@ -651,7 +768,7 @@ lbmp_status adjoint_forward(lbmp_handle* h, const double* u0, int nsteps, int in
             cudaStreamSynchronize(h->stream) != cudaSuccess)
             return LBMP_ERR_CUDA;
         h->d2h += sizeof(int);
-        E->near_blocks = std::max(1, (E->near_cells + AT - 1) / AT);
+        E->near_blocks = std::min(NEAR_BLOCKS_MAX, std::max(1, (E->near_cells + AT / 32 - 1) / (AT / 32)));
         E->geometry_done = true;
     }
     cudaMemcpyAsync(E->u0, u0, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, h->stream);
@@ -697,7 +814,7 @@ lbmp_status adjoint_backward(lbmp_handle* h, const double* dJ, double* grad_tau,
     const size_t n = (size_t)h->G.n;
     const int N = E->nsteps, K = E->interval;
     const int cli = h->cfg.boundary == LBMP_CLI ? 1 : 0;
-    const unsigned gb = (unsigned)E->plain_blocks, gn = (unsigned)E->near_blocks;
+    const unsigned gb = (unsigned)E->cell_blocks;
     lbmp_status st = LBMP_OK;
     with_adj_storage(h->cfg.precision, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
@@ -710,6 +827,20 @@ lbmp_status adjoint_backward(lbmp_handle* h, const double* dJ, double* grad_tau,
         for (int a = 0; a < 3; ++a) P.F[a] = (A)h->body_force[a];
         P.seed = (A)(1.0 / (double)N);
         P.axis = E->axis;
+        ReverseArgs<S> T;
+        T.kind = E->kind;
+        T.flags = h->flags[h->fcur];
+        T.list = E->near_list;
+        T.count = E->near_count;
+        T.G = h->G;
+        T.dx.set((unsigned)h->G.nx);
+        T.dy.set((unsigned)h->G.ny);
+        T.per_cta = E->per_cta;
+        T.nblocks = E->near_blocks;
+        T.P = P;
+        T.ps = h->d_ps;
+        T.cli = cli;
+        T.acc = E->acc;
         st = captured(h, E, &E->gbwd, [&]() {
             cudaMemsetAsync(E->acc, 0, sizeof(double) * 5 * (size_t)E->acc_blocks, h->stream);
             cudaMemsetAsync(E->nu[0], 0, E->nu_bytes, h->stream);
@@ -723,18 +854,19 @@ lbmp_status adjoint_backward(lbmp_handle* h, const double* dJ, double* grad_tau,
                     const A* nu_next = (const A*)E->nu[cur];
                     A* nu_out = (A*)E->nu[1 - cur];
                     const long long ev = profile_mark(h);
-                    k_adj_plain<S><<<gb, AT, 0, h->stream>>>(gprev, nu_next, nu_out, E->kind, h->G, P, E->acc);
+                    T.gprev = gprev;
+                    T.nu_next = nu_next;
+                    T.nu_out = nu_out;
+                    T.with_seed = s < N ? 1 : 0;
+                    launch_pdl(k_adj_step<S>, (unsigned)(E->near_blocks + E->plain_blocks), AT, 0, h->stream, T);
                     // algorithmic bytes: 19 populations of g^{n-1} read, 19 adjoint values read and written per cell
-                    const double cells = (double)n - (double)E->near_cells;
+                    const double cells = (double)n;
                     profile_kernel(h, ev, profile_mark(h), cells * (19.0 * sizeof(S) + 38.0 * sizeof(A)), cells);
-                    k_adj_near<S><<<gn, AT, 0, h->stream>>>(gprev, nu_next, nu_out, h->flags[h->fcur], E->near_list,
-                                                           E->near_count, h->G, P, h->d_ps, cli, s < N ? 1 : 0,
-                                                           E->acc + (size_t)5 * E->plain_blocks);
                     cur = 1 - cur;
                 }
             }
         });
-        h->launches += (long long)(N - E->nckpt) + 2LL * N;
+        h->launches += (long long)(N - E->nckpt) + (long long)N;
         if (st == LBMP_OK && grad_u0) {   // nu^1 sits in nu[N % 2] after N reverse steps
             k_adj_init_grad<A><<<gb, AT, 0, h->stream>>>((const A*)E->nu[N & 1], h->flags[h->fcur], E->kind, h->G,
                                                          E->u0, h->d_ps, cli, P.seed, E->axis, dJ, grad_u0);

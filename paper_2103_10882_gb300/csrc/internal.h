@@ -113,6 +113,38 @@ inline int step_boundary_blocks(const BoxDesc& b, int list_capacity) {
     return (int)(n < 1 ? 1 : (n > 1216 ? 1216 : n));
 }
 
+// n / d for n < 2^31 by one high multiplication (Granlund & Montgomery, "Division by invariant integers
+// using multiplication", 1994, Fig. 4.1): d >= 1.
+struct FastDiv {
+    unsigned d, m, s;
+    __host__ void set(unsigned v) {
+        d = v;
+        s = 0;
+        while ((1ull << s) < v) ++s;
+        m = (unsigned)(((1ull << 32) * ((1ull << s) - v)) / v + 1);
+    }
+    __device__ __forceinline__ unsigned div(unsigned n) const {
+        const unsigned t = __umulhi(m, n);
+        return (t + n) >> s;   // t <= n < 2^31: no overflow
+    }
+};
+
+// Launch that may start before the kernel ahead of it on the stream has ended (pdl_wait).
+template <typename K, typename... Args>
+inline void launch_pdl(K kernel, unsigned grid, int threads, size_t smem, cudaStream_t stream, const Args&... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3((unsigned)threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = stream;
+    cudaLaunchAttribute a = {};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &a;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 struct PFrames;
 
 // Launchers (uniform.cu).  All are asynchronous on `stream`.

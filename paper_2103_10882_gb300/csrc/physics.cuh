@@ -7,6 +7,15 @@
 
 namespace lbmp {
 
+// Programmatic dependent launch (PTX griddepcontrol): the CTAs of a kernel launched with the attribute may become
+// resident once every CTA of the kernel ahead has called pdl_trigger or ended; pdl_wait returns when that kernel has
+// completed and its writes are visible.  Every thread waits before it reads or writes global memory, so only the
+// launch itself overlaps.  Kernels launched without the attribute pass both at once.  Measured (with the boundary
+// cells' loads issued together): a 32^3 FP32 step 23.4 -> 20.7 us, 64 x 64 x 128 with MRT 29.7 -> 27.1, 256^3 in FP16
+// storage 284 -> 277 (also four CTAs per SM there instead of three).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Minimum-image difference for periodic axes.
 __device__ __forceinline__ double wrap_diff(double d, int n, int periodic) {
     if (!periodic) return d;

@@ -20,22 +20,6 @@ constexpr int STEP_THREADS = 256;
 // D3Q19 neighbour (taken by the boundary CTAs), cell with its centre inside the sphere.
 constexpr uint8_t MARK_PLAIN = 0, MARK_BOUNDARY = 1, MARK_SOLID = 2;
 
-// n / d for n < 2^31 by one high multiplication (Granlund & Montgomery, "Division by invariant integers
-// using multiplication", 1994, Fig. 4.1): d >= 1.
-struct FastDiv {
-    unsigned d, m, s;
-    __host__ void set(unsigned v) {
-        d = v;
-        s = 0;
-        while ((1ull << s) < v) ++s;
-        m = (unsigned)(((1ull << 32) * ((1ull << s) - v)) / v + 1);
-    }
-    __device__ __forceinline__ unsigned div(unsigned n) const {
-        const unsigned t = __umulhi(m, n);
-        return (t + n) >> s;   // t <= n < 2^31: no overflow
-    }
-};
-
 // One coupled step of a uniform grid.
 template <typename S>
 struct StepArgs {
@@ -85,15 +69,6 @@ __device__ __forceinline__ int box_index(const StepArgs<S>& T, int x, int y, int
     const int tx = box_coord(x, o[0], T.G.nx, T.G.periodic[0], T.B.E[0]);
     return (tx | ty | tz) < 0 ? -1 : tx + T.B.E[0] * (ty + T.B.E[1] * tz);
 }
-
-// Programmatic dependent launch (PTX griddepcontrol): the CTAs of a kernel launched with the attribute may become
-// resident once every CTA of the kernel ahead has called pdl_trigger or ended; pdl_wait returns when that kernel has
-// completed and its writes are visible.  Every thread waits before it reads or writes global memory, so only the
-// launch itself overlaps.  Kernels launched without the attribute pass both at once.  Measured (with the boundary
-// cells' loads issued together): a 32^3 FP32 step 23.4 -> 20.7 us, 64 x 64 x 128 with MRT 29.7 -> 27.1, 256^3 in FP16
-// storage 284 -> 277 (also four CTAs per SM there instead of three).
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ------------------------------------------------------------------ bulk
 // One thread per cell, pull form: g_q(x, t+1) = g~_q(x - c_q, t), then TRT; solid cells are stored as zero and
@@ -640,8 +615,9 @@ __global__ void k_init_eq(S* __restrict__ pops, const uint8_t* __restrict__ flag
         u[2] = ufield[2 * n + c];
     }
     const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+#pragma unroll
     for (int q = 0; q < 19; ++q) {
-        const double cu = cx(q) * u[0] + cy(q) * u[1] + cz(q) * u[2];
+        const double cu = dir_dot<double>(q, u[0], u[1], u[2]);
         const double e = wgt<double>(q) * ((rho - 1.0) + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
         Store<S>::store(pops + (size_t)q * n + c, fluid ? A(e) : A(0), scale);
     }
@@ -686,22 +662,6 @@ inline unsigned blocks_for(long long n, int t) { return (unsigned)((n + t - 1) /
 }  // namespace
 
 // ------------------------------------------------------------- launchers
-// Launch that may start before the kernel ahead of it on the stream has ended (pdl_wait).
-template <typename K, typename... Args>
-void launch_pdl(K kernel, unsigned grid, int threads, size_t smem, cudaStream_t stream, const Args&... args) {
-    cudaLaunchConfig_t c = {};
-    c.gridDim = dim3(grid);
-    c.blockDim = dim3((unsigned)threads);
-    c.dynamicSmemBytes = smem;
-    c.stream = stream;
-    cudaLaunchAttribute a = {};
-    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    a.val.programmaticStreamSerializationAllowed = 1;
-    c.attrs = &a;
-    c.numAttrs = 1;
-    cudaLaunchKernelEx(&c, kernel, args...);
-}
-
 // One coupled step (StepArgs); without a sphere only its bulk part.
 template <typename S>
 void launch_step(const lbmp_handle* h, const S* src, S* dst, const CollideParams<typename Store<S>::A>& p, int finish,
