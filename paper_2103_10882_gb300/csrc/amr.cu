@@ -432,9 +432,8 @@ __global__ void __maxnreg__(BND_MAXREG<S>)
     }
     block_link_sums<BNDW_THREADS>(acc, ps->x, partials + (size_t)blockIdx.x * 6);
     if (last_block_done(done, (int)gridDim.x)) {   // every other block is past its use of the frames
-        particle_block_update<BNDW_THREADS>(ps, partials, gridDim.x, G, history, hist_cap, status, frames->inv);
-        __syncthreads();
-        if (threadIdx.x < 3) pframes_axis(frames, *ps, D.n, B, threadIdx.x);   // of the moved sphere
+        particle_block_update<BNDW_THREADS>(ps, partials, gridDim.x, G, history, hist_cap, status, frames->inv,
+                                            [&](const ParticleState& Q, int a) { pframes_axis(frames, Q, D.n, B, a); });
     }
 }
 

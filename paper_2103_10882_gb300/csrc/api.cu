@@ -393,13 +393,15 @@ lbmp_status lbmp_add_sphere(lbmp_handle* h, const double pos[3], double diameter
     const double shell = 4.0 / 3.0 * M_PI * (ro * ro * ro - ri * ri * ri);
     h->list_cap = (int)std::min<double>((double)B.cells, std::ceil(shell) + 64.0);
     h->list = (int*)dev_alloc(h, sizeof(int) * (size_t)h->list_cap);
-    const int max_blocks = step_boundary_blocks(B, h->list_cap);
+    const int max_blocks = step_boundary_blocks(h->list_cap);
     h->partials = (double*)dev_alloc(h, sizeof(double) * 6 * (size_t)max_blocks);
     h->link_mask = (uint8_t*)dev_alloc(h, (size_t)B.cells);
-    h->link_blocks = (int*)dev_alloc(h, sizeof(int) * (size_t)((B.cells + 63) / 64));
+    const size_t nseg = (size_t)((B.cells + 255) / 256);
+    h->seg = (int*)dev_alloc(h, sizeof(int) * 256 * nseg);
+    h->seg_count = (int*)dev_alloc(h, sizeof(int) * nseg);
     h->frames = (PFrames*)dev_alloc(h, frames_bytes());
     h->d_done = (int*)dev_alloc(h, sizeof(int));
-    if (!h->list || !h->partials || !h->link_mask || !h->link_blocks || !h->frames || !h->d_done)
+    if (!h->list || !h->partials || !h->link_mask || !h->seg || !h->seg_count || !h->frames || !h->d_done)
         return fail(h, LBMP_ERR_OOM, "lbmp_add_sphere: device allocation failed");
     lbmp_status s = upload_particle(h);
     if (s != LBMP_OK) return s;
@@ -745,7 +747,7 @@ lbmp_status lbmp_get_links(lbmp_handle* h, int64_t* cell, int32_t* q, double* de
     }
     if (!h->has_particle || h->batch) return LBMP_OK;
     int cnt = 0;
-    launch_links_emit(h, h->frame_cur, h->stream);
+    launch_list_segments(h, h->stream);
     LBMP_CK(h, cudaMemcpyAsync(&cnt, h->count, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     LBMP_CK(h, cudaStreamSynchronize(h->stream));
     if (cnt == 0) return LBMP_OK;

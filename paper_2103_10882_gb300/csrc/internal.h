@@ -102,15 +102,19 @@ struct BoxDesc {
 };
 
 // Boundary CTAs of a coupled uniform step, also the number of force partials (8 warps each, taking the boundary
-// cells in turn).  A prefix of the counts per run of box cells finds them (MARK_CELLS_MAX bounds its shared memory,
-// 8 KB, spheres up to about 43 cells): one CTA per 128 box cells gives each warp one or two cells, enough
-// warps to hide the gathers' latency, few enough that the per-CTA set-up and the sums stay small.  Larger boxes
-// read a list: one CTA per 32 entries of its capacity (about three times the boundary cells), at most eight per SM.
-constexpr long long MARK_CELLS_MAX = 1 << 17;
-inline bool step_uses_list(const BoxDesc& b) { return b.cells > MARK_CELLS_MAX; }
-inline int step_boundary_blocks(const BoxDesc& b, int list_capacity) {
-    const long long n = step_uses_list(b) ? (list_capacity + 31) / 32 : (b.cells + 127) / 128;
-    return (int)(n < 1 ? 1 : (n > 1216 ? 1216 : n));
+// cells in turn).  The list's capacity is two to three times the boundary cells: one CTA per 20 entries gives every
+// warp about one cell, and the chain of a cell, the sums and the particle update is the step where the bulk update is
+// short (32^3: 17.6 us a step, 19.4 with one per 40; 64 x 64 x 128: 22.7 and 25.3).  Where the bulk update runs for
+// eight waves of CTAs or more the chain hides behind it and half as many cost it less (256 x 128 x 96: 92.0 and
+// 91.3 us; 256^3 in FP16 storage 272 and 270).  Coupled FP64 steps keep one per 32 entries, no slower (61 x 53 x 75:
+// 87.1 and 87.5 us): the sums then group as they always did.  At most eight per SM.
+// Boxes of up to SEG_CELLS_MAX cells (spheres up to about 70 cells) find their cells through a prefix of the segments'
+// numbers, 8 KB of shared memory at most; larger ones read a list that a further launch makes.
+constexpr long long SEG_CELLS_MAX = 2048 * 256;
+inline bool step_uses_list(const BoxDesc& b) { return b.cells > SEG_CELLS_MAX; }
+inline int step_boundary_blocks(int list_capacity, int per = 20) {   // per = 20: the most of them
+    const int n = (list_capacity + per - 1) / per;
+    return n < 1 ? 1 : (n > 1216 ? 1216 : n);
 }
 
 // n / d for n < 2^31 by one high multiplication (Granlund & Montgomery, "Division by invariant integers
@@ -159,8 +163,8 @@ template <typename S>
 int launch_remap(const lbmp_handle* h, S* pops, const uint8_t* fcur, uint8_t* fnext, int frame, bool mark_only,
                  typename Store<S>::A scale, typename Store<S>::A inv_scale, typename Store<S>::A gcoef,
                  cudaStream_t stream);
-// Boundary cells of the current marks as a list (h->list, h->count).
-void launch_links_emit(const lbmp_handle* h, int frame, cudaStream_t stream);
+// The segments' boundary cells as one list (h->list, h->count).
+void launch_list_segments(const lbmp_handle* h, cudaStream_t stream);
 void launch_export_links(const uint8_t* flags, const int* list, const int* count, int max_cells,
                          const GridDesc& g, const ParticleState* ps, int cli, int32_t* q_out, double* delta_out,
                          cudaStream_t stream);
@@ -206,7 +210,9 @@ struct lbmp_handle {
     int* count = nullptr;
     int list_cap = 0;
     uint8_t* link_mask = nullptr;        // marks of the box cells around the sphere (one byte each)
-    int* link_blocks = nullptr;          // boundary cells per run of box cells
+    int* link_blocks = nullptr;          // refined grids: boundary cells per run of box cells
+    int* seg = nullptr;                  // boundary cells by segment of the box (an entry per box cell)
+    int* seg_count = nullptr;            // and their number per segment
     double* partials = nullptr;
     int* d_done = nullptr;               // last-block-done counter of the boundary CTAs (uniform grids)
     lbmp::PFrames* frames = nullptr;     // uniform grids: two copies of the sphere's frames, a step reads one

@@ -347,6 +347,13 @@ struct LinkFrame {
 // d x 2 w_k c_k) is summed exactly by LinkSums.  Geometry and fl are
 // evaluated in the arithmetic type A of the populations (FP64 on the FP64
 // path); use_delta = false takes the wall half-way (delta = 1/2).
+// Every product and sum of the link is rounded as written (fma_rn, mul_rn: the compiler neither contracts nor splits
+// them), so the uniform, refined and batched steps get the same bits from the same populations.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // Wall distance delta along c_k (k = opp(q)) from the cell at offset d and
 // the CLI coefficients kappa0 = (1 - 2 delta) / (1 + 2 delta) and
 // alpha = 4 / (1 + 2 delta) of Sec. 2.3; use_delta = false takes delta = 1/2.
@@ -356,39 +363,65 @@ __device__ __forceinline__ void cli_coeffs(int q, const A d[3], bool use_delta, 
     const int k = opp(q);
     A delta = A(0.5);
     if (use_delta) {   // smallest root in (0,1] of |d + s c_k|^2 = r^2 (|c_k|^2 is 1 or 2)
-        const A dc = d[0] * A(cx(k)) + d[1] * A(cy(k)) + d[2] * A(cz(k));
-        const A e = d[0] * d[0] + d[1] * d[1] + d[2] * d[2] - r * r;
+        const A dc = d[0] * A(cx(k)) + d[1] * A(cy(k)) + d[2] * A(cz(k));   // products by 0 and +-1 are exact
+        const A e = fma_rn(-r, r, fma_rn(d[2], d[2], fma_rn(d[0], d[0], mul_rn(d[1], d[1]))));
         const bool face = k <= 6;
-        A disc = dc * dc - (face ? e : A(2) * e);
+        A disc = fma_rn(dc, dc, face ? -e : A(-2) * e);
         disc = disc < A(0) ? A(0) : disc;
         const A s = (-dc - sqrt(disc)) * (face ? A(1) : A(0.5));
         delta = s < A(0) ? A(0) : (s > A(1) ? A(1) : s);
     }
-    const A inv = A(1) / (A(1) + A(2) * delta);
+    const A inv = A(1) / fma_rn(A(2), delta, A(1));
     *delta_out = delta;
-    *kappa0 = (A(1) - A(2) * delta) * inv;
+    *kappa0 = mul_rn(fma_rn(A(-2), delta, A(1)), inv);
     *alpha = A(4) * inv;
+}
+
+// The part of a link that needs no populations: kappa0, alpha 3 w_k, v.c_k, the arm and the wall velocity v at the
+// link's wall point.  A caller forms it while the populations are still on their way.
+template <typename A>
+struct CliGeometry {
+    A kappa0, aw, vc, arm[3], vb[3];
+};
+
+template <typename A>
+__device__ __forceinline__ A cross_term(A a, A b, A c, A d) { return fma_rn(a, b, -mul_rn(c, d)); }   // ab - cd
+
+template <typename A>
+__device__ __forceinline__ CliGeometry<A> cli_geometry(int q, const A d[3], bool use_delta, const LinkFrame<A>& Fr) {
+    const int k = opp(q);
+    const A c[3] = {A(cx(k)), A(cy(k)), A(cz(k))};
+    CliGeometry<A> L;
+    A delta, alpha;
+    cli_coeffs<A>(q, d, use_delta, Fr.r, &delta, &L.kappa0, &alpha);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) L.arm[a] = fma_rn(delta, c[a], d[a]);
+    L.vb[0] = Fr.u[0] + cross_term(Fr.w[1], L.arm[2], Fr.w[2], L.arm[1]);
+    L.vb[1] = Fr.u[1] + cross_term(Fr.w[2], L.arm[0], Fr.w[0], L.arm[2]);
+    L.vb[2] = Fr.u[2] + cross_term(Fr.w[0], L.arm[1], Fr.w[1], L.arm[0]);
+    L.vc = L.vb[0] * c[0] + L.vb[1] * c[1] + L.vb[2] * c[2];
+    const A wk3 = k <= 6 ? A(1) / A(6) : A(1) / A(12);   // 3 w_k
+    L.aw = mul_rn(alpha, wk3);
+    return L;
+}
+
+template <typename A>
+__device__ __forceinline__ A cli_apply(int q, const CliGeometry<A>& L, A gt_k, A gt_q, A gt_far, A fl[3], A tl[3]) {
+    const int k = opp(q);
+    const A c[3] = {A(cx(k)), A(cy(k)), A(cz(k))};
+    const A gnew = fma_rn(-L.aw, L.vc, fma_rn(-L.kappa0, gt_q, fma_rn(L.kappa0, gt_far, gt_k)));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) fl[a] = fma_rn(c[a] - L.vb[a], gt_k, mul_rn(c[a] + L.vb[a], gnew));
+    tl[0] = cross_term(L.arm[1], fl[2], L.arm[2], fl[1]);
+    tl[1] = cross_term(L.arm[2], fl[0], L.arm[0], fl[2]);
+    tl[2] = cross_term(L.arm[0], fl[1], L.arm[1], fl[0]);
+    return gnew;
 }
 
 template <typename A>
 __device__ __forceinline__ A cli_link(int q, const A d[3], bool use_delta, A gt_k, A gt_q, A gt_far,
                                       const LinkFrame<A>& Fr, A fl[3], A tl[3]) {
-    const int k = opp(q);
-    const A c[3] = {A(cx(k)), A(cy(k)), A(cz(k))};
-    A delta, kappa0, alpha;
-    cli_coeffs<A>(q, d, use_delta, Fr.r, &delta, &kappa0, &alpha);
-    const A arm[3] = {d[0] + delta * c[0], d[1] + delta * c[1], d[2] + delta * c[2]};
-    const A vb[3] = {Fr.u[0] + (Fr.w[1] * arm[2] - Fr.w[2] * arm[1]), Fr.u[1] + (Fr.w[2] * arm[0] - Fr.w[0] * arm[2]),
-                     Fr.u[2] + (Fr.w[0] * arm[1] - Fr.w[1] * arm[0])};
-    const A vc = vb[0] * c[0] + vb[1] * c[1] + vb[2] * c[2];
-    const A wk3 = k <= 6 ? A(1) / A(6) : A(1) / A(12);   // 3 w_k
-    const A gnew = gt_k + kappa0 * gt_far - kappa0 * gt_q - alpha * wk3 * vc;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) fl[a] = (c[a] - vb[a]) * gt_k + (c[a] + vb[a]) * gnew;
-    tl[0] = arm[1] * fl[2] - arm[2] * fl[1];
-    tl[1] = arm[2] * fl[0] - arm[0] * fl[2];
-    tl[2] = arm[0] * fl[1] - arm[1] * fl[0];
-    return gnew;
+    return cli_apply<A>(q, cli_geometry<A>(q, d, use_delta, Fr), gt_k, gt_q, gt_far, fl, tl);
 }
 
 // Per-lane sums of the link forces and torques of one particle.  fl and tl
@@ -463,11 +496,15 @@ __device__ __forceinline__ void block_link_sums(const LinkSums<A>& acc, const do
     constexpr int SPAN = NW <= 8 ? 8 : (NW <= 16 ? 16 : 32);   // lanes of the cross-warp butterfly
     __shared__ long long si[6][NW];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    long long iv[6] = {acc.iF[0], acc.iF[1], acc.iF[2], acc.iT[0], acc.iT[1], acc.iT[2]};
+    // integers: exact warp sums by redux.sync, the torque parts in two halves of 16 low bits and the rest
+    long long iv[6];
 #pragma unroll
-    for (int c = 0; c < 6; ++c)
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) iv[c] += __shfl_down_sync(0xffffffffu, iv[c], off);
+    for (int a = 0; a < 3; ++a) {
+        iv[a] = __reduce_add_sync(0xffffffffu, acc.iF[a]);
+        const int lo = __reduce_add_sync(0xffffffffu, (int)(acc.iT[a] & 0xffff));
+        const int hi = __reduce_add_sync(0xffffffffu, (int)(acc.iT[a] >> 16));
+        iv[3 + a] = ((long long)hi << 16) + lo;
+    }
     if (lane == 0)
 #pragma unroll
         for (int c = 0; c < 6; ++c) si[c][wid] = iv[c];
@@ -475,7 +512,9 @@ __device__ __forceinline__ void block_link_sums(const LinkSums<A>& acc, const do
     int c;
     if constexpr (sizeof(A) == 4) {
         __shared__ float sh[6][NW], sl[6][NW];
-        float h[6], l[6];
+        // eight slots (six used) exchanged so that each step halves what a lane carries: 9 additions and 18 shuffles
+        // where six butterflies take 30 and 60; component c ends in lane 4 c
+        float h[8], l[8];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             h[a] = acc.F[a] + acc.eF[a];
@@ -483,19 +522,30 @@ __device__ __forceinline__ void block_link_sums(const LinkSums<A>& acc, const do
             h[3 + a] = acc.T[a] + acc.eT[a];
             l[3 + a] = acc.eT[a] - (h[3 + a] - acc.T[a]);
         }
+        h[6] = h[7] = l[6] = l[7] = 0.0f;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1)
+        for (int off = 16, m = 4; m >= 1; off >>= 1, m >>= 1) {
+            const bool up = (lane & off) != 0;
 #pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                const float oh = __shfl_xor_sync(0xffffffffu, h[k], off), ol = __shfl_xor_sync(0xffffffffu, l[k], off);
-                df_add(h[k], l[k], oh, ol);
+            for (int i = 0; i < m; ++i) {
+                const float sh_ = up ? h[i] : h[i + m], sl_ = up ? l[i] : l[i + m];
+                if (up) {
+                    h[i] = h[i + m];
+                    l[i] = l[i + m];
+                }
+                const float oh = __shfl_xor_sync(0xffffffffu, sh_, off), ol = __shfl_xor_sync(0xffffffffu, sl_, off);
+                df_add(h[i], l[i], oh, ol);
             }
-        if (lane == 0)
+        }
 #pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                sh[k][wid] = h[k];
-                sl[k][wid] = l[k];
-            }
+        for (int off = 2; off > 0; off >>= 1) {
+            const float oh = __shfl_xor_sync(0xffffffffu, h[0], off), ol = __shfl_xor_sync(0xffffffffu, l[0], off);
+            df_add(h[0], l[0], oh, ol);
+        }
+        if ((lane & 3) == 0 && lane < 24) {
+            sh[lane >> 2][wid] = h[0];
+            sl[lane >> 2][wid] = l[0];
+        }
         __syncthreads();
         if (wid >= 6) return;
         c = wid;
@@ -856,11 +906,15 @@ __device__ __forceinline__ double sum_partials(const double* partials, int nbloc
 // axes and the block writes the record back.  The partials may come from
 // other blocks of the same launch: they are read through L2.  Every thread
 // of the block must call it.
-template <int NT>
+// after(P, a): called by the thread of axis a with the advanced record (in shared memory).
+struct NoAfter {
+    __device__ __forceinline__ void operator()(const ParticleState&, int) const {}
+};
+template <int NT, typename After = NoAfter>
 __device__ __forceinline__ void particle_block_update(ParticleState* __restrict__ ps, const double* partials,
                                                       int nblocks, const GridDesc& G, double* __restrict__ history,
                                                       int hist_cap, int* __restrict__ status,
-                                                      const double* __restrict__ inv = nullptr) {
+                                                      const double* __restrict__ inv = nullptr, After after = After{}) {
     static_assert(NT % 32 == 0 && NT >= 256, "eight warps share the work");
     constexpr int words = (int)(sizeof(ParticleState) / sizeof(int));
     __shared__ double sFT[6], sinv[2];
@@ -878,9 +932,11 @@ __device__ __forceinline__ void particle_block_update(ParticleState* __restrict_
         for (int i = lane; i < words; i += 32) dstw[i] = __ldcg(srcw + i);
     }
     __syncthreads();
-    if (threadIdx.x < 3)   // the three axes in parallel
+    if (threadIdx.x < 3) {   // the three axes in parallel
         particle_advance_axis(sP, threadIdx.x, sFT[threadIdx.x], sFT[3 + threadIdx.x], sinv[0], sinv[1], G, history,
                               hist_cap, status);
+        after(sP, (int)threadIdx.x);
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         sP.steps += 1;
@@ -1025,6 +1081,47 @@ __device__ __forceinline__ int marked_cell(const int* pre, int runs, const uint8
     }
     for (; k > 0; --k) bits &= bits - 1u;   // drop the k lowest marked cells
     return (int)(r0 + base + __ffs((int)bits) - 1);
+}
+
+// Boundary cells in segments: the remap CTA of 256 box cells writes its marked cells, in box order, to the first
+// entries of its own 256, and their number.  A prefix of the numbers then gives the j-th boundary cell in one look-up
+// (a mask byte per box cell and a count per 64 took a binary search, two mask loads and a bit scan: 2,000 cycles of
+// the 5,500 that a boundary cell took).
+constexpr int SEG = 256;
+
+// The segment of boundary cell j: the largest s with pre[s] <= j, by the whole warp (two or a few ballots).
+__device__ __forceinline__ int find_segment(const int* pre, int nseg, int j) {
+    const int lane = threadIdx.x & 31;
+    const int step = (nseg + 31) >> 5;
+    const int at = lane * step;
+    const unsigned b = __ballot_sync(0xffffffffu, at < nseg && pre[at] <= j);
+    const int base = (__popc(b) - 1) * step;   // pre[0] = 0 <= j
+    int s = base;
+    for (int off = 0; off < step; off += 32) {
+        const int i = base + off + lane;
+        const unsigned m = __ballot_sync(0xffffffffu, off + lane < step && i < nseg && pre[i] <= j);
+        if (m == 0u) break;
+        s = base + off + __popc(m) - 1;
+    }
+    return s;
+}
+
+// Writes the block's marked cells (is_b, entry) into its segment.  Every thread of a block of SEG calls it.
+__device__ __forceinline__ void write_segment(bool is_b, int entry, int segment, int* __restrict__ seg,
+                                              int* __restrict__ seg_count) {
+    __shared__ int wsum[SEG / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned ballot = __ballot_sync(0xffffffffu, is_b);
+    if (lane == 0) wsum[wid] = __popc(ballot);
+    __syncthreads();
+    int base = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < SEG / 32; ++w) {
+        if (w < wid) base += wsum[w];
+        total += wsum[w];
+    }
+    if (is_b) seg[(size_t)segment * SEG + base + __popc(ballot & ((1u << lane) - 1u))] = entry;
+    if (threadIdx.x == 0) seg_count[segment] = total;
 }
 
 // Box cells of [t0, t0 + chunk) whose mask byte is set, in box order, into

@@ -33,13 +33,16 @@ struct StepArgs {
     int per_cta;           // of them per bulk CTA
     int* status;
     // the sphere's part (bblocks = 0 without a sphere)
-    int bblocks;           // boundary CTAs, first in the grid
+    int bblocks;           // boundary CTAs: every 2^bshift-th CTA from the first on
+    int bshift;
     int finish;            // last boundary CTA: 0 the particle update, 1 the force into force_out, 2 nothing
     int cli, hist_cap;
     const uint8_t* flags;
     const uint8_t* mark;
-    const int* run_count;
-    const int* list;       // boundary cells as a list, for boxes of more than MARK_CELLS_MAX cells; else null
+    const int* seg;        // boundary cells (linear indices) by segment of the box, and their numbers
+    const int* seg_count;
+    const int* list;       // boundary cells as a list, for boxes of more than SEG_CELLS_MAX cells; else null
+    FastDiv fx, fy;        // by nx and ny
     const int* count;
     BoxDesc B;
     ParticleState* ps;
@@ -224,50 +227,47 @@ __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, unsigned p
 // -------------------------------------------------------------- boundary
 // The cells next to the sphere, one warp per cell, lane q handling population q: pulls from solid cells are
 // replaced by the CLI rule of Sec. 2.3 (link geometry in the population arithmetic), then the warp collides the
-// cell cooperatively and writes it.  The marked cells are spread evenly over the warps of the boundary CTAs:
-// every CTA turns the remap's counts per run into a prefix, and warp w of W takes the marked cells w, w + W, ...
+// cell cooperatively and writes it.  The boundary cells are spread evenly over the warps of the boundary CTAs:
+// every CTA turns the remap's numbers per segment into a prefix, and warp w of W takes the cells w, w + W, ...
 // in box order (or the entries of the list, for large boxes).  The block sums of force and torque go into one
 // FP64 partial per CTA; the CTA that finishes last sums them.  Runs beside the bulk CTAs, which skip these cells.
 template <typename S, bool FORCED>
-__device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int* pre) {
+__device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int bid, int* pre) {
     using A = typename Store<S>::A;
     const GridDesc& G = T.G;
     const CollideParams<A>& P = T.P;
     const S* src = T.src;
     __shared__ LinkFrame<A> Fr;
-    __shared__ BoxFrame Bf;
-    const int runs = (int)((T.B.cells + LINK_RUN - 1) / LINK_RUN);
-    if (threadIdx.x == 0) Fr = pframe_link<A>(*T.frames);
-    if (threadIdx.x == 32) Bf = T.frames->bf;
-    const int i2 = 2 * (int)threadIdx.x;   // this thread's first two counts, in flight during the set-up
-    int first0 = 0, first1 = 0;
-    if (!T.list) {
-        if (i2 < runs) first0 = T.run_count[i2];
-        if (i2 + 1 < runs) first1 = T.run_count[i2 + 1];
+    const int nseg = (int)((T.B.cells + SEG - 1) / SEG);
+    if (threadIdx.x == STEP_THREADS - 1) Fr = pframe_link<A>(*T.frames);
+    const int i2 = 2 * (int)threadIdx.x;
+    int total;
+    if (T.list) {
+        total = *T.count;
+        __syncthreads();
+    } else {
+        const int first0 = i2 < nseg ? T.seg_count[i2] : 0, first1 = i2 + 1 < nseg ? T.seg_count[i2 + 1] : 0;
+        total = block_prefix<STEP_THREADS>(T.seg_count, nseg, pre, first0, first1);
     }
-    __syncthreads();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int total = T.list ? *T.count : block_prefix<STEP_THREADS>(T.run_count, runs, pre, first0, first1);
     const int W = T.bblocks * (STEP_THREADS / 32);
     const size_t n = (size_t)G.n;
     const int n3[3] = {G.nx, G.ny, G.nz};
+    const int q = lane < 19 ? lane : 0, k = opp(q);
+    const int c[3] = {cx(q), cy(q), cz(q)};
     LinkSums<A> acc;
-    for (int j = (int)blockIdx.x * (STEP_THREADS / 32) + wib; j < total; j += W) {
-        int xyz[3];
-        if (T.list) {
-            const int c = T.list[j];
-            xyz[0] = c % G.nx;
-            xyz[1] = (c / G.nx) % G.ny;
-            xyz[2] = c / (G.nx * G.ny);
-        } else {
-            const int t = marked_cell(pre, runs, T.mark, T.B.cells, j);
-            if (!box_cell(t, n3, G.periodic, T.B, Bf, xyz)) continue;   // marked cells are inside the domain
+    for (int j = bid * (STEP_THREADS / 32) + wib; j < total; j += W) {
+        int at = j;
+        if (!T.list) {
+            const int sg = find_segment(pre, nseg, j);
+            at = sg * SEG + (j - pre[sg]);
         }
-        const size_t cell = (size_t)xyz[0] + (size_t)G.nx * ((size_t)xyz[1] + (size_t)G.ny * (size_t)xyz[2]);
+        const int ci = T.list ? T.list[at] : T.seg[at];
+        const unsigned row = T.fx.div((unsigned)ci), plane = T.fy.div(row);
+        const int xyz[3] = {ci - (int)row * G.nx, (int)row - (int)plane * G.ny, (int)plane};
+        const size_t cell = (size_t)ci;
         A gq = A(0);
         if (lane < 19) {
-            const int q = lane;
-            const int c[3] = {cx(q), cy(q), cz(q)};
             int s3[3], f3[3];
             bool wall = false, far_ok = true;
 #pragma unroll
@@ -278,7 +278,6 @@ __device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int* pre) {
                 far_ok &= f3[a] >= 0;
             }
             // everything the pull or the link can need at once: one memory round trip instead of three
-            const int k = opp(q);
             const size_t sidx = wall ? cell : (size_t)s3[0] + (size_t)G.nx * ((size_t)s3[1] + (size_t)G.ny * (size_t)s3[2]);
             const size_t far = far_ok ? (size_t)f3[0] + (size_t)G.nx * ((size_t)f3[1] + (size_t)G.ny * (size_t)f3[2]) : cell;
             const uint8_t fsrc = T.flags[sidx], ffar = T.flags[far];
@@ -286,15 +285,19 @@ __device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int* pre) {
             const A gt_k = Store<S>::load(src + (size_t)k * n + cell, P.inv_scale);
             const A gt_q = Store<S>::load(src + (size_t)q * n + cell, P.inv_scale);
             const A vfar = Store<S>::load(src + (size_t)k * n + far, P.inv_scale);
+            // the link's geometry while they are on their way, as if the far cell were fluid (it nearly always is)
+            A d[3];
+            int pu[3];
+            Fr.offset(xyz, n3, G.periodic, d, pu);
+            CliGeometry<A> L = cli_geometry<A>(q, d, T.cli != 0, Fr);
             gq = pull;
             if (wall) {
                 gq = gt_k + wall_term<A>(G, q, xyz);
             } else if (q != 0 && fsrc != 0) {
                 far_ok = far_ok && ffar == 0;
-                A d[3], fl[3], tl[3];
-                int pu[3];
-                Fr.offset(xyz, n3, G.periodic, d, pu);
-                gq = cli_link<A>(q, d, T.cli && far_ok, gt_k, gt_q, far_ok ? vfar : A(0), Fr, fl, tl);
+                if (T.cli && !far_ok) L = cli_geometry<A>(q, d, false, Fr);
+                A fl[3], tl[3];
+                gq = cli_apply<A>(q, L, gt_k, gt_q, far_ok ? vfar : A(0), fl, tl);
                 acc.add(k, pu, fl, tl);
             }
         }
@@ -302,7 +305,7 @@ __device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int* pre) {
         if (lane < 19) Store<S>::store(T.dst + (size_t)lane * n + cell, gq, P.scale);
     }
     if (T.finish == 2) return;   // the force is not wanted
-    block_link_sums<STEP_THREADS>(acc, T.ps->x, T.partials + (size_t)blockIdx.x * 6);
+    block_link_sums<STEP_THREADS>(acc, T.ps->x, T.partials + (size_t)bid * 6);
     if (!last_block_done(T.done, T.bblocks)) return;
     if (T.finish == 1) {
         if (wib < 3) {
@@ -311,13 +314,20 @@ __device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int* pre) {
         }
         return;
     }
-    particle_block_update<STEP_THREADS>(T.ps, T.partials, T.bblocks, G, T.history, T.hist_cap, T.status, T.frames->inv);
-    __syncthreads();
-    // frames of the moved sphere, in the other copy: bulk CTAs of this launch still read this one
-    if (threadIdx.x < 3) pframes_axis(T.frames_next, *T.ps, n3, T.B, threadIdx.x);
+    // with it the frames of the moved sphere, in the other copy: bulk CTAs of this launch still read this one
+    particle_block_update<STEP_THREADS>(T.ps, T.partials, T.bblocks, G, T.history, T.hist_cap, T.status, T.frames->inv,
+                                        [&](const ParticleState& Q, int a) { pframes_axis(T.frames_next, Q, n3, T.B, a); });
 }
 
-// One launch: bblocks boundary CTAs, then the bulk CTAs.  The chain boundary cells -> force sum -> particle update
+// CTA b of the grid: boundary CTA b >> bshift (true), or the bulk CTA *bulk.
+template <typename S>
+__device__ __forceinline__ bool is_boundary_cta(const StepArgs<S>& T, unsigned b, unsigned* bulk) {
+    const unsigned before = min((unsigned)T.bblocks, (b + (1u << T.bshift) - 1u) >> T.bshift);
+    *bulk = b - before;
+    return (b & ((1u << T.bshift) - 1u)) == 0u && (b >> T.bshift) < (unsigned)T.bblocks;
+}
+
+// One launch: boundary CTAs among the first bulk CTAs (launch_step).  The chain boundary cells -> force sum -> particle update
 // (11 + 5 us as two launches of their own) runs beside the bulk update instead of after it.  With k_remap for the four
 // remap launches: a 32^3 FP32 step 46.1 -> 23.4 us, 256 x 128 x 96 with walls 123.6 -> 94.2, 61 x 53 x 75 in FP64
 // 175 -> 92 (with collide_direct), 512^3 3066 -> 2997.
@@ -327,14 +337,15 @@ constexpr int STEP_MIN_CTAS = sizeof(S) == 4 ? 5 : (sizeof(S) == 2 ? 4 : 2);
 
 template <typename S, bool WALLS, bool FORCED>
 __global__ void __launch_bounds__(STEP_THREADS, STEP_MIN_CTAS<S>) k_step(const __grid_constant__ StepArgs<S> T) {
-    extern __shared__ int pre[];   // prefix of the run counts (boundary CTAs)
+    extern __shared__ int pre[];   // prefix of the segments' numbers (boundary CTAs)
     pdl_trigger();
     pdl_wait();
-    if ((int)blockIdx.x < T.bblocks) {
-        boundary_cells<S, FORCED>(T, pre);
+    unsigned bulk;
+    if (is_boundary_cta(T, blockIdx.x, &bulk)) {
+        boundary_cells<S, FORCED>(T, (int)(blockIdx.x >> T.bshift), pre);
         return;
     }
-    const unsigned item = (blockIdx.x - (unsigned)T.bblocks) * (unsigned)T.per_cta + threadIdx.x;
+    const unsigned item = bulk * (unsigned)T.per_cta + threadIdx.x;
     if ((int)threadIdx.x >= T.per_cta || item >= T.items) return;
     bulk_cells<S, WALLS, FORCED>(T, item);
 }
@@ -344,12 +355,13 @@ __global__ void __launch_bounds__(STEP_THREADS, 4) k_step_h2(const __grid_consta
     extern __shared__ int pre[];
     pdl_trigger();
     pdl_wait();
-    if ((int)blockIdx.x < T.bblocks) {
-        boundary_cells<__half, false>(T, pre);
+    unsigned bulk;
+    if (is_boundary_cta(T, blockIdx.x, &bulk)) {
+        boundary_cells<__half, false>(T, (int)(blockIdx.x >> T.bshift), pre);
         return;
     }
     if ((int)threadIdx.x >= T.per_cta) return;   // whole warps
-    const unsigned item = (blockIdx.x - (unsigned)T.bblocks) * (unsigned)T.per_cta + threadIdx.x;
+    const unsigned item = bulk * (unsigned)T.per_cta + threadIdx.x;
     bulk_pairs<WALLS, MRT>(T, item, item < T.items);
 }
 
@@ -454,18 +466,17 @@ __device__ __forceinline__ void refill_warp(S* __restrict__ pops, const uint8_t*
 // here writes).  Neighbour flags are evaluated from the same predicate instead of being read back, so flags,
 // refill and boundary marks (four launches of 4 to 6 us before) take one pass.  mark_only: only marks and counts
 // (flags and populations already belong to the current position).
-constexpr int REMAP_THREADS = 256;
+constexpr int REMAP_THREADS = SEG;
 template <typename S>
 __global__ void __launch_bounds__(REMAP_THREADS)
     k_remap(S* __restrict__ pops, const uint8_t* __restrict__ fcur, uint8_t* __restrict__ fnext, GridDesc G, BoxDesc B,
             const ParticleState* __restrict__ ps, const PFrames* __restrict__ frames, typename Store<S>::A scale,
             typename Store<S>::A inv_scale, typename Store<S>::A gcoef, uint8_t* __restrict__ mark,
-            int* __restrict__ run_count, int mark_only) {
+            int* __restrict__ seg, int* __restrict__ seg_count, int mark_only) {
     using A = typename Store<S>::A;
     __shared__ BoxFrame F;
     __shared__ int s_n;
     __shared__ int s_g[3][REMAP_THREADS];   // uncovered cells
-    __shared__ int wsum[REMAP_THREADS / 32];
     const int n3[3] = {G.nx, G.ny, G.nz};
     pdl_trigger();
     pdl_wait();
@@ -477,16 +488,17 @@ __global__ void __launch_bounds__(REMAP_THREADS)
     const ParticleState& P = *ps;
     const size_t n = (size_t)G.n;
     const int t = blockIdx.x * REMAP_THREADS + threadIdx.x;
-    int is_b = 0;
+    bool is_b = false;
+    size_t c = 0;
     if (t < B.cells) {
         uint8_t m = MARK_PLAIN;
         int p[3];
         if (box_cell(t, n3, G.periodic, B, F, p)) {
-            const size_t c = (size_t)p[0] + (size_t)G.nx * ((size_t)p[1] + (size_t)G.ny * (size_t)p[2]);
+            c = (size_t)p[0] + (size_t)G.nx * ((size_t)p[1] + (size_t)G.ny * (size_t)p[2]);
             const bool was_solid = fcur[c] != 0;
             bool any_nb = false;
             const bool solid = ball_flag_and_neighbours(p, n3, G.periodic, F, P, &any_nb);
-            is_b = (!solid && any_nb) ? 1 : 0;
+            is_b = !solid && any_nb;
             m = solid ? MARK_SOLID : (is_b ? MARK_BOUNDARY : MARK_PLAIN);
             if (!mark_only) {
                 fnext[c] = solid ? 1 : 0;
@@ -503,65 +515,34 @@ __global__ void __launch_bounds__(REMAP_THREADS)
         }
         mark[t] = m;
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const unsigned ballot = __ballot_sync(0xffffffffu, is_b);
-    if (lane == 0) wsum[wid] = __popc(ballot);
-    __syncthreads();
-    constexpr int RUNS = REMAP_THREADS / LINK_RUN, WPR = LINK_RUN / 32;
-    if ((int)threadIdx.x < RUNS) {
-        const long long run = (long long)blockIdx.x * RUNS + threadIdx.x;
-        if (run * LINK_RUN < B.cells) {
-            int s = 0;
-#pragma unroll
-            for (int w = 0; w < WPR; ++w) s += wsum[threadIdx.x * WPR + w];
-            run_count[run] = s;
-        }
-    }
+    write_segment(is_b, (int)c, (int)blockIdx.x, seg, seg_count);   // its barrier also completes the shared list
+    const int wid = threadIdx.x >> 5;
     for (int k = wid; k < s_n; k += REMAP_THREADS / 32)
         refill_warp<S>(pops, fcur, G, n3, F, P, s_g[0][k], s_g[1][k], s_g[2][k], scale, inv_scale, gcoef);
 }
 
-// The marked cells as a list in box order (linear cell indices): every block takes 256 box cells and adds up the
-// runs before them.  Read back for inspection, and by the step itself for boxes too large for a prefix of the run
-// counts in shared memory (MARK_CELLS_MAX).
-constexpr int EMIT_THREADS = 256;
-__global__ void __launch_bounds__(EMIT_THREADS)
-    k_links_emit(const uint8_t* __restrict__ mark, const int* __restrict__ run_count, GridDesc G, BoxDesc B,
-                 const PFrames* __restrict__ frames, int* __restrict__ list, int* __restrict__ count, int capacity,
-                 int* __restrict__ status) {
-    __shared__ int red[EMIT_THREADS];
-    __shared__ int wsum[EMIT_THREADS / 32];
-    const int n3[3] = {G.nx, G.ny, G.nz};
-    const int before = (int)blockIdx.x * (EMIT_THREADS / LINK_RUN);
+// The boundary cells as one list in box order: every block copies its segment behind the cells of the segments before
+// it.  Read back for inspection, and by the step itself for boxes with too many segments for a prefix of their numbers
+// in shared memory (SEG_CELLS_MAX).
+__global__ void __launch_bounds__(SEG)
+    k_list_segments(const int* __restrict__ seg, const int* __restrict__ seg_count, int* __restrict__ list,
+                    int* __restrict__ count, int capacity, int* __restrict__ status) {
+    __shared__ int red[SEG];
     int s = 0;
-    for (int b = threadIdx.x; b < before; b += EMIT_THREADS) s += run_count[b];
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += SEG) s += seg_count[b];
     red[threadIdx.x] = s;
     __syncthreads();
-    for (int h = EMIT_THREADS / 2; h > 0; h >>= 1) {
-        if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
+    for (int h = SEG / 2; h > 0; h >>= 1) {
+        if ((int)threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
         __syncthreads();
     }
-    const int base = red[0];
-    const int t = blockIdx.x * EMIT_THREADS + threadIdx.x;
-    const int is_b = t < B.cells && mark[t] == MARK_BOUNDARY;
-    const unsigned ballot = __ballot_sync(0xffffffffu, is_b);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) wsum[warp] = __popc(ballot);
-    __syncthreads();
-    int wbase = 0;
-    for (int w = 0; w < warp; ++w) wbase += wsum[w];
-    if (is_b) {
-        int p[3];
-        const bool in = box_cell(t, n3, G.periodic, B, frames->bf, p);
-        const int pos = base + wbase + __popc(ballot & ((1u << lane) - 1u));
+    const int base = red[0], mine = seg_count[blockIdx.x];
+    if ((int)threadIdx.x < mine) {
+        const int pos = base + (int)threadIdx.x;
         if (pos >= capacity) atomicOr(status, STATUS_LINK_OVERFLOW);
-        else if (in) list[pos] = p[0] + G.nx * (p[1] + G.ny * p[2]);
+        else list[pos] = seg[(size_t)blockIdx.x * SEG + threadIdx.x];
     }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-        int tot = base;
-        for (int w = 0; w < EMIT_THREADS / 32; ++w) tot += wsum[w];
-        *count = tot < capacity ? tot : capacity;
-    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *count = min(base + mine, capacity);
 }
 
 // Link export for inspection: slot (i*18 + q-1) of the i-th boundary cell
@@ -679,7 +660,11 @@ void launch_step(const lbmp_handle* h, const S* src, S* dst, const CollideParams
     T.hist_cap = h->cfg.history_capacity;
     T.flags = h->flags[h->fcur];
     T.mark = h->link_mask;
-    T.run_count = h->link_blocks;
+    T.seg = h->seg;
+    T.seg_count = h->seg_count;
+    T.fx.set((unsigned)g.nx);
+    T.fy.set((unsigned)g.ny);
+    T.bshift = 0;
     T.list = nullptr;
     T.count = h->count;
     T.B = h->box;
@@ -690,12 +675,6 @@ void launch_step(const lbmp_handle* h, const S* src, S* dst, const CollideParams
     T.frames = h->frames + h->frame_cur;
     T.frames_next = h->frames + (1 - h->frame_cur);
     T.force_out = force_out;
-    size_t smem = 0;
-    if (h->has_particle) {
-        T.bblocks = step_boundary_blocks(h->box, h->list_cap);
-        if (step_uses_list(h->box)) T.list = h->list;
-        else smem = sizeof(int) * (size_t)((h->box.cells + LINK_RUN - 1) / LINK_RUN + 1);
-    }
     const bool walls = !(g.periodic[0] && g.periodic[1] && g.periodic[2]);
     const bool pairs = std::is_same<S, __half>::value && !p.forced && g.nx % 2 == 0;   // FP16: two cells per thread
     T.dx.set((unsigned)(pairs ? g.nx / 2 : g.nx));
@@ -705,7 +684,17 @@ void launch_step(const lbmp_handle* h, const S* src, S* dst, const CollideParams
     // bound by each scheduler's own FP64 rate, so idle SMs cost in proportion).
     T.per_cta = STEP_THREADS;
     while (T.per_cta > 32 && T.items / (unsigned)T.per_cta < 2 * 152) T.per_cta /= 2;
-    const unsigned grid = (unsigned)T.bblocks + (T.items + (unsigned)T.per_cta - 1) / (unsigned)T.per_cta;
+    const unsigned bulk = (T.items + (unsigned)T.per_cta - 1) / (unsigned)T.per_cta;
+    size_t smem = 0;
+    if (h->has_particle) {
+        T.bblocks = step_boundary_blocks(h->list_cap, bulk >= 8 * 5 * 152 ? 40 : (sizeof(S) == 8 && finish == 0 ? 32 : 20));
+        if (step_uses_list(h->box)) T.list = h->list;
+        else smem = sizeof(int) * (size_t)((h->box.cells + SEG - 1) / SEG + 1);
+    }
+    const unsigned grid = (unsigned)T.bblocks + bulk;
+    // Boundary CTAs wait on latencies: up to three bulk CTAs between two of them keep the memory busy meanwhile (a
+    // sphere of 40 cells has 900, more than a wave).
+    while (T.bshift < 2 && (unsigned)T.bblocks << (T.bshift + 1) <= grid) ++T.bshift;
     auto go = [&](auto kernel) { launch_pdl(kernel, grid, STEP_THREADS, smem, stream, T); };
     if constexpr (std::is_same<S, __half>::value) {
         if (pairs) {
@@ -740,16 +729,16 @@ int launch_remap(const lbmp_handle* h, S* pops, const uint8_t* fcur, uint8_t* fn
                  cudaStream_t stream) {
     const PFrames* F = h->frames + frame;
     launch_pdl(k_remap<S>, blocks_for(h->box.cells, REMAP_THREADS), REMAP_THREADS, 0, stream, pops, fcur, fnext, h->G,
-               h->box, (const ParticleState*)h->d_ps, F, scale, inv_scale, gcoef, h->link_mask, h->link_blocks,
+               h->box, (const ParticleState*)h->d_ps, F, scale, inv_scale, gcoef, h->link_mask, h->seg, h->seg_count,
                mark_only ? 1 : 0);
     if (!step_uses_list(h->box)) return 1;
-    launch_links_emit(h, frame, stream);
+    launch_list_segments(h, stream);
     return 2;
 }
 
-void launch_links_emit(const lbmp_handle* h, int frame, cudaStream_t stream) {
-    k_links_emit<<<blocks_for(h->box.cells, EMIT_THREADS), EMIT_THREADS, 0, stream>>>(
-        h->link_mask, h->link_blocks, h->G, h->box, h->frames + frame, h->list, h->count, h->list_cap, h->status);
+void launch_list_segments(const lbmp_handle* h, cudaStream_t stream) {
+    k_list_segments<<<blocks_for(h->box.cells, SEG), SEG, 0, stream>>>(h->seg, h->seg_count, h->list, h->count, h->list_cap,
+                                                                      h->status);
 }
 
 void launch_export_links(const uint8_t* flags, const int* list, const int* count, int max_cells, const GridDesc& g,

@@ -1,5 +1,5 @@
-"""The coupled uniform step at the edges of its launch: boundary cells found from the marks' run counts (boxes of up to
-131,072 cells) and from the list (larger ones), boxes that span a periodic axis or exceed a walled one, grids of a few
+"""The coupled uniform step at the edges of its launch: boundary cells found from the segments' numbers (boxes of up to
+524,288 cells) and from the list (larger ones), boxes that span a periodic axis or exceed a walled one, grids of a few
 cells, rows that begin inside a warp.  Tolerances of test_gpu_uniform.py: FP64 1e-10, FP16 5e-3 of max|g|."""
 import numpy as np
 import pytest
@@ -11,8 +11,9 @@ P, N = "periodic", "noslip"
 
 
 @pytest.mark.parametrize("precision,shape,d,bc,steps", [
-    ("fp64", (53, 52, 51), 41.0, (P, P, P), 6),     # 50^3 box cells, 1,954 runs: the largest prefixes
-    ("fp64", (56, 58, 57), 46.0, (P, P, P), 6),     # 54^3 box cells: the list
+    ("fp64", (53, 52, 51), 41.0, (P, P, P), 6),     # 50^3 box cells, 489 segments: a prefix in one pass
+    ("fp64", (82, 84, 83), 72.0, (P, P, P), 3),     # 80^3 box cells, 2,000 segments: the largest prefixes
+    ("fp64", (85, 86, 84), 74.0, (P, P, P), 3),     # 82^3 box cells: the list
     ("fp64", (9, 9, 9), 5.0, (P, P, P), 40),        # the box spans every axis
     ("fp64", (7, 40, 9), 3.0, (N, P, N), 40),       # the box exceeds two walled axes
     ("fp64", (8, 8, 257), 4.0, (P, N, P), 40),
