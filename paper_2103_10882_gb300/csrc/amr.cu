@@ -174,44 +174,25 @@ struct UpdateArgs {
     // levels with a coarser level C: its post-collision populations of the
     // current coarse step (csrc, read for static ghost neighbours), per group
     // of eight active ghost cells their host (real block << 12 | cell of C),
-    // per active ghost cell the mask of populations whose upwind neighbour is
-    // a static ghost cell; at the last sub-step also C's destination buffer
-    // and collision parameters, for the hosts (coalescence)
-    LevelView C;
+    // per active ghost cell and population its source in this sub-step
+    // (k_ghost_sources, [q][ghost cell]); at the last sub-step also C's
+    // destination buffer and collision parameters, for the hosts (coalescence)
     const S* csrc;
     const int* ghost_host;
-    const uint32_t* smask;
+    const uint32_t* gsrc;
     S* cdst;
     CollideParams<A> Pc;
     const uint8_t* solid;     // finest level with a sphere: solid flags of real cells
     int* status;
 };
 
-// Where an active ghost cell finds a static ghost cell upwind.  Static ghost
-// cells (the sub-cells of the second ring of coarse cells) hold the exploded
-// coarse values at the first sub-step and stream rigidly, without
-// colliding, into the second, so each of their values is that of a coarse
-// cell, which the pull reads directly: with P the host of the active cell x
-// and s in {0,1}^3 its sub-cell offset, the coarse cell containing x - c_q
-// is P + o, o_a = s_a - 1 for c_a = 1, s_a for c_a = -1, 0 for c_a = 0
-// (first sub-step); at the second sub-step the static cell has carried the
-// content of the coarse cell containing x - 2 c_q, which is P - c_q, or
-// kept its own (P + o) where that lies beyond a wall.
-struct GhostPull {
-    uint32_t smask;   // bit q: the upwind neighbour x - c_q is a static ghost cell
-    int hb, hc;       // the host P: real block and cell of the coarser level
-    int sub;          // sub-cell offset s = (sub & 1, (sub >> 1) & 1, sub >> 2)
-    bool second;      // the level's second sub-step
-};
-
 // Pull of the 19 populations of cell (b, c) into g, as stored (FP16: the
 // scaled values g * 2^s, which the collision takes in its SCALED form).  nb27 lists the pool
-// ids of block b's 26 neighbours (and itself at index 13).  GHOST: (b, c) is
-// an active ghost cell and gp says where static ghost cells lie upwind.
+// ids of block b's 26 neighbours (and itself at index 13).
 // Returns whether a source was missing (no block), which the caller reports.
-template <typename S, bool GHOST = false>
+template <typename S>
 __device__ __forceinline__ bool pull_cell(const UpdateArgs<S>& U, int b, int c, const int* nb27,
-                                          typename Store<S>::A g[19], GhostPull gp = GhostPull{}) {
+                                          typename Store<S>::A g[19]) {
     using A = typename Store<S>::A;
     const int lx = c & 15, ly = (c >> 4) & 15, lz = c >> 8;
     // source x - c_q per axis, indexed by 1 - c: block shift and local coordinate.
@@ -234,18 +215,7 @@ __device__ __forceinline__ bool pull_cell(const UpdateArgs<S>& U, int b, int c, 
         const int sb = own ? b : nbk, sq = own ? opp(q) : q;
         const int sc = own ? c : lsx[ix] + lsy[iy] + lsz[iz];
         const S* src = U.src + (unsigned)((sb * 19 + sq) * B3 + sc);   // pools hold < 2^31 elements
-        bool lost = nbk == -1;
-        if (GHOST && q > 0 && ((gp.smask >> q) & 1u)) {   // static ghost upwind: its coarse cell
-            const int hx = gp.hc & 15, hy = (gp.hc >> 4) & 15, hz = gp.hc >> 8;
-            const int ox = cx(q) == 1 ? (gp.sub & 1) - 1 : (cx(q) == -1 ? (gp.sub & 1) : 0);
-            const int oy = cy(q) == 1 ? ((gp.sub >> 1) & 1) - 1 : (cy(q) == -1 ? ((gp.sub >> 1) & 1) : 0);
-            const int oz = cz(q) == 1 ? (gp.sub >> 2) - 1 : (cz(q) == -1 ? (gp.sub >> 2) : 0);
-            int cc;
-            int cb = gp.second ? nbr_cell(U.C, gp.hb, hx, hy, hz, -cx(q), -cy(q), -cz(q), &cc) : -2;
-            if (cb == -2) cb = nbr_cell(U.C, gp.hb, hx, hy, hz, ox, oy, oz, &cc);
-            lost = cb < 0;
-            src = U.csrc + (unsigned)(((lost ? 0 : cb) * 19 + q) * B3 + cc);
-        }
+        const bool lost = nbk == -1;
         const A v = Store<S>::load_raw(src);
         missing |= lost;
         g[q] = lost ? A(0) : v;
@@ -253,6 +223,29 @@ __device__ __forceinline__ bool pull_cell(const UpdateArgs<S>& U, int b, int c, 
     return missing;
 }
 
+
+// Source of a ghost cell's population (k_ghost_sources): an element offset into the level's pool, or with bit 31 set
+// into the coarser level's; GHOST_MISSING where no block holds it.
+constexpr uint32_t GHOST_COARSE = 0x80000000u, GHOST_MISSING = 0xffffffffu;
+
+// Pull of active ghost cell i, as stored; returns whether a source was missing.
+template <typename S>
+__device__ __forceinline__ bool pull_ghost(const UpdateArgs<S>& U, int i, int nglist, typename Store<S>::A g[19]) {
+    using A = typename Store<S>::A;
+    uint32_t off[19];
+#pragma unroll
+    for (int q = 0; q < 19; ++q) off[q] = U.gsrc[(size_t)q * nglist + i];
+    bool missing = false;
+#pragma unroll
+    for (int q = 0; q < 19; ++q) {
+        const bool lost = off[q] == GHOST_MISSING;
+        const S* base = (off[q] & GHOST_COARSE) ? U.csrc : U.src;
+        const A v = Store<S>::load_raw(base + (lost ? 0u : off[q] & ~GHOST_COARSE));
+        missing |= lost;
+        g[q] = lost ? A(0) : v;
+    }
+    return missing;
+}
 
 // One launch per level step: the first gblocks CTAs stream the active ghost
 // cells of the level (glist: pool block << 12 | cell, eight consecutive
@@ -284,8 +277,7 @@ __global__ void __launch_bounds__(UPD_THREADS, sizeof(S) == 8 ? 1 : UPD_MIN_CTAS
             b = e >> 12;
             c = e & 4095;
             hp = U.ghost_host[i >> 3];
-            const GhostPull gp{U.smask[i], hp >> 12, hp & 4095, i & 7, coalesce != 0};
-            if (pull_cell<S, true>(U, b, c, U.D.nbr + (size_t)b * 27, g, gp)) atomicOr(U.status, STATUS_AMR_MISSING);
+            if (pull_ghost<S>(U, i, nglist, g)) atomicOr(U.status, STATUS_AMR_MISSING);
             if (!coalesce) {
 #pragma unroll
                 for (int q = 0; q < 19; ++q) Store<S>::store_raw(U.dst + paddr(b, q, c), g[q]);
@@ -738,35 +730,55 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// Static-neighbour masks of the active ghost cells of level F (list and
-// hosts of k_ghost_lists, n entries): bit q is set when the upwind
-// neighbour x - c_q lies in a ghost block and its coarse cell (P + o, see
-// GhostPull) is a second-ring cell of level C (host flag 2).  A ghost
-// neighbour whose coarse cell is neither a host nor in the second ring is
-// an error of the layout.
+// Sources of the active ghost cells of level F (list and hosts of k_ghost_lists, n entries), which depend on the layout
+// alone: per population q the element that the pull of q reads at the level's first sub-step (table 0) and at its
+// second (table 1), laid out [table][q][ghost cell].
+//   - Mostly the upwind neighbour x - c_q in F's pool (real or active ghost cell), or beyond a domain wall the cell's
+//     own opposite population (bounce-back).
+//   - Where the upwind neighbour is a static ghost cell (a sub-cell of the second ring of coarse cells, host flag 2):
+//     static ghost cells hold the exploded coarse values at the first sub-step and stream rigidly, without colliding,
+//     into the second, so each of their values is that of a coarse cell, read directly.  With P the host of the active
+//     cell x and s in {0,1}^3 its sub-cell offset, the coarse cell containing x - c_q is P + o, o_a = s_a - 1 for
+//     c_a = 1, s_a for c_a = -1, 0 for c_a = 0 (first sub-step); at the second the static cell has carried the content
+//     of the coarse cell containing x - 2 c_q, which is P - c_q, or kept its own (P + o) where that lies beyond a wall.
+// Found here once per layout: the step's ghost CTAs walked the neighbour tables of both levels in divergent code for
+// each of the 19 populations, and ended long after the real blocks' CTAs.  A ghost neighbour whose coarse cell is
+// neither a host nor in the second ring is an error of the layout.
 __global__ void __launch_bounds__(256)
-    k_ghost_smask(LevelView C, LevelView F, const int* __restrict__ list, const int* __restrict__ hosts, int n,
-                  uint32_t* __restrict__ smask, int* __restrict__ status) {
+    k_ghost_sources(LevelView C, LevelView F, const int* __restrict__ list, const int* __restrict__ hosts, int n,
+                    uint32_t* __restrict__ gsrc, int* __restrict__ status) {
     const int i = blockIdx.x * 256 + threadIdx.x;
     if (i >= n) return;
     const int e = list[i], hp = hosts[i >> 3];
     const int b = e >> 12, c = e & 4095, hb = hp >> 12, hc = hp & 4095, sub = i & 7;
     const int s[3] = {sub & 1, (sub >> 1) & 1, sub >> 2};
-    uint32_t m = 0;
-    for (int q = 1; q < 19; ++q) {
+    for (int q = 0; q < 19; ++q) {
         const int cq[3] = {cx(q), cy(q), cz(q)};
         int nc;
         const int nbk = nbr_cell(F, b, c & 15, (c >> 4) & 15, c >> 8, -cq[0], -cq[1], -cq[2], &nc);
-        if (nbk < F.nreal) continue;   // a real cell, a wall or no block: the ordinary pull
-        int o[3];
-        for (int a = 0; a < 3; ++a) o[a] = cq[a] == 1 ? s[a] - 1 : (cq[a] == -1 ? s[a] : 0);
-        int pc;
-        const int pb = nbr_cell(C, hb, hc & 15, (hc >> 4) & 15, hc >> 8, o[0], o[1], o[2], &pc);
-        const int kind = (pb >= 0 && pb < C.nreal) ? C.host[(size_t)pb * B3 + pc] : 0;
-        if (kind == 2) m |= 1u << q;
-        else if (kind != 1) atomicOr(status, STATUS_AMR_MISSING);
+        uint32_t first, second;
+        int kind = 1;
+        int o[3], pc, pb = -1;
+        if (nbk >= F.nreal) {   // a ghost block: its coarse cell is a host (active ghost cell) or in the second ring
+            for (int a = 0; a < 3; ++a) o[a] = cq[a] == 1 ? s[a] - 1 : (cq[a] == -1 ? s[a] : 0);
+            if (q == 0) o[0] = o[1] = o[2] = 0;
+            pb = nbr_cell(C, hb, hc & 15, (hc >> 4) & 15, hc >> 8, o[0], o[1], o[2], &pc);
+            kind = (pb >= 0 && pb < C.nreal) ? C.host[(size_t)pb * B3 + pc] : 0;
+            if (kind != 1 && kind != 2) atomicOr(status, STATUS_AMR_MISSING);
+        }
+        if (kind == 2) {
+            first = GHOST_COARSE | (uint32_t)((pb * 19 + q) * B3 + pc);
+            int sc;
+            const int sb = nbr_cell(C, hb, hc & 15, (hc >> 4) & 15, hc >> 8, -cq[0], -cq[1], -cq[2], &sc);
+            second = sb >= 0 ? GHOST_COARSE | (uint32_t)((sb * 19 + q) * B3 + sc) : (sb == -2 ? first : GHOST_MISSING);
+        } else if (nbk >= 0) {
+            first = second = (uint32_t)((nbk * 19 + q) * B3 + nc);
+        } else {
+            first = second = nbk == -2 ? (uint32_t)((b * 19 + opp(q)) * B3 + c) : GHOST_MISSING;
+        }
+        gsrc[(size_t)q * n + i] = first;
+        gsrc[(size_t)(19 + q) * n + i] = second;
     }
-    smask[i] = m;
 }
 
 __global__ void k_amr_flags_full(LevelView D, uint8_t* __restrict__ f0, uint8_t* __restrict__ f1,
@@ -1012,7 +1024,7 @@ struct Level {
     bool ghosts_valid = false;   // the active ghost cells of the current buffer hold the coarser level's hosts
     int* d_glist = nullptr;      // the active ghost cells, pool block << 12 | cell, eight per host
     int* d_ghost_host = nullptr; // per eight: the host, real block << 12 | cell of the coarser level
-    uint32_t* d_smask = nullptr; // per active ghost cell: populations with a static ghost cell upwind
+    uint32_t* d_gsrc = nullptr;  // per sub-step, population and active ghost cell: the element it pulls (k_ghost_sources)
     void* d_pops[2] = {nullptr, nullptr};
     int cur = 0;
     uint8_t* d_flags[2] = {nullptr, nullptr};   // finest level only
@@ -1291,7 +1303,7 @@ void free_level(lbmp_handle* h, Level& V) {
     handle_free(h, V.d_host);
     handle_free(h, V.d_glist);
     handle_free(h, V.d_ghost_host);
-    handle_free(h, V.d_smask);
+    handle_free(h, V.d_gsrc);
     handle_free(h, V.d_pops[0]);
     handle_free(h, V.d_pops[1]);
     handle_free(h, V.d_flags[0]);
@@ -1456,16 +1468,16 @@ lbmp_status build_layout(lbmp_handle* h, const std::vector<Mask>& R) {
         const size_t ng = std::max<size_t>((size_t)F.nglist, 8);
         F.d_glist = (int*)handle_alloc(h, sizeof(int) * ng);
         F.d_ghost_host = (int*)handle_alloc(h, sizeof(int) * (ng / 8));
-        F.d_smask = (uint32_t*)handle_alloc(h, sizeof(uint32_t) * ng);
-        if (!F.d_glist || !F.d_ghost_host || !F.d_smask) {
+        F.d_gsrc = (uint32_t*)handle_alloc(h, sizeof(uint32_t) * 2 * 19 * ng);
+        if (!F.d_glist || !F.d_ghost_host || !F.d_gsrc) {
             ok = false;
             break;
         }
         if (F.nglist > 0) {
             k_ghost_lists<<<(unsigned)C.nreal * 16, 256, 0, h->stream>>>(view(E, C), C.d_host, d_runs[l], view(E, F),
                                                                            F.d_glist, F.d_ghost_host, h->status);
-            k_ghost_smask<<<(unsigned)((F.nglist + 255) / 256), 256, 0, h->stream>>>(
-                view(E, C), view(E, F), F.d_glist, F.d_ghost_host, F.nglist, F.d_smask, h->status);
+            k_ghost_sources<<<(unsigned)((F.nglist + 255) / 256), 256, 0, h->stream>>>(
+                view(E, C), view(E, F), F.d_glist, F.d_ghost_host, F.nglist, F.d_gsrc, h->status);
         }
     }
     if (ok && cudaStreamSynchronize(h->stream) != cudaSuccess) ok = false;
@@ -1626,10 +1638,9 @@ void enqueue_advance(lbmp_handle* h, int l, int sub) {
     U.src = (const S*)V.d_pops[V.cur];
     U.dst = (S*)V.d_pops[1 - V.cur];
     U.P = P;
-    U.C = U.D;
     U.csrc = nullptr;
     U.ghost_host = nullptr;
-    U.smask = nullptr;
+    U.gsrc = nullptr;
     U.cdst = nullptr;
     U.Pc = P;
     U.solid = nullptr;
@@ -1638,10 +1649,9 @@ void enqueue_advance(lbmp_handle* h, int l, int sub) {
     const int coalesce = (has_coarse && sub == 1) ? 1 : 0;   // this sub-step ends the coarser level's step
     if (has_coarse) {
         Level& C = E->lv[l - 1];
-        U.C = view(E, C);
         U.csrc = (const S*)C.d_pops[C.cur];   // the coarser level's step flips cur after both sub-steps
         U.ghost_host = V.d_ghost_host;
-        U.smask = V.d_smask;
+        U.gsrc = V.d_gsrc + (size_t)(coalesce ? 19 : 0) * V.nglist;
         if (coalesce) {
             U.cdst = (S*)C.d_pops[1 - C.cur];
             U.Pc = level_params<S>(h, C);
