@@ -345,77 +345,79 @@ __global__ void __launch_bounds__(UPD_THREADS, sizeof(S) == 8 ? 1 : UPD_MIN_CTAS
 
 // ---------------------------------------------------------------- coupling
 constexpr int BNDW_THREADS = 256;
-constexpr int BND_CHUNK = 128;     // box cells per boundary CTA (sizes the grid)
 // Register cap of the boundary kernel (BNDW_THREADS threads).  It runs beside the finest level's
 // update for most of that update, so every register it holds is taken from the update's CTAs: at
 // 56 in FP32 a boundary CTA (14,336 registers) leaves room for 1,280 update threads of 40 registers
 // instead of 1,024.
 template <typename S>
 constexpr int BND_MAXREG = sizeof(S) == 8 ? 128 : (sizeof(S) == 4 ? 56 : 64);
-constexpr int REMAP_THREADS = 256;   // remap blocks: their uncovered cells are spread over the eight warps
+constexpr int REMAP_THREADS = SEG;   // remap blocks: their uncovered cells are spread over the eight warps
 
 // Boundary cells of the finest level (flag 2: fluid with a solid
-// neighbour), from the mask the remap wrote in box order and its count of
-// marked cells per run of LINK_RUN box cells.  The marked cells are
-// spread evenly over all warps of the grid: every CTA turns the counts into
-// a prefix, and warp w of W takes the marked cells w, w + W, ... (box
-// order), one cell per warp at a time, lane q handling population q (CLI
-// links of Sec. 2.3, geometry in the population arithmetic, FP64 force
-// partials per CTA), with a cooperative collision.  The level update skips
-// these cells, so this kernel runs beside it.  The block that finishes
-// last sums the partials and runs the particle update of Algorithm 1.
-// Dynamic shared memory: (runs + 1) ints.
+// neighbour), from the segments the remap wrote (pool block << 12 | cell).
+// They are spread evenly over all warps of the grid: every CTA turns the
+// segments' numbers into a prefix, and warp w of W takes the cells w, w + W,
+// ... in box order, lane q handling population q (CLI links of Sec. 2.3,
+// geometry in the population arithmetic, FP64 force partials per CTA), with
+// a cooperative collision.  A cell takes three memory round trips: its
+// segment entry; the neighbour blocks on both sides of every lane's link;
+// then both flags and all populations at once, with the link's geometry
+// formed meanwhile.  The level update skips these cells, so this kernel runs
+// beside it.  The block that finishes last sums the partials and runs the
+// particle update of Algorithm 1.  Dynamic shared memory: (segments + 1) ints.
 template <typename S>
 __global__ void __maxnreg__(BND_MAXREG<S>)
-    k_amr_boundary(LevelView D, const S* __restrict__ src, S* __restrict__ dst, const uint8_t* __restrict__ solid,
-                   const uint8_t* __restrict__ mask, const int* __restrict__ run_count, BoxDesc B,
-                   CollideParams<typename Store<S>::A> P, ParticleState* ps, int cli, double* partials, int* done,
-                   GridDesc G, double* __restrict__ history, int hist_cap, int* __restrict__ status,
+    k_amr_boundary(const __grid_constant__ LevelView D, const S* __restrict__ src, S* __restrict__ dst, const uint8_t* __restrict__ solid,
+                   const int* __restrict__ seg, const int* __restrict__ seg_count,
+                   const __grid_constant__ BoxDesc B,
+                   const __grid_constant__ CollideParams<typename Store<S>::A> P, ParticleState* ps, int cli, double* partials, int* done,
+                   const __grid_constant__ GridDesc G, double* __restrict__ history, int hist_cap, int* __restrict__ status,
                    PFrames* __restrict__ frames) {
     using A = typename Store<S>::A;
-    extern __shared__ int pre[];   // [runs + 1]
+    extern __shared__ int pre[];   // [segments + 1]
     __shared__ LinkFrame<A> Fr;
-    __shared__ BoxFrame Bf;
-    const int runs = (int)((B.cells + LINK_RUN - 1) / LINK_RUN);
-    const int i2 = 2 * (int)threadIdx.x;   // this thread's first two counts, in flight during the set-up
-    const int first0 = i2 < runs ? run_count[i2] : 0, first1 = i2 + 1 < runs ? run_count[i2 + 1] : 0;
-    if (threadIdx.x == 0) Fr = pframe_link<A>(*frames);   // formed by the last particle update
-    if (threadIdx.x == 32) Bf = frames->bf;
-    __syncthreads();
+    const int nseg = (int)((B.cells + SEG - 1) / SEG);
+    const int i2 = 2 * (int)threadIdx.x;   // this thread's first two numbers, in flight during the set-up
+    const int first0 = i2 < nseg ? seg_count[i2] : 0, first1 = i2 + 1 < nseg ? seg_count[i2 + 1] : 0;
+    if (threadIdx.x == BNDW_THREADS - 1) Fr = pframe_link<A>(*frames);   // formed by the last particle update
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int total = block_prefix<BNDW_THREADS>(run_count, runs, pre, first0, first1);
+    const int total = block_prefix<BNDW_THREADS>(seg_count, nseg, pre, first0, first1);
     const int W = (int)gridDim.x * (BNDW_THREADS / 32);
+    const int q = lane < 19 ? lane : 0, k = opp(q);
+    const int cq[3] = {cx(q), cy(q), cz(q)};
     LinkSums<A> acc;
     for (int j = (int)blockIdx.x * (BNDW_THREADS / 32) + wib; j < total; j += W) {
-        const int t = marked_cell(pre, runs, mask, B.cells, j);
-        int g[3], c;
-        if (!box_cell(t, D.n, D.periodic, B, Bf, g)) continue;   // marked cells are inside the domain
-        const int b = locate(D, g, &c);
+        const int sg = find_segment(pre, nseg, j);
+        const int e = seg[sg * SEG + (j - pre[sg])];
+        const int b = e >> 12, c = e & 4095;
         const int lx = c & 15, ly = (c >> 4) & 15, lz = c >> 8;
         A gq = A(0);
         if (lane < 19) {
-            const int q = lane;
-            const int cq[3] = {cx(q), cy(q), cz(q)};
-            int sc;
+            int sc, fc;
             const int sb = nbr_cell(D, b, lx, ly, lz, -cq[0], -cq[1], -cq[2], &sc);
+            const int fb = nbr_cell(D, b, lx, ly, lz, cq[0], cq[1], cq[2], &fc);   // x - c_k
+            const int g[3] = {D.bpos[3 * b] * BS + lx, D.bpos[3 * b + 1] * BS + ly, D.bpos[3 * b + 2] * BS + lz};
+            const bool sreal = sb >= 0 && sb < D.nreal, freal = fb >= 0 && fb < D.nreal;
+            const uint8_t ssolid = solid[sreal ? (size_t)sb * B3 + sc : 0], fsolid = solid[freal ? (size_t)fb * B3 + fc : 0];
+            const A pull = Store<S>::load(src + (sb >= 0 ? paddr(sb, q, sc) : paddr(b, q, c)), P.inv_scale);
+            const A gt_k = Store<S>::load(src + paddr(b, k, c), P.inv_scale);
+            const A gt_q = Store<S>::load(src + paddr(b, q, c), P.inv_scale);
+            const A vfar = Store<S>::load(src + (freal ? paddr(fb, k, fc) : paddr(b, k, c)), P.inv_scale);
+            A d[3];
+            int pu[3];
+            Fr.offset(g, D.n, D.periodic, d, pu);
+            CliGeometry<A> Lk = cli_geometry<A>(q, d, cli != 0, Fr);   // as if the far cell were fluid
+            gq = pull;
             if (sb == -2) {
-                gq = Store<S>::load(src + paddr(b, opp(q), c), P.inv_scale);
+                gq = gt_k;
             } else if (sb < 0) {
+                gq = A(0);
                 atomicOr(status, STATUS_AMR_MISSING);
-            } else if (q == 0 || sb >= D.nreal || solid[(size_t)sb * B3 + sc] != FLAG_SOLID) {
-                gq = Store<S>::load(src + paddr(sb, q, sc), P.inv_scale);
-            } else {
-                const int k = opp(q);
-                int fc;
-                const int fb = nbr_cell(D, b, lx, ly, lz, cq[0], cq[1], cq[2], &fc);   // x - c_k
-                const bool far_ok = fb >= 0 && fb < D.nreal && solid[(size_t)fb * B3 + fc] != FLAG_SOLID;
-                A d[3], fl[3], tl3[3];
-                int pu[3];
-                Fr.offset(g, D.n, D.periodic, d, pu);
-                const A gt_k = Store<S>::load(src + paddr(b, k, c), P.inv_scale);
-                const A gt_q = Store<S>::load(src + paddr(b, q, c), P.inv_scale);
-                const A gt_far = far_ok ? Store<S>::load(src + paddr(fb, k, fc), P.inv_scale) : A(0);
-                gq = cli_link<A>(q, d, cli && far_ok, gt_k, gt_q, gt_far, Fr, fl, tl3);
+            } else if (q != 0 && sreal && ssolid == FLAG_SOLID) {
+                const bool far_ok = freal && fsolid != FLAG_SOLID;
+                if (cli && !far_ok) Lk = cli_geometry<A>(q, d, false, Fr);
+                A fl[3], tl3[3];
+                gq = cli_apply<A>(q, Lk, gt_k, gt_q, far_ok ? vfar : A(0), fl, tl3);
                 acc.add(k, pu, fl, tl3);
             }
         }
@@ -533,15 +535,14 @@ __global__ void k_pframes(const ParticleState* __restrict__ ps, PFrames* __restr
 // are listed in shared memory and refilled afterwards, each by one warp of
 // the block in turn (refill_cell_warp: it reads only cells that are fluid
 // before and after the move, which nothing here writes); fluid cells with a
-// solid neighbour are marked for the boundary list (counts per run of
-// LINK_RUN box cells for the ordered compaction).  Neighbour flags are
+// solid neighbour go to the block's segment.  Neighbour flags are
 // evaluated from the same predicate instead of being read back, so no
 // second pass is needed.
 template <typename S>
 __global__ void __launch_bounds__(REMAP_THREADS)
     k_amr_remap(LevelView D, S* __restrict__ pops, const uint8_t* __restrict__ fcur, uint8_t* __restrict__ fnext,
                 BoxDesc B, const ParticleState* __restrict__ ps, typename Store<S>::A scale,
-                typename Store<S>::A inv_scale, uint8_t* __restrict__ mask, int* __restrict__ block_count,
+                typename Store<S>::A inv_scale, int* __restrict__ seg, int* __restrict__ seg_count,
                 int* __restrict__ status, typename Store<S>::A gcoef, const PFrames* __restrict__ frames) {
     using A = typename Store<S>::A;
     __shared__ BoxFrame F;
@@ -555,12 +556,14 @@ __global__ void __launch_bounds__(REMAP_THREADS)
     __syncthreads();
     const ParticleState& P = *ps;
     const int t = blockIdx.x * REMAP_THREADS + threadIdx.x;
-    int is_b = 0;
+    bool is_b = false;
+    int entry = 0;
     if (t < B.cells) {
         int g[3];
         if (box_cell(t, D.n, D.periodic, B, F, g)) {
             int c;
             const int b = locate(D, g, &c);
+            entry = (b << 12) | c;
             if (b < 0 || b >= D.nreal) {
                 atomicOr(status, STATUS_NOT_FINEST);
             } else {
@@ -574,7 +577,7 @@ __global__ void __launch_bounds__(REMAP_THREADS)
 #pragma unroll
                         for (int q = 0; q < 19; ++q) Store<S>::store(pops + paddr(b, q, c), A(0), scale);
                 } else {
-                    is_b = any_nb ? 1 : 0;
+                    is_b = any_nb;
                     fnext[x] = is_b ? FLAG_BOUNDARY : FLAG_FLUID;
                     if (was_solid) {   // uncovered: fluid after the move, solid before
                         const int k = atomicAdd(&s_n, 1);
@@ -587,67 +590,13 @@ __global__ void __launch_bounds__(REMAP_THREADS)
                 }
             }
         }
-        mask[t] = (uint8_t)is_b;
     }
-    __syncthreads();
+    write_segment(is_b, entry, (int)blockIdx.x, seg, seg_count);   // its barrier also completes the shared list
     const int wid = threadIdx.x >> 5;
     for (int k = wid; k < s_n; k += REMAP_THREADS / 32) {
         const int g3[3] = {s_g[0][k], s_g[1][k], s_g[2][k]};
         refill_cell_warp<S>(D, pops, fcur, F, P, s_cell[0][k], s_cell[1][k], g3, scale, inv_scale, gcoef,
                             frames ? &frames->lf : nullptr);
-    }
-    const unsigned ballot = __ballot_sync(0xffffffffu, is_b);
-    __shared__ int wsum[REMAP_THREADS / 32];
-    if ((threadIdx.x & 31) == 0) wsum[wid] = __popc(ballot);
-    __syncthreads();
-    constexpr int RUNS = REMAP_THREADS / LINK_RUN, WPR = LINK_RUN / 32;
-    if ((int)threadIdx.x < RUNS) {
-        const long long run = (long long)blockIdx.x * RUNS + threadIdx.x;
-        if (run * LINK_RUN < B.cells) {
-            int s = 0;
-            for (int w = 0; w < WPR; ++w) s += wsum[threadIdx.x * WPR + w];
-            block_count[run] = s;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(LINK_RUN)
-    k_amr_links_emit(LevelView D, const uint8_t* __restrict__ mask, const int* __restrict__ block_count, BoxDesc B,
-                     const ParticleState* __restrict__ ps, int* __restrict__ list, int* __restrict__ count,
-                     int capacity, int* __restrict__ status) {
-    __shared__ int red[LINK_RUN];
-    __shared__ int wsum[LINK_RUN / 32];
-    __shared__ BoxFrame F;
-    if (threadIdx.x == 0) box_frame_init(F, D.n, D.periodic, B, *ps);
-    int s = 0;
-    for (int b = threadIdx.x; b < (int)blockIdx.x; b += LINK_RUN) s += block_count[b];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int h = LINK_RUN / 2; h > 0; h >>= 1) {
-        if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-        __syncthreads();
-    }
-    const int base = red[0];
-    const int t = blockIdx.x * LINK_RUN + threadIdx.x;
-    const int is_b = t < B.cells ? mask[t] : 0;
-    const unsigned ballot = __ballot_sync(0xffffffffu, is_b);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) wsum[warp] = __popc(ballot);
-    __syncthreads();
-    int wbase = 0;
-    for (int w = 0; w < warp; ++w) wbase += wsum[w];
-    if (is_b) {
-        int g[3], c;
-        const bool in = box_cell(t, D.n, D.periodic, B, F, g);
-        const int b = in ? locate(D, g, &c) : -1;
-        const int pos = base + wbase + __popc(ballot & ((1u << lane) - 1u));
-        if (pos >= capacity) atomicOr(status, STATUS_LINK_OVERFLOW);
-        else if (b >= 0) list[pos] = (b << 12) | c;
-    }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-        int tot = base;
-        for (int w = 0; w < LINK_RUN / 32; ++w) tot += wsum[w];
-        *count = tot < capacity ? tot : capacity;
     }
 }
 
@@ -1532,7 +1481,7 @@ lbmp_status build_layout(lbmp_handle* h, const std::vector<Mask>& R) {
             using A = typename Store<S>::A;
             k_amr_remap<S><<<nb, REMAP_THREADS, 0, h->stream>>>(view(E, Ff), (S*)Ff.d_pops[Ff.cur], Ff.d_flags[1],
                                                                Ff.d_flags[0], h->box, h->d_ps, (A)1, (A)1,
-                                                               h->link_mask, h->link_blocks, h->status, (A)0, nullptr);
+                                                               h->seg, h->seg_count, h->status, (A)0, nullptr);
         });
     }
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(h->stream) != cudaSuccess) return LBMP_ERR_CUDA;
@@ -1674,9 +1623,9 @@ void enqueue_advance(lbmp_handle* h, int l, int sub) {
         }
         cudaEventRecord(E->ev_fork, st);
         cudaStreamWaitEvent(E->side, E->ev_fork, 0);
-        const size_t pre_bytes = sizeof(int) * (size_t)((h->box.cells + LINK_RUN - 1) / LINK_RUN + 1);
+        const size_t pre_bytes = sizeof(int) * (size_t)((h->box.cells + SEG - 1) / SEG + 1);
         k_amr_boundary<S><<<E->boundary_blocks, BNDW_THREADS, pre_bytes, E->side>>>(
-            D, U.src, U.dst, U.solid, h->link_mask, h->link_blocks, h->box, P, h->d_ps, h->cfg.boundary == LBMP_CLI ? 1 : 0,
+            D, U.src, U.dst, U.solid, h->seg, h->seg_count, h->box, P, h->d_ps, h->cfg.boundary == LBMP_CLI ? 1 : 0,
             h->partials, E->d_done, G, h->history, h->cfg.history_capacity, h->status, E->d_frames);
         cudaEventRecord(E->ev_join, E->side);
         h->launches += 1;
@@ -1717,7 +1666,7 @@ void enqueue_advance(lbmp_handle* h, int l, int sub) {
             cudaStreamWaitEvent(st, E->ev_join, 0);
         }
         k_amr_remap<S><<<nl, REMAP_THREADS, 0, rs>>>(D, U.dst, V.d_flags[V.fcur], fnext, h->box, h->d_ps, P.scale,
-                                                    P.inv_scale, h->link_mask, h->link_blocks, h->status,
+                                                    P.inv_scale, h->seg, h->seg_count, h->status,
                                                     (A)grad_refill_coef(h->cfg.refill, V.taup), E->d_frames);
         if (beside) {
             cudaEventRecord(E->ev_remap, E->side);
@@ -1812,15 +1761,17 @@ lbmp_status amr_add_sphere(lbmp_handle* h) {
     const double shell = 4.0 / 3.0 * M_PI * (ro * ro * ro - ri * ri * ri);
     h->list_cap = (int)std::min<double>((double)B.cells, std::ceil(shell) + 64.0);
     h->list = (int*)handle_alloc(h, sizeof(int) * (size_t)h->list_cap);
-    E->boundary_blocks = (int)((B.cells + BND_CHUNK - 1) / BND_CHUNK);
+    E->boundary_blocks = step_boundary_blocks(h->list_cap);
     h->partials = (double*)handle_alloc(h, sizeof(double) * 6 * (size_t)E->boundary_blocks);
     if (!E->d_frames) E->d_frames = (PFrames*)handle_alloc(h, sizeof(PFrames));
     if (!E->d_frames) return LBMP_ERR_OOM;
-    h->link_mask = (uint8_t*)handle_alloc(h, (size_t)B.cells);
-    h->link_blocks = (int*)handle_alloc(h, sizeof(int) * (size_t)((B.cells + LINK_RUN - 1) / LINK_RUN));
-    if (!h->list || !h->partials || !h->link_mask || !h->link_blocks) return LBMP_ERR_OOM;
-    // the boundary kernel keeps a prefix of the remap's run counts in dynamic shared memory
-    const int pre_bytes = (int)(sizeof(int) * ((B.cells + LINK_RUN - 1) / LINK_RUN + 1));
+    const size_t nseg = (size_t)((B.cells + SEG - 1) / SEG);
+    h->seg = (int*)handle_alloc(h, sizeof(int) * SEG * nseg);
+    h->seg_count = (int*)handle_alloc(h, sizeof(int) * nseg);
+    if (!h->list || !h->partials || !h->seg || !h->seg_count) return LBMP_ERR_OOM;
+    // the boundary kernel keeps a prefix of the segments' numbers in dynamic shared memory; the limit on the sphere
+    // is that of a count per 64 box cells
+    const int pre_bytes = (int)(sizeof(int) * ((B.cells + 63) / 64 + 1));
     bool attr_ok = true;
     with_storage_amr(h->cfg.precision, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
@@ -2217,13 +2168,7 @@ lbmp_status amr_links(lbmp_handle* h, int64_t* cell, int32_t* q, double* delta, 
     AmrEngine* E = h->amr;
     *n = 0;
     if (!h->has_particle) return LBMP_OK;
-    // the step keeps the boundary cells as a mask in box order; compact it for the export
-    {
-        const Level& Vf = E->lv[E->L - 1];
-        const unsigned nl = (unsigned)((h->box.cells + LINK_RUN - 1) / LINK_RUN);
-        k_amr_links_emit<<<nl, LINK_RUN, 0, h->stream>>>(view(E, Vf), h->link_mask, h->link_blocks, h->box,
-                                                             h->d_ps, h->list, h->count, h->list_cap, h->status);
-    }
+    launch_list_segments(h, h->stream);   // the step keeps the boundary cells in segments
     int cnt = 0;
     if (cudaMemcpyAsync(&cnt, h->count, sizeof(int), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
         cudaStreamSynchronize(h->stream) != cudaSuccess)

@@ -209,8 +209,7 @@ struct lbmp_handle {
     int* list = nullptr;                 // boundary cells
     int* count = nullptr;
     int list_cap = 0;
-    uint8_t* link_mask = nullptr;        // marks of the box cells around the sphere (one byte each)
-    int* link_blocks = nullptr;          // refined grids: boundary cells per run of box cells
+    uint8_t* link_mask = nullptr;        // uniform grids: marks of the box cells around the sphere (one byte each)
     int* seg = nullptr;                  // boundary cells by segment of the box (an entry per box cell)
     int* seg_count = nullptr;            // and their number per segment
     double* partials = nullptr;

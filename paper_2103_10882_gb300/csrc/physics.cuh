@@ -1007,8 +1007,6 @@ __device__ __forceinline__ bool last_block_done(int* counter, int nblocks) {
     return last != 0;
 }
 
-constexpr int LINK_RUN = 64;   // box cells per run of the boundary marks (one count per run)
-
 // Exclusive prefix of n counts into pre[0..n] (pre[n] = total), computed by
 // the whole CTA (NT threads, two consecutive counts per thread and pass);
 // every thread must call it.  first0, first1: counts 2 threadIdx.x and
@@ -1052,35 +1050,6 @@ __device__ __forceinline__ int block_prefix(const int* __restrict__ count, int n
     if (threadIdx.x == 0) pre[0] = 0;
     __syncthreads();
     return pre[n];
-}
-
-// Box cell of the j-th marked one (mask byte 1, box order): the run r that holds it is the largest with
-// pre[r] <= j (pre: the prefix of the runs' counts), the cell the (j - pre[r])-th marked one of that run.  The whole
-// warp calls it with the same j.
-__device__ __forceinline__ int marked_cell(const int* pre, int runs, const uint8_t* __restrict__ mask, long long cells,
-                                           int j) {
-    static_assert(LINK_RUN == 64, "two ballots per run");
-    const int lane = threadIdx.x & 31;
-    int lo = 0, hi = runs;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (pre[mid] <= j) lo = mid;
-        else hi = mid;
-    }
-    const long long r0 = (long long)lo * LINK_RUN;
-    const bool m0 = r0 + lane < cells && mask[r0 + lane] == 1;
-    const bool m1 = r0 + 32 + lane < cells && mask[r0 + 32 + lane] == 1;
-    const unsigned b0 = __ballot_sync(0xffffffffu, m0), b1 = __ballot_sync(0xffffffffu, m1);
-    int k = j - pre[lo];
-    unsigned bits = b0;
-    int base = 0;
-    if (k >= __popc(b0)) {
-        k -= __popc(b0);
-        bits = b1;
-        base = 32;
-    }
-    for (; k > 0; --k) bits &= bits - 1u;   // drop the k lowest marked cells
-    return (int)(r0 + base + __ffs((int)bits) - 1);
 }
 
 // Boundary cells in segments: the remap CTA of 256 box cells writes its marked cells, in box order, to the first
