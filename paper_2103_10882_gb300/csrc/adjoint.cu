@@ -351,7 +351,7 @@ __device__ __forceinline__ void reverse_plain(const ReverseArgs<S>& T, unsigned 
     for (int q = 0; q < 19; ++q) {
         const int src = xs[1 + cx(q)] + G.nx * (ys[1 + cy(q)] + G.ny * zs[1 + cz(q)]);
         const int dn = xs[1 - cx(q)] + G.nx * (ys[1 - cy(q)] + G.ny * zs[1 - cz(q)]);
-        h[q] = Store<S>::load(T.gprev + (size_t)q * n + src, A(1));
+        h[q] = Store<S>::fetch(T.gprev + (size_t)q * n + src, A(1));
         lam[q] = T.nu_next[(size_t)q * n + dn];
     }
     if (kd == KIND_SOLID) {
@@ -393,10 +393,10 @@ __device__ __forceinline__ void reverse_near(const ReverseArgs<S>& T, typename S
             const long long y = cell_at(G, p[0] + c[0], p[1] + c[1], p[2] + c[2]);
             const long long yy = cell_at(G, p[0] + 2 * c[0], p[1] + 2 * c[1], p[2] + 2 * c[2]);
             const bool s_solid = T.flags[s] != 0, y_solid = T.flags[y] != 0, yy_solid = T.flags[yy] != 0;
-            const A g_s = Store<S>::load(T.gprev + (size_t)q * n + s, A(1));
-            const A g_k = Store<S>::load(T.gprev + (size_t)k * n + x, A(1));
-            const A g_q = Store<S>::load(T.gprev + (size_t)q * n + x, A(1));
-            const A g_far = Store<S>::load(T.gprev + (size_t)k * n + y, A(1));
+            const A g_s = Store<S>::fetch(T.gprev + (size_t)q * n + s, A(1));
+            const A g_k = Store<S>::fetch(T.gprev + (size_t)k * n + x, A(1));
+            const A g_q = Store<S>::fetch(T.gprev + (size_t)q * n + x, A(1));
+            const A g_far = Store<S>::fetch(T.gprev + (size_t)k * n + y, A(1));
             const A nu_y = T.nu_next[(size_t)q * n + y], nu_yk = T.nu_next[(size_t)k * n + y];
             const A nu_k = T.nu_next[(size_t)k * n + x], nu_q = T.nu_next[(size_t)q * n + x];
             const int ca = c[T.P.axis];

@@ -379,14 +379,21 @@ __global__ void __maxnreg__(BND_MAXREG<S>)
     const int nseg = (int)((B.cells + SEG - 1) / SEG);
     const int i2 = 2 * (int)threadIdx.x;   // this thread's first two numbers, in flight during the set-up
     const int first0 = i2 < nseg ? seg_count[i2] : 0, first1 = i2 + 1 < nseg ? seg_count[i2 + 1] : 0;
+    __shared__ double sX[3];
     if (threadIdx.x == BNDW_THREADS - 1) Fr = pframe_link<A>(*frames);   // formed by the last particle update
+    if (threadIdx.x >= BNDW_THREADS - 32 && threadIdx.x < BNDW_THREADS - 29)
+        sX[threadIdx.x - (BNDW_THREADS - 32)] = ps->x[threadIdx.x - (BNDW_THREADS - 32)];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int total = block_prefix<BNDW_THREADS>(seg_count, nseg, pre, first0, first1);
     const int W = (int)gridDim.x * (BNDW_THREADS / 32);
     const int q = lane < 19 ? lane : 0, k = opp(q);
     const int cq[3] = {cx(q), cy(q), cz(q)};
     LinkSums<A> acc;
+    // a warp's last cell is stored after the hand-off: the hand-off's release waits for the stores before it
+    A kept = A(0);
+    S* kept_at = nullptr;
     for (int j = (int)blockIdx.x * (BNDW_THREADS / 32) + wib; j < total; j += W) {
+        if (kept_at) Store<S>::store(kept_at, kept, P.scale);
         const int sg = find_segment(pre, nseg, j);
         const int e = seg[sg * SEG + (j - pre[sg])];
         const int b = e >> 12, c = e & 4095;
@@ -421,14 +428,16 @@ __global__ void __maxnreg__(BND_MAXREG<S>)
                 acc.add(k, pu, fl, tl3);
             }
         }
-        gq = warp_trt_collide<A, false>(gq, lane, P, status);
-        if (lane < 19) Store<S>::store(dst + paddr(b, lane, c), gq, P.scale);
+        kept = warp_trt_collide<A, false>(gq, lane, P, status);
+        if (lane < 19) kept_at = dst + paddr(b, lane, c);
     }
-    block_link_sums<BNDW_THREADS>(acc, ps->x, partials + (size_t)blockIdx.x * 6);
-    if (last_block_done(done, (int)gridDim.x)) {   // every other block is past its use of the frames
-        particle_block_update<BNDW_THREADS>(ps, partials, gridDim.x, G, history, hist_cap, status, frames->inv,
-                                            [&](const ParticleState& Q, int a) { pframes_axis(frames, Q, D.n, B, a); });
-    }
+    block_link_sums<BNDW_THREADS>(acc, sX, partials + blockIdx.x, (int)gridDim.x);
+    const bool last = last_block_done(done, (int)gridDim.x);   // every other block is past its use of the frames
+    if (kept_at) Store<S>::store(kept_at, kept, P.scale);
+    if (last)
+        particle_block_update<BNDW_THREADS>(
+            ps, partials, gridDim.x, G, history, hist_cap, status, frames->inv,
+            [&](const ParticleState& Q, int a, int part) { pframes_axis(frames, Q, D.n, B, a, part); });
 }
 
 

@@ -170,7 +170,7 @@ __global__ void __maxnreg__(BND_MAXREG<S>)
         gq = warp_trt_collide<A, false>(gq, lane, P, status);
         if (lane < 19) Store<S>::store(d0 + (size_t)lane * n + cell, gq, P.scale);
     }
-    block_link_sums<BW>(acc, ps[sim].x, partials + (size_t)blockIdx.x * 6);
+    block_link_sums<BW>(acc, ps[sim].x, partials + (size_t)D.bnd_off * 6 + (blockIdx.x - D.bnd_off), D.bnd_n);
     if (last_block_done(done + sim, D.bnd_n))
         particle_block_update<BW>(ps + sim, partials + (size_t)D.bnd_off * 6, D.bnd_n, G,
                                   history + (size_t)D.hist_off * 15, hist_cap, status);

@@ -38,12 +38,15 @@ __host__ __device__ constexpr T wgt(int q) {
 //   double : FP64 storage, FP64 arithmetic
 //   float  : FP32 storage, FP32 arithmetic
 //   __half : FP16 storage of g * 2^s, FP32 arithmetic
+// load reads through the non-coherent path (data that nothing writes while the kernel is resident); fetch is an
+// ordinary load, for kernels that become resident while the kernel ahead still writes (pdl_wait).
 template <typename S>
 struct Store;
 template <>
 struct Store<double> {
     using A = double;
     __device__ static __forceinline__ A load(const double* p, A) { return __ldg(p); }
+    __device__ static __forceinline__ A fetch(const double* p, A) { return *p; }
     __device__ static __forceinline__ void store(double* p, A v, A) { __stcs(p, v); }
     __device__ static __forceinline__ A load_raw(const double* p) { return __ldg(p); }
     __device__ static __forceinline__ void store_raw(double* p, A v) { __stcs(p, v); }
@@ -52,6 +55,7 @@ template <>
 struct Store<float> {
     using A = float;
     __device__ static __forceinline__ A load(const float* p, A) { return __ldg(p); }
+    __device__ static __forceinline__ A fetch(const float* p, A) { return *p; }
     __device__ static __forceinline__ void store(float* p, A v, A) { __stcs(p, v); }
     __device__ static __forceinline__ A load_raw(const float* p) { return __ldg(p); }
     __device__ static __forceinline__ void store_raw(float* p, A v) { __stcs(p, v); }
@@ -63,6 +67,7 @@ struct Store<__half> {
     __device__ static __forceinline__ A load(const __half* p, A inv_scale) {
         return __half2float(__ldg(p)) * inv_scale;
     }
+    __device__ static __forceinline__ A fetch(const __half* p, A inv_scale) { return __half2float(*p) * inv_scale; }
     __device__ static __forceinline__ void store(__half* p, A v, A scale) { *p = __float2half_rn(v * scale); }
     // the stored value g * 2^s itself (kernels that work on the scaled values)
     __device__ static __forceinline__ A load_raw(const __half* p) { return __half2float(__ldg(p)); }

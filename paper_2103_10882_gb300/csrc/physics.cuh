@@ -3,6 +3,8 @@
 // the CLI boundary (Sec. 2.3).
 #pragma once
 
+#include <cstddef>
+
 #include "internal.h"
 
 namespace lbmp {
@@ -10,7 +12,8 @@ namespace lbmp {
 // Programmatic dependent launch (PTX griddepcontrol): the CTAs of a kernel launched with the attribute may become
 // resident once every CTA of the kernel ahead has called pdl_trigger or ended; pdl_wait returns when that kernel has
 // completed and its writes are visible.  Every thread waits before it reads or writes global memory, so only the
-// launch itself overlaps.  Kernels launched without the attribute pass both at once.  Measured (with the boundary
+// launch itself overlaps; loads are ordinary ones (Store::fetch), as the kernel ahead may write while this one is
+// resident.  Kernels launched without the attribute pass both at once.  Measured (with the boundary
 // cells' loads issued together): a 32^3 FP32 step 23.4 -> 20.7 us, 64 x 64 x 128 with MRT 29.7 -> 27.1, 256^3 in FP16
 // storage 284 -> 277 (also four CTAs per SM there instead of three).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -477,8 +480,8 @@ __device__ __forceinline__ void df_add(float& h, float& l, float bh, float bl) {
     l = e - (h - s);
 }
 
-// Deterministic block sum of the threads' link sums into out[0..5]: force,
-// and torque about X.  Every thread of the block must call it.  FP64
+// Deterministic block sum of the threads' link sums into out[c * stride], c = 0..5: force,
+// and torque about X (best in shared memory: it is read last).  Every thread of the block must call it.  FP64
 // additions, and conversions to FP64, are slow and narrow on this GPU, so
 // in FP32 the lanes' sums (each with its TwoSum error) are reduced as
 // double-float pairs, a butterfly within each warp and, after one barrier,
@@ -490,7 +493,8 @@ __device__ __forceinline__ void df_add(float& h, float& l, float bh, float bl) {
 // the reciprocals.  A last-block hand-off after this call is ordered by its
 // barrier and release (the writers need no fence of their own).
 template <int NT, typename A>
-__device__ __forceinline__ void block_link_sums(const LinkSums<A>& acc, const double X[3], double* __restrict__ out) {
+__device__ __forceinline__ void block_link_sums(const LinkSums<A>& acc, const double X[3], double* __restrict__ out,
+                                                int stride) {
     static_assert(NT % 32 == 0 && NT >= 192 && NT <= 1024, "six warps take the six components");
     constexpr int NW = NT / 32;
     constexpr int SPAN = NW <= 8 ? 8 : (NW <= 16 ? 16 : 32);   // lanes of the cross-warp butterfly
@@ -590,10 +594,10 @@ __device__ __forceinline__ void block_link_sums(const LinkSums<A>& acc, const do
     const double r36 = 1.0 / 36.0, r72 = 1.0 / 72.0;
     const double fr[3] = {(double)iF[0] * r36, (double)iF[1] * r36, (double)iF[2] * r36};
     if (c < 3) {
-        out[c] = t + pick3(fr, c);
+        out[(size_t)c * stride] = t + pick3(fr, c);
     } else {
         const int a1 = c == 3 ? 1 : (c == 4 ? 2 : 0), a2 = c == 3 ? 2 : (c == 4 ? 0 : 1);
-        out[c] = t + ((double)iT * r72 - (X[a1] * pick3(fr, a2) - X[a2] * pick3(fr, a1)));
+        out[(size_t)c * stride] = t + ((double)iT * r72 - (X[a1] * pick3(fr, a2) - X[a2] * pick3(fr, a1)));
     }
 }
 
@@ -690,25 +694,33 @@ __device__ __forceinline__ void pframes_form(PFrames* __restrict__ F, const Part
     else if (threadIdx.x == 97) F->inv[1] = 1.0 / particle_inertia(P);
 }
 
-// The parts of F that follow the sphere along axis a (a = 0, 1, 2 by lanes
-// 0, 1, 2 of one warp) after the particle update: the same values as
-// pframes_form, from a shorter FP64 sequence (floor by one conversion, the
-// box origin from the fraction); the radius and the FP32 pre-test bounds do
-// not change during a run and keep the values pframes_form gave them.
+// |v| as an integer that orders like it (NaN above infinity).
+__device__ __forceinline__ long long abs_bits(double v) { return __double_as_longlong(v) & 0x7fffffffffffffffll; }
+
+// The parts of F that follow the sphere along axis a after the particle update, positions (part 0) and velocities
+// (part 1) by different warps: the same values as pframes_form, from a shorter FP64 sequence (floor by one conversion,
+// the box origin from the fraction); the radius and the FP32 pre-test bounds do not change during a run and keep the
+// values pframes_form gave them.
 __device__ __forceinline__ void pframes_axis(PFrames* __restrict__ F, const ParticleState& P, const int n[3],
-                                             const BoxDesc& B, int a) {
+                                             const BoxDesc& B, int a, int part) {
+    if (part == 1) {
+        F->lf.u[a] = (float)P.u[a];
+        F->lf.w[a] = (float)P.w[a];
+        F->ld.u[a] = P.u[a];
+        F->ld.w[a] = P.w[a];
+        return;
+    }
     const double xr = P.x[a];
-    const double x = fabs(xr) < 1e9 ? xr : 0.0;   // as box_frame_init: keep the box arithmetic in range
-    const int xi = __double2int_rd(xr), bi = __double2int_rd(x);
-    const double frac = xr - (double)xi, bfrac = x - (double)bi;
+    const bool sane = abs_bits(xr) < abs_bits(1e9);   // as box_frame_init: keep the box arithmetic in range
+    const int xi = __double2int_rd(xr);
+    const double frac = xr - (double)xi;
+    const int bi = sane ? xi : 0;
+    const double bfrac = sane ? frac : 0.0;
+    const double xh = 0.5 - frac;
     F->lf.Xi[a] = xi;
     F->ld.Xi[a] = xi;
-    F->ld.Xh[a] = 0.5 - frac;
-    F->lf.Xh[a] = (float)(0.5 - frac);
-    F->lf.u[a] = (float)P.u[a];
-    F->lf.w[a] = (float)P.w[a];
-    F->ld.u[a] = P.u[a];
-    F->ld.w[a] = P.w[a];
+    F->ld.Xh[a] = xh;
+    F->lf.Xh[a] = (float)xh;
     F->bf.Xi[a] = bi;
     F->bf.Xh[a] = (float)(0.5 - bfrac);
     // floor(x - 1/2): x - 1/2 and x - floor(x) are exact
@@ -805,75 +817,70 @@ __device__ __forceinline__ double particle_inertia(const ParticleState& P) {
     return 0.4 * (P.rho_p + P.cvw) * P.V * P.r * P.r;
 }
 
-// One axis a of Algorithm 1's particle update: average of the hydrodynamic
-// force and torque over two steps, gravity/buoyancy, the virtual force and
-// torque from the previous accelerations, and the kick-drift-kick update
-// with the virtually increased mass and moment of inertia, whose inverses
-// the caller passes (particle_mass, particle_inertia).  The axes are
-// independent; P.steps is advanced once afterwards.
-__device__ __forceinline__ void particle_advance_axis(ParticleState& P, int a, double Fh, double Th, double inv_m,
-                                                      double inv_I, const GridDesc& G, double* __restrict__ history,
-                                                      int hist_cap, int* __restrict__ status) {
-    const double V = P.V, r = P.r;
-    const bool avg = P.force_average && P.steps > 0;
-    const double Fbar = avg ? 0.5 * (Fh + P.Fh_old[a]) : Fh;
-    const double Tbar = avg ? 0.5 * (Th + P.Th_old[a]) : Th;
-    P.Fh[a] = Fh;
-    P.Th[a] = Th;
-    P.Fh_old[a] = Fh;
-    P.Th_old[a] = Th;
-    const double Fg = (P.rho_p - 1.0) * P.g[a] * V;
-    const double Fv = P.cv * V * P.a[a];
-    const double Tv = 0.4 * P.cvw * V * r * r * P.b[a];
-    const double Fp = Fbar + Fg + Fv;
-    const double Tp = Tbar + Tv;
-    P.Fp[a] = Fp;
-    const double xold = P.x[a];
-    const double acc = Fp * inv_m, bet = Tp * inv_I;
-    // A held group (translation; rotation) keeps its velocity and records zero acceleration, so the
-    // virtual force or torque after it is zero; a group released in this step starts afresh, with
-    // no half kick completing a previous step.
-    const bool tfree = P.fixed == 0, rfree = P.fixed != 1;
-    const bool tprev = P.steps > 0 && P.prev_fixed == 0, rprev = P.steps > 0 && P.prev_fixed != 1;
-    if (tfree) {
-        if (tprev) P.u[a] += 0.5 * acc;   // second half kick of the previous step completes u(t)
-        P.a[a] = acc;
-        P.u[a] += 0.5 * acc;   // first half kick, then drift with u(t + 1/2)
-        P.x[a] += P.u[a];
-    } else {
-        P.a[a] = 0.0;
-    }
-    if (rfree) {
-        if (rprev) P.w[a] += 0.5 * bet;
-        P.b[a] = bet;
-        P.w[a] += 0.5 * bet;
-    } else {
-        P.b[a] = 0.0;
-    }
-    if (!(fabs(P.x[a] - xold) <= 0.5) || !(fabs(P.u[a]) < 0.5) || !(fabs(P.w[a]) < 1e30)) {
-        // a jump or a non-finite state: flag it, and keep the sphere where it was and at rest, so that
-        // the box kernels that follow until the host reads the status stay inside the domain
-        atomicOr(status, STATUS_PARTICLE_JUMP);
-        P.x[a] = xold;
-        P.u[a] = P.w[a] = P.a[a] = P.b[a] = 0.0;
-    }
+// One axis a of Algorithm 1's particle update, translation and rotation each by a thread of its own (of different
+// warps: a scheduler issues one FP64 instruction in about 76 cycles): average of the hydrodynamic force or torque over
+// two steps, gravity/buoyancy (Fg) and the virtual force (Fv) or torque (Tv) from the previous accelerations, and the
+// kick-drift-kick update with the virtually increased mass or moment of inertia, whose inverses the caller passes.
+// A held group (translation; rotation) keeps its velocity and records zero acceleration, so the virtual force or
+// torque after it is zero; a group released in this step starts afresh, with no half kick completing a previous step.
+// Both return false for a jump or a non-finite state (!(|x - xold| <= 1/2), !(|u| < 1/2); !(|w| < 1e30)), compared as
+// integers, which order non-negative doubles alike and put NaN above infinity.
+
+__device__ __forceinline__ void wrap_centre(ParticleState& P, int a, const GridDesc& G) {   // into the periodic box
     const int n = a == 0 ? G.nx : (a == 1 ? G.ny : G.nz);
-    if (G.periodic[a]) {   // keep the centre inside the periodic box
+    if (G.periodic[a]) {
         const double L = (double)n;
         if (P.x[a] >= L) P.x[a] -= L;
         else if (P.x[a] < 0.0) P.x[a] += L;
     }
-    if (hist_cap > 0) {
-        double* h = history + (size_t)(P.steps % hist_cap) * 15;
-        h[a] = Fh;
-        h[3 + a] = Th;
-        h[6 + a] = P.x[a];
-        h[9 + a] = P.u[a];
-        h[12 + a] = P.w[a];
-    }
 }
 
-// Sum of component comp over the nblocks force partials by one warp, in a fixed order (every lane gets it).
+__device__ __forceinline__ bool advance_translation(ParticleState& P, int a, double Fh, double Fg, double Fv, double inv_m,
+                                                    const GridDesc& G) {
+    const bool avg = P.force_average && P.steps > 0;
+    const double Fbar = avg ? 0.5 * (Fh + P.Fh_old[a]) : Fh;
+    P.Fh[a] = Fh;
+    P.Fh_old[a] = Fh;
+    const double Fp = Fbar + Fg + Fv;
+    P.Fp[a] = Fp;
+    const double xold = P.x[a];
+    const double acc = Fp * inv_m;
+    if (P.fixed == 0) {
+        double u = P.u[a];
+        if (P.steps > 0 && P.prev_fixed == 0) u += 0.5 * acc;   // second half kick of the previous step completes u(t)
+        u += 0.5 * acc;   // first half kick, then drift with u(t + 1/2)
+        P.a[a] = acc;
+        P.u[a] = u;
+        P.x[a] = xold + u;
+    } else {
+        P.a[a] = 0.0;
+    }
+    const bool ok = abs_bits(P.x[a] - xold) <= abs_bits(0.5) && abs_bits(P.u[a]) < abs_bits(0.5);
+    if (ok) wrap_centre(P, a, G);
+    return ok;
+}
+
+__device__ __forceinline__ bool advance_rotation(ParticleState& P, int a, double Th, double Tv, double inv_I) {
+    const bool avg = P.force_average && P.steps > 0;
+    const double Tbar = avg ? 0.5 * (Th + P.Th_old[a]) : Th;
+    P.Th[a] = Th;
+    P.Th_old[a] = Th;
+    const double Tp = Tbar + Tv;
+    const double bet = Tp * inv_I;
+    if (P.fixed != 1) {
+        double w = P.w[a];
+        if (P.steps > 0 && P.prev_fixed != 1) w += 0.5 * bet;
+        w += 0.5 * bet;
+        P.b[a] = bet;
+        P.w[a] = w;
+    } else {
+        P.b[a] = 0.0;
+    }
+    return abs_bits(P.w[a]) < abs_bits(1e30);
+}
+
+// Sum of component comp over the nblocks force partials ([component][block]) by one warp, in a fixed order (every lane
+// gets it).
 __device__ __forceinline__ double sum_partials(const double* partials, int nblocks, int comp) {
     const int lane = threadIdx.x & 31;
     // Lane l sums partials l, l + 64, ... into s0 and l + 32, l + 96, ... into s1, in that
@@ -884,7 +891,7 @@ __device__ __forceinline__ double sum_partials(const double* partials, int nbloc
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int b = base + lane + 32 * k;
-            v[k] = b < nblocks ? __ldcg(partials + (size_t)b * 6 + comp) : 0.0;
+            v[k] = b < nblocks ? __ldcg(partials + (size_t)comp * nblocks + b) : 0.0;
         }
 #pragma unroll
         for (int k = 0; k < 8; k += 2) {
@@ -899,16 +906,19 @@ __device__ __forceinline__ double sum_partials(const double* partials, int nbloc
 }
 
 // Particle update by one block of NT >= 256 threads once the nblocks force
-// partials are complete: warps 0..5 sum one component each in a fixed
-// order (lane l takes partials l, l + 32, ... in two alternating sums, then
-// a butterfly runs across the lanes), warp 6 forms 1/m and 1/I, warp 7
-// stages the record in shared memory; threads 0..2 then advance the three
-// axes and the block writes the record back.  The partials may come from
-// other blocks of the same launch: they are read through L2.  Every thread
-// of the block must call it.
-// after(P, a): called by the thread of axis a with the advanced record (in shared memory).
+// partials ([component][block]) are complete: warps 0..5 sum one component
+// each in a fixed order (lane l takes partials l, l + 32, ... in two
+// alternating sums, then a butterfly runs across the lanes), warp 6 forms
+// 1/m, 1/I and the forces known beforehand, warp 7 stages the record in
+// shared memory.  Then warp 0 advances the translation and warp 1 the
+// rotation, a lane per axis, and all of the block writes record and history.
+// The partials may come from other blocks of the same launch: they are read
+// through L2.  Every thread of the block must call it.
+// after(P, a, part): called with the advanced record (in shared memory) by the lanes of warp 2 (part 0, for what
+// follows the position) and of warp 3 (part 1, the velocities), a lane per axis.
+// Measured on the rising sphere's boundary launch: 3.7 us when one warp advanced both groups and all else followed it.
 struct NoAfter {
-    __device__ __forceinline__ void operator()(const ParticleState&, int) const {}
+    __device__ __forceinline__ void operator()(const ParticleState&, int, int) const {}
 };
 template <int NT, typename After = NoAfter>
 __device__ __forceinline__ void particle_block_update(ParticleState* __restrict__ ps, const double* partials,
@@ -917,14 +927,25 @@ __device__ __forceinline__ void particle_block_update(ParticleState* __restrict_
                                                       const double* __restrict__ inv = nullptr, After after = After{}) {
     static_assert(NT % 32 == 0 && NT >= 256, "eight warps share the work");
     constexpr int words = (int)(sizeof(ParticleState) / sizeof(int));
-    __shared__ double sFT[6], sinv[2];
+    __shared__ double sFT[6], sinv[2], sFg[3], sFv[3], sTv[3];
     __shared__ ParticleState sP;
+    __shared__ double xold[3];
+    __shared__ int bad[2][3];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (wid < 6) {
         const double t = sum_partials(partials, nblocks, wid);
         if (lane == 0) sFT[wid] = t;
     } else if (wid == 6) {
-        if (lane < 2) sinv[lane] = inv ? inv[lane] : 1.0 / (lane == 0 ? particle_mass(*ps) : particle_inertia(*ps));
+        if (lane < 2) {
+            sinv[lane] = inv ? inv[lane] : 1.0 / (lane == 0 ? particle_mass(*ps) : particle_inertia(*ps));
+        } else if (lane >= 8 && lane < 11) {
+            const int a = lane - 8;
+            const double V = ps->V, r = ps->r;
+            sFg[a] = (ps->rho_p - 1.0) * ps->g[a] * V;
+            sFv[a] = ps->cv * V * ps->a[a];
+            sTv[a] = 0.4 * ps->cvw * V * r * r * ps->b[a];
+            xold[a] = ps->x[a];
+        }
     } else if (wid == 7) {
         const int* srcw = reinterpret_cast<const int*>(ps);
         int* dstw = reinterpret_cast<int*>(&sP);
@@ -932,21 +953,40 @@ __device__ __forceinline__ void particle_block_update(ParticleState* __restrict_
         for (int i = lane; i < words; i += 32) dstw[i] = __ldcg(srcw + i);
     }
     __syncthreads();
-    if (threadIdx.x < 3) {   // the three axes in parallel
-        particle_advance_axis(sP, threadIdx.x, sFT[threadIdx.x], sFT[3 + threadIdx.x], sinv[0], sinv[1], G, history,
-                              hist_cap, status);
-        after(sP, (int)threadIdx.x);
-    }
+    if (wid == 0 && lane < 3) bad[0][lane] = !advance_translation(sP, lane, sFT[lane], sFg[lane], sFv[lane], sinv[0], G);
+    if (wid == 1 && lane < 3) bad[1][lane] = !advance_rotation(sP, lane, sFT[3 + lane], sTv[lane], sinv[1]);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        sP.steps += 1;
-        sP.prev_fixed = sP.fixed;
+    if ((bad[0][0] | bad[0][1] | bad[0][2] | bad[1][0] | bad[1][1] | bad[1][2]) != 0) {   // uniform across the block
+        // a jump or a non-finite state: flag it, and keep the sphere where it was and at rest, so that
+        // the box kernels that follow until the host reads the status stay inside the domain
+        const int a = threadIdx.x;
+        if (a < 3 && (bad[0][a] | bad[1][a])) {
+            atomicOr(status, STATUS_PARTICLE_JUMP);
+            sP.x[a] = xold[a];
+            sP.u[a] = sP.w[a] = sP.a[a] = sP.b[a] = 0.0;
+            wrap_centre(sP, a, G);
+        }
+        __syncthreads();
     }
-    __syncthreads();
+    if (wid == 2 && lane < 3) after(sP, lane, 0);
+    if (wid == 3 && lane < 3) after(sP, lane, 1);
+    if (wid == 0 && lane < 15 && hist_cap > 0) {   // F_hyd, T_hyd, x_p, u_p, omega_p
+        const int a = lane % 3, f = lane / 3;
+        const double v = f == 0 ? sP.Fh[a] : (f == 1 ? sP.Th[a] : (f == 2 ? sP.x[a] : (f == 3 ? sP.u[a] : sP.w[a])));
+        history[(size_t)(sP.steps % hist_cap) * 15 + lane] = v;
+    }
     {
         const int* srcw = reinterpret_cast<const int*>(&sP);
         int* dstw = reinterpret_cast<int*>(ps);
-        for (int i = threadIdx.x; i < words; i += NT) dstw[i] = srcw[i];
+        constexpr int at_steps = (int)(offsetof(ParticleState, steps) / sizeof(int));
+        constexpr int at_prev = (int)(offsetof(ParticleState, prev_fixed) / sizeof(int));
+        for (int i = (int)threadIdx.x - 128; i >= 0 && i < words; i += NT - 128) {
+            int v = srcw[i];
+            if (i == at_steps) v = (int)(unsigned)(unsigned long long)(sP.steps + 1);
+            if (i == at_steps + 1) v = (int)((sP.steps + 1) >> 32);
+            if (i == at_prev) v = sP.fixed;
+            dstw[i] = v;
+        }
     }
 }
 

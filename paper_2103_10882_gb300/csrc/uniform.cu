@@ -105,10 +105,10 @@ __device__ __forceinline__ void bulk_cells(const StepArgs<S>& T, unsigned item) 
         const int sx = xs[cx(q) + 1], sy = ys[cy(q) + 1], sz = zs[cz(q) + 1];
         if (WALLS && (sx < 0 || sy < 0 || sz < 0)) {   // no-slip wall: bounce-back (moving: Ladd's term)
             const int xyz[3] = {x, y, z};
-            g[q] = Store<S>::load(T.src + (size_t)opp(q) * n + cell, T.P.inv_scale) + wall_term<A>(G, q, xyz);
+            g[q] = Store<S>::fetch(T.src + (size_t)opp(q) * n + cell, T.P.inv_scale) + wall_term<A>(G, q, xyz);
         } else {
             const int off = sx + nx * (sy + ny * sz);
-            g[q] = Store<S>::load(T.src + (size_t)q * n + off, T.P.inv_scale);
+            g[q] = Store<S>::fetch(T.src + (size_t)q * n + off, T.P.inv_scale);
         }
     }
     const uint8_t mark = box >= 0 ? T.mark[box] : MARK_PLAIN;   // beside the pulls, not before them
@@ -166,11 +166,11 @@ __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, unsigned p
         yw[q] = WALLS && (sy < 0 || sz < 0);
         const int row = nx * ((yw[q] ? yy : sy) + ny * (yw[q] ? z : sz));
         const __half* pq = src + (size_t)q * n;
-        pr[q] = __ldg(reinterpret_cast<const __half2*>(pq + row + x));
+        pr[q] = *reinterpret_cast<const __half2*>(pq + row + x);
         if (cx(q) != 0) {
             const int xe = cx(q) == 1 ? xm : xq;
             const bool need = cx(q) == 1 ? first : last;
-            ex[q] = __ldg(pq + row + ((need && xe >= 0) ? xe : x));
+            ex[q] = pq[row + ((need && xe >= 0) ? xe : x)];
         }
     }
     const uint8_t mark0 = box0 >= 0 ? T.mark[box0] : MARK_PLAIN, mark1 = box1 >= 0 ? T.mark[box1] : MARK_PLAIN;
@@ -239,7 +239,10 @@ __device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int bid, in
     const S* src = T.src;
     __shared__ LinkFrame<A> Fr;
     const int nseg = (int)((T.B.cells + SEG - 1) / SEG);
+    __shared__ double sX[3];
     if (threadIdx.x == STEP_THREADS - 1) Fr = pframe_link<A>(*T.frames);
+    if (threadIdx.x >= STEP_THREADS - 32 && threadIdx.x < STEP_THREADS - 29)
+        sX[threadIdx.x - (STEP_THREADS - 32)] = T.ps->x[threadIdx.x - (STEP_THREADS - 32)];
     const int i2 = 2 * (int)threadIdx.x;
     int total;
     if (T.list) {
@@ -256,7 +259,11 @@ __device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int bid, in
     const int q = lane < 19 ? lane : 0, k = opp(q);
     const int c[3] = {cx(q), cy(q), cz(q)};
     LinkSums<A> acc;
+    // a warp's last cell is stored after the hand-off: the hand-off's release waits for the stores before it
+    A kept = A(0);
+    S* kept_at = nullptr;
     for (int j = bid * (STEP_THREADS / 32) + wib; j < total; j += W) {
+        if (kept_at) Store<S>::store(kept_at, kept, P.scale);
         int at = j;
         if (!T.list) {
             const int sg = find_segment(pre, nseg, j);
@@ -281,10 +288,10 @@ __device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int bid, in
             const size_t sidx = wall ? cell : (size_t)s3[0] + (size_t)G.nx * ((size_t)s3[1] + (size_t)G.ny * (size_t)s3[2]);
             const size_t far = far_ok ? (size_t)f3[0] + (size_t)G.nx * ((size_t)f3[1] + (size_t)G.ny * (size_t)f3[2]) : cell;
             const uint8_t fsrc = T.flags[sidx], ffar = T.flags[far];
-            const A pull = Store<S>::load(src + (size_t)q * n + sidx, P.inv_scale);
-            const A gt_k = Store<S>::load(src + (size_t)k * n + cell, P.inv_scale);
-            const A gt_q = Store<S>::load(src + (size_t)q * n + cell, P.inv_scale);
-            const A vfar = Store<S>::load(src + (size_t)k * n + far, P.inv_scale);
+            const A pull = Store<S>::fetch(src + (size_t)q * n + sidx, P.inv_scale);
+            const A gt_k = Store<S>::fetch(src + (size_t)k * n + cell, P.inv_scale);
+            const A gt_q = Store<S>::fetch(src + (size_t)q * n + cell, P.inv_scale);
+            const A vfar = Store<S>::fetch(src + (size_t)k * n + far, P.inv_scale);
             // the link's geometry while they are on their way, as if the far cell were fluid (it nearly always is)
             A d[3];
             int pu[3];
@@ -301,12 +308,17 @@ __device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int bid, in
                 acc.add(k, pu, fl, tl);
             }
         }
-        gq = warp_trt_collide<A, FORCED>(gq, lane, P, T.status);
-        if (lane < 19) Store<S>::store(T.dst + (size_t)lane * n + cell, gq, P.scale);
+        kept = warp_trt_collide<A, FORCED>(gq, lane, P, T.status);
+        if (lane < 19) kept_at = T.dst + (size_t)lane * n + cell;
     }
-    if (T.finish == 2) return;   // the force is not wanted
-    block_link_sums<STEP_THREADS>(acc, T.ps->x, T.partials + (size_t)bid * 6);
-    if (!last_block_done(T.done, T.bblocks)) return;
+    if (T.finish == 2) {   // the force is not wanted
+        if (kept_at) Store<S>::store(kept_at, kept, P.scale);
+        return;
+    }
+    block_link_sums<STEP_THREADS>(acc, sX, T.partials + bid, T.bblocks);
+    const bool last = last_block_done(T.done, T.bblocks);
+    if (kept_at) Store<S>::store(kept_at, kept, P.scale);
+    if (!last) return;
     if (T.finish == 1) {
         if (wib < 3) {
             const double f = sum_partials(T.partials, T.bblocks, wib);
@@ -316,7 +328,9 @@ __device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int bid, in
     }
     // with it the frames of the moved sphere, in the other copy: bulk CTAs of this launch still read this one
     particle_block_update<STEP_THREADS>(T.ps, T.partials, T.bblocks, G, T.history, T.hist_cap, T.status, T.frames->inv,
-                                        [&](const ParticleState& Q, int a) { pframes_axis(T.frames_next, Q, n3, T.B, a); });
+                                        [&](const ParticleState& Q, int a, int part) {
+                                            pframes_axis(T.frames_next, Q, n3, T.B, a, part);
+                                        });
 }
 
 // CTA b of the grid: boundary CTA b >> bshift (true), or the bulk CTA *bulk.
@@ -390,7 +404,7 @@ __global__ void k_frames(const ParticleState* __restrict__ ps, PFrames* __restri
 // the equilibrium, plus Grad's term when gcoef != 0; lane q < 19 writes
 // population q.  Every lane calls it with the same cell.
 template <typename S>
-__device__ __forceinline__ void refill_warp(S* __restrict__ pops, const uint8_t* __restrict__ fcur, const GridDesc& G,
+__device__ __forceinline__ void refill_warp(S* pops, const uint8_t* fcur, const GridDesc& G,
                                             const int n3[3], const BoxFrame& F, const ParticleState& P, int i, int j,
                                             int k, typename Store<S>::A scale, typename Store<S>::A inv_scale,
                                             typename Store<S>::A gcoef) {
@@ -415,7 +429,7 @@ __device__ __forceinline__ void refill_warp(S* __restrict__ pops, const uint8_t*
             // the populations are loaded beside the flag (not after it): a solid neighbour's are dropped
             A gp[19];
 #pragma unroll
-            for (int q = 0; q < 19; ++q) gp[q] = Store<S>::load(pops + (size_t)q * n + y, inv_scale);
+            for (int q = 0; q < 19; ++q) gp[q] = Store<S>::fetch(pops + (size_t)q * n + y, inv_scale);
             ok = fcur[y] == 0;
             r = A(1);
 #pragma unroll
@@ -469,10 +483,10 @@ __device__ __forceinline__ void refill_warp(S* __restrict__ pops, const uint8_t*
 constexpr int REMAP_THREADS = SEG;
 template <typename S>
 __global__ void __launch_bounds__(REMAP_THREADS)
-    k_remap(S* __restrict__ pops, const uint8_t* __restrict__ fcur, uint8_t* __restrict__ fnext, GridDesc G, BoxDesc B,
-            const ParticleState* __restrict__ ps, const PFrames* __restrict__ frames, typename Store<S>::A scale,
-            typename Store<S>::A inv_scale, typename Store<S>::A gcoef, uint8_t* __restrict__ mark,
-            int* __restrict__ seg, int* __restrict__ seg_count, int mark_only) {
+    k_remap(S* pops, const uint8_t* fcur, uint8_t* fnext, const __grid_constant__ GridDesc G,
+            const __grid_constant__ BoxDesc B, const ParticleState* ps, const PFrames* frames, typename Store<S>::A scale,
+            typename Store<S>::A inv_scale, typename Store<S>::A gcoef, uint8_t* mark, int* seg, int* seg_count,
+            int mark_only) {
     using A = typename Store<S>::A;
     __shared__ BoxFrame F;
     __shared__ int s_n;
