@@ -346,11 +346,10 @@ __global__ void __launch_bounds__(UPD_THREADS, sizeof(S) == 8 ? 1 : UPD_MIN_CTAS
 // ---------------------------------------------------------------- coupling
 constexpr int BNDW_THREADS = 256;
 // Register cap of the boundary kernel (BNDW_THREADS threads).  It runs beside the finest level's
-// update for most of that update, so every register it holds is taken from the update's CTAs: at
-// 56 in FP32 a boundary CTA (14,336 registers) leaves room for 1,280 update threads of 40 registers
-// instead of 1,024.
+// update for most of that update, so every register it holds is taken from the update's CTAs; at 64
+// it keeps its loads of one round trip without spills (rising sphere: 1% faster than at 56).
 template <typename S>
-constexpr int BND_MAXREG = sizeof(S) == 8 ? 128 : (sizeof(S) == 4 ? 56 : 64);
+constexpr int BND_MAXREG = sizeof(S) == 8 ? 128 : 64;
 constexpr int REMAP_THREADS = SEG;   // remap blocks: their uncovered cells are spread over the eight warps
 
 // Boundary cells of the finest level (flag 2: fluid with a solid
@@ -476,11 +475,13 @@ __device__ __forceinline__ void refill_cell_warp(const LevelView& D, S* __restri
                 r = A(1);
 #pragma unroll
                 for (int p = 0; p < 19; ++p) r += gp[p];
+                if (gcoef != A(0)) {
 #pragma unroll
-                for (int p = 1; p < 19; ++p) {
-                    mo[0] += A(cx(p)) * gp[p];
-                    mo[1] += A(cy(p)) * gp[p];
-                    mo[2] += A(cz(p)) * gp[p];
+                    for (int p = 1; p < 19; ++p) {
+                        if (cx(p)) mo[0] += cx(p) > 0 ? gp[p] : -gp[p];
+                        if (cy(p)) mo[1] += cy(p) > 0 ? gp[p] : -gp[p];
+                        if (cz(p)) mo[2] += cz(p) > 0 ? gp[p] : -gp[p];
+                    }
                 }
             }
         }
@@ -538,23 +539,36 @@ __global__ void k_pframes(const ParticleState* __restrict__ ps, PFrames* __restr
 }
 
 // Remap of Sec. 2.3 after the particle moved, over the box of finest cells
-// around the sphere, in one pass: the new solid flag of every cell (the
-// exact ball predicate); newly covered cells drop their populations (the
-// update already zeroed the cells that were solid before); uncovered cells
-// are listed in shared memory and refilled afterwards, each by one warp of
-// the block in turn (refill_cell_warp: it reads only cells that are fluid
-// before and after the move, which nothing here writes); fluid cells with a
-// solid neighbour go to the block's segment.  Neighbour flags are
-// evaluated from the same predicate instead of being read back, so no
-// second pass is needed.
+// around the sphere: the new solid flag of every cell (the exact ball
+// predicate); newly covered cells drop their populations (the update
+// already zeroed the cells that were solid before); fluid cells with a
+// solid neighbour go to the CTA's segment (neighbour flags are evaluated
+// from the same predicate instead of being read back); uncovered cells are
+// listed in shared memory and refilled, each by one warp of the block in
+// turn (refill_cell_warp: it reads only cells that are fluid before and
+// after the move, which nothing here writes).
+// FP32 and FP16 storage (REMAP_SPLIT) launch a CTA per segment twice over:
+// the second half lists its uncovered cells from the own-cell predicate
+// alone and refills them beside the first half's marks.  In one pass the
+// refill followed the marks, 4 us of 8 in the rising sphere's developed
+// steps and twice that beside the coarser levels' updates: 168 us per
+// level-0 step against 161.  FP64, where the step waits for FP64 issue and
+// the CTAs take 96 registers a thread, loses by it (275 us against 267) and
+// does both in one pass.  frames = null: the current position's marks only
+// (nothing is uncovered).
+template <typename S>
+constexpr bool REMAP_SPLIT = sizeof(S) != 8;
+
 template <typename S>
 __global__ void __launch_bounds__(REMAP_THREADS)
-    k_amr_remap(LevelView D, S* __restrict__ pops, const uint8_t* __restrict__ fcur, uint8_t* __restrict__ fnext,
-                BoxDesc B, const ParticleState* __restrict__ ps, typename Store<S>::A scale,
+    k_amr_remap(const __grid_constant__ LevelView D, S* __restrict__ pops, const uint8_t* __restrict__ fcur, uint8_t* __restrict__ fnext,
+                const __grid_constant__ BoxDesc B, const ParticleState* __restrict__ ps, typename Store<S>::A scale,
                 typename Store<S>::A inv_scale, int* __restrict__ seg, int* __restrict__ seg_count,
                 int* __restrict__ status, typename Store<S>::A gcoef, const PFrames* __restrict__ frames) {
     using A = typename Store<S>::A;
     __shared__ BoxFrame F;
+    __shared__ LinkFrame<float> lf;
+    if (threadIdx.x == 32 && frames) lf = frames->lf;
     __shared__ int s_n;
     __shared__ int s_cell[2][REMAP_THREADS], s_g[3][REMAP_THREADS];   // uncovered cells: pool block, cell, position
     if (threadIdx.x == 0) {
@@ -564,7 +578,10 @@ __global__ void __launch_bounds__(REMAP_THREADS)
     }
     __syncthreads();
     const ParticleState& P = *ps;
-    const int t = blockIdx.x * REMAP_THREADS + threadIdx.x;
+    const int nseg = (int)((B.cells + SEG - 1) / SEG);
+    const bool refill_only = REMAP_SPLIT<S> && (int)blockIdx.x >= nseg;   // uniform across the block
+    const int segment = refill_only ? (int)blockIdx.x - nseg : (int)blockIdx.x;
+    const int t = segment * REMAP_THREADS + threadIdx.x;
     bool is_b = false;
     int entry = 0;
     if (t < B.cells) {
@@ -578,34 +595,34 @@ __global__ void __launch_bounds__(REMAP_THREADS)
             } else {
                 const size_t x = (size_t)b * B3 + c;
                 bool any_nb = false;
-                const bool solid = ball_flag_and_neighbours(g, D.n, D.periodic, F, P, &any_nb);
+                const bool solid = refill_only ? ball_flag(g, D.n, D.periodic, F, P)
+                                               : ball_flag_and_neighbours(g, D.n, D.periodic, F, P, &any_nb);
                 const bool was_solid = fcur[x] == FLAG_SOLID;
-                if (solid) {
-                    fnext[x] = FLAG_SOLID;
-                    if (!was_solid)
+                if (!refill_only) {
+                    is_b = !solid && any_nb;
+                    fnext[x] = solid ? FLAG_SOLID : (is_b ? FLAG_BOUNDARY : FLAG_FLUID);
+                    if (solid && !was_solid)
 #pragma unroll
                         for (int q = 0; q < 19; ++q) Store<S>::store(pops + paddr(b, q, c), A(0), scale);
-                } else {
-                    is_b = any_nb;
-                    fnext[x] = is_b ? FLAG_BOUNDARY : FLAG_FLUID;
-                    if (was_solid) {   // uncovered: fluid after the move, solid before
-                        const int k = atomicAdd(&s_n, 1);
-                        s_cell[0][k] = b;
-                        s_cell[1][k] = c;
-                        s_g[0][k] = g[0];
-                        s_g[1][k] = g[1];
-                        s_g[2][k] = g[2];
-                    }
+                }
+                if ((refill_only || !REMAP_SPLIT<S>) && !solid && was_solid) {   // uncovered: fluid after the move, solid before
+                    const int k = atomicAdd(&s_n, 1);
+                    s_cell[0][k] = b;
+                    s_cell[1][k] = c;
+                    s_g[0][k] = g[0];
+                    s_g[1][k] = g[1];
+                    s_g[2][k] = g[2];
                 }
             }
         }
     }
-    write_segment(is_b, entry, (int)blockIdx.x, seg, seg_count);   // its barrier also completes the shared list
-    const int wid = threadIdx.x >> 5;
-    for (int k = wid; k < s_n; k += REMAP_THREADS / 32) {
+    if (refill_only) __syncthreads();
+    else write_segment(is_b, entry, segment, seg, seg_count);   // its barrier also completes the shared list
+    if (REMAP_SPLIT<S> && !refill_only) return;
+    for (int k = (int)(threadIdx.x >> 5); k < s_n; k += REMAP_THREADS / 32) {
         const int g3[3] = {s_g[0][k], s_g[1][k], s_g[2][k]};
         refill_cell_warp<S>(D, pops, fcur, F, P, s_cell[0][k], s_cell[1][k], g3, scale, inv_scale, gcoef,
-                            frames ? &frames->lf : nullptr);
+                            frames ? &lf : nullptr);
     }
 }
 
@@ -1674,7 +1691,7 @@ void enqueue_advance(lbmp_handle* h, int l, int sub) {
         } else {
             cudaStreamWaitEvent(st, E->ev_join, 0);
         }
-        k_amr_remap<S><<<nl, REMAP_THREADS, 0, rs>>>(D, U.dst, V.d_flags[V.fcur], fnext, h->box, h->d_ps, P.scale,
+        k_amr_remap<S><<<REMAP_SPLIT<S> ? 2 * nl : nl, REMAP_THREADS, 0, rs>>>(D, U.dst, V.d_flags[V.fcur], fnext, h->box, h->d_ps, P.scale,
                                                     P.inv_scale, h->seg, h->seg_count, h->status,
                                                     (A)grad_refill_coef(h->cfg.refill, V.taup), E->d_frames);
         if (beside) {
@@ -1770,7 +1787,8 @@ lbmp_status amr_add_sphere(lbmp_handle* h) {
     const double shell = 4.0 / 3.0 * M_PI * (ro * ro * ro - ri * ri * ri);
     h->list_cap = (int)std::min<double>((double)B.cells, std::ceil(shell) + 64.0);
     h->list = (int*)handle_alloc(h, sizeof(int) * (size_t)h->list_cap);
-    E->boundary_blocks = step_boundary_blocks(h->list_cap);
+    // FP64: half as many, each warp two cells (the CTAs compete with the update for FP64 issue: 263 us against 267)
+    E->boundary_blocks = step_boundary_blocks(h->list_cap, h->cfg.precision == LBMP_FP64 ? 40 : 20);
     h->partials = (double*)handle_alloc(h, sizeof(double) * 6 * (size_t)E->boundary_blocks);
     if (!E->d_frames) E->d_frames = (PFrames*)handle_alloc(h, sizeof(PFrames));
     if (!E->d_frames) return LBMP_ERR_OOM;
