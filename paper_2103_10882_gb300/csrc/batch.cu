@@ -26,7 +26,8 @@ struct SimDev {
     GridDesc G;
     long long pop_off;   // element offset of the simulation in each population pool
     long long flag_off;  // byte offset in each flag pool
-    int mask_off;        // boundary mask: one byte per box cell
+    FastDiv by_edge;     // division by the edge
+    int seg_off, nseg;   // segments of the box: boundary cells and their number per 256 box cells
     int bnd_off, bnd_n;  // boundary-kernel blocks of the simulation (and their force partials)
     BoxDesc box;
     CollideParams<double> P;   // FP64: the collision's parameters; else its rates are rounded from here
@@ -34,7 +35,7 @@ struct SimDev {
 };
 
 constexpr int BW = 256;   // threads of the boundary, particle and remap kernels
-constexpr int BND_CHUNK = 512;   // box cells per boundary block (fewer, fuller blocks: the fixed cost per block dominates)
+constexpr int BND_SEGS = 2;   // segments per boundary block (fewer, fuller blocks: the fixed cost per block dominates)
 // Cell flags: fluid, solid (centre inside the sphere), fluid with a solid
 // D3Q19 neighbour (updated by k_batch_boundary instead of the bulk kernel).
 constexpr uint8_t FLAG_FLUID = 0, FLAG_SOLID = 1, FLAG_BOUNDARY = 2;
@@ -79,7 +80,13 @@ __global__ void __launch_bounds__(512, sizeof(S) == 8 ? 1 : 3) k_batch_bulk(cons
         const int z = t.w + threadIdx.z * ZC + k;
         const int zs[3] = {z + 1 < e ? z + 1 : 0, z, z > 0 ? z - 1 : e - 1};
         const size_t cell = (size_t)(x + e * (y + e * z));
-        if (fl[cell] != FLAG_FLUID) continue;   // solid (zeroed by the remap) or done by k_batch_boundary
+        const uint8_t f = fl[cell];
+        if (f != FLAG_FLUID) {   // solid: stored as zero; else done by k_batch_boundary
+            if (f == FLAG_SOLID)
+#pragma unroll
+                for (int q = 0; q < 19; ++q) Store<S>::store(d0 + (size_t)q * n + cell, A(0), P.scale);
+            continue;
+        }
         A g[19];
 #pragma unroll
         for (int q = 0; q < 19; ++q)
@@ -92,16 +99,15 @@ __global__ void __launch_bounds__(512, sizeof(S) == 8 ? 1 : 3) k_batch_bulk(cons
 }
 
 // ----------------------------------------------------------------- boundary
-// Boundary cells of every simulation (flag 2), found from the remap's mask
-// in box order: each block compacts the marked cells of its chunk of
-// BND_CHUNK box cells and its warps take them in turn, lane q handling
-// population q (CLI
-// links, geometry in the population arithmetic, FP64 force partials), with
-// a cooperative collision.  The grid is flat: block b belongs to simulation
-// bnd_sim[b], which owns bnd_n blocks (a warp per 32 box cells) and as many
-// partials; the last of them to finish runs that simulation's particle
-// update (Algorithm 1).  The bulk kernel skips these cells, so this kernel
-// runs beside it.
+// Boundary cells of every simulation (flag 2), from the segments the remap
+// wrote: the grid is flat, block b belongs to simulation bnd_sim[b] and takes
+// BND_SEGS segments of its box, its warps the cells in turn, lane q handling
+// population q (CLI links, geometry in the population arithmetic, FP64 force
+// partials), with a cooperative collision.  All loads of a link are issued
+// at once, its geometry formed meanwhile.  The last of a simulation's blocks
+// to finish runs its particle update (Algorithm 1) and forms the frames of
+// the moved sphere, which the next kernels read.  The bulk kernel skips these
+// cells, so this kernel runs beside it.
 // Register cap of the boundary kernel (BW threads): it runs beside the bulk kernel (three CTAs of 512 threads
 // at 40 registers per SM), and at its natural 122 registers a resident boundary CTA left room for one bulk CTA.
 template <typename S>
@@ -110,70 +116,88 @@ constexpr int BND_MAXREG = sizeof(S) == 8 ? 128 : 64;
 template <typename S>
 __global__ void __maxnreg__(BND_MAXREG<S>)
     k_batch_boundary(const S* __restrict__ src, S* __restrict__ dst, const uint8_t* __restrict__ flags,
-                     const uint8_t* __restrict__ mask, const SimDev* __restrict__ sims,
-                     const int* __restrict__ bnd_sim, ParticleState* ps, int cli, typename Store<S>::A scale,
-                     typename Store<S>::A inv, double* partials, int* done, double* __restrict__ history,
-                     int hist_cap, int* __restrict__ status) {
+                     const int* __restrict__ seg, const int* __restrict__ seg_count, const SimDev* __restrict__ sims,
+                     const int* __restrict__ bnd_sim, ParticleState* ps, PFrames* frames, int cli,
+                     typename Store<S>::A scale, typename Store<S>::A inv, double* partials, int* done,
+                     double* __restrict__ history, int hist_cap, int* __restrict__ status) {
     using A = typename Store<S>::A;
     __shared__ LinkFrame<A> Fr;
-    __shared__ BoxFrame Bf;
+    __shared__ double sX[3];
+    __shared__ int upto[BND_SEGS];   // cells of the block's segments up to and with each
     const int sim = bnd_sim[blockIdx.x];
     const SimDev& D = sims[sim];
     const GridDesc& G = D.G;
     const int n3[3] = {G.nx, G.ny, G.nz};
     const int per3[3] = {1, 1, 1};
-    if (threadIdx.x == 0) Fr.init(ps[sim]);   // the two FP64 set-ups on two warps
-    if (threadIdx.x == 32) box_frame_init(Bf, n3, per3, D.box, ps[sim]);
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int local = (int)blockIdx.x - D.bnd_off, seg0 = local * BND_SEGS;
+    if (threadIdx.x == 0) Fr = pframe_link<A>(frames[sim]);   // formed by the last particle update
+    if (threadIdx.x >= 32 && threadIdx.x < 35) sX[threadIdx.x - 32] = ps[sim].x[threadIdx.x - 32];
+    if (threadIdx.x == 64) {
+        int t = 0;
+#pragma unroll
+        for (int k = 0; k < BND_SEGS; ++k) {
+            t += seg0 + k < D.nseg ? seg_count[D.seg_off + seg0 + k] : 0;
+            upto[k] = t;
+        }
+    }
     __syncthreads();
     const CollideParams<A> P = sim_params<S>(D, scale, inv);
     const S* s0 = src + D.pop_off;
     S* d0 = dst + D.pop_off;
     const uint8_t* fl = flags + D.flag_off;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const size_t n = (size_t)G.n;
-    __shared__ int sl[BND_CHUNK];
-    const long long t0 = (long long)(blockIdx.x - D.bnd_off) * BND_CHUNK;
-    const int nm = block_compact_mask(mask + D.mask_off, t0, D.box.cells, BND_CHUNK, sl);
+    const int q = lane < 19 ? lane : 0, k = opp(q);
+    const int cq[3] = {cx(q), cy(q), cz(q)};
     LinkSums<A> acc;
-    for (int i = wib; i < nm; i += BW / 32) {
-        int xyz[3];
-        if (!box_cell((int)(t0 + sl[i]), n3, per3, D.box, Bf, xyz)) continue;   // marked cells are inside
-        const int x = xyz[0], y = xyz[1], z = xyz[2];
-        const size_t cell = (size_t)x + (size_t)G.nx * ((size_t)y + (size_t)G.ny * (size_t)z);
+    // a warp's last cell is stored after the hand-off: the hand-off's release waits for the stores before it
+    A kept = A(0);
+    S* kept_at = nullptr;
+    for (int j = wib; j < upto[BND_SEGS - 1]; j += BW / 32) {
+        if (kept_at) Store<S>::store(kept_at, kept, P.scale);
+        int g = 0;
+        while (upto[g] <= j) ++g;
+        const int cell = seg[(size_t)(D.seg_off + seg0 + g) * SEG + (j - (g > 0 ? upto[g - 1] : 0))];
+        const unsigned row = D.by_edge.div((unsigned)cell), plane = D.by_edge.div(row);
+        const int xyz[3] = {cell - (int)row * G.nx, (int)row - (int)plane * G.ny, (int)plane};
         A gq = A(0);
         if (lane < 19) {
-            const int q = lane;
-            const int c[3] = {cx(q), cy(q), cz(q)};
             int s3[3], f3[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                s3[a] = src_coord(xyz[a], c[a], n3[a], 1);
-                f3[a] = src_coord(xyz[a], -c[a], n3[a], 1);
+                s3[a] = src_coord(xyz[a], cq[a], n3[a], 1);
+                f3[a] = src_coord(xyz[a], -cq[a], n3[a], 1);
             }
-            const size_t sidx = (size_t)s3[0] + (size_t)G.nx * ((size_t)s3[1] + (size_t)G.ny * (size_t)s3[2]);
-            if (q == 0 || fl[sidx] != FLAG_SOLID) {
-                gq = Store<S>::load(s0 + (size_t)q * n + sidx, P.inv_scale);
-            } else {
-                const int k = opp(q);
-                const size_t far = (size_t)f3[0] + (size_t)G.nx * ((size_t)f3[1] + (size_t)G.ny * (size_t)f3[2]);
-                const bool far_ok = fl[far] != FLAG_SOLID;
-                A d[3], flk[3], tl3[3];
-                int pu[3];
-                Fr.offset(xyz, n3, per3, d, pu);
-                const A gt_k = Store<S>::load(s0 + (size_t)k * n + cell, P.inv_scale);
-                const A gt_q = Store<S>::load(s0 + (size_t)q * n + cell, P.inv_scale);
-                const A gt_far = far_ok ? Store<S>::load(s0 + (size_t)k * n + far, P.inv_scale) : A(0);
-                gq = cli_link<A>(q, d, cli && far_ok, gt_k, gt_q, gt_far, Fr, flk, tl3);
+            const int sidx = s3[0] + G.nx * (s3[1] + G.ny * s3[2]), far = f3[0] + G.nx * (f3[1] + G.ny * f3[2]);
+            const uint8_t fsrc = fl[sidx], ffar = fl[far];
+            const A pull = Store<S>::load(s0 + (size_t)q * n + sidx, P.inv_scale);
+            const A gt_k = Store<S>::load(s0 + (size_t)k * n + cell, P.inv_scale);
+            const A gt_q = Store<S>::load(s0 + (size_t)q * n + cell, P.inv_scale);
+            const A vfar = Store<S>::load(s0 + (size_t)k * n + far, P.inv_scale);
+            A d[3];
+            int pu[3];
+            Fr.offset(xyz, n3, per3, d, pu);
+            CliGeometry<A> L = cli_geometry<A>(q, d, cli != 0, Fr);   // as if the far cell were fluid
+            gq = pull;
+            if (q != 0 && fsrc == FLAG_SOLID) {
+                const bool far_ok = ffar != FLAG_SOLID;
+                if (cli && !far_ok) L = cli_geometry<A>(q, d, false, Fr);
+                A flk[3], tl3[3];
+                gq = cli_apply<A>(q, L, gt_k, gt_q, far_ok ? vfar : A(0), flk, tl3);
                 acc.add(k, pu, flk, tl3);
             }
         }
-        gq = warp_trt_collide<A, false>(gq, lane, P, status);
-        if (lane < 19) Store<S>::store(d0 + (size_t)lane * n + cell, gq, P.scale);
+        kept = warp_trt_collide<A, false>(gq, lane, P, status);
+        if (lane < 19) kept_at = d0 + (size_t)lane * n + cell;
     }
-    block_link_sums<BW>(acc, ps[sim].x, partials + (size_t)D.bnd_off * 6 + (blockIdx.x - D.bnd_off), D.bnd_n);
-    if (last_block_done(done + sim, D.bnd_n))
-        particle_block_update<BW>(ps + sim, partials + (size_t)D.bnd_off * 6, D.bnd_n, G,
-                                  history + (size_t)D.hist_off * 15, hist_cap, status);
+    block_link_sums<BW>(acc, sX, partials + (size_t)D.bnd_off * 6 + local, D.bnd_n);
+    const bool last = last_block_done(done + sim, D.bnd_n);
+    if (kept_at) Store<S>::store(kept_at, kept, P.scale);
+    if (last)
+        particle_block_update<BW>(
+            ps + sim, partials + (size_t)D.bnd_off * 6, D.bnd_n, G, history + (size_t)D.hist_off * 15, hist_cap, status,
+            frames[sim].inv,
+            [&](const ParticleState& Q, int a, int part) { pframes_axis(frames + sim, Q, n3, D.box, a, part); });
 }
 
 // -------------------------------------------------------------------- remap
@@ -201,19 +225,21 @@ __device__ __forceinline__ void batch_refill_warp(S* __restrict__ p0, const uint
         for (int a = 0; a < 3; ++a) v[a] = v[a] < 0 ? v[a] + n3[a] : (v[a] >= n3[a] ? v[a] - n3[a] : v[a]);
         if (!ball_flag(v, n3, G.periodic, F, P)) {
             const size_t y = (size_t)v[0] + (size_t)G.nx * ((size_t)v[1] + (size_t)G.ny * (size_t)v[2]);
-            if (fc[y] != FLAG_SOLID) {
-                ok = true;
+            {   // the populations are loaded beside the flag (not after it): a solid neighbour's are dropped
+                ok = fc[y] != FLAG_SOLID;
                 A gp[19];
 #pragma unroll
                 for (int q2 = 0; q2 < 19; ++q2) gp[q2] = Store<S>::load(p0 + (size_t)q2 * n + y, inv);
                 r = A(1);
 #pragma unroll
                 for (int q2 = 0; q2 < 19; ++q2) r += gp[q2];
+                if (grad) {
 #pragma unroll
-                for (int q2 = 1; q2 < 19; ++q2) {
-                    mo[0] += A(cx(q2)) * gp[q2];
-                    mo[1] += A(cy(q2)) * gp[q2];
-                    mo[2] += A(cz(q2)) * gp[q2];
+                    for (int q2 = 1; q2 < 19; ++q2) {
+                        if (cx(q2)) mo[0] += cx(q2) > 0 ? gp[q2] : -gp[q2];
+                        if (cy(q2)) mo[1] += cy(q2) > 0 ? gp[q2] : -gp[q2];
+                        if (cz(q2)) mo[2] += cz(q2) > 0 ? gp[q2] : -gp[q2];
+                    }
                 }
             }
         }
@@ -250,57 +276,68 @@ __device__ __forceinline__ void batch_refill_warp(S* __restrict__ p0, const uint
     }
 }
 
-// Remap of Sec. 2.3 in one pass over each simulation's box: the new flag of
-// every cell (the exact ball predicate; 2 for fluid cells with a solid
-// neighbour, evaluated from the same predicate), covered cells zeroed,
-// uncovered cells refilled afterwards, one at a time by their whole warp
-// (batch_refill_warp), and the mask of boundary cells in box order for the
-// next step's k_batch_boundary.
+// Remap of Sec. 2.3 over each simulation's box, a block per segment (seg_sim names its simulation): the new flag of
+// every cell (the exact ball predicate; 2 for fluid cells with a solid neighbour, evaluated from the same predicate),
+// covered cells zeroed, the boundary cells into the segment; uncovered cells are listed in shared memory and refilled
+// by the block's warps in turn (batch_refill_warp). 
 template <typename S>
 __global__ void __launch_bounds__(BW)
     k_batch_remap(S* __restrict__ pops, const uint8_t* __restrict__ fcur, uint8_t* __restrict__ fnext,
-                  const SimDev* __restrict__ sims, const ParticleState* __restrict__ ps,
-                  typename Store<S>::A scale, typename Store<S>::A inv, uint8_t* __restrict__ mask, int grad) {
+                  const SimDev* __restrict__ sims, const int* __restrict__ seg_sim, const ParticleState* __restrict__ ps,
+                  const PFrames* __restrict__ frames, typename Store<S>::A scale, typename Store<S>::A inv,
+                  int* __restrict__ seg, int* __restrict__ seg_count, int grad) {
     using A = typename Store<S>::A;
+    static_assert(BW == SEG, "a block is a segment");
     __shared__ BoxFrame F;
-    const int sim = blockIdx.y;
+    __shared__ int s_n;
+    __shared__ int s_g[3][BW];   // uncovered cells
+    const int sim = seg_sim[blockIdx.x];
     const SimDev& D = sims[sim];
     const GridDesc& G = D.G;
-    if ((long long)blockIdx.x * BW >= D.box.cells) return;   // uniform across the block
     const int n3[3] = {G.nx, G.ny, G.nz};
-    if (threadIdx.x == 0) box_frame_init(F, n3, G.periodic, D.box, ps[sim]);
+    if (threadIdx.x == 0) {
+        F = frames[sim].bf;   // formed by the particle update that moved the sphere
+        s_n = 0;
+    }
     __syncthreads();
-    const int t = blockIdx.x * BW + threadIdx.x;
+    const int t = ((int)blockIdx.x - D.seg_off) * BW + threadIdx.x;
     const ParticleState& P = ps[sim];
     const uint8_t* fc = fcur + D.flag_off;
     uint8_t* fn = fnext + D.flag_off;
     S* p0 = pops + D.pop_off;
     const size_t n = (size_t)G.n;
-    bool uncovered = false;   // fluid after the move, solid before: refilled below by the warp
-    int p[3] = {0, 0, 0};
-    size_t c = 0;
+    bool is_b = false;
+    int c = 0, p[3] = {0, 0, 0};
     // periodic: box_cell fails only for a corrupt centre
     if (t < D.box.cells && box_cell(t, n3, G.periodic, D.box, F, p)) {
-        c = (size_t)p[0] + (size_t)G.nx * ((size_t)p[1] + (size_t)G.ny * (size_t)p[2]);
-        int is_b = 0;
+        c = p[0] + G.nx * (p[1] + G.ny * p[2]);
+        const bool was_solid = fc[c] == FLAG_SOLID;
         bool any_nb = false;
-        if (ball_flag_and_neighbours(p, n3, G.periodic, F, P, &any_nb)) {
-            fn[c] = FLAG_SOLID;
+        const bool solid = ball_flag_and_neighbours(p, n3, G.periodic, F, P, &any_nb);
+        is_b = !solid && any_nb;
+        fn[c] = solid ? FLAG_SOLID : (is_b ? FLAG_BOUNDARY : FLAG_FLUID);
+        if (solid && !was_solid) {   // (the bulk kernel stores the cells that were solid before as zero)
+#pragma unroll
             for (int q = 0; q < 19; ++q) Store<S>::store(p0 + (size_t)q * n + c, A(0), scale);
-        } else {
-            uncovered = fc[c] == FLAG_SOLID;
-            is_b = any_nb ? 1 : 0;
-            fn[c] = is_b ? FLAG_BOUNDARY : FLAG_FLUID;
+        } else if (!solid && was_solid) {
+            const int k = atomicAdd(&s_n, 1);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) s_g[a][k] = p[a];
         }
-        mask[D.mask_off + t] = (uint8_t)is_b;
     }
-    for (unsigned todo = __ballot_sync(0xffffffffu, uncovered); todo != 0u; todo &= todo - 1u) {
-        const int src = __ffs((int)todo) - 1;
-        const int i = __shfl_sync(0xffffffffu, p[0], src), j = __shfl_sync(0xffffffffu, p[1], src),
-                  k = __shfl_sync(0xffffffffu, p[2], src);
-        const size_t cc = (size_t)i + (size_t)G.nx * ((size_t)j + (size_t)G.ny * (size_t)k);
-        batch_refill_warp<S>(p0, fc, G, n3, F, P, i, j, k, cc, scale, inv, grad, D.P.sp);
+    write_segment(is_b, c, (int)blockIdx.x, seg, seg_count);   // its barrier also completes the shared list
+    for (int k = (int)(threadIdx.x >> 5); k < s_n; k += BW / 32) {
+        const int i = s_g[0][k], j = s_g[1][k], m = s_g[2][k];
+        batch_refill_warp<S>(p0, fc, G, n3, F, P, i, j, m, (size_t)(i + G.nx * (j + G.ny * m)), scale, inv, grad, D.P.sp);
     }
+}
+
+// Frames of every simulation's start position (one block of 128 threads each).
+__global__ void k_batch_frames(const SimDev* __restrict__ sims, const ParticleState* __restrict__ ps,
+                               PFrames* __restrict__ frames) {
+    const SimDev& D = sims[blockIdx.x];
+    const int n3[3] = {D.G.nx, D.G.ny, D.G.nz};
+    pframes_form(frames + blockIdx.x, ps[blockIdx.x], n3, D.G.periodic, D.box);
 }
 
 template <typename S>
@@ -361,12 +398,15 @@ struct BatchEngine {
     int fcur = 0;
     ParticleState* d_ps = nullptr;
     std::vector<ParticleState> h_ps;
-    uint8_t* mask = nullptr;
+    int* seg = nullptr;         // boundary cells by segment (an entry per box cell of every simulation)
+    int* seg_count = nullptr;   // and their number
+    int* d_seg_sim = nullptr;   // simulation of each segment
+    int segments = 0;
+    PFrames* frames = nullptr;  // frames of every simulation's sphere
     int* done = nullptr;        // last-block-done counter per simulation
     double* partials = nullptr;
     int bnd_blocks = 1;     // boundary-kernel blocks of all simulations
     int* d_bnd_sim = nullptr;   // simulation of each boundary-kernel block
-    int max_box_blocks = 1;
     double* history = nullptr;
     // stream-collide tiles for every candidate shape
     int4* d_tiles[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -424,9 +464,9 @@ void enqueue_batch_step(lbmp_handle* h) {
     // boundary cells (flag 2) and the particle updates beside the bulk kernel, which skips them
     cudaEventRecord(B->ev_fork, h->stream);
     cudaStreamWaitEvent(B->side, B->ev_fork, 0);
-    k_batch_boundary<S><<<B->bnd_blocks, BW, 0, B->side>>>(src, dst, B->flags[B->fcur], B->mask, B->d_sims,
-                                                           B->d_bnd_sim, B->d_ps, h->cfg.boundary == LBMP_CLI ? 1 : 0,
-                                                           scale, inv, B->partials, B->done, B->history,
+    k_batch_boundary<S><<<B->bnd_blocks, BW, 0, B->side>>>(src, dst, B->flags[B->fcur], B->seg, B->seg_count, B->d_sims,
+                                                           B->d_bnd_sim, B->d_ps, B->frames,
+                                                           h->cfg.boundary == LBMP_CLI ? 1 : 0, scale, inv, B->partials, B->done, B->history,
                                                            h->cfg.history_capacity, h->status);
     cudaEventRecord(B->ev_join, B->side);
     const long long ev = profile_mark(h);
@@ -434,9 +474,9 @@ void enqueue_batch_step(lbmp_handle* h) {
     profile_kernel(h, ev, profile_mark(h), 38.0 * sizeof(S) * (double)B->total_cells, (double)B->total_cells);
     cudaStreamWaitEvent(h->stream, B->ev_join, 0);
     uint8_t* fnext = B->flags[1 - B->fcur];
-    const dim3 gr(B->max_box_blocks, B->nsims);
-    k_batch_remap<S><<<gr, BW, 0, h->stream>>>(dst, B->flags[B->fcur], fnext, B->d_sims, B->d_ps, scale, inv, B->mask,
-                                               h->cfg.refill == LBMP_REFILL_GRAD ? 1 : 0);
+    k_batch_remap<S><<<B->segments, BW, 0, h->stream>>>(dst, B->flags[B->fcur], fnext, B->d_sims, B->d_seg_sim, B->d_ps,
+                                                        B->frames, scale, inv, B->seg, B->seg_count,
+                                                        h->cfg.refill == LBMP_REFILL_GRAD ? 1 : 0);
     B->cur = 1 - B->cur;
     B->fcur = 1 - B->fcur;
     h->launches += 3;
@@ -466,9 +506,8 @@ lbmp_status batch_create(lbmp_handle* h, const lbmp_batch_sim* sims, int n) {
     B->h_ps.resize(n);
     B->cell_off.resize(n + 1, 0);
     const size_t es = h->cfg.precision == LBMP_FP64 ? 8 : (h->cfg.precision == LBMP_FP32 ? 4 : 2);
-    long long cells = 0, mask_total = 0;
-    int max_box = 1;
-    std::vector<int> bnd_sim;
+    long long cells = 0;
+    std::vector<int> bnd_sim, seg_sim;
     for (int s = 0; s < n; ++s) {
         const lbmp_batch_sim& in = sims[s];
         SimDev& D = B->sims[s];
@@ -507,18 +546,18 @@ lbmp_status batch_create(lbmp_handle* h, const lbmp_batch_sim* sims, int n) {
             if (X.E[a] >= in.edge) X.E[a] = in.edge;
             X.cells *= X.E[a];
         }
-        D.mask_off = (int)mask_total;
-        mask_total += X.cells;
-        const int nbx = (int)((X.cells + BW - 1) / BW);
-        max_box = std::max(max_box, nbx);
+        D.by_edge.set((unsigned)in.edge);
+        D.seg_off = (int)seg_sim.size();
+        D.nseg = (int)((X.cells + SEG - 1) / SEG);
+        seg_sim.insert(seg_sim.end(), (size_t)D.nseg, s);
         D.bnd_off = (int)bnd_sim.size();
-        D.bnd_n = (int)((X.cells + BND_CHUNK - 1) / BND_CHUNK);
-        for (int j = 0; j < D.bnd_n; ++j) bnd_sim.push_back(s);
+        D.bnd_n = (D.nseg + BND_SEGS - 1) / BND_SEGS;
+        bnd_sim.insert(bnd_sim.end(), (size_t)D.bnd_n, s);
         D.hist_off = (long long)s * std::max(1, h->cfg.history_capacity);
     }
     B->cell_off[n] = cells;
     B->total_cells = cells;
-    B->max_box_blocks = max_box;
+    B->segments = (int)seg_sim.size();
     B->bnd_blocks = (int)bnd_sim.size();
     const size_t pop_bytes = es * 19 * (size_t)cells;
     B->pops[0] = handle_alloc(h, pop_bytes);
@@ -528,19 +567,23 @@ lbmp_status batch_create(lbmp_handle* h, const lbmp_batch_sim* sims, int n) {
     B->d_sims = (SimDev*)handle_alloc(h, sizeof(SimDev) * n);
     B->d_cell_off = (long long*)handle_alloc(h, sizeof(long long) * (n + 1));
     B->d_ps = (ParticleState*)handle_alloc(h, sizeof(ParticleState) * n);
-    B->mask = (uint8_t*)handle_alloc(h, (size_t)mask_total);
+    B->seg = (int*)handle_alloc(h, sizeof(int) * SEG * seg_sim.size());
+    B->seg_count = (int*)handle_alloc(h, sizeof(int) * seg_sim.size());
+    B->d_seg_sim = (int*)handle_alloc(h, sizeof(int) * seg_sim.size());
+    B->frames = (PFrames*)handle_alloc(h, sizeof(PFrames) * (size_t)n);
     B->done = (int*)handle_alloc(h, sizeof(int) * n);
     B->partials = (double*)handle_alloc(h, sizeof(double) * 6 * (size_t)B->bnd_blocks);
     B->d_bnd_sim = (int*)handle_alloc(h, sizeof(int) * (size_t)B->bnd_blocks);
     B->history = (double*)handle_alloc(h, sizeof(double) * 15 * (size_t)n * std::max(1, h->cfg.history_capacity));
     if (!B->pops[0] || !B->pops[1] || !B->flags[0] || !B->flags[1] || !B->d_sims || !B->d_cell_off || !B->d_ps ||
-        !B->mask || !B->done || !B->partials || !B->d_bnd_sim || !B->history)
+        !B->seg || !B->seg_count || !B->d_seg_sim || !B->frames || !B->done || !B->partials || !B->d_bnd_sim || !B->history)
         return LBMP_ERR_OOM;
     if (cudaStreamCreateWithFlags(&B->side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&B->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&B->ev_join, cudaEventDisableTiming) != cudaSuccess)
         return LBMP_ERR_CUDA;
     cudaMemcpyAsync(B->d_bnd_sim, bnd_sim.data(), sizeof(int) * bnd_sim.size(), cudaMemcpyHostToDevice, h->stream);
+    cudaMemcpyAsync(B->d_seg_sim, seg_sim.data(), sizeof(int) * seg_sim.size(), cudaMemcpyHostToDevice, h->stream);
     // stream-collide tiles for every candidate shape (edges are multiples of 16)
     for (int c = 0; c < 4; ++c) {
         std::vector<int4> tiles;
@@ -571,13 +614,14 @@ lbmp_status batch_create(lbmp_handle* h, const lbmp_batch_sim* sims, int n) {
         using A = typename Store<S>::A;
         A scale, inv;
         batch_scales<S>(h, &scale, &inv);
-        // boundary flags and mask of the start position (both flag buffers hold its solid cells)
-        const dim3 gr(B->max_box_blocks, B->nsims);
-        k_batch_remap<S><<<gr, BW, 0, h->stream>>>((S*)B->pops[0], B->flags[1], B->flags[0], B->d_sims, B->d_ps,
-                                                   scale, inv, B->mask, 0);   // nothing is uncovered here
+        // frames, boundary flags and segments of the start position (both flag buffers hold its solid cells)
+        k_batch_frames<<<n, 128, 0, h->stream>>>(B->d_sims, B->d_ps, B->frames);
+        k_batch_remap<S><<<B->segments, BW, 0, h->stream>>>((S*)B->pops[0], B->flags[1], B->flags[0], B->d_sims,
+                                                            B->d_seg_sim, B->d_ps, B->frames, scale, inv, B->seg,
+                                                            B->seg_count, 0);   // nothing is uncovered here
     });
     h->h2d += (long long)(sizeof(SimDev) + sizeof(ParticleState) + sizeof(long long)) * n +
-              (long long)(sizeof(int) * bnd_sim.size());
+              (long long)(sizeof(int) * (bnd_sim.size() + seg_sim.size()));
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(h->stream) != cudaSuccess) return LBMP_ERR_CUDA;
     h->has_particle = true;
     return LBMP_OK;

@@ -1133,31 +1133,4 @@ __device__ __forceinline__ void write_segment(bool is_b, int entry, int segment,
     if (threadIdx.x == 0) seg_count[segment] = total;
 }
 
-// Box cells of [t0, t0 + chunk) whose mask byte is set, in box order, into
-// the shared list sl (offsets from t0); returns their number.  blockDim.x
-// is a multiple of 32; chunk may be smaller or larger.  Every thread of the
-// block must call it.
-__device__ __forceinline__ int block_compact_mask(const uint8_t* __restrict__ mask, long long t0, long long cells,
-                                                  int chunk, int* sl) {
-    __shared__ int wcount[32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-    int total = 0;
-    for (int off = 0; off < chunk; off += (int)blockDim.x) {
-        const long long t = t0 + off + threadIdx.x;
-        const bool m = off + (int)threadIdx.x < chunk && t < cells && mask[t] != 0;
-        const unsigned bits = __ballot_sync(0xffffffffu, m);
-        if (lane == 0) wcount[wid] = __popc(bits);
-        __syncthreads();
-        int base = total, add = 0;
-        for (int w = 0; w < nw; ++w) {
-            if (w < wid) base += wcount[w];
-            add += wcount[w];
-        }
-        if (m) sl[base + __popc(bits & ((1u << lane) - 1u))] = off + threadIdx.x;
-        total += add;
-        __syncthreads();
-    }
-    return total;
-}
-
 }  // namespace lbmp
