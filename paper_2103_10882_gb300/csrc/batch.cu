@@ -1,11 +1,14 @@
 // Batched sweep: many independent uniform periodic simulations of uneven size
 // (the paper's (density ratio, Ga) parameter study, Sec. 5) advanced together.
-// Every phase of the coupled step (Algorithm 1) is one launch covering all
-// simulations: stream-collide over a flat tile list, CLI/momentum-exchange
-// boundary (one grid row per simulation), particle update (one CTA per
-// simulation), remap.  Two steps are captured in a CUDA graph and replayed.
-// The stream-collide tile shape is chosen by timing the candidates on the
-// batch itself (autotuner).
+// The coupled step (Algorithm 1) of all simulations is two launches:
+//   k_batch_step   stream-collide over a flat list of runs; among its CTAs
+//                  those of the cells next to the spheres (CLI links,
+//                  momentum exchange), the last of each simulation running
+//                  its particle update
+//   k_batch_remap  flags, refill and boundary cells
+// Two steps are captured in a CUDA graph and replayed.  The stream-collide
+// CTA shape is chosen by timing the candidates on the batch itself
+// (autotuner).
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -35,7 +38,8 @@ struct SimDev {
 };
 
 constexpr int BW = 256;   // threads of the boundary, particle and remap kernels
-constexpr int BND_SEGS = 2;   // segments per boundary block (fewer, fuller blocks: the fixed cost per block dominates)
+constexpr int BND_SEGS = 2;     // segments per boundary CTA of a large batch (fewer, fuller CTAs: the fixed cost dominates)
+constexpr int BND_PARTS = 4;    // CTAs that share a segment's cells in a small batch (there the chain of a warp's cells is the step)
 // Cell flags: fluid, solid (centre inside the sphere), fluid with a solid
 // D3Q19 neighbour (updated by k_batch_boundary instead of the bulk kernel).
 constexpr uint8_t FLAG_FLUID = 0, FLAG_SOLID = 1, FLAG_BOUNDARY = 2;
@@ -55,44 +59,82 @@ __host__ __device__ __forceinline__ CollideParams<typename Store<S>::A> sim_para
     return p;
 }
 
-// ------------------------------------------------------------ stream-collide
-// tile = (simulation, x0, y0, z0); block (16, TY); each thread ZC cells along z.
-template <typename S, int ZC>
-__global__ void __launch_bounds__(512, sizeof(S) == 8 ? 1 : 3) k_batch_bulk(const S* __restrict__ src, S* __restrict__ dst,
-                                                    const uint8_t* __restrict__ flags,
-                                                    const int4* __restrict__ tiles, const SimDev* __restrict__ sims,
-                                                    typename Store<S>::A scale, typename Store<S>::A inv,
-                                                    int* __restrict__ status) {
+// Bulk CTA: its simulation, first item, and what the stream-collide needs of the simulation, so that its pulls wait for
+// one load and not for a chain of two (FP64 takes the collision's parameters from SimDev).
+struct alignas(16) BulkRun {
+    long long pop_off;   // also 19 times the flag offset
+    int sim, item, edge;
+    FastDiv by_edge;
+    float sp, sm, db;
+};
+
+// One step of all simulations.
+template <typename S>
+struct BatchArgs {
     using A = typename Store<S>::A;
-    const int4 t = tiles[blockIdx.x];
-    const SimDev& D = sims[t.x];
-    const CollideParams<A> P = sim_params<S>(D, scale, inv);
-    const int e = D.G.nx;
-    const int x = t.y + threadIdx.x, y = t.z + threadIdx.y;
-    const size_t n = (size_t)D.G.n;
-    const S* s0 = src + D.pop_off;
-    S* d0 = dst + D.pop_off;
-    const uint8_t* fl = flags + D.flag_off;
+    const S* src;
+    S* dst;
+    const uint8_t* flags;
+    const BulkRun* runs;
+    const SimDev* sims;
+    A scale, inv;
+    int* status;
+    int bblocks, bshift;   // boundary CTAs: every 2^bshift-th CTA from the first on
+    int segs, parts;       // segments of a boundary CTA, CTAs that share them
+    const int* seg;
+    const int* seg_count;
+    const int* bnd_sim;
+    ParticleState* ps;
+    PFrames* frames;
+    int cli, hist_cap;
+    double* partials;
+    int* done;
+    double* history;
+};
+
+// ------------------------------------------------------------ stream-collide
+// Item i of a simulation: with ZC = 1 cell i, with ZC = 2 the two cells i mod e^2 of the planes 2 (i / e^2) and the
+// next, one after the other.  Items are taken in memory order.
+template <typename S, int ZC>
+__device__ __forceinline__ void batch_bulk(const BatchArgs<S>& T, const BulkRun& R, int item) {
+    using A = typename Store<S>::A;
+    CollideParams<A> P;
+    if constexpr (sizeof(S) == 8) {
+        P = T.sims[R.sim].P;
+    } else {
+        P.sp = R.sp;
+        P.sm = R.sm;
+        P.db = R.db;
+        P.scale = T.scale;
+        P.inv_scale = T.inv;
+    }
+    const int e = R.edge;
+    const unsigned row = R.by_edge.div((unsigned)item), plane = R.by_edge.div(row);
+    const int x = item - (int)row * e, y = (int)row - (int)plane * e;
+    const size_t n = (size_t)e * (size_t)e * (size_t)e;
+    const S* s0 = T.src + R.pop_off;
+    S* d0 = T.dst + R.pop_off;
+    const uint8_t* fl = T.flags + R.pop_off / 19;
     const int xs[3] = {x + 1 < e ? x + 1 : 0, x, x > 0 ? x - 1 : e - 1};
     const int ys[3] = {y + 1 < e ? y + 1 : 0, y, y > 0 ? y - 1 : e - 1};
 #pragma unroll
     for (int k = 0; k < ZC; ++k) {
-        const int z = t.w + threadIdx.z * ZC + k;
+        const int z = (int)plane * ZC + k;
         const int zs[3] = {z + 1 < e ? z + 1 : 0, z, z > 0 ? z - 1 : e - 1};
         const size_t cell = (size_t)(x + e * (y + e * z));
         const uint8_t f = fl[cell];
-        if (f != FLAG_FLUID) {   // solid: stored as zero; else done by k_batch_boundary
+        A g[19];
+#pragma unroll
+        for (int q = 0; q < 19; ++q)
+            g[q] = Store<S>::fetch(s0 + (size_t)q * n + (size_t)(xs[cx(q) + 1] + e * (ys[cy(q) + 1] + e * zs[cz(q) + 1])),
+                                   P.inv_scale);
+        if (f != FLAG_FLUID) {   // solid: stored as zero; else a boundary CTA's cell
             if (f == FLAG_SOLID)
 #pragma unroll
                 for (int q = 0; q < 19; ++q) Store<S>::store(d0 + (size_t)q * n + cell, A(0), P.scale);
             continue;
         }
-        A g[19];
-#pragma unroll
-        for (int q = 0; q < 19; ++q)
-            g[q] = Store<S>::load(s0 + (size_t)q * n + (size_t)(xs[cx(q) + 1] + e * (ys[cy(q) + 1] + e * zs[cz(q) + 1])),
-                                  P.inv_scale);
-        trt_collide<A, false>(g, P, status);
+        trt_collide<A, false>(g, P, T.status);
 #pragma unroll
         for (int q = 0; q < 19; ++q) Store<S>::store(d0 + (size_t)q * n + cell, g[q], P.scale);
     }
@@ -100,52 +142,41 @@ __global__ void __launch_bounds__(512, sizeof(S) == 8 ? 1 : 3) k_batch_bulk(cons
 
 // ----------------------------------------------------------------- boundary
 // Boundary cells of every simulation (flag 2), from the segments the remap
-// wrote: the grid is flat, block b belongs to simulation bnd_sim[b] and takes
-// BND_SEGS segments of its box, its warps the cells in turn, lane q handling
-// population q (CLI links, geometry in the population arithmetic, FP64 force
-// partials), with a cooperative collision.  All loads of a link are issued
-// at once, its geometry formed meanwhile.  The last of a simulation's blocks
+// wrote: boundary CTA b belongs to simulation bnd_sim[b] and takes some
+// segments of its box, or a part of one's cells, its warps the cells in
+// turn, lane q handling population q (CLI links, geometry in the population
+// arithmetic, FP64 force partials), with a cooperative collision.  All loads of a link are issued
+// at once, its geometry formed meanwhile.  The last of a simulation's CTAs
 // to finish runs its particle update (Algorithm 1) and forms the frames of
-// the moved sphere, which the next kernels read.  The bulk kernel skips these
-// cells, so this kernel runs beside it.
-// Register cap of the boundary kernel (BW threads): it runs beside the bulk kernel (three CTAs of 512 threads
-// at 40 registers per SM), and at its natural 122 registers a resident boundary CTA left room for one bulk CTA.
+// the moved sphere, which the next kernels read.
 template <typename S>
-constexpr int BND_MAXREG = sizeof(S) == 8 ? 128 : 64;
-
-template <typename S>
-__global__ void __maxnreg__(BND_MAXREG<S>)
-    k_batch_boundary(const S* __restrict__ src, S* __restrict__ dst, const uint8_t* __restrict__ flags,
-                     const int* __restrict__ seg, const int* __restrict__ seg_count, const SimDev* __restrict__ sims,
-                     const int* __restrict__ bnd_sim, ParticleState* ps, PFrames* frames, int cli,
-                     typename Store<S>::A scale, typename Store<S>::A inv, double* partials, int* done,
-                     double* __restrict__ history, int hist_cap, int* __restrict__ status) {
+__device__ __forceinline__ void batch_boundary(const BatchArgs<S>& T, int bid) {
     using A = typename Store<S>::A;
     __shared__ LinkFrame<A> Fr;
     __shared__ double sX[3];
-    __shared__ int upto[BND_SEGS];   // cells of the block's segments up to and with each
-    const int sim = bnd_sim[blockIdx.x];
-    const SimDev& D = sims[sim];
+    __shared__ int upto[BND_SEGS];   // cells of the CTA's segments up to and with each
+    const int sim = T.bnd_sim[bid];
+    const SimDev& D = T.sims[sim];
     const GridDesc& G = D.G;
     const int n3[3] = {G.nx, G.ny, G.nz};
     const int per3[3] = {1, 1, 1};
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int local = (int)blockIdx.x - D.bnd_off, seg0 = local * BND_SEGS;
-    if (threadIdx.x == 0) Fr = pframe_link<A>(frames[sim]);   // formed by the last particle update
-    if (threadIdx.x >= 32 && threadIdx.x < 35) sX[threadIdx.x - 32] = ps[sim].x[threadIdx.x - 32];
+    const int local = bid - D.bnd_off, seg0 = local / T.parts * T.segs, part = local % T.parts;
+    if (threadIdx.x == 0) Fr = pframe_link<A>(T.frames[sim]);   // formed by the last particle update
+    if (threadIdx.x >= 32 && threadIdx.x < 35) sX[threadIdx.x - 32] = T.ps[sim].x[threadIdx.x - 32];
     if (threadIdx.x == 64) {
         int t = 0;
 #pragma unroll
         for (int k = 0; k < BND_SEGS; ++k) {
-            t += seg0 + k < D.nseg ? seg_count[D.seg_off + seg0 + k] : 0;
+            t += (k < T.segs && seg0 + k < D.nseg) ? T.seg_count[D.seg_off + seg0 + k] : 0;
             upto[k] = t;
         }
     }
     __syncthreads();
-    const CollideParams<A> P = sim_params<S>(D, scale, inv);
-    const S* s0 = src + D.pop_off;
-    S* d0 = dst + D.pop_off;
-    const uint8_t* fl = flags + D.flag_off;
+    const CollideParams<A> P = sim_params<S>(D, T.scale, T.inv);
+    const S* s0 = T.src + D.pop_off;
+    S* d0 = T.dst + D.pop_off;
+    const uint8_t* fl = T.flags + D.flag_off;
     const size_t n = (size_t)G.n;
     const int q = lane < 19 ? lane : 0, k = opp(q);
     const int cq[3] = {cx(q), cy(q), cz(q)};
@@ -153,11 +184,11 @@ __global__ void __maxnreg__(BND_MAXREG<S>)
     // a warp's last cell is stored after the hand-off: the hand-off's release waits for the stores before it
     A kept = A(0);
     S* kept_at = nullptr;
-    for (int j = wib; j < upto[BND_SEGS - 1]; j += BW / 32) {
+    for (int j = part * (BW / 32) + wib; j < upto[BND_SEGS - 1]; j += T.parts * (BW / 32)) {
         if (kept_at) Store<S>::store(kept_at, kept, P.scale);
         int g = 0;
         while (upto[g] <= j) ++g;
-        const int cell = seg[(size_t)(D.seg_off + seg0 + g) * SEG + (j - (g > 0 ? upto[g - 1] : 0))];
+        const int cell = T.seg[(size_t)(D.seg_off + seg0 + g) * SEG + (j - (g > 0 ? upto[g - 1] : 0))];
         const unsigned row = D.by_edge.div((unsigned)cell), plane = D.by_edge.div(row);
         const int xyz[3] = {cell - (int)row * G.nx, (int)row - (int)plane * G.ny, (int)plane};
         A gq = A(0);
@@ -170,34 +201,55 @@ __global__ void __maxnreg__(BND_MAXREG<S>)
             }
             const int sidx = s3[0] + G.nx * (s3[1] + G.ny * s3[2]), far = f3[0] + G.nx * (f3[1] + G.ny * f3[2]);
             const uint8_t fsrc = fl[sidx], ffar = fl[far];
-            const A pull = Store<S>::load(s0 + (size_t)q * n + sidx, P.inv_scale);
-            const A gt_k = Store<S>::load(s0 + (size_t)k * n + cell, P.inv_scale);
-            const A gt_q = Store<S>::load(s0 + (size_t)q * n + cell, P.inv_scale);
-            const A vfar = Store<S>::load(s0 + (size_t)k * n + far, P.inv_scale);
+            const A pull = Store<S>::fetch(s0 + (size_t)q * n + sidx, P.inv_scale);
+            const A gt_k = Store<S>::fetch(s0 + (size_t)k * n + cell, P.inv_scale);
+            const A gt_q = Store<S>::fetch(s0 + (size_t)q * n + cell, P.inv_scale);
+            const A vfar = Store<S>::fetch(s0 + (size_t)k * n + far, P.inv_scale);
             A d[3];
             int pu[3];
             Fr.offset(xyz, n3, per3, d, pu);
-            CliGeometry<A> L = cli_geometry<A>(q, d, cli != 0, Fr);   // as if the far cell were fluid
+            CliGeometry<A> L = cli_geometry<A>(q, d, T.cli != 0, Fr);   // as if the far cell were fluid
             gq = pull;
             if (q != 0 && fsrc == FLAG_SOLID) {
                 const bool far_ok = ffar != FLAG_SOLID;
-                if (cli && !far_ok) L = cli_geometry<A>(q, d, false, Fr);
+                if (T.cli && !far_ok) L = cli_geometry<A>(q, d, false, Fr);
                 A flk[3], tl3[3];
                 gq = cli_apply<A>(q, L, gt_k, gt_q, far_ok ? vfar : A(0), flk, tl3);
                 acc.add(k, pu, flk, tl3);
             }
         }
-        kept = warp_trt_collide<A, false>(gq, lane, P, status);
+        kept = warp_trt_collide<A, false>(gq, lane, P, T.status);
         if (lane < 19) kept_at = d0 + (size_t)lane * n + cell;
     }
-    block_link_sums<BW>(acc, sX, partials + (size_t)D.bnd_off * 6 + local, D.bnd_n);
-    const bool last = last_block_done(done + sim, D.bnd_n);
+    block_link_sums<BW>(acc, sX, T.partials + (size_t)D.bnd_off * 6 + local, D.bnd_n);
+    const bool last = last_block_done(T.done + sim, D.bnd_n);
     if (kept_at) Store<S>::store(kept_at, kept, P.scale);
     if (last)
         particle_block_update<BW>(
-            ps + sim, partials + (size_t)D.bnd_off * 6, D.bnd_n, G, history + (size_t)D.hist_off * 15, hist_cap, status,
-            frames[sim].inv,
-            [&](const ParticleState& Q, int a, int part) { pframes_axis(frames + sim, Q, n3, D.box, a, part); });
+            T.ps + sim, T.partials + (size_t)D.bnd_off * 6, D.bnd_n, G, T.history + (size_t)D.hist_off * 15, T.hist_cap,
+            T.status, T.frames[sim].inv,
+            [&](const ParticleState& Q, int a, int part) { pframes_axis(T.frames + sim, Q, n3, D.box, a, part); });
+}
+
+// One launch, bound by HBM in FP32 and FP16 and by the FP64 pipe in FP64.  As two kernels on two streams the boundary
+// CTAs, launched beside the bulk kernel, filled the SMs first and held it back: 566 us a step for the sweep's 64 boxes,
+// whose bulk kernel takes 500 alone, now 544 (FP16 467 to 455, 16 boxes in FP64 1643 to 1565).  Spread among the first
+// half of the bulk CTAs they take few slots at a time.  A box by itself and four small ones are bound by the chain
+// from a boundary CTA's first load to the remap's last store: 49 to 34 and 34 to 23 us, most of it from BND_PARTS and
+// from the bulk CTA's one load before its pulls.
+// ZC cells per thread along z, CTAS resident CTAs per SM asked of the compiler: the autotuner's choice.  Neither
+// touches the arithmetic, so the results do not depend on it.
+template <typename S, int ZC, int CTAS>
+__global__ void __launch_bounds__(BW, CTAS) k_batch_step(const __grid_constant__ BatchArgs<S> T) {
+    pdl_trigger();
+    pdl_wait();
+    const unsigned before = min((unsigned)T.bblocks, (blockIdx.x + (1u << T.bshift) - 1u) >> T.bshift);
+    if ((blockIdx.x & ((1u << T.bshift) - 1u)) == 0u && (blockIdx.x >> T.bshift) < (unsigned)T.bblocks) {
+        batch_boundary<S>(T, (int)(blockIdx.x >> T.bshift));
+        return;
+    }
+    const BulkRun R = T.runs[blockIdx.x - before];
+    batch_bulk<S, ZC>(T, R, R.item + (int)threadIdx.x);
 }
 
 // -------------------------------------------------------------------- remap
@@ -210,7 +262,7 @@ __global__ void __maxnreg__(BND_MAXREG<S>)
 // term when grad is set; lane q < 19 writes population q.  Every lane calls
 // it with the same cell.
 template <typename S>
-__device__ __forceinline__ void batch_refill_warp(S* __restrict__ p0, const uint8_t* __restrict__ fc, const GridDesc& G,
+__device__ __forceinline__ void batch_refill_warp(S* p0, const uint8_t* fc, const GridDesc& G,
                                                   const int n3[3], const BoxFrame& F, const ParticleState& P, int i,
                                                   int j, int k, size_t c, typename Store<S>::A scale,
                                                   typename Store<S>::A inv, int grad, double sp) {
@@ -229,7 +281,7 @@ __device__ __forceinline__ void batch_refill_warp(S* __restrict__ p0, const uint
                 ok = fc[y] != FLAG_SOLID;
                 A gp[19];
 #pragma unroll
-                for (int q2 = 0; q2 < 19; ++q2) gp[q2] = Store<S>::load(p0 + (size_t)q2 * n + y, inv);
+                for (int q2 = 0; q2 < 19; ++q2) gp[q2] = Store<S>::fetch(p0 + (size_t)q2 * n + y, inv);
                 r = A(1);
 #pragma unroll
                 for (int q2 = 0; q2 < 19; ++q2) r += gp[q2];
@@ -282,15 +334,16 @@ __device__ __forceinline__ void batch_refill_warp(S* __restrict__ p0, const uint
 // by the block's warps in turn (batch_refill_warp). 
 template <typename S>
 __global__ void __launch_bounds__(BW)
-    k_batch_remap(S* __restrict__ pops, const uint8_t* __restrict__ fcur, uint8_t* __restrict__ fnext,
-                  const SimDev* __restrict__ sims, const int* __restrict__ seg_sim, const ParticleState* __restrict__ ps,
-                  const PFrames* __restrict__ frames, typename Store<S>::A scale, typename Store<S>::A inv,
-                  int* __restrict__ seg, int* __restrict__ seg_count, int grad) {
+    k_batch_remap(S* pops, const uint8_t* fcur, uint8_t* fnext, const SimDev* sims, const int* seg_sim,
+                  const ParticleState* ps, const PFrames* frames, typename Store<S>::A scale, typename Store<S>::A inv,
+                  int* seg, int* seg_count, int grad) {
     using A = typename Store<S>::A;
     static_assert(BW == SEG, "a block is a segment");
     __shared__ BoxFrame F;
     __shared__ int s_n;
     __shared__ int s_g[3][BW];   // uncovered cells
+    pdl_trigger();
+    pdl_wait();
     const int sim = seg_sim[blockIdx.x];
     const SimDev& D = sims[sim];
     const GridDesc& G = D.G;
@@ -378,8 +431,8 @@ __global__ void k_batch_to_f64(const S* __restrict__ pops, double* __restrict__ 
     if (i < count) out[i] = (double)Store<S>::load(pops + i, inv);
 }
 
-struct Tile {
-    int threads_y, zc;
+struct Shape {
+    int zc, dense;   // cells per thread along z; more resident CTAs (fewer registers)
 };
 
 }  // namespace
@@ -402,27 +455,26 @@ struct BatchEngine {
     int* seg_count = nullptr;   // and their number
     int* d_seg_sim = nullptr;   // simulation of each segment
     int segments = 0;
+    int bnd_segs = 1, bnd_parts = 1;   // segments of a boundary CTA, CTAs that share them
     PFrames* frames = nullptr;  // frames of every simulation's sphere
     int* done = nullptr;        // last-block-done counter per simulation
     double* partials = nullptr;
     int bnd_blocks = 1;     // boundary-kernel blocks of all simulations
     int* d_bnd_sim = nullptr;   // simulation of each boundary-kernel block
     double* history = nullptr;
-    // stream-collide tiles for every candidate shape
-    int4* d_tiles[4] = {nullptr, nullptr, nullptr, nullptr};
-    int ntiles[4] = {0, 0, 0, 0};
-    int tile_choice = 1;
-    float tile_ms[4] = {0, 0, 0, 0};
+    // runs of items per bulk CTA for every candidate shape
+    BulkRun* d_runs[2] = {nullptr, nullptr};   // with one and with two cells a thread
+    int nruns[2] = {0, 0};
+    int shape = 0;
+    float shape_ms[4] = {0, 0, 0, 0};
     cudaGraphExec_t graph = nullptr;
     cudaStream_t capture_stream = nullptr;
     long long graph_launches = 0;
-    cudaStream_t side = nullptr;               // k_batch_boundary runs here, beside the bulk kernel
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
 
 namespace {
 
-const Tile TILES[4] = {{8, 1}, {16, 1}, {8, 2}, {16, 2}};   // block (16, threads_y, 1), zc cells per thread
+const Shape SHAPES[4] = {{1, 0}, {2, 0}, {1, 1}, {2, 1}};
 
 template <typename F>
 void with_storage_batch(int prec, F&& f) {
@@ -438,19 +490,40 @@ void batch_scales(const lbmp_handle* h, typename Store<S>::A* scale, typename St
     *inv = (typename Store<S>::A)(f16 ? std::ldexp(1.0, -h->cfg.fp16_scale_log2) : 1.0);
 }
 
+// One step's stream-collide launch in a candidate shape; coupled: with the boundary CTAs.
 template <typename S>
-void launch_bulk_choice(lbmp_handle* h, BatchEngine* B, int choice, const S* src, S* dst) {
-    using A = typename Store<S>::A;
-    A scale, inv;
-    batch_scales<S>(h, &scale, &inv);
-    const Tile t = TILES[choice];
-    const dim3 block(16, t.threads_y, 1);
-    if (t.zc == 1)
-        k_batch_bulk<S, 1><<<B->ntiles[choice], block, 0, h->stream>>>(src, dst, B->flags[B->fcur], B->d_tiles[choice], B->d_sims, scale,
-                                                                       inv, h->status);
-    else
-        k_batch_bulk<S, 2><<<B->ntiles[choice], block, 0, h->stream>>>(src, dst, B->flags[B->fcur], B->d_tiles[choice], B->d_sims, scale,
-                                                                       inv, h->status);
+void launch_step_shape(lbmp_handle* h, BatchEngine* B, int shape, const S* src, S* dst, bool coupled) {
+    BatchArgs<S> T;
+    batch_scales<S>(h, &T.scale, &T.inv);
+    T.src = src;
+    T.dst = dst;
+    T.flags = B->flags[B->fcur];
+    const Shape s = SHAPES[shape];
+    T.runs = B->d_runs[s.zc - 1];
+    T.sims = B->d_sims;
+    T.status = h->status;
+    T.bblocks = coupled ? B->bnd_blocks : 0;
+    T.bshift = 0;
+    T.segs = B->bnd_segs;
+    T.parts = B->bnd_parts;
+    T.seg = B->seg;
+    T.seg_count = B->seg_count;
+    T.bnd_sim = B->d_bnd_sim;
+    T.ps = B->d_ps;
+    T.frames = B->frames;
+    T.cli = h->cfg.boundary == LBMP_CLI ? 1 : 0;
+    T.hist_cap = h->cfg.history_capacity;
+    T.partials = B->partials;
+    T.done = B->done;
+    T.history = B->history;
+    const unsigned grid = (unsigned)(T.bblocks + B->nruns[s.zc - 1]);
+    while (T.bshift < 5 && (unsigned)T.bblocks << (T.bshift + 2) <= grid) ++T.bshift;   // in the first half of the grid
+    auto go = [&](auto kernel) { launch_pdl(kernel, grid, BW, 0, h->stream, T); };
+    constexpr int FEW = sizeof(S) == 8 ? 1 : 5, MORE = sizeof(S) == 8 ? 2 : 6;
+    if (s.zc == 1 && !s.dense) go(k_batch_step<S, 1, FEW>);
+    else if (!s.dense) go(k_batch_step<S, 2, FEW>);
+    else if (s.zc == 1) go(k_batch_step<S, 1, MORE>);
+    else go(k_batch_step<S, 2, MORE>);
 }
 
 template <typename S>
@@ -461,25 +534,15 @@ void enqueue_batch_step(lbmp_handle* h) {
     batch_scales<S>(h, &scale, &inv);
     const S* src = (const S*)B->pops[B->cur];
     S* dst = (S*)B->pops[1 - B->cur];
-    // boundary cells (flag 2) and the particle updates beside the bulk kernel, which skips them
-    cudaEventRecord(B->ev_fork, h->stream);
-    cudaStreamWaitEvent(B->side, B->ev_fork, 0);
-    k_batch_boundary<S><<<B->bnd_blocks, BW, 0, B->side>>>(src, dst, B->flags[B->fcur], B->seg, B->seg_count, B->d_sims,
-                                                           B->d_bnd_sim, B->d_ps, B->frames,
-                                                           h->cfg.boundary == LBMP_CLI ? 1 : 0, scale, inv, B->partials, B->done, B->history,
-                                                           h->cfg.history_capacity, h->status);
-    cudaEventRecord(B->ev_join, B->side);
     const long long ev = profile_mark(h);
-    launch_bulk_choice<S>(h, B, B->tile_choice, src, dst);
+    launch_step_shape<S>(h, B, B->shape, src, dst, true);
     profile_kernel(h, ev, profile_mark(h), 38.0 * sizeof(S) * (double)B->total_cells, (double)B->total_cells);
-    cudaStreamWaitEvent(h->stream, B->ev_join, 0);
-    uint8_t* fnext = B->flags[1 - B->fcur];
-    k_batch_remap<S><<<B->segments, BW, 0, h->stream>>>(dst, B->flags[B->fcur], fnext, B->d_sims, B->d_seg_sim, B->d_ps,
-                                                        B->frames, scale, inv, B->seg, B->seg_count,
-                                                        h->cfg.refill == LBMP_REFILL_GRAD ? 1 : 0);
+    launch_pdl(k_batch_remap<S>, (unsigned)B->segments, BW, 0, h->stream, dst, (const uint8_t*)B->flags[B->fcur],
+               B->flags[1 - B->fcur], (const SimDev*)B->d_sims, (const int*)B->d_seg_sim, (const ParticleState*)B->d_ps,
+               (const PFrames*)B->frames, scale, inv, B->seg, B->seg_count, h->cfg.refill == LBMP_REFILL_GRAD ? 1 : 0);
     B->cur = 1 - B->cur;
     B->fcur = 1 - B->fcur;
-    h->launches += 3;
+    h->launches += 2;
     h->updates += B->total_cells;
 }
 
@@ -490,9 +553,6 @@ void batch_destroy(lbmp_handle* h) {
     if (!B) return;
     if (B->graph) cudaGraphExecDestroy(B->graph);
     if (B->capture_stream) cudaStreamDestroy(B->capture_stream);
-    if (B->side) cudaStreamDestroy(B->side);
-    if (B->ev_fork) cudaEventDestroy(B->ev_fork);
-    if (B->ev_join) cudaEventDestroy(B->ev_join);
     delete B;
     h->batch = nullptr;   // device memory is released with the handle's allocations
 }
@@ -550,10 +610,16 @@ lbmp_status batch_create(lbmp_handle* h, const lbmp_batch_sim* sims, int n) {
         D.seg_off = (int)seg_sim.size();
         D.nseg = (int)((X.cells + SEG - 1) / SEG);
         seg_sim.insert(seg_sim.end(), (size_t)D.nseg, s);
-        D.bnd_off = (int)bnd_sim.size();
-        D.bnd_n = (D.nseg + BND_SEGS - 1) / BND_SEGS;
-        bnd_sim.insert(bnd_sim.end(), (size_t)D.bnd_n, s);
         D.hist_off = (long long)s * std::max(1, h->cfg.history_capacity);
+    }
+    // boundary CTAs: two segments each where that is two or more CTAs per SM, else one, shared by up to BND_PARTS CTAs
+    B->bnd_segs = (int)seg_sim.size() >= 2 * 152 * BND_SEGS ? BND_SEGS : 1;
+    while (B->bnd_segs == 1 && B->bnd_parts < BND_PARTS && (int)seg_sim.size() * B->bnd_parts < 2 * 152) B->bnd_parts *= 2;
+    for (int s = 0; s < n; ++s) {
+        SimDev& D = B->sims[s];
+        D.bnd_off = (int)bnd_sim.size();
+        D.bnd_n = (D.nseg + B->bnd_segs - 1) / B->bnd_segs * B->bnd_parts;
+        bnd_sim.insert(bnd_sim.end(), (size_t)D.bnd_n, s);
     }
     B->cell_off[n] = cells;
     B->total_cells = cells;
@@ -578,26 +644,33 @@ lbmp_status batch_create(lbmp_handle* h, const lbmp_batch_sim* sims, int n) {
     if (!B->pops[0] || !B->pops[1] || !B->flags[0] || !B->flags[1] || !B->d_sims || !B->d_cell_off || !B->d_ps ||
         !B->seg || !B->seg_count || !B->d_seg_sim || !B->frames || !B->done || !B->partials || !B->d_bnd_sim || !B->history)
         return LBMP_ERR_OOM;
-    if (cudaStreamCreateWithFlags(&B->side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&B->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&B->ev_join, cudaEventDisableTiming) != cudaSuccess)
-        return LBMP_ERR_CUDA;
     cudaMemcpyAsync(B->d_bnd_sim, bnd_sim.data(), sizeof(int) * bnd_sim.size(), cudaMemcpyHostToDevice, h->stream);
     cudaMemcpyAsync(B->d_seg_sim, seg_sim.data(), sizeof(int) * seg_sim.size(), cudaMemcpyHostToDevice, h->stream);
-    // stream-collide tiles for every candidate shape (edges are multiples of 16)
-    for (int c = 0; c < 4; ++c) {
-        std::vector<int4> tiles;
-        const int ty = TILES[c].threads_y, zc = TILES[c].zc;
+    // bulk runs with zc = c + 1 cells a thread: a CTA takes BW consecutive items (edges are multiples of 16, e^3 / zc
+    // of 2,048, so runs are whole)
+    long long run_bytes = 0;
+    for (int c = 0; c < 2; ++c) {
+        std::vector<BulkRun> runs;
         for (int s = 0; s < n; ++s) {
-            const int e = B->sims[s].G.nx;
-            for (int z = 0; z < e; z += zc)
-                for (int y = 0; y < e; y += ty)
-                    for (int x = 0; x < e; x += 16) tiles.push_back(make_int4(s, x, y, z));
+            const SimDev& D = B->sims[s];
+            BulkRun R = {};
+            R.pop_off = D.pop_off;
+            R.sim = s;
+            R.edge = D.G.nx;
+            R.by_edge = D.by_edge;
+            R.sp = (float)D.P.sp;
+            R.sm = (float)D.P.sm;
+            R.db = (float)D.P.db;
+            for (long long i = 0; i < D.G.n / (c + 1); i += BW) {
+                R.item = (int)i;
+                runs.push_back(R);
+            }
         }
-        B->ntiles[c] = (int)tiles.size();
-        B->d_tiles[c] = (int4*)handle_alloc(h, sizeof(int4) * tiles.size());
-        if (!B->d_tiles[c]) return LBMP_ERR_OOM;
-        cudaMemcpyAsync(B->d_tiles[c], tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice, h->stream);
+        B->nruns[c] = (int)runs.size();
+        B->d_runs[c] = (BulkRun*)handle_alloc(h, sizeof(BulkRun) * runs.size());
+        if (!B->d_runs[c]) return LBMP_ERR_OOM;
+        cudaMemcpyAsync(B->d_runs[c], runs.data(), sizeof(BulkRun) * runs.size(), cudaMemcpyHostToDevice, h->stream);
+        run_bytes += (long long)(sizeof(BulkRun) * runs.size());
     }
     cudaMemcpyAsync(B->d_sims, B->sims.data(), sizeof(SimDev) * n, cudaMemcpyHostToDevice, h->stream);
     cudaMemcpyAsync(B->d_cell_off, B->cell_off.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, h->stream);
@@ -621,7 +694,7 @@ lbmp_status batch_create(lbmp_handle* h, const lbmp_batch_sim* sims, int n) {
                                                             B->seg_count, 0);   // nothing is uncovered here
     });
     h->h2d += (long long)(sizeof(SimDev) + sizeof(ParticleState) + sizeof(long long)) * n +
-              (long long)(sizeof(int) * (bnd_sim.size() + seg_sim.size()));
+              (long long)(sizeof(int) * (bnd_sim.size() + seg_sim.size())) + run_bytes;
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(h->stream) != cudaSuccess) return LBMP_ERR_CUDA;
     h->has_particle = true;
     return LBMP_OK;
@@ -643,17 +716,17 @@ lbmp_status batch_autotune(lbmp_handle* h, int reps) {
         const S* src = (const S*)B->pops[B->cur];
         S* dst = (S*)B->pops[1 - B->cur];
         for (int c = 0; c < 4; ++c) {
-            launch_bulk_choice<S>(h, B, c, src, dst);   // warm-up
+            launch_step_shape<S>(h, B, c, src, dst, false);   // warm-up
             cudaEventRecord(a, h->stream);
-            for (int r = 0; r < reps; ++r) launch_bulk_choice<S>(h, B, c, src, dst);
+            for (int r = 0; r < reps; ++r) launch_step_shape<S>(h, B, c, src, dst, false);
             cudaEventRecord(b, h->stream);
             cudaEventSynchronize(b);
             float ms = 0.f;
             cudaEventElapsedTime(&ms, a, b);
-            B->tile_ms[c] = ms / reps;
-            if (B->tile_ms[c] < best) {
-                best = B->tile_ms[c];
-                B->tile_choice = c;
+            B->shape_ms[c] = ms / reps;
+            if (B->shape_ms[c] < best) {
+                best = B->shape_ms[c];
+                B->shape = c;
             }
         }
     });
@@ -772,9 +845,9 @@ void batch_info(const lbmp_handle* h, int64_t out[8]) {
     const BatchEngine* B = h->batch;
     out[0] = B->nsims;
     out[1] = B->total_cells;
-    out[2] = 16 * TILES[B->tile_choice].threads_y;
-    out[3] = TILES[B->tile_choice].zc;
-    for (int c = 0; c < 4; ++c) out[4 + c] = (int64_t)(B->tile_ms[c] * 1e6);   // ns per launch
+    out[2] = BW;
+    out[3] = SHAPES[B->shape].zc;
+    for (int c = 0; c < 4; ++c) out[4 + c] = (int64_t)(B->shape_ms[c] * 1e6);   // ns per launch
 }
 
 }  // namespace lbmp

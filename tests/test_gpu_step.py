@@ -32,3 +32,25 @@ def test_step_edges(orc, lib, precision, shape, d, bc, steps):  # noqa: F811
     if precision == "fp64":
         assert np.array_equal(o.flags(), g.flags())
         assert_links_equal(o, g)
+
+
+@pytest.mark.parametrize("edges", [
+    (16,), (32,) * 15, (32,) * 30, (16, 48, 32) * 24,
+], ids=["four CTAs a segment", "two", "one", "two segments a CTA"])
+def test_batch_step_splits(lib, edges):  # noqa: F811
+    """Boundary CTAs of a batch: a segment of a box shared by several, or several segments each (here with an odd last
+    one); first, middle and last simulation against a run of its own (FP64 1e-10)."""
+    sims = [dict(edge=e, pos=np.full(3, e / 2) + 0.01 * i * np.array([1, -1, 0.5]), diameter=max(5.0, e / 6), tau=0.7,
+                 density_ratio=0.6, cv=0.5, gravity=(0.0, 0.0, -2e-5)) for i, e in enumerate(edges)]
+    b = lib.BatchSimulation(sims, precision="fp64")
+    b.step(12)
+    for i in sorted({0, len(sims) // 2, len(sims) - 1}):
+        s = sims[i]
+        g = lib.Simulation((s["edge"],) * 3, precision="fp64", tau=s["tau"])
+        g.add_sphere(s["pos"], s["diameter"], s["density_ratio"], cv=s["cv"])
+        g.set_gravity(s["gravity"])
+        g.init_fluid()
+        g.step(12)
+        a, c = g.populations(), b.populations(i)
+        assert np.abs(a - c).max() <= 1e-10 * np.abs(a).max()
+        np.testing.assert_allclose(b.particle(i)[6:12], g.particle()[6:12], rtol=1e-10, atol=1e-12)
