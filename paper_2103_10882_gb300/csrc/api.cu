@@ -128,14 +128,16 @@ void mark_boundary(lbmp_handle* h) {
 }
 
 lbmp_status read_status(lbmp_handle* h) {
-    int st = 0;
-    LBMP_CK(h, cudaMemcpyAsync(&st, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    // the particle record comes back with the status word (one synchronisation), so that reading
-    // it right after a step costs no second one
+    // the particle record comes back with the status word behind it (one copy, one synchronisation), so that reading it
+    // right after a step costs no second one
     const bool with_ps = h->has_particle && !h->batch;
-    if (with_ps) LBMP_CK(h, cudaMemcpyAsync(&h->h_ps, h->d_ps, sizeof(ParticleState), cudaMemcpyDeviceToHost, h->stream));
+    RecordStatus back;
+    if (with_ps) LBMP_CK(h, cudaMemcpyAsync(&back, h->d_ps, sizeof(back), cudaMemcpyDeviceToHost, h->stream));
+    else LBMP_CK(h, cudaMemcpyAsync(&back.status, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     LBMP_CK(h, cudaStreamSynchronize(h->stream));
-    h->d2h += sizeof(int) + (with_ps ? sizeof(ParticleState) : 0);
+    const int st = back.status;
+    if (with_ps) h->h_ps = back.ps;
+    h->d2h += with_ps ? sizeof(back) : sizeof(int);
     h->ps_current = with_ps;
     if (st != 0) {
         int zero = 0;
@@ -295,8 +297,11 @@ lbmp_status lbmp_create(const lbmp_config* cfg, lbmp_handle** out) {
         h->flags[0] = (uint8_t*)dev_alloc(h, (size_t)n);
         h->flags[1] = (uint8_t*)dev_alloc(h, (size_t)n);
     }
-    h->d_ps = (ParticleState*)dev_alloc(h, sizeof(ParticleState));
-    h->status = (int*)dev_alloc(h, sizeof(int));
+    RecordStatus* record = (RecordStatus*)dev_alloc(h, sizeof(RecordStatus));
+    if (record) {
+        h->d_ps = &record->ps;
+        h->status = &record->status;
+    }
     h->count = (int*)dev_alloc(h, sizeof(int));
     h->history = (double*)dev_alloc(h, sizeof(double) * 15 * (size_t)std::max(1, cfg->history_capacity));
     if ((!refined && (!h->pops[0] || !h->pops[1] || !h->flags[0] || !h->flags[1])) || !h->d_ps || !h->status ||
@@ -702,8 +707,10 @@ lbmp_status lbmp_get_history(lbmp_handle* h, int id, double* out, int max_steps,
         if (batch_get_particle(h, id, &tmp) != LBMP_OK) return fail(h, LBMP_ERR_INVALID_ARG, "lbmp_get_history: no such simulation");
     } else {
         if (!h->has_particle || id != 0) return fail(h, LBMP_ERR_INVALID_ARG, "lbmp_get_history: no such sphere");
-        lbmp_status s = download_particle(h);
-        if (s != LBMP_OK) return s;
+        if (!h->ps_current) {
+            lbmp_status s = download_particle(h);
+            if (s != LBMP_OK) return s;
+        }
         tmp = h->h_ps;
     }
     const long long steps = tmp.steps;
@@ -711,20 +718,17 @@ lbmp_status lbmp_get_history(lbmp_handle* h, int id, double* out, int max_steps,
     const long long avail = std::min<long long>(steps, cap);
     if (n) *n = (int)avail;
     if (!out || max_steps <= 0 || avail == 0) return LBMP_OK;
-    std::vector<double> ring((size_t)cap * 15);
-    if (h->batch) {
-        if (batch_history(h, id, ring.data(), cap) != LBMP_OK) return fail(h, LBMP_ERR_CUDA, "lbmp_get_history: copy failed");
-    } else {
-        LBMP_CK(h, cudaMemcpyAsync(ring.data(), h->history, sizeof(double) * 15 * (size_t)cap, cudaMemcpyDeviceToHost,
-                                   h->stream));
-        LBMP_CK(h, cudaStreamSynchronize(h->stream));
-    }
     const long long m = std::min<long long>(avail, max_steps);
     const long long first = steps - m;   // oldest step returned
-    for (long long i = 0; i < m; ++i) {
-        const long long st = first + i;
-        std::memcpy(out + i * 15, ring.data() + (size_t)(st % cap) * 15, sizeof(double) * 15);
-    }
+    // the ring's rows first % cap on, then its rows from 0 on: straight into out, without the rest of the ring
+    const double* ring = h->batch ? batch_history(h, id) : h->history;
+    const long long at = first % cap, head = std::min<long long>(m, cap - at);
+    LBMP_CK(h, cudaMemcpyAsync(out, ring + at * 15, sizeof(double) * 15 * (size_t)head, cudaMemcpyDeviceToHost, h->stream));
+    if (m > head)
+        LBMP_CK(h, cudaMemcpyAsync(out + head * 15, ring, sizeof(double) * 15 * (size_t)(m - head), cudaMemcpyDeviceToHost,
+                                   h->stream));
+    LBMP_CK(h, cudaStreamSynchronize(h->stream));
+    h->d2h += (long long)sizeof(double) * 15 * m;
     if (n) *n = (int)m;
     return LBMP_OK;
 }

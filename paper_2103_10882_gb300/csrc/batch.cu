@@ -39,6 +39,7 @@ struct SimDev {
 
 constexpr int BW = 256;   // threads of the boundary, particle and remap kernels
 constexpr int BND_SEGS = 2;     // segments per boundary CTA of a large batch (fewer, fuller CTAs: the fixed cost dominates)
+constexpr int RECORDS = 32;      // particle records read back at once (a copy of one record takes as long, 12 us)
 constexpr int BND_PARTS = 4;    // CTAs that share a segment's cells in a small batch (there the chain of a warp's cells is the step)
 // Cell flags: fluid, solid (centre inside the sphere), fluid with a solid
 // D3Q19 neighbour (updated by k_batch_boundary instead of the bulk kernel).
@@ -450,7 +451,8 @@ struct BatchEngine {
     uint8_t* flags[2] = {nullptr, nullptr};
     int fcur = 0;
     ParticleState* d_ps = nullptr;
-    std::vector<ParticleState> h_ps;
+    std::vector<ParticleState> h_ps;   // host copies: of the start, then of what was read back
+    std::vector<char> read;            // per RECORDS records: h_ps holds them as they are on the device
     int* seg = nullptr;         // boundary cells by segment (an entry per box cell of every simulation)
     int* seg_count = nullptr;   // and their number
     int* d_seg_sim = nullptr;   // simulation of each segment
@@ -564,6 +566,7 @@ lbmp_status batch_create(lbmp_handle* h, const lbmp_batch_sim* sims, int n) {
     B->nsims = n;
     B->sims.resize(n);
     B->h_ps.resize(n);
+    B->read.assign((size_t)((n + RECORDS - 1) / RECORDS), 0);
     B->cell_off.resize(n + 1, 0);
     const size_t es = h->cfg.precision == LBMP_FP64 ? 8 : (h->cfg.precision == LBMP_FP32 ? 4 : 2);
     long long cells = 0;
@@ -737,6 +740,7 @@ lbmp_status batch_autotune(lbmp_handle* h, int reps) {
 
 lbmp_status batch_step(lbmp_handle* h, int n) {
     BatchEngine* B = h->batch;
+    std::fill(B->read.begin(), B->read.end(), 0);
     auto one = [&]() {
         with_storage_batch(h->cfg.precision, [&](auto tag) {
             using S = std::remove_pointer_t<decltype(tag)>;
@@ -790,16 +794,23 @@ lbmp_status batch_step(lbmp_handle* h, int n) {
 lbmp_status batch_get_particle(lbmp_handle* h, int sim, ParticleState* out) {
     BatchEngine* B = h->batch;
     if (sim < 0 || sim >= B->nsims) return LBMP_ERR_INVALID_ARG;
-    if (cudaMemcpyAsync(out, B->d_ps + sim, sizeof(ParticleState), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
-        cudaStreamSynchronize(h->stream) != cudaSuccess)
-        return LBMP_ERR_CUDA;
-    h->d2h += sizeof(ParticleState);
+    const int block = sim / RECORDS, first = block * RECORDS;
+    if (!B->read[block]) {
+        const size_t bytes = sizeof(ParticleState) * (size_t)std::min(RECORDS, B->nsims - first);
+        if (cudaMemcpyAsync(B->h_ps.data() + first, B->d_ps + first, bytes, cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
+            cudaStreamSynchronize(h->stream) != cudaSuccess)
+            return LBMP_ERR_CUDA;
+        h->d2h += (long long)bytes;
+        B->read[block] = 1;
+    }
+    *out = B->h_ps[sim];
     return LBMP_OK;
 }
 
 lbmp_status batch_set_particle(lbmp_handle* h, int sim, const ParticleState* in) {
     BatchEngine* B = h->batch;
     if (sim < 0 || sim >= B->nsims) return LBMP_ERR_INVALID_ARG;
+    B->read[sim / RECORDS] = 0;
     if (cudaMemcpyAsync(B->d_ps + sim, in, sizeof(ParticleState), cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
         cudaStreamSynchronize(h->stream) != cudaSuccess)
         return LBMP_ERR_CUDA;
@@ -807,15 +818,8 @@ lbmp_status batch_set_particle(lbmp_handle* h, int sim, const ParticleState* in)
     return LBMP_OK;
 }
 
-lbmp_status batch_history(lbmp_handle* h, int sim, double* ring, int cap) {
-    BatchEngine* B = h->batch;
-    if (sim < 0 || sim >= B->nsims) return LBMP_ERR_INVALID_ARG;
-    if (cudaMemcpyAsync(ring, B->history + (size_t)B->sims[sim].hist_off * 15, sizeof(double) * 15 * (size_t)cap,
-                        cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
-        cudaStreamSynchronize(h->stream) != cudaSuccess)
-        return LBMP_ERR_CUDA;
-    h->d2h += (long long)sizeof(double) * 15 * cap;
-    return LBMP_OK;
+const double* batch_history(const lbmp_handle* h, int sim) {
+    return h->batch->history + (size_t)h->batch->sims[sim].hist_off * 15;
 }
 
 lbmp_status batch_populations(lbmp_handle* h, int sim, double* out, size_t cap) {

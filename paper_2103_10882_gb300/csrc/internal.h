@@ -197,6 +197,14 @@ void handle_free(lbmp_handle* h, void* p);
 
 }  // namespace lbmp
 
+namespace lbmp {
+// The particle record and the status word, side by side on the device so that one copy brings both back.
+struct RecordStatus {
+    ParticleState ps;
+    int status;
+};
+}  // namespace lbmp
+
 // One simulation (opaque to callers of the C ABI).
 struct lbmp_handle {
     lbmp_config cfg;
@@ -216,7 +224,7 @@ struct lbmp_handle {
     int* d_done = nullptr;               // last-block-done counter of the boundary CTAs (uniform grids)
     lbmp::PFrames* frames = nullptr;     // uniform grids: two copies of the sphere's frames, a step reads one
     int frame_cur = 0;                   // (frame_cur) while its particle update writes the other
-    lbmp::ParticleState* d_ps = nullptr;
+    lbmp::ParticleState* d_ps = nullptr;       // of a RecordStatus, as status
     lbmp::ParticleState h_ps;                  // host copy of the parameters
     double* history = nullptr;
     int* status = nullptr;

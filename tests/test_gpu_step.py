@@ -54,3 +54,30 @@ def test_batch_step_splits(lib, edges):  # noqa: F811
         a, c = g.populations(), b.populations(i)
         assert np.abs(a - c).max() <= 1e-10 * np.abs(a).max()
         np.testing.assert_allclose(b.particle(i)[6:12], g.particle()[6:12], rtol=1e-10, atol=1e-12)
+
+
+def test_records_read_back(lib):  # noqa: F811
+    """Histories from a ring that has wrapped, whole and in part, and the particle records of a batch of more than one
+    copy's 32 before and after further steps: equal to those of runs that read nothing in between."""
+    def run(cap, parts):
+        g = lib.Simulation((16, 16, 16), precision="fp64", tau=0.7, history_capacity=cap)
+        g.add_sphere((8.2, 7.9, 8.1), 5.0, 0.6, cv=0.5)
+        g.set_gravity((0, 0, -2e-5))
+        g.init_fluid()
+        for n in parts:
+            g.step(n)
+            g.particle()
+        return g
+    full, ring = run(32, (13,)).history(), run(8, (5, 8))
+    assert full.shape == (13, 15) and np.array_equal(ring.history(), full[5:])
+    assert np.array_equal(run(13, (13,)).history(), full)
+    sims = [dict(edge=16, pos=(8.0, 8.0, 8.0), diameter=5.0, density_ratio=0.3 + 0.01 * i, cv=0.5, tau=0.7,
+                 gravity=(0, 0, -2e-5)) for i in range(34)]
+    a, b = (lib.BatchSimulation(sims, precision="fp64") for _ in range(2))
+    a.step(3)
+    first = [a.particle(i) for i in (0, 31, 32, 33)]
+    a.step(4)
+    b.step(7)
+    for i, was in zip((33, 0, 31, 32), (first[3], *first[:3])):
+        assert np.array_equal(a.particle(i), b.particle(i)) and not np.array_equal(a.particle(i), was)
+        assert np.array_equal(a.history(i), b.history(i)) and a.history(i).shape == (7, 15)
