@@ -37,8 +37,17 @@ namespace lbmp {
 namespace {
 
 constexpr int AT = 256;   // threads per block of the cell kernels
-constexpr int NEAR_BLOCKS_MAX = 608;   // CTAs of the cells next to the sphere (four per SM, each warp takes several of a large sphere's)
-constexpr int ADJ_MIN_CTAS = 4;   // resident reverse-step CTAs per SM asked of the compiler (FP32): 64 registers
+constexpr int NEAR_WARPS_MAX = 4864;   // warps for the cells next to the sphere (32 per SM, each takes several of a large sphere's)
+
+// Threads of a reverse-step CTA, and resident CTAs per SM asked of the compiler: 64 registers in FP32, 128 in FP64.
+// In FP64 an SM runs one instruction in 19 cycles and a warp of its own one in 64, so three or four busy warps fill it:
+// CTAs of two warps, all resident, even out what each SM gets, 25 us a step of 24^3 cells (1,700 instructions on an SM,
+// 17 us).  Of 256 threads, one per SM, its 500 CTAs took 3.3 rounds, 57 us.  FP32 at 64^3 16.2 ms per gradient with
+// CTAs of 128 threads, 16.6 with 256.
+template <typename S>
+constexpr int ADJ_THREADS = sizeof(S) == 8 ? 64 : 128;
+template <typename S>
+constexpr int ADJ_MIN_CTAS = (sizeof(S) == 8 ? 512 : 1024) / ADJ_THREADS<S>;
 
 enum : uint8_t { KIND_PLAIN = 0, KIND_SOLID = 1, KIND_NEAR = 2 };
 
@@ -149,13 +158,13 @@ __device__ __forceinline__ void trt_adjoint(const A (&h)[19], A (&lam)[19], cons
     lam[0] = lam[0] - P.sp * lam[0] + a0;
 }
 
-// Sums of 16 values over the warp's lanes: each exchange halves the values a lane still carries, 16 shuffles where 16
-// separate sums take 80.  Value i ends in the lanes sum16_lane(i) and the one after.
-template <typename A>
-__device__ __forceinline__ A warp_sum16(A (&v)[16]) {
+// Sums of N = 16 or 8 values over the warp's lanes: each exchange halves the values a lane still carries, 16 shuffles
+// where 16 separate sums take 80.  Value i ends in the 32 / N lanes from lane 32 / N * i on.
+template <int N, typename A>
+__device__ __forceinline__ A warp_sums(A (&v)[N]) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int off = 16, m = 8; m >= 1; off >>= 1, m >>= 1) {
+    for (int off = 16, m = N / 2; m >= 1; off >>= 1, m >>= 1) {
         const bool up = (lane & off) != 0;
 #pragma unroll
         for (int i = 0; i < m; ++i) {
@@ -163,7 +172,9 @@ __device__ __forceinline__ A warp_sum16(A (&v)[16]) {
             v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
         }
     }
-    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+#pragma unroll
+    for (int off = 16 / N; off >= 1; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+    return v[0];
 }
 __host__ __device__ constexpr int sum16_lane(int i) { return 2 * i; }
 
@@ -176,7 +187,7 @@ __device__ __forceinline__ A warp_trt_adjoint(A h, A lam, int lane, const AdjPar
     const A f0 = A(c0), f1 = A(c1), f2 = A(c2), wl = w * lam;
     A v[16] = {h,           f0 * h,      f1 * h,      f2 * h,       wl,           f0 * wl,      f1 * wl, f2 * wl,
                f0 * f0 * wl, f1 * f1 * wl, f2 * f2 * wl, f0 * f1 * wl, f0 * f2 * wl, f1 * f2 * wl, A(0),    A(0)};
-    const A mine = warp_sum16<A>(v);
+    const A mine = warp_sums<16>(v);
     A s[14];
 #pragma unroll
     for (int i = 0; i < 14; ++i) s[i] = __shfl_sync(0xffffffffu, mine, sum16_lane(i));
@@ -217,27 +228,28 @@ __device__ __forceinline__ A warp_trt_adjoint(A h, A lam, int lane, const AdjPar
 // FP32 the warps' sums are added as a double-float pair (TwoSum, exact to
 // far below FP32 resolution) and converted once: FP64 arithmetic is slow on
 // this part and every block ends with it.
-template <typename A>
-__device__ __forceinline__ void accumulate_parts(const A part[5], double* __restrict__ acc) {
-    __shared__ A red[5][AT / 32];
+template <int THREADS, typename A>
+__device__ __forceinline__ void accumulate_parts(const A part[5], bool busy, double* __restrict__ acc) {
+    __shared__ A red[5][THREADS / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-        A v = part[c];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-        if (lane == 0) red[c][wid] = v;
+    if (busy) {
+        A v[8] = {part[0], part[1], part[2], part[3], part[4], A(0), A(0), A(0)};
+        const A s = warp_sums<8>(v);
+        const int c = lane >> 2;
+        if ((lane & 3) == 0 && c < 5) red[c][wid] = s;
+    } else if (lane < 5) {
+        red[lane][wid] = A(0);
     }
     __syncthreads();
     if (threadIdx.x < 5) {
         double s;
         if constexpr (sizeof(A) == 4) {
             float h = 0.0f, l = 0.0f;
-            for (int w = 0; w < AT / 32; ++w) df_add(h, l, red[threadIdx.x][w], 0.0f);
+            for (int w = 0; w < THREADS / 32; ++w) df_add(h, l, red[threadIdx.x][w], 0.0f);
             s = (double)h + (double)l;
         } else {
             s = 0.0;
-            for (int w = 0; w < AT / 32; ++w) s += red[threadIdx.x][w];
+            for (int w = 0; w < THREADS / 32; ++w) s += red[threadIdx.x][w];
         }
         acc[(size_t)blockIdx.x * 5 + threadIdx.x] += s;
     }
@@ -378,9 +390,9 @@ __device__ __forceinline__ void reverse_near(const ReverseArgs<S>& T, typename S
     const size_t n = (size_t)G.n;
     const int n3[3] = {G.nx, G.ny, G.nz}, per[3] = {1, 1, 1};
     const int lane = threadIdx.x & 31;
-    const int total = *T.count, W = T.nblocks * (AT / 32);
+    const int total = *T.count, W = T.nblocks * (ADJ_THREADS<S> / 32);
     __syncthreads();
-    for (int t = (int)blockIdx.x * (AT / 32) + (int)(threadIdx.x >> 5); t < total; t += W) {
+    for (int t = (int)blockIdx.x * (ADJ_THREADS<S> / 32) + (int)(threadIdx.x >> 5); t < total; t += W) {
         const int x = T.list[t];
         const unsigned row = T.dx.div((unsigned)x), plane = T.dy.div(row);
         const int p[3] = {x - (int)row * G.nx, (int)row - (int)plane * G.ny, (int)plane};
@@ -436,19 +448,21 @@ __device__ __forceinline__ void reverse_near(const ReverseArgs<S>& T, typename S
 }
 
 template <typename S>
-__global__ void __launch_bounds__(AT, sizeof(S) == 8 ? 1 : ADJ_MIN_CTAS)
+__global__ void __launch_bounds__(ADJ_THREADS<S>, ADJ_MIN_CTAS<S>)
     k_adj_step(const __grid_constant__ ReverseArgs<S> T) {
     using A = typename Store<S>::A;
-    pdl_trigger();
     pdl_wait();
     A part[5] = {A(0), A(0), A(0), A(0), A(0)};
+    bool busy = true;
     if ((int)blockIdx.x < T.nblocks) {
         reverse_near<S>(T, part);
     } else {
-        const unsigned item = (blockIdx.x - (unsigned)T.nblocks) * (unsigned)T.per_cta + threadIdx.x;
-        if ((int)threadIdx.x < T.per_cta && item < (unsigned)T.G.n) reverse_plain<S>(T, item, part);
+        const unsigned cta = blockIdx.x - (unsigned)T.nblocks;
+        const unsigned t = threadIdx.x, item = cta * (unsigned)T.per_cta + t;
+        busy = (int)t < T.per_cta;   // whole warps
+        if (busy && item < (unsigned)T.G.n) reverse_plain<S>(T, item, part);
     }
-    accumulate_parts<A>(part, T.acc);
+    accumulate_parts<ADJ_THREADS<S>>(part, busy, T.acc);
 }
 
 // lambda at a fluid cell next to the sphere: S^T nu with the link terms,
@@ -590,6 +604,7 @@ struct AdjointEngine {
     double* acc = nullptr;    // [acc_blocks][5]
     int acc_blocks = 0, near_blocks = 0, near_cells = 0;
     int cell_blocks = 0;                   // blocks of AT cells
+    int threads = AT;                      // of a reverse-step CTA
     int per_cta = AT, plain_blocks = 0;    // plain cells per reverse-step CTA, and those CTAs
     uint8_t* kind = nullptr;
     int* blk = nullptr;
@@ -720,12 +735,13 @@ lbmp_status adjoint_forward(lbmp_handle* h, const double* u0, int nsteps, int in
         E->state_bytes = es * 19 * n;
         E->nu_bytes = es * 19 * n;
         E->cell_blocks = (int)((n + AT - 1) / AT);
-        E->per_cta = AT;   // small grids over all SMs, as in launch_step
-        while (E->per_cta > 32 && (int)n / E->per_cta < 2 * 152) E->per_cta /= 2;
+        E->threads = h->cfg.precision == LBMP_FP64 ? ADJ_THREADS<double> : ADJ_THREADS<float>;
+        E->per_cta = E->threads;   // small grids over all SMs: four CTAs on each (32^3 FP32 0.3 us a step less than two)
+        while (E->per_cta > 32 && (int)n / E->per_cta < 4 * 152) E->per_cta /= 2;
         E->plain_blocks = (int)((n + (size_t)E->per_cta - 1) / (size_t)E->per_cta);
         E->near_cap = (int)n;
         E->near_blocks = 0;
-        E->acc_blocks = NEAR_BLOCKS_MAX + E->plain_blocks;
+        E->acc_blocks = NEAR_WARPS_MAX / (E->threads / 32) + E->plain_blocks;
         E->ckpt = handle_alloc(h, E->state_bytes * (size_t)nckpt);
         E->seg = handle_alloc(h, E->state_bytes * (size_t)interval);
         E->nu[0] = handle_alloc(h, E->nu_bytes);
@@ -768,7 +784,8 @@ lbmp_status adjoint_forward(lbmp_handle* h, const double* u0, int nsteps, int in
             cudaStreamSynchronize(h->stream) != cudaSuccess)
             return LBMP_ERR_CUDA;
         h->d2h += sizeof(int);
-        E->near_blocks = std::min(NEAR_BLOCKS_MAX, std::max(1, (E->near_cells + AT / 32 - 1) / (AT / 32)));
+        const int warps = E->threads / 32;
+        E->near_blocks = std::min(NEAR_WARPS_MAX / warps, std::max(1, (E->near_cells + warps - 1) / warps));
         E->geometry_done = true;
     }
     cudaMemcpyAsync(E->u0, u0, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, h->stream);
@@ -858,7 +875,7 @@ lbmp_status adjoint_backward(lbmp_handle* h, const double* dJ, double* grad_tau,
                     T.nu_next = nu_next;
                     T.nu_out = nu_out;
                     T.with_seed = s < N ? 1 : 0;
-                    launch_pdl(k_adj_step<S>, (unsigned)(E->near_blocks + E->plain_blocks), AT, 0, h->stream, T);
+                    launch_pdl(k_adj_step<S>, (unsigned)(E->near_blocks + E->plain_blocks), ADJ_THREADS<S>, 0, h->stream, T);
                     // algorithmic bytes: 19 populations of g^{n-1} read, 19 adjoint values read and written per cell
                     const double cells = (double)n;
                     profile_kernel(h, ev, profile_mark(h), cells * (19.0 * sizeof(S) + 38.0 * sizeof(A)), cells);

@@ -398,7 +398,7 @@ lbmp_status lbmp_add_sphere(lbmp_handle* h, const double pos[3], double diameter
     const double shell = 4.0 / 3.0 * M_PI * (ro * ro * ro - ri * ri * ri);
     h->list_cap = (int)std::min<double>((double)B.cells, std::ceil(shell) + 64.0);
     h->list = (int*)dev_alloc(h, sizeof(int) * (size_t)h->list_cap);
-    const int max_blocks = step_boundary_blocks(h->list_cap);
+    const int max_blocks = step_boundary_blocks(h->list_cap, h->cfg.precision == LBMP_FP64 ? BOUNDARY_PER_FP64 : BOUNDARY_PER);
     h->partials = (double*)dev_alloc(h, sizeof(double) * 6 * (size_t)max_blocks);
     h->link_mask = (uint8_t*)dev_alloc(h, (size_t)B.cells);
     const size_t nseg = (size_t)((B.cells + 255) / 256);

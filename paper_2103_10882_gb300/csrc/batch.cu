@@ -242,7 +242,6 @@ __device__ __forceinline__ void batch_boundary(const BatchArgs<S>& T, int bid) {
 // touches the arithmetic, so the results do not depend on it.
 template <typename S, int ZC, int CTAS>
 __global__ void __launch_bounds__(BW, CTAS) k_batch_step(const __grid_constant__ BatchArgs<S> T) {
-    pdl_trigger();
     pdl_wait();
     const unsigned before = min((unsigned)T.bblocks, (blockIdx.x + (1u << T.bshift) - 1u) >> T.bshift);
     if ((blockIdx.x & ((1u << T.bshift) - 1u)) == 0u && (blockIdx.x >> T.bshift) < (unsigned)T.bblocks) {
@@ -343,7 +342,6 @@ __global__ void __launch_bounds__(BW)
     __shared__ BoxFrame F;
     __shared__ int s_n;
     __shared__ int s_g[3][BW];   // uncovered cells
-    pdl_trigger();
     pdl_wait();
     const int sim = seg_sim[blockIdx.x];
     const SimDev& D = sims[sim];

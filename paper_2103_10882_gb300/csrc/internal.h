@@ -104,15 +104,15 @@ struct BoxDesc {
 // Boundary CTAs of a coupled uniform step, also the number of force partials (8 warps each, taking the boundary
 // cells in turn).  The list's capacity is two to three times the boundary cells: one CTA per 20 entries gives every
 // warp about one cell, and the chain of a cell, the sums and the particle update is the step where the bulk update is
-// short (32^3: 17.6 us a step, 19.4 with one per 40; 64 x 64 x 128: 22.7 and 25.3).  Where the bulk update runs for
-// eight waves of CTAs or more the chain hides behind it and half as many cost it less (256 x 128 x 96: 92.0 and
-// 91.3 us; 256^3 in FP16 storage 272 and 270).  Coupled FP64 steps keep one per 32 entries, no slower (61 x 53 x 75:
-// 87.1 and 87.5 us): the sums then group as they always did.  At most eight per SM.
+// short (one per 40 costs a 32^3 step 10%, one per 10 4%).  Where the bulk update runs for eight waves of CTAs or more
+// the chain hides behind it and half as many cost it less (256 x 128 x 96: 92.0 and 91.3 us; 256^3 in FP16 storage 272
+// and 270).  FP64 in launch_step.  At most eight per SM.
 // Boxes of up to SEG_CELLS_MAX cells (spheres up to about 70 cells) find their cells through a prefix of the segments'
 // numbers, 8 KB of shared memory at most; larger ones read a list that a further launch makes.
+constexpr int BOUNDARY_PER = 20, BOUNDARY_PER_FP64 = 8;   // list entries per CTA where there are most CTAs
 constexpr long long SEG_CELLS_MAX = 2048 * 256;
 inline bool step_uses_list(const BoxDesc& b) { return b.cells > SEG_CELLS_MAX; }
-inline int step_boundary_blocks(int list_capacity, int per = 20) {   // per = 20: the most of them
+inline int step_boundary_blocks(int list_capacity, int per) {
     const int n = (list_capacity + per - 1) / per;
     return n < 1 ? 1 : (n > 1216 ? 1216 : n);
 }

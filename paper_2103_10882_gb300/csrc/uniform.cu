@@ -35,6 +35,7 @@ struct StepArgs {
     // the sphere's part (bblocks = 0 without a sphere)
     int bblocks;           // boundary CTAs: every 2^bshift-th CTA from the first on
     int bshift;
+    int thin;              // a warp of every boundary CTA before a second one of any
     int finish;            // last boundary CTA: 0 the particle update, 1 the force into force_out, 2 nothing
     int cli, hist_cap;
     const uint8_t* flags;
@@ -262,7 +263,7 @@ __device__ __forceinline__ void boundary_cells(const StepArgs<S>& T, int bid, in
     // a warp's last cell is stored after the hand-off: the hand-off's release waits for the stores before it
     A kept = A(0);
     S* kept_at = nullptr;
-    for (int j = bid * (STEP_THREADS / 32) + wib; j < total; j += W) {
+    for (int j = sizeof(S) == 8 && T.thin ? wib * T.bblocks + bid : bid * (STEP_THREADS / 32) + wib; j < total; j += W) {
         if (kept_at) Store<S>::store(kept_at, kept, P.scale);
         int at = j;
         if (!T.list) {
@@ -352,30 +353,28 @@ constexpr int STEP_MIN_CTAS = sizeof(S) == 4 ? 5 : (sizeof(S) == 2 ? 4 : 2);
 template <typename S, bool WALLS, bool FORCED>
 __global__ void __launch_bounds__(STEP_THREADS, STEP_MIN_CTAS<S>) k_step(const __grid_constant__ StepArgs<S> T) {
     extern __shared__ int pre[];   // prefix of the segments' numbers (boundary CTAs)
-    pdl_trigger();
     pdl_wait();
     unsigned bulk;
     if (is_boundary_cta(T, blockIdx.x, &bulk)) {
         boundary_cells<S, FORCED>(T, (int)(blockIdx.x >> T.bshift), pre);
         return;
     }
-    const unsigned item = bulk * (unsigned)T.per_cta + threadIdx.x;
-    if ((int)threadIdx.x >= T.per_cta || item >= T.items) return;
+    const unsigned t = threadIdx.x, item = bulk * (unsigned)T.per_cta + t;
+    if ((int)t >= T.per_cta || item >= T.items) return;
     bulk_cells<S, WALLS, FORCED>(T, item);
 }
 
 template <bool WALLS, bool MRT>
 __global__ void __launch_bounds__(STEP_THREADS, 4) k_step_h2(const __grid_constant__ StepArgs<__half> T) {
     extern __shared__ int pre[];
-    pdl_trigger();
     pdl_wait();
     unsigned bulk;
     if (is_boundary_cta(T, blockIdx.x, &bulk)) {
         boundary_cells<__half, false>(T, (int)(blockIdx.x >> T.bshift), pre);
         return;
     }
-    if ((int)threadIdx.x >= T.per_cta) return;   // whole warps
-    const unsigned item = bulk * (unsigned)T.per_cta + threadIdx.x;
+    const unsigned t = threadIdx.x, item = bulk * (unsigned)T.per_cta + t;
+    if ((int)t >= T.per_cta) return;   // whole warps
     bulk_pairs<WALLS, MRT>(T, item, item < T.items);
 }
 
@@ -492,7 +491,6 @@ __global__ void __launch_bounds__(REMAP_THREADS)
     __shared__ int s_n;
     __shared__ int s_g[3][REMAP_THREADS];   // uncovered cells
     const int n3[3] = {G.nx, G.ny, G.nz};
-    pdl_trigger();
     pdl_wait();
     if (threadIdx.x == 0) {
         F = frames->bf;
@@ -694,16 +692,33 @@ void launch_step(const lbmp_handle* h, const S* src, S* dst, const CollideParams
     T.dx.set((unsigned)(pairs ? g.nx / 2 : g.nx));
     T.dy.set((unsigned)g.ny);
     T.items = (unsigned)(pairs ? g.n / 2 : g.n);
-    // Small grids are spread over the SMs: CTAs of fewer cells until there are two per SM (FP64 in particular is
-    // bound by each scheduler's own FP64 rate, so idle SMs cost in proportion).
+    // Small grids are spread over the SMs: CTAs of fewer cells until there is one per SM (with two per SM 24^3 cells
+    // take 14.5 us a step instead of 13.7, 32^3 15.5 instead of 15.2).
+    // FP64: an SM runs one instruction in 19 cycles and a warp of its own one in 64, so three or four busy warps fill
+    // it, and two CTAs' registers.  As long as the launch is resident at once, CTAs are made smaller; and up to 2.5
+    // rounds the boundary cells go to many CTAs of few busy warps each, not eight warps to an SM: 32^3 cells 38.1 to
+    // 25.7 us a step, 40^3 43 to 38, a forward step of the 24^3 gradient 20 to 14.  In longer launches the bulk update
+    // fills the SMs anyway (60^3: 66.9 us with one CTA per 32 entries, 71.5 with one per 8).
+    auto ctas = [&](int per_cta) { return (T.items + (unsigned)per_cta - 1) / (unsigned)per_cta; };
     T.per_cta = STEP_THREADS;
-    while (T.per_cta > 32 && T.items / (unsigned)T.per_cta < 2 * 152) T.per_cta /= 2;
-    const unsigned bulk = (T.items + (unsigned)T.per_cta - 1) / (unsigned)T.per_cta;
+    if (sizeof(S) != 8)
+        while (T.per_cta > 32 && T.items / (unsigned)T.per_cta < 152) T.per_cta /= 2;
+    unsigned bulk = ctas(T.per_cta);
     size_t smem = 0;
     if (h->has_particle) {
-        T.bblocks = step_boundary_blocks(h->list_cap, bulk >= 8 * 5 * 152 ? 40 : (sizeof(S) == 8 && finish == 0 ? 32 : 20));
+        if constexpr (sizeof(S) == 8) {
+            T.bblocks = step_boundary_blocks(h->list_cap, BOUNDARY_PER_FP64);
+            T.thin = bulk + (unsigned)T.bblocks <= 5 * 152;
+            if (!T.thin) T.bblocks = step_boundary_blocks(h->list_cap, bulk >= 8 * 5 * 152 ? 40 : 32);
+        } else {
+            T.bblocks = step_boundary_blocks(h->list_cap, bulk >= 8 * 5 * 152 ? 40 : BOUNDARY_PER);
+        }
         if (step_uses_list(h->box)) T.list = h->list;
         else smem = sizeof(int) * (size_t)((h->box.cells + SEG - 1) / SEG + 1);
+    }
+    if (sizeof(S) == 8) {
+        while (T.per_cta > 32 && (unsigned)T.bblocks + ctas(T.per_cta / 2) <= 2 * 152) T.per_cta /= 2;
+        bulk = ctas(T.per_cta);
     }
     const unsigned grid = (unsigned)T.bblocks + bulk;
     // Boundary CTAs wait on latencies: up to three bulk CTAs between two of them keep the memory busy meanwhile (a
