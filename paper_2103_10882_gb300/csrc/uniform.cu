@@ -124,6 +124,123 @@ __device__ __forceinline__ void bulk_cells(const StepArgs<S>& T, unsigned item) 
     for (int q = 0; q < 19; ++q) Store<S>::store(T.dst + (size_t)q * n + cell, g[q], T.P.scale);
 }
 
+// Two cells side by side in the packed FP32 arithmetic of the part (PTX f32x2): one instruction for both.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(v));
+    return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// Coefficients of collide_pair, each twice.
+struct PairConsts {
+    float2 sp, hp, hm, r0, kF, kE, mF, mE, c15, wF, wE, w0;   // as in CollideConsts; c15 negated
+    float2 one_m;                                             // -1
+    float2 third, u3, h15, half, two, d0, dF, dE;             // MRT: 1/3, c15/3, 3/2, 1/2, -2, -db w of rest, +2 db w, -db w
+};
+inline PairConsts pair_consts(const CollideParams<float>& P) {
+    auto both = [](double v) { return make_float2((float)v, (float)v); };
+    const CollideConsts<float>& k = P.k;
+    PairConsts c;
+    c.sp = both(P.sp);
+    c.hp = both(k.hp);
+    c.hm = both(k.hm);
+    c.r0 = both(k.r0);
+    c.kF = both(k.kF);
+    c.kE = both(k.kE);
+    c.mF = both(k.mF);
+    c.mE = both(k.mE);
+    c.c15 = both(-k.c15);
+    c.wF = both(1.0 / 18.0);
+    c.wE = both(1.0 / 36.0);
+    c.w0 = both(1.0 / 3.0);
+    c.one_m = both(-1.0);
+    c.third = both(-1.0 / 3.0);
+    c.u3 = both(k.c15 / 3.0);
+    c.h15 = both(1.5);
+    c.half = both(0.5);
+    c.two = both(-2.0);
+    c.d0 = both(-P.db / 3.0);
+    c.dF = both(P.db / 9.0);
+    c.dE = both(-P.db / 36.0);
+    return c;
+}
+
+// collide_direct (unforced, scaled) of two cells at once; check0, check1: the cell's velocity is looked at.
+template <bool MRT>
+__device__ __forceinline__ void collide_pair(f32x2 (&g)[19], const PairConsts& C, float inv_scale, bool check0, bool check1,
+                                             int* status) {
+    auto K = [](const float2& v) { return pack2(v.x, v.y); };
+    auto sub2 = [&](f32x2 a, f32x2 b) { return fma2(b, K(C.one_m), a); };
+    f32x2 ps[9], pd[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        ps[k] = add2(g[2 * k + 1], g[2 * k + 2]);
+        pd[k] = sub2(g[2 * k + 1], g[2 * k + 2]);
+    }
+    const f32x2 pF = add2(add2(ps[0], ps[1]), ps[2]);
+    const f32x2 pE = add2(add2(add2(ps[3], ps[4]), add2(ps[5], ps[6])), add2(ps[7], ps[8]));
+    const f32x2 drho = add2(add2(g[0], pF), pE);
+    const f32x2 u[3] = {add2(pd[0], add2(add2(pd[3], pd[4]), add2(pd[5], pd[6]))),
+                        add2(pd[1], add2(sub2(pd[3], pd[4]), add2(pd[7], pd[8]))),
+                        add2(pd[2], add2(sub2(pd[5], pd[6]), sub2(pd[7], pd[8])))};
+    const f32x2 u2[3] = {mul2(u[0], u[0]), mul2(u[1], u[1]), mul2(u[2], u[2])};
+    const f32x2 uu = add2(add2(u2[0], u2[1]), u2[2]);
+    const float2 v = unpack2(uu);
+    const float limit = inv_scale * inv_scale;
+    if ((check0 && !(v.x * limit <= 0.09f)) || (check1 && !(v.y * limit <= 0.09f))) atomicOr(status, STATUS_UNSTABLE_FLUID);
+    const f32x2 R = mul2(K(C.sp), fma2(K(C.c15), uu, drho));
+    f32x2 bF = mul2(K(C.wF), R), bE = mul2(K(C.wE), R), b0 = mul2(K(C.w0), R);
+    if (MRT) {
+        const f32x2 u3 = mul2(K(C.u3), uu);
+        const f32x2 nR = add2(fma2(K(C.third), drho, g[0]), u3), nF = fma2(K(C.third), drho, pF);
+        const f32x2 nE = sub2(fma2(K(C.third), drho, pE), u3);
+        const f32x2 c4 = mul2(K(C.h15), sub2(nE, nR)), c16 = mul2(K(C.half), add2(fma2(K(C.two), nF, nR), nE));
+        b0 = fma2(K(C.d0), sub2(c16, c4), b0);
+        bF = fma2(K(C.dF), c16, bF);
+        bE = fma2(K(C.dE), add2(c4, c16), bE);
+    }
+    g[0] = fma2(K(C.r0), g[0], b0);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int q = 2 * k + 1;
+        f32x2 e, d;
+        if (k < 3) {
+            e = fma2(K(C.kF), u2[k], bF);
+            d = mul2(K(C.mF), u[k]);
+        } else {
+            // pairs 3..8: (+x+y), (+x-y), (+x+z), (+x-z), (+y+z), (+y-z)
+            const int a = k < 7 ? 0 : 1, b = k < 5 ? 1 : 2;
+            const f32x2 cu = (k & 1) ? add2(u[a], u[b]) : sub2(u[a], u[b]);
+            e = fma2(mul2(K(C.kE), cu), cu, bE);
+            d = mul2(K(C.mE), cu);
+        }
+        const f32x2 Sy = fma2(K(C.hp), ps[k], e), Da = fma2(K(C.hm), pd[k], d);
+        g[q] = add2(Sy, Da);
+        g[q + 1] = sub2(Sy, Da);
+    }
+}
+
 // FP16 storage, unforced: the same update, two cells (x, x + 1, x even) per
 // thread.  Every population is read as the aligned pair of halves of its
 // source row; the populations shifted along x take their outer half from the
@@ -134,7 +251,7 @@ __device__ __forceinline__ void bulk_cells(const StepArgs<S>& T, unsigned item) 
 // chosen at compile time.  nx is even; rows hold whole pairs.  Every lane of
 // the warp calls it (valid: the lane has a pair).
 template <bool WALLS, bool MRT>
-__device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, unsigned pair, bool valid) {
+__device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, const PairConsts& K, unsigned pair, bool valid) {
     const GridDesc& G = T.G;
     const int nx = G.nx, ny = G.ny, nz = G.nz;
     const int lane = threadIdx.x & 31;
@@ -175,7 +292,7 @@ __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, unsigned p
         }
     }
     const uint8_t mark0 = box0 >= 0 ? T.mark[box0] : MARK_PLAIN, mark1 = box1 >= 0 ? T.mark[box1] : MARK_PLAIN;
-    float g0[19], g1[19];
+    f32x2 g[19];
 #pragma unroll
     for (int q = 0; q < 19; ++q) {
         const __half2 p = pr[q];
@@ -202,26 +319,25 @@ __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, unsigned p
                 if (wb) b = __high2float(o) + wall_term<float>(G, q, xyz1) * T.P.scale;
             }
         }
-        g0[q] = a;
-        g1[q] = b;
+        g[q] = pack2(a, b);
     }
     if (!valid) return;
     __half* dst = T.dst;
+    collide_pair<MRT>(g, K, T.P.inv_scale, mark0 == MARK_PLAIN, mark1 == MARK_PLAIN, T.status);
     if ((mark0 | mark1) == MARK_PLAIN) {
-        trt_collide<float, false, true, MRT ? 1 : 0, true>(g0, T.P, T.status);
-        trt_collide<float, false, true, MRT ? 1 : 0, true>(g1, T.P, T.status);
 #pragma unroll
-        for (int q = 0; q < 19; ++q)
-            __stcs(reinterpret_cast<__half2*>(dst + (size_t)q * n + cell), __floats2half2_rn(g0[q], g1[q]));
+        for (int q = 0; q < 19; ++q) {
+            const float2 v = unpack2(g[q]);
+            __stcs(reinterpret_cast<__half2*>(dst + (size_t)q * n + cell), __floats2half2_rn(v.x, v.y));
+        }
         return;
     }
     // one of the two is solid or a boundary cell: each by itself
-    if (mark0 == MARK_PLAIN) trt_collide<float, false, true, MRT ? 1 : 0, true>(g0, T.P, T.status);
-    if (mark1 == MARK_PLAIN) trt_collide<float, false, true, MRT ? 1 : 0, true>(g1, T.P, T.status);
 #pragma unroll
     for (int q = 0; q < 19; ++q) {
-        if (mark0 != MARK_BOUNDARY) dst[(size_t)q * n + cell] = __float2half_rn(mark0 == MARK_SOLID ? 0.0f : g0[q]);
-        if (mark1 != MARK_BOUNDARY) dst[(size_t)q * n + cell + 1] = __float2half_rn(mark1 == MARK_SOLID ? 0.0f : g1[q]);
+        const float2 v = unpack2(g[q]);
+        if (mark0 != MARK_BOUNDARY) dst[(size_t)q * n + cell] = __float2half_rn(mark0 == MARK_SOLID ? 0.0f : v.x);
+        if (mark1 != MARK_BOUNDARY) dst[(size_t)q * n + cell + 1] = __float2half_rn(mark1 == MARK_SOLID ? 0.0f : v.y);
     }
 }
 
@@ -365,7 +481,7 @@ __global__ void __launch_bounds__(STEP_THREADS, STEP_MIN_CTAS<S>) k_step(const _
 }
 
 template <bool WALLS, bool MRT>
-__global__ void __launch_bounds__(STEP_THREADS, 4) k_step_h2(const __grid_constant__ StepArgs<__half> T) {
+__global__ void __launch_bounds__(STEP_THREADS, 4) k_step_h2(const __grid_constant__ StepArgs<__half> T, const __grid_constant__ PairConsts K) {
     extern __shared__ int pre[];
     pdl_wait();
     unsigned bulk;
@@ -375,7 +491,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 4) k_step_h2(const __grid_consta
     }
     const unsigned t = threadIdx.x, item = bulk * (unsigned)T.per_cta + t;
     if ((int)t >= T.per_cta) return;   // whole warps
-    bulk_pairs<WALLS, MRT>(T, item, item < T.items);
+    bulk_pairs<WALLS, MRT>(T, K, item, item < T.items);
 }
 
 // ------------------------------------------------------------------ remap
@@ -728,10 +844,12 @@ void launch_step(const lbmp_handle* h, const S* src, S* dst, const CollideParams
     if constexpr (std::is_same<S, __half>::value) {
         if (pairs) {
             const bool mrt = p.db != 0.0f;
-            if (walls && mrt) go(k_step_h2<true, true>);
-            else if (walls) go(k_step_h2<true, false>);
-            else if (mrt) go(k_step_h2<false, true>);
-            else go(k_step_h2<false, false>);
+            const PairConsts K = pair_consts(p);
+            auto go2 = [&](auto kernel) { launch_pdl(kernel, grid, STEP_THREADS, smem, stream, T, K); };
+            if (walls && mrt) go2(k_step_h2<true, true>);
+            else if (walls) go2(k_step_h2<true, false>);
+            else if (mrt) go2(k_step_h2<false, true>);
+            else go2(k_step_h2<false, false>);
             return;
         }
     }
