@@ -246,10 +246,14 @@ __device__ __forceinline__ void collide_pair(f32x2 (&g)[19], const PairConsts& C
 // source row; the populations shifted along x take their outer half from the
 // neighbouring lane (a shuffle); the first lane of a warp or row and the last
 // pair of a warp or row load that one half themselves.  The collision runs on
-// the stored, scaled values (trt_collide's SCALED form, collide_direct), so
-// neither the loads nor the stores multiply by the scale, and TRT or MRT is
-// chosen at compile time.  nx is even; rows hold whole pairs.  Every lane of
-// the warp calls it (valid: the lane has a pair).
+// the stored, scaled values (collide_pair), so neither the loads nor the
+// stores multiply by the scale, and TRT or MRT is chosen at compile time.  nx
+// is even; rows hold whole pairs.  Every lane of the warp calls it (valid:
+// the lane has a pair).
+// Bound by what it issues as much as by HBM (188 us at 256^3): 262 us a step
+// with two scalar collisions, 255 packed, 251 with ordinary stores, 235 with
+// one load for the outer halves of a population and its mirror image (not
+// with walls, where it spills and costs 6%).
 template <bool WALLS, bool MRT>
 __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, const PairConsts& K, unsigned pair, bool valid) {
     const GridDesc& G = T.G;
@@ -285,11 +289,21 @@ __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, const Pair
         const int row = nx * ((yw[q] ? yy : sy) + ny * (yw[q] ? z : sz));
         const __half* pq = src + (size_t)q * n;
         pr[q] = *reinterpret_cast<const __half2*>(pq + row + x);
-        if (cx(q) != 0) {
+        if (WALLS && cx(q) != 0) {
             const int xe = cx(q) == 1 ? xm : xq;
             const bool need = cx(q) == 1 ? first : last;
             ex[q] = pq[row + ((need && xe >= 0) ? xe : x)];
+        } else if (cx(q) == 1) {
+            // its mirror image along x reads the same row: one load for the two, few lanes need both
+            const int m = q == 1 ? 2 : (q == 7 ? 10 : (q == 9 ? 8 : (q == 11 ? 14 : 12)));
+            ex[q] = src[(size_t)(first ? q : m) * n + (size_t)(row + (first ? xm : (last ? xq : x)))];
+            ex[m] = ex[q];
         }
+    }
+    if (!WALLS && first && last) {
+#pragma unroll
+        for (int q = 1; q < 19; ++q)
+            if (cx(q) == -1) ex[q] = src[(size_t)q * n + (size_t)(nx * (ys[cy(q) + 1] + ny * zs[cz(q) + 1]) + xq)];
     }
     const uint8_t mark0 = box0 >= 0 ? T.mark[box0] : MARK_PLAIN, mark1 = box1 >= 0 ? T.mark[box1] : MARK_PLAIN;
     f32x2 g[19];
@@ -328,7 +342,7 @@ __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, const Pair
 #pragma unroll
         for (int q = 0; q < 19; ++q) {
             const float2 v = unpack2(g[q]);
-            __stcs(reinterpret_cast<__half2*>(dst + (size_t)q * n + cell), __floats2half2_rn(v.x, v.y));
+            *reinterpret_cast<__half2*>(dst + (size_t)q * n + cell) = __floats2half2_rn(v.x, v.y);
         }
         return;
     }
