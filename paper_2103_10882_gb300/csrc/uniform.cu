@@ -78,7 +78,8 @@ __device__ __forceinline__ int box_index(const StepArgs<S>& T, int x, int y, int
 // One thread per cell, pull form: g_q(x, t+1) = g~_q(x - c_q, t), then TRT; solid cells are stored as zero and
 // boundary cells left to the boundary CTAs.  Cells are taken in memory order, so full warps touch whole lines
 // whatever the extents (a 2-D tile of a 75-cell row left two threads in five idle).  WALLS: some axis has
-// no-slip walls (bounce-back at the domain edge); FORCED: fluid body force present.
+// no-slip walls (bounce-back at the domain edge, by the address of the load, not by a branch around it: 256 x 128 x 96
+// 87.0 -> 81.3 us a step, 61 x 53 x 75 in FP64 82.4 -> 79.2); FORCED: fluid body force present.
 template <typename S, bool WALLS, bool FORCED>
 __device__ __forceinline__ void bulk_cells(const StepArgs<S>& T, unsigned item) {
     using A = typename Store<S>::A;
@@ -104,13 +105,9 @@ __device__ __forceinline__ void bulk_cells(const StepArgs<S>& T, unsigned item) 
 #pragma unroll
     for (int q = 0; q < 19; ++q) {
         const int sx = xs[cx(q) + 1], sy = ys[cy(q) + 1], sz = zs[cz(q) + 1];
-        if (WALLS && (sx < 0 || sy < 0 || sz < 0)) {   // no-slip wall: bounce-back (moving: Ladd's term)
-            const int xyz[3] = {x, y, z};
-            g[q] = Store<S>::fetch(T.src + (size_t)opp(q) * n + cell, T.P.inv_scale) + wall_term<A>(G, q, xyz);
-        } else {
-            const int off = sx + nx * (sy + ny * sz);
-            g[q] = Store<S>::fetch(T.src + (size_t)q * n + off, T.P.inv_scale);
-        }
+        const bool wall = WALLS && (sx < 0 || sy < 0 || sz < 0);   // no-slip wall: bounce-back
+        const size_t at = wall ? (size_t)opp(q) * n + (size_t)cell : (size_t)q * n + (size_t)(sx + nx * (sy + ny * sz));
+        g[q] = Store<S>::fetch(T.src + at, T.P.inv_scale);
     }
     const uint8_t mark = box >= 0 ? T.mark[box] : MARK_PLAIN;   // beside the pulls, not before them
     if (mark != MARK_PLAIN) {
@@ -118,6 +115,12 @@ __device__ __forceinline__ void bulk_cells(const StepArgs<S>& T, unsigned item) 
 #pragma unroll
             for (int q = 0; q < 19; ++q) Store<S>::store(T.dst + (size_t)q * n + cell, A(0), T.P.scale);
         return;
+    }
+    if (WALLS && G.moving && ((xs[0] | xs[2] | ys[0] | ys[2] | zs[0] | zs[2]) < 0)) {   // moving walls: Ladd's term
+        const int xyz[3] = {x, y, z};
+#pragma unroll
+        for (int q = 1; q < 19; ++q)
+            if ((xs[cx(q) + 1] | ys[cy(q) + 1] | zs[cz(q) + 1]) < 0) g[q] += wall_term<A>(G, q, xyz);
     }
     trt_collide<A, FORCED>(g, T.P, T.status);
 #pragma unroll
@@ -252,8 +255,10 @@ __device__ __forceinline__ void collide_pair(f32x2 (&g)[19], const PairConsts& C
 // the lane has a pair).
 // Bound by what it issues as much as by HBM (188 us at 256^3): 262 us a step
 // with two scalar collisions, 255 packed, 251 with ordinary stores, 235 with
-// one load for the outer halves of a population and its mirror image (not
-// with walls, where it spills and costs 6%).
+// one load for the outer halves of a population and its mirror image.  With
+// walls the bounced populations are chosen by their address, the moving
+// walls' term added after the loads: 256 x 128 x 96 74.7 us a step with a
+// branch around every load, 70.4 packed, 62.0 so.
 template <bool WALLS, bool MRT>
 __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, const PairConsts& K, unsigned pair, bool valid) {
     const GridDesc& G = T.G;
@@ -281,29 +286,29 @@ __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, const Pair
     // loading one: the lanes that need none read their own pair's first half), then the shuffles
     __half2 pr[19];
     __half ex[19];
-    bool yw[19];
+    auto behind = [&](int q) { return WALLS && (ys[cy(q) + 1] < 0 || zs[cz(q) + 1] < 0); };   // a wall in y or z
+    auto row_of = [&](int q) { return nx * (ys[cy(q) + 1] + ny * zs[cz(q) + 1]); };
 #pragma unroll
     for (int q = 0; q < 19; ++q) {
-        const int sy = ys[cy(q) + 1], sz = zs[cz(q) + 1];
-        yw[q] = WALLS && (sy < 0 || sz < 0);
-        const int row = nx * ((yw[q] ? yy : sy) + ny * (yw[q] ? z : sz));
-        const __half* pq = src + (size_t)q * n;
-        pr[q] = *reinterpret_cast<const __half2*>(pq + row + x);
-        if (WALLS && cx(q) != 0) {
-            const int xe = cx(q) == 1 ? xm : xq;
-            const bool need = cx(q) == 1 ? first : last;
-            ex[q] = pq[row + ((need && xe >= 0) ? xe : x)];
-        } else if (cx(q) == 1) {
+        const bool yw = behind(q);
+        const int row = yw ? nx * (yy + ny * z) : row_of(q);
+        pr[q] = *reinterpret_cast<const __half2*>(src + (size_t)(yw ? opp(q) : q) * n + row + x);
+        if (cx(q) == 1) {
             // its mirror image along x reads the same row: one load for the two, few lanes need both
             const int m = q == 1 ? 2 : (q == 7 ? 10 : (q == 9 ? 8 : (q == 11 ? 14 : 12)));
-            ex[q] = src[(size_t)(first ? q : m) * n + (size_t)(row + (first ? xm : (last ? xq : x)))];
+            const bool wall = WALLS && (first ? xm : xq) < 0;   // bounce-back: the cell's own opposite population
+            const int pop = wall ? (first ? opp(q) : opp(m)) : (first ? q : m);
+            ex[q] = src[(size_t)pop * n + (size_t)(wall ? cell + (first ? 0 : 1) : row + (first ? xm : (last ? xq : x)))];
             ex[m] = ex[q];
         }
     }
-    if (!WALLS && first && last) {
+    if (first && last) {
 #pragma unroll
         for (int q = 1; q < 19; ++q)
-            if (cx(q) == -1) ex[q] = src[(size_t)q * n + (size_t)(nx * (ys[cy(q) + 1] + ny * zs[cz(q) + 1]) + xq)];
+            if (cx(q) == -1) {
+                const bool wall = WALLS && xq < 0;
+                ex[q] = src[(size_t)(wall ? opp(q) : q) * n + (size_t)(wall ? cell + 1 : (behind(q) ? nx * (yy + ny * z) : row_of(q)) + xq)];
+            }
     }
     const uint8_t mark0 = box0 >= 0 ? T.mark[box0] : MARK_PLAIN, mark1 = box1 >= 0 ? T.mark[box1] : MARK_PLAIN;
     f32x2 g[19];
@@ -314,29 +319,35 @@ __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, const Pair
         if (cx(q) == 0) {
             a = __low2float(p);
             b = __high2float(p);
-        } else if (cx(q) == 1) {   // sources x - 1 and x
-            const float prev = __shfl_up_sync(0xffffffffu, __high2float(p), 1);
-            a = first ? __half2float(ex[q]) : prev;
-            b = __low2float(p);
-        } else {                   // sources x + 1 and x + 2
-            const float next = __shfl_down_sync(0xffffffffu, __low2float(p), 1);
-            a = __high2float(p);
-            b = last ? __half2float(ex[q]) : next;
-        }
-        if (WALLS) {   // bounce-back (moving walls: Ladd's term, scaled like the stored values)
-            const bool wa = yw[q] || (cx(q) == 1 && xm < 0);
-            const bool wb = yw[q] || (cx(q) == -1 && xq < 0);
-            if (wa || wb) {
-                const __half2 o = *reinterpret_cast<const __half2*>(src + (size_t)opp(q) * n + cell);
-                const int xyz0[3] = {x, yy, z}, xyz1[3] = {x + 1, yy, z};
-                if (wa) a = __low2float(o) + wall_term<float>(G, q, xyz0) * T.P.scale;
-                if (wb) b = __high2float(o) + wall_term<float>(G, q, xyz1) * T.P.scale;
+        } else {
+            if (cx(q) == 1) {   // sources x - 1 and x
+                const float prev = __shfl_up_sync(0xffffffffu, __high2float(p), 1);
+                a = first ? __half2float(ex[q]) : prev;
+                b = __low2float(p);
+            } else {            // sources x + 1 and x + 2
+                const float next = __shfl_down_sync(0xffffffffu, __low2float(p), 1);
+                a = __high2float(p);
+                b = last ? __half2float(ex[q]) : next;
+            }
+            if (behind(q)) {
+                a = __low2float(p);
+                b = __high2float(p);
             }
         }
         g[q] = pack2(a, b);
     }
     if (!valid) return;
     __half* dst = T.dst;
+    if (WALLS && G.moving && ((xm | xq | ys[0] | ys[2] | zs[0] | zs[2]) < 0)) {   // Ladd's term, scaled like the stored values
+        const int xyz0[3] = {x, yy, z}, xyz1[3] = {x + 1, yy, z};
+#pragma unroll
+        for (int q = 1; q < 19; ++q) {
+            const bool wa = behind(q) || (cx(q) == 1 && xm < 0), wb = behind(q) || (cx(q) == -1 && xq < 0);
+            if (wa || wb)
+                g[q] = add2(g[q], pack2(wa ? wall_term<float>(G, q, xyz0) * T.P.scale : 0.0f,
+                                        wb ? wall_term<float>(G, q, xyz1) * T.P.scale : 0.0f));
+        }
+    }
     collide_pair<MRT>(g, K, T.P.inv_scale, mark0 == MARK_PLAIN, mark1 == MARK_PLAIN, T.status);
     if ((mark0 | mark1) == MARK_PLAIN) {
 #pragma unroll

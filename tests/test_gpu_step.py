@@ -81,3 +81,17 @@ def test_records_read_back(lib):  # noqa: F811
     for i, was in zip((33, 0, 31, 32), (first[3], *first[:3])):
         assert np.array_equal(a.particle(i), b.particle(i)) and not np.array_equal(a.particle(i), was)
         assert np.array_equal(a.history(i), b.history(i)) and a.history(i).shape == (7, 15)
+
+
+@pytest.mark.parametrize("precision,shape", [("fp64", (10, 9, 11)), ("fp32", (33, 8, 9)), ("fp16", (10, 9, 11)),
+                                             ("fp16", (66, 8, 9)), ("fp16", (4, 9, 8)), ("fp16", (9, 8, 11))])
+def test_moving_walls_on_every_axis(orc, lib, precision, shape):  # noqa: F811
+    """Walls on all axes, those of x and z moving, gravity-free but forced by the walls: faces, edges and corners of
+    the domain, in FP16 pairs with lanes that begin a row, end one, or both.  Tolerances of test_gpu_uniform.py."""
+    o, g = make_pair(orc, lib, shape, precision=precision, tau=0.7, bc=(N, N, N))
+    for axis, side, u in ((0, 0, (0.0, 0.02, -0.01)), (0, 1, (0.0, -0.01, 0.03)), (2, 1, (0.03, 0.01, 0.0))):
+        o.set_wall_velocity(axis, side, u)
+        g.set_wall_velocity(axis, side, u)
+    o.step(40)
+    g.step(40)
+    assert_pops_close(o, g, {"fp64": 1e-10, "fp32": 1e-5, "fp16": 5e-3}[precision])
