@@ -39,7 +39,8 @@ namespace {
 constexpr int AT = 256;   // threads per block of the cell kernels
 constexpr int NEAR_WARPS_MAX = 4864;   // warps for the cells next to the sphere (32 per SM, each takes several of a large sphere's)
 
-// Threads of a reverse-step CTA, and resident CTAs per SM asked of the compiler: 64 registers in FP32, 128 in FP64.
+// Threads of a reverse-step CTA, and resident CTAs per SM asked of the compiler: 56 registers in FP32 (64^3
+// 2% faster per gradient than 64), 128 in FP64.
 // In FP64 an SM runs one instruction in 19 cycles and a warp of its own one in 64, so three or four busy warps fill it:
 // CTAs of two warps, all resident, even out what each SM gets, 25 us a step of 24^3 cells (1,700 instructions on an SM,
 // 17 us).  Of 256 threads, one per SM, its 500 CTAs took 3.3 rounds, 57 us.  FP32 at 64^3 16.2 ms per gradient with
@@ -47,7 +48,7 @@ constexpr int NEAR_WARPS_MAX = 4864;   // warps for the cells next to the sphere
 template <typename S>
 constexpr int ADJ_THREADS = sizeof(S) == 8 ? 64 : 128;
 template <typename S>
-constexpr int ADJ_MIN_CTAS = (sizeof(S) == 8 ? 512 : 1024) / ADJ_THREADS<S>;
+constexpr int ADJ_MIN_CTAS = sizeof(S) == 8 ? 8 : 9;
 
 enum : uint8_t { KIND_PLAIN = 0, KIND_SOLID = 1, KIND_NEAR = 2 };
 

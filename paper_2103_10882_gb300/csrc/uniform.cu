@@ -16,6 +16,7 @@ namespace lbmp {
 namespace {
 
 constexpr int STEP_THREADS = 256;
+constexpr unsigned WAVES_8 = 8 * 5 * 152;   // bulk CTAs of eight waves, five per SM
 // Marks of the box cells around the sphere, written by the remap: plain fluid cell, fluid cell with a solid
 // D3Q19 neighbour (taken by the boundary CTAs), cell with its centre inside the sphere.
 constexpr uint8_t MARK_PLAIN = 0, MARK_BOUNDARY = 1, MARK_SOLID = 2;
@@ -487,12 +488,9 @@ __device__ __forceinline__ bool is_boundary_cta(const StepArgs<S>& T, unsigned b
 // (11 + 5 us as two launches of their own) runs beside the bulk update instead of after it.  With k_remap for the four
 // remap launches: a 32^3 FP32 step 46.1 -> 23.4 us, 256 x 128 x 96 with walls 123.6 -> 94.2, 61 x 53 x 75 in FP64
 // 175 -> 92 (with collide_direct), 512^3 3066 -> 2997.
-// Registers: 5 CTAs of 256 threads per SM (48 registers) where the bulk update waits on memory.
-template <typename S>
-constexpr int STEP_MIN_CTAS = sizeof(S) == 4 ? 5 : (sizeof(S) == 2 ? 4 : 2);
-
-template <typename S, bool WALLS, bool FORCED>
-__global__ void __launch_bounds__(STEP_THREADS, STEP_MIN_CTAS<S>) k_step(const __grid_constant__ StepArgs<S> T) {
+// CTAS: resident CTAs of 256 threads per SM asked of the compiler (launch_step): FP64 2, FP16 4, FP32 4 or 5.
+template <typename S, bool WALLS, bool FORCED, int CTAS>
+__global__ void __launch_bounds__(STEP_THREADS, CTAS) k_step(const __grid_constant__ StepArgs<S> T) {
     extern __shared__ int pre[];   // prefix of the segments' numbers (boundary CTAs)
     pdl_wait();
     unsigned bulk;
@@ -850,9 +848,9 @@ void launch_step(const lbmp_handle* h, const S* src, S* dst, const CollideParams
         if constexpr (sizeof(S) == 8) {
             T.bblocks = step_boundary_blocks(h->list_cap, BOUNDARY_PER_FP64);
             T.thin = bulk + (unsigned)T.bblocks <= 5 * 152;
-            if (!T.thin) T.bblocks = step_boundary_blocks(h->list_cap, bulk >= 8 * 5 * 152 ? 40 : 32);
+            if (!T.thin) T.bblocks = step_boundary_blocks(h->list_cap, bulk >= WAVES_8 ? 40 : 32);
         } else {
-            T.bblocks = step_boundary_blocks(h->list_cap, bulk >= 8 * 5 * 152 ? 40 : BOUNDARY_PER);
+            T.bblocks = step_boundary_blocks(h->list_cap, bulk >= WAVES_8 ? 40 : BOUNDARY_PER);
         }
         if (step_uses_list(h->box)) T.list = h->list;
         else smem = sizeof(int) * (size_t)((h->box.cells + SEG - 1) / SEG + 1);
@@ -878,10 +876,23 @@ void launch_step(const lbmp_handle* h, const S* src, S* dst, const CollideParams
             return;
         }
     }
-    if (walls && p.forced) go(k_step<S, true, true>);
-    else if (walls) go(k_step<S, true, false>);
-    else if (p.forced) go(k_step<S, false, true>);
-    else go(k_step<S, false, false>);
+    // FP32: a bulk update of more than four waves waits on HBM and wants five CTAs per SM (48 registers, some spilled in
+    // the boundary cells: 512^3 2990 us a step, 3095 with four; 88^3 21.3 and 21.7).  In a shorter one the boundary
+    // cells' chain counts, which four (64 registers) shorten: 32^3 15.2 -> 14.8 us a step, 64 x 64 x 128 with MRT 20.9
+    // -> 19.5, 84^3 20.0 -> 19.3.
+    auto pick = [&](auto ctas) {
+        constexpr int C = decltype(ctas)::value;
+        if (walls && p.forced) go(k_step<S, true, true, C>);
+        else if (walls) go(k_step<S, true, false, C>);
+        else if (p.forced) go(k_step<S, false, true, C>);
+        else go(k_step<S, false, false, C>);
+    };
+    if constexpr (std::is_same<S, float>::value) {
+        if (bulk > 4 * 4 * 152) pick(std::integral_constant<int, 5>());
+        else pick(std::integral_constant<int, 4>());
+    } else {
+        pick(std::integral_constant<int, sizeof(S) == 8 ? 2 : 4>());
+    }
 }
 
 void launch_flags_full(uint8_t* flags, const GridDesc& g, const ParticleState* ps, cudaStream_t stream) {
