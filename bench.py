@@ -518,8 +518,8 @@ def adjoint_line(L, workloads, torch, prec, reps):
         "ms_forward": float(np.median(tf)), "ms_backward": float(np.median(tb)),
         "reverse_mlups": N * n / (float(np.median(tb)) * 1e-3) / 1e6,
         "J": J.item(), "dJ_dtau": gt.item(), "dJ_dgx": gf[0].item(),
-        "roofline": roofline(prof, "k_adj_plain (reverse stream-collide, %s)" % prec,
-                             profiled_traffic("k_adj_plain_%s_adjoint64.md" % prec, "traffic_bytes_per_launch")),
+        "roofline": roofline(prof, "k_adj_step (reverse stream-collide, %s)" % prec,
+                             profiled_traffic("k_adj_step_%s_adjoint64.md" % prec, "traffic_bytes_per_launch")),
         "bytes_per_cell_reverse": 19 * (8 if prec == "fp64" else 4) * 3,
     }
     sim.close()
@@ -696,8 +696,8 @@ def main():
             "workload": uniform_name(e, prec) + ("" if bulk == 1.0 else ", " + model),
             "value": (u1[1] - u0[1]) / (ums * 1e-3) / 1e6, "unit": "MLUPS",
             "ms_per_step": ums / args.uniform_steps,
-            "roofline": roofline(uprof, "k_bulk (stream + %s collide, %s)" % (model, prec),
-                                 profiled_traffic("k_bulk_%s_uniform256.md" % prec, "traffic_bytes_per_launch_512")
+            "roofline": roofline(uprof, "k_step (stream + %s collide, %s)" % (model, prec),
+                                 profiled_traffic("k_step_%s_uniform256.md" % prec, "traffic_bytes_per_launch_512")
                                  if e == 512 and bulk == 1.0 else None),
             "roofline_mlups": measured_peak()[0] * 1e9 / (38 * bpp) / 1e6,
             "clocks": clk_u.summary(),
@@ -730,8 +730,8 @@ def main():
             "ms_per_step": bms / args.batch_steps, "launches_per_step": (b1[2] - b0[2]) / args.batch_steps,
             "autotuner": {"threads_per_tile": int(info[2]), "z_cells_per_thread": int(info[3]),
                           "candidate_us": [v / 1e3 for v in info[4:8]]},
-            "roofline": roofline(bprof, "k_batch_bulk (%s)" % prec,
-                                 profiled_traffic("k_batch_bulk_%s_batch64.md" % prec, "traffic_bytes_per_launch")),
+            "roofline": roofline(bprof, "k_batch_step (%s)" % prec,
+                                 profiled_traffic("k_batch_step_%s_batch64.md" % prec, "traffic_bytes_per_launch")),
             "clocks": clk_b.summary(),
         }
     # --------------------------------------------- differentiation (adjoint)

@@ -274,10 +274,10 @@ typedef struct {
 } lbmp_batch_sim;
 
 lbmp_status lbmp_batch_create(const lbmp_config* cfg, const lbmp_batch_sim* sims, int n, lbmp_handle** out);
-/* Times the candidate stream-collide tile shapes on the batch (reps launches
+/* Times the candidate stream-collide launch shapes on the batch (reps launches
  * each, without advancing the simulations) and keeps the fastest. */
 lbmp_status lbmp_batch_autotune(lbmp_handle* h, int reps);
-/* [0] simulations, [1] cells, [2] threads per tile, [3] cells per thread
+/* [0] simulations, [1] cells, [2] threads per CTA, [3] cells per thread
  * along z, [4..7] measured ns per launch of the four candidate shapes. */
 lbmp_status lbmp_batch_info(lbmp_handle* h, int64_t out[8]);
 /* FP64 deviations [19][edge^3] of one simulation (host memory). */

@@ -31,18 +31,18 @@ struct SimDev {
     long long flag_off;  // byte offset in each flag pool
     FastDiv by_edge;     // division by the edge
     int seg_off, nseg;   // segments of the box: boundary cells and their number per 256 box cells
-    int bnd_off, bnd_n;  // boundary-kernel blocks of the simulation (and their force partials)
+    int bnd_off, bnd_n;  // boundary CTAs of the simulation (and their force partials)
     BoxDesc box;
     CollideParams<double> P;   // FP64: the collision's parameters; else its rates are rounded from here
     long long hist_off;  // records
 };
 
-constexpr int BW = 256;   // threads of the boundary, particle and remap kernels
+constexpr int BW = 256;   // threads of a CTA
 constexpr int BND_SEGS = 2;     // segments per boundary CTA of a large batch (fewer, fuller CTAs: the fixed cost dominates)
 constexpr int RECORDS = 32;      // particle records read back at once (a copy of one record takes as long, 12 us)
 constexpr int BND_PARTS = 4;    // CTAs that share a segment's cells in a small batch (there the chain of a warp's cells is the step)
 // Cell flags: fluid, solid (centre inside the sphere), fluid with a solid
-// D3Q19 neighbour (updated by k_batch_boundary instead of the bulk kernel).
+// D3Q19 neighbour (updated by the boundary CTAs instead of the bulk ones).
 constexpr uint8_t FLAG_FLUID = 0, FLAG_SOLID = 1, FLAG_BOUNDARY = 2;
 
 template <typename S>
@@ -460,7 +460,7 @@ struct BatchEngine {
     int* done = nullptr;        // last-block-done counter per simulation
     double* partials = nullptr;
     int bnd_blocks = 1;     // boundary-kernel blocks of all simulations
-    int* d_bnd_sim = nullptr;   // simulation of each boundary-kernel block
+    int* d_bnd_sim = nullptr;   // simulation of each boundary CTA
     double* history = nullptr;
     // runs of items per bulk CTA for every candidate shape
     BulkRun* d_runs[2] = {nullptr, nullptr};   // with one and with two cells a thread

@@ -46,12 +46,12 @@ __device__ __forceinline__ A wall_term(const GridDesc& G, int q, const int xyz[3
     return t;
 }
 
-// Coefficients of collide_direct, formed once on the host in FP64 (collide_consts): the relaxation and
+// Coefficients of collide_direct and collide_pair, formed once on the host in FP64 (collide_consts): the relaxation and
 // equilibrium factors of a pair's sum and difference, and per pair of directions the constant part of the
 // Guo source.  The quadratic ones include the FP16 storage factor.
 template <typename A>
 struct CollideConsts {
-    A hp, hm, hsm, r0;    // (1 - s+)/2, (1 - s-)/2, s-/2, 1 - s+
+    A hp, hm, hsm, r0;    // (1 - s+)/2, (1 - s-)/2 (collide_pair), s-/2 (collide_direct), 1 - s+
     A kF, kE, mF, mE;     // s+ 9/2 w, s- 3 w on faces and edges
     A c15, cF;            // 3/2, 3 (1 - s+/2)
     A gs[9], ga[9];       // 9 (1 - s+/2) w c_q.F, 3 (1 - s-/2) w c_q.F for q = 1, 3, ..., 17

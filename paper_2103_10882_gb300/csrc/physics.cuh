@@ -60,23 +60,21 @@ __device__ __forceinline__ A dir_dot(int q, A x, A y, A z) {
     return t;
 }
 
-// The collision of trt_collide with the fewest instructions, for the kernels whose time is instructions: FP64
-// (GB300 issues one FP64 warp instruction per scheduler in about 76 cycles: k_bulk in FP64 ran at 242 of them per
-// cell, 0.51e12 a second) and FP16 storage (two cells per thread, issue-bound).  With the sums ps and differences pd
-// of the opposite pairs, both new populations of a pair are S + D and S - D,
+// The collision of trt_collide with the fewest instructions, for FP64, whose time is instructions (an SM issues one FP64
+// warp instruction in 19 cycles, a warp by itself one in 64: at 242 of them per cell the update ran at that rate,
+// 0.51e12 a second), and in packed form for FP16 storage (collide_pair).  With the sums ps and differences pd of the
+// opposite pairs, both new populations of a pair are S + D and S - D,
 //   S = (1 - s+)/2 ps + s+ e+ + (1 - s+/2) S+,   D = (1 - s-)/2 pd + s- e- + (1 - s-/2) S-,
 // the coefficients and the direction's part of the Guo source come from the host (collide_consts), the density part of
 // e+ and the MRT correction are one number per class of directions: 121 instructions per cell unforced (13 more forced).
 // (1 - s+)/2 is exact for s+ in [1/2, 2]; (1 - s-)/2 is not for s- < 1/2, and its rounding would change every cell's
 // momentum by the same relative 6e-17 in every step, so FP64 takes pd/2 - (s-/2) pd in two operations.
-// Measured: a coupled FP64 step of 61 x 53 x 75 cells 175 -> 129 us, a refined FP64 step (1.1 M updates) 394 -> 261 us,
-// an FP16-storage step of 256^3 301 -> 293 us.
+// Measured: a coupled FP64 step of 61 x 53 x 75 cells 175 -> 129 us, a refined FP64 step (1.1 M updates) 394 -> 261 us.
 // The MRT sums over a class follow from ps alone: sum_faces 2 e+ = rho/3, sum_edges 2 e+ = rho/3 + uu/2, and the half
 // source sums to -uF/2, 0 and uF/2 over rest, faces and edges.
 // FP32 storage keeps the plain form below: its kernels wait on memory, not on instructions, and there the rounded
 // coefficient would be a relative 3e-8 a step.  FP16 storage itself rounds at 5e-4 and takes (1 - s-)/2 in one.
-// Populations may be scaled by 2^s (SCALED): quadratic terms then carry 2^-s, which the host's coefficients include.
-template <typename A, bool FORCED, bool SCALED, int MRT_MODE>
+template <typename A, bool FORCED>
 __device__ __forceinline__ void collide_direct(A (&g)[19], const CollideParams<A>& P, int* status) {
     const CollideConsts<A>& K = P.k;
     A ps[9], pd[9];
@@ -98,8 +96,8 @@ __device__ __forceinline__ void collide_direct(A (&g)[19], const CollideParams<A
         uz += A(0.5) * P.F[2];
     }
     const A u2[3] = {ux * ux, uy * uy, uz * uz};
-    const A uu = u2[0] + u2[1] + u2[2];   // SCALED: times 2^2s
-    if (!(uu * (SCALED ? P.inv_scale * P.inv_scale : A(1)) <= A(0.09))) atomicOr(status, STATUS_UNSTABLE_FLUID);
+    const A uu = u2[0] + u2[1] + u2[2];
+    if (!(uu <= A(0.09))) atomicOr(status, STATUS_UNSTABLE_FLUID);
     A R = P.sp * (drho - K.c15 * uu);
     A uF = A(0);
     if (FORCED) {
@@ -107,9 +105,8 @@ __device__ __forceinline__ void collide_direct(A (&g)[19], const CollideParams<A
         R -= K.cF * uF;
     }
     A bF = wgt<A>(1) * R, bE = wgt<A>(7) * R, b0 = wgt<A>(0) * R;
-    const bool mrt = MRT_MODE < 0 ? P.db != A(0) : MRT_MODE == 1;
-    if (mrt) {   // as in trt_collide
-        const A t = drho * (A(1) / A(3)), u3 = K.c15 * (A(1) / A(3)) * uu;   // u3 = uu / 2 (scaled as a population)
+    if (P.db != A(0)) {   // MRT, as in trt_collide
+        const A t = drho * (A(1) / A(3)), u3 = K.c15 * (A(1) / A(3)) * uu;   // u3 = uu / 2
         A nR = g[0] - t + u3;
         const A nF = pF - t;
         A nE = pE - t - u3;
@@ -138,7 +135,7 @@ __device__ __forceinline__ void collide_direct(A (&g)[19], const CollideParams<A
             d = (face ? K.mF : K.mE) * cu;
         }
         const A Sy = K.hp * ps[k] + e;
-        const A Da = sizeof(A) == 8 ? (A(0.5) * pd[k] + d) - K.hsm * pd[k] : K.hm * pd[k] + d;
+        const A Da = (A(0.5) * pd[k] + d) - K.hsm * pd[k];
         g[q] = Sy + Da;
         g[q + 1] = Sy - Da;
     }
@@ -150,14 +147,11 @@ __device__ __forceinline__ void collide_direct(A (&g)[19], const CollideParams<A
 // SCALED: g holds the deviations times 2^s (FP16 storage kept in its scaled
 // form); the collision is linear in g except for the equilibrium's two
 // quadratic terms, which then take one factor 2^-s (P.inv_scale).
-// MRT_MODE: -1 decides TRT or MRT from P.db at run time, 0 is TRT only, 1
-// MRT only (kernels that know which one runs carry no code of the other).
-// DIRECT: collide_direct (FP64, and where a kernel asks for it).
-template <typename A, bool FORCED, bool SCALED = false, int MRT_MODE = -1, bool DIRECT = sizeof(A) == 8>
+template <typename A, bool FORCED, bool SCALED = false>
 __device__ __forceinline__ void trt_collide(A (&g)[19], const CollideParams<A>& P, int* status) {
     static_assert(!(FORCED && SCALED), "the scaled form is for the unforced collision");
-    if constexpr (DIRECT) {
-        collide_direct<A, FORCED, SCALED, MRT_MODE>(g, P, status);
+    if constexpr (sizeof(A) == 8) {
+        collide_direct<A, FORCED>(g, P, status);
         return;
     }
     const A q2 = SCALED ? P.inv_scale : A(1);
@@ -181,7 +175,7 @@ __device__ __forceinline__ void trt_collide(A (&g)[19], const CollideParams<A>& 
     const A uu = (ux * ux + uy * uy + uz * uz) * q2;
     if (!(uu * q2 <= A(0.09))) atomicOr(status, STATUS_UNSTABLE_FLUID);
     const A sp = P.sp, sm = P.sm;
-    const bool mrt = MRT_MODE < 0 ? P.db != A(0) : MRT_MODE == 1;
+    const bool mrt = P.db != A(0);
     // MRT bulk correction: sums of (f - f_eq + source/2) over the rest,
     // face and edge populations (the even modes' inputs)
     A nR = A(0), nF = A(0), nE = A(0);
