@@ -392,21 +392,6 @@ __global__ void k_batch_frames(const SimDev* __restrict__ sims, const ParticleSt
     pframes_form(frames + blockIdx.x, ps[blockIdx.x], n3, D.G.periodic, D.box);
 }
 
-template <typename S>
-__global__ void k_batch_init(S* __restrict__ pops, const uint8_t* __restrict__ flags, const SimDev* __restrict__ sims,
-                             const long long* __restrict__ cell_off, int nsims, long long total,
-                             typename Store<S>::A scale) {
-    using A = typename Store<S>::A;
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= total) return;
-    int sim = 0;
-    while (sim + 1 < nsims && cell_off[sim + 1] <= g) ++sim;
-    const SimDev& D = sims[sim];
-    const long long c = g - cell_off[sim];
-    for (int q = 0; q < 19; ++q) Store<S>::store(pops + D.pop_off + (size_t)q * D.G.n + c, A(0), scale);
-    (void)flags;
-}
-
 __global__ void k_batch_flags_full(uint8_t* __restrict__ f0, uint8_t* __restrict__ f1, const SimDev* __restrict__ sims,
                                    const ParticleState* __restrict__ ps, const long long* __restrict__ cell_off,
                                    int nsims, long long total) {

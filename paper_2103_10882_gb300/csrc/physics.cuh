@@ -415,12 +415,6 @@ __device__ __forceinline__ A cli_apply(int q, const CliGeometry<A>& L, A gt_k, A
     return gnew;
 }
 
-template <typename A>
-__device__ __forceinline__ A cli_link(int q, const A d[3], bool use_delta, A gt_k, A gt_q, A gt_far,
-                                      const LinkFrame<A>& Fr, A fl[3], A tl[3]) {
-    return cli_apply<A>(q, cli_geometry<A>(q, d, use_delta, Fr), gt_k, gt_q, gt_far, fl, tl);
-}
-
 // Per-lane sums of the link forces and torques of one particle.  fl and tl
 // of every link are added in the arithmetic type A; in FP32 each running
 // sum carries its rounding error (Knuth's TwoSum, exact for every

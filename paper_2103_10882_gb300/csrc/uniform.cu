@@ -487,7 +487,7 @@ __device__ __forceinline__ bool is_boundary_cta(const StepArgs<S>& T, unsigned b
 // One launch: boundary CTAs among the first bulk CTAs (launch_step).  The chain boundary cells -> force sum -> particle update
 // (11 + 5 us as two launches of their own) runs beside the bulk update instead of after it.  With k_remap for the four
 // remap launches: a 32^3 FP32 step 46.1 -> 23.4 us, 256 x 128 x 96 with walls 123.6 -> 94.2, 61 x 53 x 75 in FP64
-// 175 -> 92 (with collide_direct), 512^3 3066 -> 2997.
+// 175 -> 92 (with collide_direct), 512^3 3066 -> 2997.  With what the parts below took off since: 14.7, 81.3, 79.2 and 2990.
 // CTAS: resident CTAs of 256 threads per SM asked of the compiler (launch_step): FP64 2, FP16 4, FP32 4 or 5.
 template <typename S, bool WALLS, bool FORCED, int CTAS>
 __global__ void __launch_bounds__(STEP_THREADS, CTAS) k_step(const __grid_constant__ StepArgs<S> T) {
