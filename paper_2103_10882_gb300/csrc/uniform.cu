@@ -64,15 +64,16 @@ __device__ __forceinline__ int box_coord(int v, int o, int n, int periodic, int 
     return (t >= 0 && t < E) ? t : -1;
 }
 
-// Box cell of (x, y, z), -1 outside the sphere's box (and without a sphere).
+// Index of the box cells of row (y, z), -1 outside the sphere's box (and without a sphere).  Most rows lie outside, so
+// only there a cell's own place in the row is looked for, after its loads: 256^3 in FP16 storage 237 -> 228 us a step,
+// the 64^3 gradient 15.7 -> 15.5 ms, 512^3 2989 -> 2976 us.
 template <typename S>
-__device__ __forceinline__ int box_index(const StepArgs<S>& T, int x, int y, int z) {
+__device__ __forceinline__ int box_row(const StepArgs<S>& T, int y, int z) {
     if (T.bblocks == 0) return -1;
     const int* o = T.frames->bf.o;
     const int tz = box_coord(z, o[2], T.G.nz, T.G.periodic[2], T.B.E[2]);
     const int ty = box_coord(y, o[1], T.G.ny, T.G.periodic[1], T.B.E[1]);
-    const int tx = box_coord(x, o[0], T.G.nx, T.G.periodic[0], T.B.E[0]);
-    return (tx | ty | tz) < 0 ? -1 : tx + T.B.E[0] * (ty + T.B.E[1] * tz);
+    return (ty | tz) < 0 ? -1 : T.B.E[0] * (ty + T.B.E[1] * tz);
 }
 
 // ------------------------------------------------------------------ bulk
@@ -101,7 +102,6 @@ __device__ __forceinline__ void bulk_cells(const StepArgs<S>& T, unsigned item) 
     ys[2] = y > 0 ? y - 1 : (WALLS && !G.periodic[1] ? -1 : ny - 1);
     zs[0] = z + 1 < nz ? z + 1 : (WALLS && !G.periodic[2] ? -1 : 0);
     zs[2] = z > 0 ? z - 1 : (WALLS && !G.periodic[2] ? -1 : nz - 1);
-    const int box = box_index<S>(T, x, y, z);
     A g[19];
 #pragma unroll
     for (int q = 0; q < 19; ++q) {
@@ -110,7 +110,12 @@ __device__ __forceinline__ void bulk_cells(const StepArgs<S>& T, unsigned item) 
         const size_t at = wall ? (size_t)opp(q) * n + (size_t)cell : (size_t)q * n + (size_t)(sx + nx * (sy + ny * sz));
         g[q] = Store<S>::fetch(T.src + at, T.P.inv_scale);
     }
-    const uint8_t mark = box >= 0 ? T.mark[box] : MARK_PLAIN;   // beside the pulls, not before them
+    uint8_t mark = MARK_PLAIN;   // beside the pulls, not before them
+    const int box = box_row(T, y, z);
+    if (box >= 0) {
+        const int tx = box_coord(x, T.frames->bf.o[0], nx, G.periodic[0], T.B.E[0]);
+        if (tx >= 0) mark = T.mark[box + tx];
+    }
     if (mark != MARK_PLAIN) {
         if (mark == MARK_SOLID)
 #pragma unroll
@@ -256,10 +261,11 @@ __device__ __forceinline__ void collide_pair(f32x2 (&g)[19], const PairConsts& C
 // the lane has a pair).
 // Bound by what it issues as much as by HBM (188 us at 256^3): 262 us a step
 // with two scalar collisions, 255 packed, 251 with ordinary stores, 235 with
-// one load for the outer halves of a population and its mirror image.  With
+// one load for the outer halves of a population and its mirror image, 228 with
+// the marks after the loads (box_row).  With
 // walls the bounced populations are chosen by their address, the moving
 // walls' term added after the loads: 256 x 128 x 96 74.7 us a step with a
-// branch around every load, 70.4 packed, 62.0 so.
+// branch around every load, 70.4 packed, 62.0 so, 59.0 with box_row.
 template <bool WALLS, bool MRT>
 __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, const PairConsts& K, unsigned pair, bool valid) {
     const GridDesc& G = T.G;
@@ -282,7 +288,6 @@ __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, const Pair
     const int xm = x > 0 ? x - 1 : (WALLS && !G.periodic[0] ? -1 : nx - 1);
     const int xq = x + 2 < nx ? x + 2 : (WALLS && !G.periodic[0] ? -1 : 0);
     const bool first = lane == 0 || x == 0, last = lane == 31 || x + 2 >= nx;   // warp or row ends
-    const int box0 = box_index<__half>(T, x, yy, z), box1 = box_index<__half>(T, x + 1, yy, z);
     // all loads first (the pairs, then the outer halves of the shifted populations, every lane
     // loading one: the lanes that need none read their own pair's first half), then the shuffles
     __half2 pr[19];
@@ -311,7 +316,14 @@ __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, const Pair
                 ex[q] = src[(size_t)(wall ? opp(q) : q) * n + (size_t)(wall ? cell + 1 : (behind(q) ? nx * (yy + ny * z) : row_of(q)) + xq)];
             }
     }
-    const uint8_t mark0 = box0 >= 0 ? T.mark[box0] : MARK_PLAIN, mark1 = box1 >= 0 ? T.mark[box1] : MARK_PLAIN;
+    uint8_t mark0 = MARK_PLAIN, mark1 = MARK_PLAIN;
+    const int box = box_row(T, yy, z);
+    if (box >= 0) {
+        const int t0 = box_coord(x, T.frames->bf.o[0], nx, G.periodic[0], T.B.E[0]);
+        const int t1 = box_coord(x + 1, T.frames->bf.o[0], nx, G.periodic[0], T.B.E[0]);
+        if (t0 >= 0) mark0 = T.mark[box + t0];
+        if (t1 >= 0) mark1 = T.mark[box + t1];
+    }
     f32x2 g[19];
 #pragma unroll
     for (int q = 0; q < 19; ++q) {
