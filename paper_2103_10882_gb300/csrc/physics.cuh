@@ -10,13 +10,14 @@
 namespace lbmp {
 
 // Programmatic dependent launch (PTX griddepcontrol): the CTAs of a kernel launched with the attribute may become
-// resident once every CTA of the kernel ahead has ended (launch_dependents would allow it earlier); pdl_wait returns
-// when that kernel has completed and its writes are visible.  Every thread waits before it reads or writes global
-// memory, so only the launch itself overlaps; loads are ordinary ones (Store::fetch).
-// No kernel calls launch_dependents: CTAs that become resident while the kernel ahead still runs take the slots that
+// resident once every CTA of the kernel ahead has ended or called pdl_trigger; pdl_wait returns when that kernel has
+// completed and its writes are visible.  Every thread waits before it reads or writes global memory, so only the
+// launch itself overlaps; loads are ordinary ones (Store::fetch).
+// No kernel triggers at its start: CTAs that become resident while the kernel ahead still runs take the slots that
 // happen to be free, several of the first, longest ones on one SM, instead of one on each.  Without the attribute, with
-// launch_dependents at the start, and as it is, a 32^3 FP32 step takes 19.3, 16.9 and 15.5 us, a 24^3 FP64 gradient
-// 1.80, 2.92 and 1.79 ms, 256 x 128 x 96 with walls 91.8, 89.2 and 87.4 us a step.
+// a trigger at the start, and with none, a 32^3 FP32 step takes 19.3, 16.9 and 15.5 us, a 24^3 FP64 gradient 1.80, 2.92
+// and 1.79 ms, 256 x 128 x 96 with walls 91.8, 89.2 and 87.4 us a step.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Minimum-image difference for periodic axes.
