@@ -512,16 +512,21 @@ __device__ __forceinline__ void near_lambda(const A* __restrict__ nu, const uint
 }
 
 // lambda^0 and dJ/du0 = (dE/du0)^T lambda^0 with
-// dE_q/du = w_q (3 c_q + 9 (c_q.u0) c_q - 3 u0), times the incoming dJ.
+// dE_q/du = w_q (3 c_q + 9 (c_q.u0) c_q - 3 u0), times the incoming dJ.  In
+// FP64 (u0's type) whatever the field's: bound by its instructions, about 100
+// a cell on the sums and differences of the opposite pairs instead of 320,
+// and in CTAs of two warps for all SMs of a small grid: 63 -> 41 us for 24^3
+// FP64 cells (what is left are the link quotients of the cells by the sphere).
+constexpr int INIT_THREADS = 64;
 template <typename A>
-__global__ void __launch_bounds__(AT)
+__global__ void __launch_bounds__(INIT_THREADS)
     k_adj_init_grad(const A* __restrict__ nu, const uint8_t* __restrict__ flags, const uint8_t* __restrict__ kind,
                     GridDesc G, const double* __restrict__ u0, const ParticleState* __restrict__ ps, int cli, A seed,
                     int axis, const double* __restrict__ dJ, double* __restrict__ grad_u0) {
     __shared__ LinkFrame<A> Fr;
     if (threadIdx.x == 0) Fr.init(*ps);
     __syncthreads();
-    const long long x = (long long)blockIdx.x * AT + threadIdx.x;
+    const long long x = (long long)blockIdx.x * INIT_THREADS + threadIdx.x;
     if (x >= G.n) return;
     const size_t n = (size_t)G.n;
     if (kind[x] == KIND_SOLID) {
@@ -536,17 +541,22 @@ __global__ void __launch_bounds__(AT)
         near_lambda<A>(nu, flags, G, i, j, k, Fr, cli, true, seed, axis, lam);
     }
     const double u[3] = {u0[x], u0[n + x], u0[2 * n + x]};
-    double L0 = 0.0, L1[3] = {0.0, 0.0, 0.0}, L2u[3] = {0.0, 0.0, 0.0};
-    for (int q = 0; q < 19; ++q) {
-        const double wl = wgt<double>(q) * (double)lam[q];
-        const double c[3] = {(double)cx(q), (double)cy(q), (double)cz(q)};
-        const double cu = c[0] * u[0] + c[1] * u[1] + c[2] * u[2];
-        L0 += wl;
-        for (int a = 0; a < 3; ++a) {
-            L1[a] += wl * c[a];
-            L2u[a] += wl * cu * c[a];
-        }
+    double p[9], m[9];   // pairs 0..2 are the faces, 3..8 (+x+y), (+x-y), (+x+z), (+x-z), (+y+z), (+y-z)
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const double a = (double)lam[2 * q + 1], b = (double)lam[2 * q + 2];
+        p[q] = a + b;
+        m[q] = a - b;
     }
+    const double wF = wgt<double>(1), wE = wgt<double>(7);
+    const double exy = p[3] + p[4], exz = p[5] + p[6], eyz = p[7] + p[8];
+    const double L0 = wgt<double>(0) * (double)lam[0] + wF * ((p[0] + p[1]) + p[2]) + wE * ((exy + exz) + eyz);
+    const double L1[3] = {wF * m[0] + wE * ((m[3] + m[4]) + (m[5] + m[6])), wF * m[1] + wE * ((m[3] - m[4]) + (m[7] + m[8])),
+                          wF * m[2] + wE * ((m[5] - m[6]) + (m[7] - m[8]))};
+    const double xy = wE * (p[3] - p[4]), xz = wE * (p[5] - p[6]), yz = wE * (p[7] - p[8]);
+    const double L2u[3] = {(wF * p[0] + wE * (exy + exz)) * u[0] + xy * u[1] + xz * u[2],
+                           xy * u[0] + (wF * p[1] + wE * (exy + eyz)) * u[1] + yz * u[2],
+                           xz * u[0] + yz * u[1] + (wF * p[2] + wE * (exz + eyz)) * u[2]};
     const double s = *dJ;
     for (int a = 0; a < 3; ++a) grad_u0[(size_t)a * n + x] = s * (3.0 * L1[a] + 9.0 * L2u[a] - 3.0 * L0 * u[a]);
 }
@@ -832,7 +842,6 @@ lbmp_status adjoint_backward(lbmp_handle* h, const double* dJ, double* grad_tau,
     const size_t n = (size_t)h->G.n;
     const int N = E->nsteps, K = E->interval;
     const int cli = h->cfg.boundary == LBMP_CLI ? 1 : 0;
-    const unsigned gb = (unsigned)E->cell_blocks;
     lbmp_status st = LBMP_OK;
     with_adj_storage(h->cfg.precision, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
@@ -886,8 +895,8 @@ lbmp_status adjoint_backward(lbmp_handle* h, const double* dJ, double* grad_tau,
         });
         h->launches += (long long)(N - E->nckpt) + (long long)N;
         if (st == LBMP_OK && grad_u0) {   // nu^1 sits in nu[N % 2] after N reverse steps
-            k_adj_init_grad<A><<<gb, AT, 0, h->stream>>>((const A*)E->nu[N & 1], h->flags[h->fcur], E->kind, h->G,
-                                                         E->u0, h->d_ps, cli, P.seed, E->axis, dJ, grad_u0);
+            k_adj_init_grad<A><<<(unsigned)((n + INIT_THREADS - 1) / INIT_THREADS), INIT_THREADS, 0, h->stream>>>(
+                (const A*)E->nu[N & 1], h->flags[h->fcur], E->kind, h->G, E->u0, h->d_ps, cli, P.seed, E->axis, dJ, grad_u0);
             h->launches += 1;
         }
     });
