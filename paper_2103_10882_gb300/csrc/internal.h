@@ -46,12 +46,12 @@ __device__ __forceinline__ A wall_term(const GridDesc& G, int q, const int xyz[3
     return t;
 }
 
-// Coefficients of collide_direct and collide_pair, formed once on the host in FP64 (collide_consts): the relaxation and
+// Coefficients of collide_direct, formed once on the host in FP64 (collide_consts): the relaxation and
 // equilibrium factors of a pair's sum and difference, and per pair of directions the constant part of the
-// Guo source.  The quadratic ones include the FP16 storage factor.
+// Guo source.
 template <typename A>
 struct CollideConsts {
-    A hp, hm, hsm, r0;    // (1 - s+)/2, (1 - s-)/2 (collide_pair), s-/2 (collide_direct), 1 - s+
+    A hp, hsm, r0;        // (1 - s+)/2, s-/2, 1 - s+
     A kF, kE, mF, mE;     // s+ 9/2 w, s- 3 w on faces and edges
     A c15, cF;            // 3/2, 3 (1 - s+/2)
     A gs[9], ga[9];       // 9 (1 - s+/2) w c_q.F, 3 (1 - s-/2) w c_q.F for q = 1, 3, ..., 17
@@ -71,18 +71,17 @@ struct CollideParams {
 // Fills p.k from the rates and the force of p (already rounded to A: the coefficients belong to them).
 template <typename A>
 inline void collide_consts(CollideParams<A>& p) {
-    const double sp = p.sp, sm = p.sm, q2 = p.inv_scale;
+    const double sp = p.sp, sm = p.sm;
     const double wF = 1.0 / 18.0, wE = 1.0 / 36.0;
     CollideConsts<A>& k = p.k;
     k.hp = (A)(0.5 * (1.0 - sp));
-    k.hm = (A)(0.5 * (1.0 - sm));
     k.hsm = (A)(0.5 * sm);
     k.r0 = (A)(1.0 - sp);
-    k.kF = (A)(4.5 * sp * wF * q2);
-    k.kE = (A)(4.5 * sp * wE * q2);
+    k.kF = (A)(4.5 * sp * wF);
+    k.kE = (A)(4.5 * sp * wE);
     k.mF = (A)(3.0 * sm * wF);
     k.mE = (A)(3.0 * sm * wE);
-    k.c15 = (A)(1.5 * q2);
+    k.c15 = (A)1.5;
     k.cF = (A)(3.0 * (1.0 - 0.5 * sp));
     for (int i = 0; i < 9; ++i) {
         const int q = 2 * i + 1;

@@ -63,18 +63,19 @@ __device__ __forceinline__ A dir_dot(int q, A x, A y, A z) {
 
 // The collision of trt_collide with the fewest instructions, for FP64, whose time is instructions (an SM issues one FP64
 // warp instruction in 19 cycles, a warp by itself one in 64: at 242 of them per cell the update ran at that rate,
-// 0.51e12 a second), and in packed form for FP16 storage (collide_pair).  With the sums ps and differences pd of the
-// opposite pairs, both new populations of a pair are S + D and S - D,
+// 0.51e12 a second).  With the sums ps and differences pd of the opposite pairs, both new populations of a pair are
+// S + D and S - D,
 //   S = (1 - s+)/2 ps + s+ e+ + (1 - s+/2) S+,   D = (1 - s-)/2 pd + s- e- + (1 - s-/2) S-,
 // the coefficients and the direction's part of the Guo source come from the host (collide_consts), the density part of
 // e+ and the MRT correction are one number per class of directions: 121 instructions per cell unforced (13 more forced).
-// (1 - s+)/2 is exact for s+ in [1/2, 2]; (1 - s-)/2 is not for s- < 1/2, and its rounding would change every cell's
-// momentum by the same relative 6e-17 in every step, so FP64 takes pd/2 - (s-/2) pd in two operations.
+// (1 - s+)/2 is exact for s+ in [1/2, 2] (below, tau above 2, its rounding scales a cell's density by up to 6e-17 a
+// step, where that of the weights does by 1.1e-16 at tau 0.5); (1 - s-)/2 is not for s- < 1/2, and its rounding would
+// change every cell's momentum by the same relative 6e-17 in every step, so pd/2 - (s-/2) pd takes two operations.
 // Measured: a coupled FP64 step of 61 x 53 x 75 cells 175 -> 129 us, a refined FP64 step (1.1 M updates) 394 -> 261 us.
 // The MRT sums over a class follow from ps alone: sum_faces 2 e+ = rho/3, sum_edges 2 e+ = rho/3 + uu/2, and the half
 // source sums to -uF/2, 0 and uF/2 over rest, faces and edges.
-// FP32 storage keeps the plain form below: its kernels wait on memory, not on instructions, and there the rounded
-// coefficient would be a relative 3e-8 a step.  FP16 storage itself rounds at 5e-4 and takes (1 - s-)/2 in one.
+// FP32 and FP16 storage keep the plain form below (collide_pair: two cells in one): their kernels wait on memory as much
+// as on instructions, and in FP32 arithmetic the rounded coefficient would be a relative 1.5e-8 to 6e-8 a step.
 template <typename A, bool FORCED>
 __device__ __forceinline__ void collide_direct(A (&g)[19], const CollideParams<A>& P, int* status) {
     const CollideConsts<A>& K = P.k;

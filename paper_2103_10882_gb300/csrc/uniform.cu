@@ -161,41 +161,43 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
     return d;
 }
 
-// Coefficients of collide_pair, each twice.
+// Coefficients of collide_pair, each twice (c...: of the quadratic terms, with the FP16 storage factor).
 struct PairConsts {
-    float2 sp, hp, hm, r0, kF, kE, mF, mE, c15, wF, wE, w0;   // as in CollideConsts; c15 negated
-    float2 one_m;                                             // -1
-    float2 third, u3, h15, half, two, d0, dF, dE;             // MRT: 1/3, c15/3, 3/2, 1/2, -2, -db w of rest, +2 db w, -db w
+    float2 one_m, half, three, c15, c45;   // -1, 1/2, 3, -3/2, 9/2
+    float2 w0, wF, wE;                     // lattice weights, negated
+    float2 sp, sm, sm_m;                   // -s+, s-, -s-
+    float2 two, h15, d0, dF, dE;           // MRT: -2, 3/2, -db w of rest, 2 db w of faces, -db w of edges
 };
 inline PairConsts pair_consts(const CollideParams<float>& P) {
-    auto both = [](double v) { return make_float2((float)v, (float)v); };
-    const CollideConsts<float>& k = P.k;
+    auto both = [](float v) { return make_float2(v, v); };
+    const float w0 = wgt<float>(0), wF = wgt<float>(1), wE = wgt<float>(7);
     PairConsts c;
-    c.sp = both(P.sp);
-    c.hp = both(k.hp);
-    c.hm = both(k.hm);
-    c.r0 = both(k.r0);
-    c.kF = both(k.kF);
-    c.kE = both(k.kE);
-    c.mF = both(k.mF);
-    c.mE = both(k.mE);
-    c.c15 = both(-k.c15);
-    c.wF = both(1.0 / 18.0);
-    c.wE = both(1.0 / 36.0);
-    c.w0 = both(1.0 / 3.0);
-    c.one_m = both(-1.0);
-    c.third = both(-1.0 / 3.0);
-    c.u3 = both(k.c15 / 3.0);
-    c.h15 = both(1.5);
-    c.half = both(0.5);
-    c.two = both(-2.0);
-    c.d0 = both(-P.db / 3.0);
-    c.dF = both(P.db / 9.0);
-    c.dE = both(-P.db / 36.0);
+    c.one_m = both(-1.0f);
+    c.half = both(0.5f);
+    c.three = both(3.0f);
+    c.c15 = both(-1.5f * P.inv_scale);
+    c.c45 = both(4.5f * P.inv_scale);
+    c.w0 = both(-w0);
+    c.wF = both(-wF);
+    c.wE = both(-wE);
+    c.sp = both(-P.sp);
+    c.sm = both(P.sm);
+    c.sm_m = both(-P.sm);
+    c.two = both(-2.0f);
+    c.h15 = both(1.5f);
+    c.d0 = both(-(P.db * w0));
+    c.dF = both(2.0f * (P.db * wF));
+    c.dE = both(-(P.db * wE));
     return c;
 }
 
-// collide_direct (unforced, scaled) of two cells at once; check0, check1: the cell's velocity is looked at.
+// trt_collide (unforced, scaled) of two cells at once, the moments from the sums and differences of the opposite pairs;
+// check0, check1: the cell's velocity is looked at.  A population relaxes by s+ and s- times its distance from the
+// equilibrium, g - s+ (g+ - e+) - s- (g- - e-), so that the rounding of the rates is multiplied by that distance: the
+// momentum, which a collision keeps, is scaled by 1 + 2e-10 (tau 0.506) to 1 + 1.5e-8 in a step, by the rounding of the
+// weights.  Sums and differences multiplied by rounded coefficients (1 - s+)/2 and (1 - s-)/2 take 116 instructions
+// instead of 177 (a step of 256^3 cells 224 us and 229; 256 x 128 x 96 with walls, where the instructions are the time,
+// 57 and 67), but scale it by 1 + 1.5e-8 to 1 + 6e-8.  Every product and sum is rounded as written.
 template <bool MRT>
 __device__ __forceinline__ void collide_pair(f32x2 (&g)[19], const PairConsts& C, float inv_scale, bool check0, bool check1,
                                              int* status) {
@@ -207,46 +209,58 @@ __device__ __forceinline__ void collide_pair(f32x2 (&g)[19], const PairConsts& C
         ps[k] = add2(g[2 * k + 1], g[2 * k + 2]);
         pd[k] = sub2(g[2 * k + 1], g[2 * k + 2]);
     }
-    const f32x2 pF = add2(add2(ps[0], ps[1]), ps[2]);
-    const f32x2 pE = add2(add2(add2(ps[3], ps[4]), add2(ps[5], ps[6])), add2(ps[7], ps[8]));
-    const f32x2 drho = add2(add2(g[0], pF), pE);
-    const f32x2 u[3] = {add2(pd[0], add2(add2(pd[3], pd[4]), add2(pd[5], pd[6]))),
-                        add2(pd[1], add2(sub2(pd[3], pd[4]), add2(pd[7], pd[8]))),
-                        add2(pd[2], add2(sub2(pd[5], pd[6]), sub2(pd[7], pd[8])))};
-    const f32x2 u2[3] = {mul2(u[0], u[0]), mul2(u[1], u[1]), mul2(u[2], u[2])};
-    const f32x2 uu = add2(add2(u2[0], u2[1]), u2[2]);
+    f32x2 drho = g[0];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) drho = add2(drho, ps[k]);
+    // pairs 3..8: (+x+y), (+x-y), (+x+z), (+x-z), (+y+z), (+y-z)
+    const f32x2 u[3] = {add2(add2(add2(add2(pd[0], pd[3]), pd[4]), pd[5]), pd[6]),
+                        add2(add2(sub2(add2(pd[1], pd[3]), pd[4]), pd[7]), pd[8]),
+                        sub2(add2(sub2(add2(pd[2], pd[5]), pd[6]), pd[7]), pd[8])};
+    const f32x2 uu = fma2(u[2], u[2], fma2(u[1], u[1], mul2(u[0], u[0])));
     const float2 v = unpack2(uu);
     const float limit = inv_scale * inv_scale;
     if ((check0 && !(v.x * limit <= 0.09f)) || (check1 && !(v.y * limit <= 0.09f))) atomicOr(status, STATUS_UNSTABLE_FLUID);
-    const f32x2 R = mul2(K(C.sp), fma2(K(C.c15), uu, drho));
-    f32x2 bF = mul2(K(C.wF), R), bE = mul2(K(C.wE), R), b0 = mul2(K(C.w0), R);
-    if (MRT) {
-        const f32x2 u3 = mul2(K(C.u3), uu);
-        const f32x2 nR = add2(fma2(K(C.third), drho, g[0]), u3), nF = fma2(K(C.third), drho, pF);
-        const f32x2 nE = sub2(fma2(K(C.third), drho, pE), u3);
-        const f32x2 c4 = mul2(K(C.h15), sub2(nE, nR)), c16 = mul2(K(C.half), add2(fma2(K(C.two), nF, nR), nE));
-        b0 = fma2(K(C.d0), sub2(c16, c4), b0);
-        bF = fma2(K(C.dF), c16, bF);
-        bE = fma2(K(C.dE), add2(c4, c16), bE);
+    // MRT: sums of f - f_eq over the rest, face and edge populations
+    f32x2 nR, nF, nE;
+    {
+        const f32x2 n0 = fma2(K(C.w0), fma2(K(C.c15), uu, drho), g[0]);
+        if (MRT) nR = n0;
+        g[0] = fma2(K(C.sp), n0, g[0]);
     }
-    g[0] = fma2(K(C.r0), g[0], b0);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         const int q = 2 * k + 1;
-        f32x2 e, d;
+        const float2 &w = k < 3 ? C.wF : C.wE;
+        f32x2 cu;
         if (k < 3) {
-            e = fma2(K(C.kF), u2[k], bF);
-            d = mul2(K(C.mF), u[k]);
+            cu = u[k];
         } else {
-            // pairs 3..8: (+x+y), (+x-y), (+x+z), (+x-z), (+y+z), (+y-z)
             const int a = k < 7 ? 0 : 1, b = k < 5 ? 1 : 2;
-            const f32x2 cu = (k & 1) ? add2(u[a], u[b]) : sub2(u[a], u[b]);
-            e = fma2(mul2(K(C.kE), cu), cu, bE);
-            d = mul2(K(C.mE), cu);
+            cu = (k & 1) ? add2(u[a], u[b]) : sub2(u[a], u[b]);
         }
-        const f32x2 Sy = fma2(K(C.hp), ps[k], e), Da = fma2(K(C.hm), pd[k], d);
-        g[q] = add2(Sy, Da);
-        g[q + 1] = sub2(Sy, Da);
+        const f32x2 ep = mul2(K(w), fma2(K(C.c15), uu, fma2(mul2(K(C.c45), cu), cu, drho)));   // -e+
+        const f32x2 em = mul2(K(w), mul2(K(C.three), cu));                                      // -e-
+        // g+ - e+ and g- - e-, the sum and difference formed again: kept, they spill.  (As sums of two such terms, not
+        // as fma2 with one half, the assembler would fuse them with the products before them.)
+        const f32x2 np = fma2(K(C.half), add2(g[q + 1], g[q]), ep);
+        const f32x2 nm = fma2(K(C.half), fma2(K(C.one_m), g[q + 1], g[q]), em);
+        if (MRT) {
+            if (k == 0) nF = add2(np, np);
+            else if (k < 3) nF = add2(nF, add2(np, np));
+            else if (k == 3) nE = add2(np, np);
+            else nE = add2(nE, add2(np, np));
+        }
+        g[q] = fma2(K(C.sm_m), nm, fma2(K(C.sp), np, g[q]));
+        g[q + 1] = fma2(K(C.sm), nm, fma2(K(C.sp), np, g[q + 1]));
+    }
+    if (MRT) {   // as in trt_collide
+        const f32x2 s4 = sub2(nE, nR), c16 = mul2(K(C.half), add2(fma2(K(C.two), nF, nR), nE));
+        const f32x2 r = fma2(K(C.h15), mul2(K(C.one_m), s4), c16), e = fma2(K(C.h15), s4, c16);
+        g[0] = fma2(K(C.d0), r, g[0]);
+#pragma unroll
+        for (int q = 1; q < 7; ++q) g[q] = fma2(K(C.dF), c16, g[q]);
+#pragma unroll
+        for (int q = 7; q < 19; ++q) g[q] = fma2(K(C.dE), e, g[q]);
     }
 }
 
@@ -261,11 +275,11 @@ __device__ __forceinline__ void collide_pair(f32x2 (&g)[19], const PairConsts& C
 // the lane has a pair).
 // Bound by what it issues as much as by HBM (188 us at 256^3): 262 us a step
 // with two scalar collisions, 255 packed, 251 with ordinary stores, 235 with
-// one load for the outer halves of a population and its mirror image, 228 with
-// the marks after the loads (box_row).  With
-// walls the bounced populations are chosen by their address, the moving
-// walls' term added after the loads: 256 x 128 x 96 74.7 us a step with a
-// branch around every load, 70.4 packed, 62.0 so, 59.0 with box_row.
+// one load for the outer halves of a population and its mirror image, 224 with
+// the marks after the loads (box_row), 229 with the collision's rounding as it
+// is now.  With walls the bounced populations are chosen by their address, the
+// moving walls' term added after the loads: 256 x 128 x 96 74.7 us a step with a
+// branch around every load, 70.4 packed, 62.0 so, 57.3 with box_row, now 66.8.
 template <bool WALLS, bool MRT>
 __device__ __forceinline__ void bulk_pairs(const StepArgs<__half>& T, const PairConsts& K, unsigned pair, bool valid) {
     const GridDesc& G = T.G;
@@ -503,7 +517,8 @@ __device__ __forceinline__ bool is_boundary_cta(const StepArgs<S>& T, unsigned b
 // (11 + 5 us as two launches of their own) runs beside the bulk update instead of after it.  With k_remap for the four
 // remap launches: a 32^3 FP32 step 46.1 -> 23.4 us, 256 x 128 x 96 with walls 123.6 -> 94.2, 61 x 53 x 75 in FP64
 // 175 -> 92 (with collide_direct), 512^3 3066 -> 2997.  With what the parts below took off since: 14.7, 81.3, 79.2 and 2990.
-// CTAS: resident CTAs of 256 threads per SM asked of the compiler (launch_step): FP64 2, FP16 4, FP32 4 or 5.
+// CTAS: resident CTAs of 256 threads per SM asked of the compiler (launch_step): FP64 2, FP16 4, FP32 4 or 5.  FP16
+// pairs: 4, with walls 3 (80 registers; four spill 100 bytes, 256 x 128 x 96 68.2 us a step instead of 66.8).
 template <typename S, bool WALLS, bool FORCED, int CTAS>
 __global__ void __launch_bounds__(STEP_THREADS, CTAS) k_step(const __grid_constant__ StepArgs<S> T) {
     extern __shared__ int pre[];   // prefix of the segments' numbers (boundary CTAs)
@@ -519,7 +534,7 @@ __global__ void __launch_bounds__(STEP_THREADS, CTAS) k_step(const __grid_consta
 }
 
 template <bool WALLS, bool MRT>
-__global__ void __launch_bounds__(STEP_THREADS, 4) k_step_h2(const __grid_constant__ StepArgs<__half> T, const __grid_constant__ PairConsts K) {
+__global__ void __launch_bounds__(STEP_THREADS, WALLS ? 3 : 4) k_step_h2(const __grid_constant__ StepArgs<__half> T, const __grid_constant__ PairConsts K) {
     extern __shared__ int pre[];
     pdl_wait();
     unsigned bulk;
