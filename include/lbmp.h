@@ -372,7 +372,8 @@ const char* lbmp_last_error(const lbmp_handle* h);
  *   grad_tau    device double, dJ * dJ/dtau               (may be NULL)
  *   grad_force  device double[3], dJ * dJ/dF (body force)  (may be NULL)
  *   grad_u0     device array like u0, dJ * dJ/du0          (may be NULL)
- * It needs the preceding forward call with the same tau and body force.
+ * It needs the preceding forward call with the same tau and body force and
+ * the sphere where it was then.
  * Both calls are asynchronous on the handle's stream except for one
  * synchronisation on the first forward call after the geometry is set.
  * Errors: LBMP_ERR_UNSUPPORTED for a refined or batched handle, FP16

@@ -624,10 +624,11 @@ struct AdjointEngine {
     int near_cap = 0;
     bool forward_done = false;
     bool geometry_done = false;   // kind bytes and near list of the (fixed) sphere
+    long long placed = -1;        // the handle's `placed` that they, the graphs and the forward pass belong to
     double tau = 0, F[3] = {0, 0, 0};
     // the forward pass (one per parity of the handle's buffers) and the reverse
-    // sweep replayed from CUDA graphs; dropped when tau, the body force or the
-    // objective's axis change
+    // sweep replayed from CUDA graphs; dropped when tau, the body force, the
+    // objective's axis or the sphere's place (with it the flag buffer) change
     cudaGraphExec_t gfwd[2] = {nullptr, nullptr};
     cudaGraphExec_t gbwd = nullptr;
     double graph_tau = -1.0, graph_F[3] = {0, 0, 0};
@@ -636,6 +637,14 @@ struct AdjointEngine {
 };
 
 namespace {
+
+// The step's frames after the host changed the record.
+void renew_frames(lbmp_handle* h) {
+    if (!h->frames_stale) return;
+    launch_frames(h, h->stream);
+    h->frames_stale = false;
+    h->launches += 1;
+}
 
 // One forward step with the sphere held at rest; the force of the step into force_out (null: not wanted).
 template <typename S>
@@ -780,11 +789,12 @@ lbmp_status adjoint_forward(lbmp_handle* h, const double* u0, int nsteps, int in
         E->graph_axis = axis;
         for (int a = 0; a < 3; ++a) E->graph_F[a] = h->body_force[a];
     }
-    if (h->frames_stale) {   // the host changed the record: the step's frames first
-        launch_frames(h, h->stream);
-        h->frames_stale = false;
-        h->launches += 1;
+    if (E->placed != h->placed) {   // released, moved and held again, or another one loaded
+        drop_graphs(E);
+        E->geometry_done = false;
+        E->placed = h->placed;
     }
+    renew_frames(h);
     if (!E->geometry_done) {   // cells of the reverse step next to the (fixed) sphere
         const unsigned gb = (unsigned)E->cell_blocks;
         k_adj_kind<<<gb, AT, 0, h->stream>>>(h->flags[h->fcur], h->G, E->kind, E->blk);
@@ -839,6 +849,8 @@ lbmp_status adjoint_backward(lbmp_handle* h, const double* dJ, double* grad_tau,
     if (!E || !E->forward_done) return *why = "lbmp_drag_backward needs a preceding lbmp_drag_forward", LBMP_ERR_INVALID_ARG;
     if (E->tau != h->tau || E->F[0] != h->body_force[0] || E->F[1] != h->body_force[1] || E->F[2] != h->body_force[2])
         return *why = "tau or the body force changed since lbmp_drag_forward", LBMP_ERR_INVALID_ARG;
+    if (E->placed != h->placed) return *why = "the sphere moved since lbmp_drag_forward", LBMP_ERR_INVALID_ARG;
+    renew_frames(h);   // the held sphere's velocities may have been others in between
     const size_t n = (size_t)h->G.n;
     const int N = E->nsteps, K = E->interval;
     const int cli = h->cfg.boundary == LBMP_CLI ? 1 : 0;

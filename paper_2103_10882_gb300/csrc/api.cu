@@ -107,6 +107,7 @@ void enqueue_step(lbmp_handle* h) {
                                            (A)fp16_scale(h, false), (A)fp16_scale(h, true),
                                            (A)grad_refill_coef(h->cfg.refill, h->tau), h->stream);
             h->fcur = 1 - h->fcur;
+            if (h->h_ps.fixed == 0) h->placed += 1;
         }
     });
     profile_step(h, ev_step, profile_mark(h));
@@ -1098,6 +1099,7 @@ lbmp_status lbmp_load(lbmp_handle* h, const char* path) {
         h->G.moving = moving;
     }
     if (H.has_particle) {
+        if (h->h_ps.x[0] != P.x[0] || h->h_ps.x[1] != P.x[1] || h->h_ps.x[2] != P.x[2]) h->placed += 1;
         h->h_ps = P;
         const lbmp_status s = upload_particle(h);
         if (s != LBMP_OK) return s;

@@ -230,6 +230,8 @@ struct lbmp_handle {
     lbmp::BoxDesc box;
     bool has_particle = false;
     bool frames_stale = true;            // the host changed the particle record since the refined step formed its frames
+    long long placed = 0;                // uniform grids: raised where the sphere's place may change (a step that does not
+                                         // hold it, a load)
     bool ps_current = false;             // h_ps equals the device record (read with the status after a step)
     double tau = 0.6, magic = 3.0 / 16.0;
     double body_force[3] = {0, 0, 0};
