@@ -1820,14 +1820,21 @@ lbmp_status amr_add_sphere(lbmp_handle* h) {
     h->seg = (int*)handle_alloc(h, sizeof(int) * SEG * nseg);
     h->seg_count = (int*)handle_alloc(h, sizeof(int) * nseg);
     if (!h->list || !h->partials || !h->seg || !h->seg_count) return LBMP_ERR_OOM;
-    // the boundary kernel keeps a prefix of the segments' numbers in dynamic shared memory; the limit on the sphere
-    // is that of a count per 64 box cells
-    const int pre_bytes = (int)(sizeof(int) * ((B.cells + 63) / 64 + 1));
+    // The boundary kernel keeps a prefix of the segments' numbers in dynamic shared memory.  The kernel's limit belongs to
+    // the process, so it is never set to this sphere's size but always to all that the device gives a CTA.  The largest
+    // sphere is the one whose counts per 64 box cells would fit.
+    const size_t pre_bytes = sizeof(int) * (size_t)((B.cells + 63) / 64 + 1);
     bool attr_ok = true;
     with_storage_amr(h->cfg.precision, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
-        attr_ok = cudaFuncSetAttribute(k_amr_boundary<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       std::max(pre_bytes, 1024)) == cudaSuccess;
+        int device = 0, optin = 0;
+        cudaFuncAttributes fa;
+        attr_ok = cudaGetDevice(&device) == cudaSuccess &&
+                  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) == cudaSuccess &&
+                  cudaFuncGetAttributes(&fa, k_amr_boundary<S>) == cudaSuccess &&
+                  pre_bytes + fa.sharedSizeBytes <= (size_t)optin &&
+                  cudaFuncSetAttribute(k_amr_boundary<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       optin - (int)fa.sharedSizeBytes) == cudaSuccess;
     });
     if (!attr_ok) return amr_cuda_error(h, "sphere too large for the boundary kernel's shared memory");
     if (cudaMemcpyAsync(h->d_ps, &h->h_ps, sizeof(ParticleState), cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
