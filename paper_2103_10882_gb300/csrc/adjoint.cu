@@ -621,7 +621,6 @@ struct AdjointEngine {
     int* blk = nullptr;
     int* near_list = nullptr;
     int* near_count = nullptr;
-    int near_cap = 0;
     bool forward_done = false;
     bool geometry_done = false;   // kind bytes and near list of the (fixed) sphere
     long long placed = -1;        // the handle's `placed` that they, the graphs and the forward pass belong to
@@ -759,7 +758,6 @@ lbmp_status adjoint_forward(lbmp_handle* h, const double* u0, int nsteps, int in
         E->per_cta = E->threads;   // small grids over all SMs: four CTAs on each (32^3 FP32 0.3 us a step less than two)
         while (E->per_cta > 32 && (int)n / E->per_cta < 4 * 152) E->per_cta /= 2;
         E->plain_blocks = (int)((n + (size_t)E->per_cta - 1) / (size_t)E->per_cta);
-        E->near_cap = (int)n;
         E->near_blocks = 0;
         E->acc_blocks = NEAR_WARPS_MAX / (E->threads / 32) + E->plain_blocks;
         E->ckpt = handle_alloc(h, E->state_bytes * (size_t)nckpt);

@@ -407,7 +407,7 @@ __global__ void k_batch_flags_full(uint8_t* __restrict__ f0, uint8_t* __restrict
     f1[D.flag_off + c] = v;
 }
 
-// Initial boundary-cell lists (uses the refill/mark kernel on unchanged flags).
+// Stored populations as FP64 deviations, for the read-back.
 template <typename S>
 __global__ void k_batch_to_f64(const S* __restrict__ pops, double* __restrict__ out, long long count,
                                typename Store<S>::A inv) {
@@ -787,17 +787,6 @@ lbmp_status batch_get_particle(lbmp_handle* h, int sim, ParticleState* out) {
         B->read[block] = 1;
     }
     *out = B->h_ps[sim];
-    return LBMP_OK;
-}
-
-lbmp_status batch_set_particle(lbmp_handle* h, int sim, const ParticleState* in) {
-    BatchEngine* B = h->batch;
-    if (sim < 0 || sim >= B->nsims) return LBMP_ERR_INVALID_ARG;
-    B->read[sim / RECORDS] = 0;
-    if (cudaMemcpyAsync(B->d_ps + sim, in, sizeof(ParticleState), cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
-        cudaStreamSynchronize(h->stream) != cudaSuccess)
-        return LBMP_ERR_CUDA;
-    h->h2d += sizeof(ParticleState);
     return LBMP_OK;
 }
 
