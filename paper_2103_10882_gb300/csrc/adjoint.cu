@@ -37,7 +37,7 @@ namespace lbmp {
 namespace {
 
 constexpr int AT = 256;   // threads per block of the cell kernels
-constexpr int NEAR_WARPS_MAX = 4864;   // warps for the cells next to the sphere (32 per SM, each takes several of a large sphere's)
+constexpr int NEAR_WARPS_MAX = 32 * SMS;   // warps for the cells next to the sphere (4,864, each takes several of a large sphere's)
 
 // Threads of a reverse-step CTA, and resident CTAs per SM asked of the compiler: 56 registers in FP32 (64^3
 // 2% faster per gradient than 64), 128 in FP64.
@@ -756,7 +756,7 @@ lbmp_status adjoint_forward(lbmp_handle* h, const double* u0, int nsteps, int in
         E->cell_blocks = (int)((n + AT - 1) / AT);
         E->threads = h->cfg.precision == LBMP_FP64 ? ADJ_THREADS<double> : ADJ_THREADS<float>;
         E->per_cta = E->threads;   // small grids over all SMs: four CTAs on each (32^3 FP32 0.3 us a step less than two)
-        while (E->per_cta > 32 && (int)n / E->per_cta < 4 * 152) E->per_cta /= 2;
+        while (E->per_cta > 32 && (int)n / E->per_cta < 4 * SMS) E->per_cta /= 2;
         E->plain_blocks = (int)((n + (size_t)E->per_cta - 1) / (size_t)E->per_cta);
         E->near_blocks = 0;
         E->acc_blocks = NEAR_WARPS_MAX / (E->threads / 32) + E->plain_blocks;

@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(UPD_THREADS, sizeof(S) == 8 ? 1 : UPD_MIN_CTAS
 constexpr int BNDW_THREADS = 256;
 // Register cap of the boundary kernel (BNDW_THREADS threads).  It runs beside the finest level's
 // update for most of that update, so every register it holds is taken from the update's CTAs; at 64
-// it keeps its loads of one round trip without spills (rising sphere: 1% faster than at 56).
+// it keeps its loads of one round trip with 20 bytes spilled, 16 in FP16 (rising sphere: 1% faster than at 56).
 template <typename S>
 constexpr int BND_MAXREG = sizeof(S) == 8 ? 128 : 64;
 constexpr int REMAP_THREADS = SEG;   // remap blocks: their uncovered cells are spread over the eight warps

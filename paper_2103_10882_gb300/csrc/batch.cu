@@ -238,8 +238,9 @@ __device__ __forceinline__ void batch_boundary(const BatchArgs<S>& T, int bid) {
 // half of the bulk CTAs they take few slots at a time.  A box by itself and four small ones are bound by the chain
 // from a boundary CTA's first load to the remap's last store: 49 to 34 and 34 to 23 us, most of it from BND_PARTS and
 // from the bulk CTA's one load before its pulls.
-// ZC cells per thread along z, CTAS resident CTAs per SM asked of the compiler: the autotuner's choice.  Neither
-// touches the arithmetic, so the results do not depend on it.
+// ZC cells per thread along z, CTAS resident CTAs per SM asked of the compiler: the autotuner's choice, timed on the bulk
+// CTAs alone (boundary CTAs would advance the spheres).  Neither touches the arithmetic, so the results do not depend on
+// it.
 template <typename S, int ZC, int CTAS>
 __global__ void __launch_bounds__(BW, CTAS) k_batch_step(const __grid_constant__ BatchArgs<S> T) {
     pdl_wait();
@@ -599,8 +600,8 @@ lbmp_status batch_create(lbmp_handle* h, const lbmp_batch_sim* sims, int n) {
         D.hist_off = (long long)s * std::max(1, h->cfg.history_capacity);
     }
     // boundary CTAs: two segments each where that is two or more CTAs per SM, else one, shared by up to BND_PARTS CTAs
-    B->bnd_segs = (int)seg_sim.size() >= 2 * 152 * BND_SEGS ? BND_SEGS : 1;
-    while (B->bnd_segs == 1 && B->bnd_parts < BND_PARTS && (int)seg_sim.size() * B->bnd_parts < 2 * 152) B->bnd_parts *= 2;
+    B->bnd_segs = (int)seg_sim.size() >= 2 * SMS * BND_SEGS ? BND_SEGS : 1;
+    while (B->bnd_segs == 1 && B->bnd_parts < BND_PARTS && (int)seg_sim.size() * B->bnd_parts < 2 * SMS) B->bnd_parts *= 2;
     for (int s = 0; s < n; ++s) {
         SimDev& D = B->sims[s];
         D.bnd_off = (int)bnd_sim.size();

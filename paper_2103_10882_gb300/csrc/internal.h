@@ -16,6 +16,8 @@
 
 namespace lbmp {
 
+constexpr int SMS = 152;   // streaming multiprocessors of the part, by which launches are sized
+
 struct GridDesc {
     int nx, ny, nz;
     int periodic[3];
@@ -103,7 +105,7 @@ struct BoxDesc {
 // Boundary CTAs of a coupled uniform step, also the number of force partials (8 warps each, taking the boundary
 // cells in turn).  The list's capacity is two to three times the boundary cells: one CTA per 20 entries gives every
 // warp about one cell, and the chain of a cell, the sums and the particle update is the step where the bulk update is
-// short (one per 40 costs a 32^3 step 10%, one per 10 4%).  Where the bulk update runs for eight waves of CTAs or more
+// short (one per 40 costs a 32^3 step 10%, one per 10 4%).  Where the bulk update runs for 6,080 CTAs or more (BULK_LONG)
 // the chain hides behind it and half as many cost it less (256 x 128 x 96: 92.0 and 91.3 us; 256^3 in FP16 storage 272
 // and 270).  FP64 in launch_step.  At most eight per SM.
 // Boxes of up to SEG_CELLS_MAX cells (spheres up to about 70 cells) find their cells through a prefix of the segments'
@@ -113,7 +115,7 @@ constexpr long long SEG_CELLS_MAX = 2048 * 256;
 inline bool step_uses_list(const BoxDesc& b) { return b.cells > SEG_CELLS_MAX; }
 inline int step_boundary_blocks(int list_capacity, int per) {
     const int n = (list_capacity + per - 1) / per;
-    return n < 1 ? 1 : (n > 1216 ? 1216 : n);
+    return n < 1 ? 1 : (n > 8 * SMS ? 8 * SMS : n);
 }
 
 // n / d for n < 2^31 by one high multiplication (Granlund & Montgomery, "Division by invariant integers

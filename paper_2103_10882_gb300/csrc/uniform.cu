@@ -16,7 +16,7 @@ namespace lbmp {
 namespace {
 
 constexpr int STEP_THREADS = 256;
-constexpr unsigned WAVES_8 = 8 * 5 * 152;   // bulk CTAs of eight waves, five per SM
+constexpr unsigned BULK_LONG = 40 * SMS;   // bulk CTAs: eight waves in FP32, ten in FP16, twenty in FP64
 // Marks of the box cells around the sphere, written by the remap: plain fluid cell, fluid cell with a solid
 // D3Q19 neighbour (taken by the boundary CTAs), cell with its centre inside the sphere.
 constexpr uint8_t MARK_PLAIN = 0, MARK_BOUNDARY = 1, MARK_SOLID = 2;
@@ -871,22 +871,22 @@ void launch_step(const lbmp_handle* h, const S* src, S* dst, const CollideParams
     auto ctas = [&](int per_cta) { return (T.items + (unsigned)per_cta - 1) / (unsigned)per_cta; };
     T.per_cta = STEP_THREADS;
     if (sizeof(S) != 8)
-        while (T.per_cta > 32 && T.items / (unsigned)T.per_cta < 152) T.per_cta /= 2;
+        while (T.per_cta > 32 && T.items / (unsigned)T.per_cta < SMS) T.per_cta /= 2;
     unsigned bulk = ctas(T.per_cta);
     size_t smem = 0;
     if (h->has_particle) {
         if constexpr (sizeof(S) == 8) {
             T.bblocks = step_boundary_blocks(h->list_cap, BOUNDARY_PER_FP64);
-            T.thin = bulk + (unsigned)T.bblocks <= 5 * 152;
-            if (!T.thin) T.bblocks = step_boundary_blocks(h->list_cap, bulk >= WAVES_8 ? 40 : 32);
+            T.thin = bulk + (unsigned)T.bblocks <= 5 * SMS;
+            if (!T.thin) T.bblocks = step_boundary_blocks(h->list_cap, bulk >= BULK_LONG ? 40 : 32);
         } else {
-            T.bblocks = step_boundary_blocks(h->list_cap, bulk >= WAVES_8 ? 40 : BOUNDARY_PER);
+            T.bblocks = step_boundary_blocks(h->list_cap, bulk >= BULK_LONG ? 40 : BOUNDARY_PER);
         }
         if (step_uses_list(h->box)) T.list = h->list;
         else smem = sizeof(int) * (size_t)((h->box.cells + SEG - 1) / SEG + 1);
     }
     if (sizeof(S) == 8) {
-        while (T.per_cta > 32 && (unsigned)T.bblocks + ctas(T.per_cta / 2) <= 2 * 152) T.per_cta /= 2;
+        while (T.per_cta > 32 && (unsigned)T.bblocks + ctas(T.per_cta / 2) <= 2 * SMS) T.per_cta /= 2;
         bulk = ctas(T.per_cta);
     }
     const unsigned grid = (unsigned)T.bblocks + bulk;
@@ -918,7 +918,7 @@ void launch_step(const lbmp_handle* h, const S* src, S* dst, const CollideParams
         else go(k_step<S, false, false, C>);
     };
     if constexpr (std::is_same<S, float>::value) {
-        if (bulk > 4 * 4 * 152) pick(std::integral_constant<int, 5>());
+        if (bulk > 4 * 4 * SMS) pick(std::integral_constant<int, 5>());
         else pick(std::integral_constant<int, 4>());
     } else {
         pick(std::integral_constant<int, sizeof(S) == 8 ? 2 : 4>());
